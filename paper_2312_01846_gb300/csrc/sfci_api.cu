@@ -214,6 +214,11 @@ sfci_status sfci_system_create(sfci_system **out, int n, int na, int nb, const d
     if (fp32) o = a256(o + nh * 4);
     const size_t off_gf = o;
     if (fp32) o = a256(o + ng * 4);
+    const size_t off_pi = o;
+    {
+        const size_t np = size_t(n) * (n - 1) / 2;
+        o = a256(o + np * np * 8);
+    }
     std::vector<float> hf, gf;
     if (fp32) {
         hf.resize(nh), gf.resize(ng);
@@ -264,9 +269,21 @@ sfci_status sfci_system_create(sfci_system **out, int n, int na, int nb, const d
     }
     d.bound_ab = reinterpret_cast<const double *>(blk + off_bab);
     d.bound_ss = reinterpret_cast<const double *>(blk + off_bss);
+    for (int a = 0; a < n; ++a)
+        for (int i = 0; i < n; ++i)
+            if (a != i && bab[size_t(a) * n + i] != 0.0) d.ab_any = 1;
     d.ss_any = std::any_of(bss.begin(), bss.end(), [](double x) { return x != 0.0; }) ? 1 : 0;
     s->d = d;
     s->dev_block = blk;
+    s->pair_int = reinterpret_cast<double *>(blk + off_pi);
+    e = launch_pair_integrals(d, s->pair_int, nullptr);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    if (e != cudaSuccess) {
+        cudaFree(blk);
+        cudaFree(s->dev_status);
+        delete s;
+        return cuda_fail(e, "sfci_system_create");
+    }
     *out = s;
     return SFCI_OK;
 }

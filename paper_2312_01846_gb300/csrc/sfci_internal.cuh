@@ -139,6 +139,7 @@ struct SysDev {
     // for every (b, j); bound_ss[i*n+j] >= |(ai|bj) - (aj|bi)| for every (a, b)
     const double *bound_ab;
     const double *bound_ss;
+    int ab_any;          // 1: some (ai|bj) with a != i is non-zero (else every opposite-spin double is zero)
     int ss_any;          // 1: some bound_ss entry is non-zero (else every same-spin double is zero)
     double hbound;       // |<D'|H|D>| <= hbound for every pair of determinants
 };
@@ -149,6 +150,7 @@ struct sfci_system {
     sfci::SysDev d;
     void *dev_block;  // one allocation holding h, g, binom, pairs
     int *dev_status;  // scratch status words for rank/unrank
+    double *pair_int; // (ai|bj) - (aj|bi) over orbital pairs (a < b), (i < j)
     int device;
 };
 
@@ -563,6 +565,155 @@ cudaError_t min_abs(const double *val, const unsigned long long *n_dev, long lon
 size_t aligned_dots_ws_bytes(int nvec);
 cudaError_t aligned_dots(const VecRef *vecs, double *const *sig, int nvec, double *out_dev, void *ws,
                          cudaStream_t st);
+
+// sfci_lanczos.cu: sfci_lanczos_create with the device bytes a batch leaves the solver (0: no batch)
+sfci_status lanczos_create(sfci_lanczos **out, const sfci_system *sys, const sfci_params *params,
+                           const uint64_t *init_rank, const double *init_coef, int64_t n_init, void *stream,
+                           int64_t share);
+
+// sfci_gather.cu -- sigma by target rows (see the file's header)
+constexpr int kGatherMaxElectrons = 12;  // per spin
+struct GatherShape {
+    int bb, bs;                      // bits of pi(beta'), its xor-shift
+    unsigned bmask, m1, m2, i1, i2;  // its mask, multipliers and their inverses
+    int kb1, kb2;                    // log2 of the bins of the singles' and doubles' tables
+    int nd2;                         // beta-beta doubles per string
+    unsigned nk1, nk2;               // substrings of n_alpha - 1 and n_alpha - 2 electrons
+    unsigned npair;                  // orbital pairs
+};
+struct RowPlanArgs {
+    unsigned long long half;  // a row of more weight is heavy (units of its own); a group weighs at most 2 half
+    double fill;              // distinct entries a class should hold
+    unsigned w_fixed;         // weight of a row besides its elements (a group holds at most 2 half / w_fixed rows)
+};
+// a group of light rows or one class of a heavy row, as ranges of its lists
+struct GatherUnit {
+    unsigned long long rec0, rec1;  // ready elements
+    unsigned ab0, ab1;              // one-hop sources
+    unsigned src0, src1;            // own sources
+    unsigned k0, k1;                // active rows
+    unsigned lo, hi;                // range of pi
+    unsigned bin, n_cls;            // weight bin of a heavy row (light: 0), its classes
+    unsigned pad[2];
+};
+static_assert(sizeof(GatherUnit) == 64, "read as four 16-byte words");
+constexpr int kSeenBins = 128;
+struct GatherBufs {
+    unsigned long long *words;  // [8]: runs, n
+    unsigned long long *skey;   // [n] row << bb | pi(beta), runs in the order of pi
+    double *sc;                 // [n]
+    void *sort_ws, *scan_ws;
+    unsigned *bflag;            // [cb] beta strings seen
+    unsigned long long *bid;    // [cb + 1] their numbers
+    unsigned *s_pi, *s_b;       // [n] per source: pi(beta), number of its beta string
+    unsigned *s_kb;             // [n] number of its row in its group << bb
+    double *s_diag;             // [n] <D|H|D>
+    unsigned *cnt1, *cnt2;      // one block: sources per substring
+    unsigned long long *off1, *off2;      // [nk1 + 1], [nk2 + 1] list offsets
+    unsigned *s1, *s2, *act;    // [ca] sources one hop away; listed under the substrings; any at all
+    unsigned long long *apos;   // [ca + 1]
+    unsigned *act_row;          // [ca] rows with elements
+    unsigned long long *act_str, *wpre;   // their strings, weight prefix
+    unsigned long long *aw;     // weights; aw | nrec | nab | np | nu are one block
+    unsigned *nrec, *nab, *np, *nu;       // records, one-hop sources, list parts, units per active row
+    unsigned long long *uoff, *poff, *rec_off, *ab_off;
+    unsigned long long *seen;   // [2 * kSeenBins] elements and distinct entries by row weight (kept by the solver)
+    unsigned long long *bstr;   // [nd] distinct beta strings
+    uint2 *t1;                  // [nd * s_b]
+    unsigned short *idx1;       // [nd * (2^kb1 + 1)]
+    unsigned *t2p;              // [nd * nd2]
+    double *t2e;
+    unsigned *idx2;             // [nd * (2^kb2 + 1)]
+    uint4 *ent1, *ent2;         // [n * n_alpha], [n * C(n_alpha, 2)]
+    GatherUnit *units;
+    unsigned *part_k;           // row of each list part
+    unsigned *cursor, *split;   // per row (one block): one-hop sources written; steps its classes split into
+    unsigned *split_rows;       // rows summed in classes (words[2] of them)
+    unsigned *rkey, *okey;      // records; those of split rows in class order
+    double *rval, *oval;
+    uint4 *ab;                  // one-hop sources
+};
+struct ListArgs {
+    SysDev d;
+    GatherShape gs;
+    const double *W;
+    const unsigned *act_row;
+    const unsigned long long *act_str;
+    const unsigned *part_k;
+    unsigned n_parts;
+    const unsigned *nu;
+    const unsigned long long *poff, *uoff, *rec_off, *ab_off;
+    const GatherUnit *units;
+    const unsigned *s1, *s2, *rp;
+    const unsigned long long *off1, *off2;
+    const uint4 *ent1, *ent2;
+    const unsigned *s_pi, *s_b;
+    const double *s_c, *s_diag;
+    const unsigned long long *bstr;
+    const uint2 *t1;
+    unsigned *cursor, *rkey;
+    double *rval;
+    uint4 *ab;
+    unsigned *s_kb;
+};
+struct GatherArgs {
+    GatherShape gs;
+    unsigned long long cb;
+    const double *g;
+    const float *gf;     // float32 elements, else null
+    unsigned sb, nd2;    // single and double excitations per beta string (nd2 = 0: every double is zero)
+    const GatherUnit *units;
+    unsigned n_units;
+    const unsigned *act_row;
+    const unsigned *rkey, *okey;
+    const double *rval, *oval;
+    unsigned *split;
+    const uint4 *ab;
+    const unsigned long long *rec_off, *ab_off;
+    const unsigned *rp;
+    const unsigned *s_b, *s_kb;
+    const double *s_c;
+    const uint2 *t1;
+    const unsigned short *idx1;
+    const unsigned *t2p;
+    const double *t2e;
+    const unsigned *idx2;
+    unsigned long long *seen;
+    unsigned long long min_bits;  // smallest |element * c| generated, as bits (at least 1: zeros are dropped)
+    int nvec, ja, jb;
+    const unsigned *vrp[kMaxVec];
+    const unsigned long long *vrank[kMaxVec];
+    double *sigw[kMaxVec];
+    double eps;
+    unsigned long long *out_key;
+    double *out_val;
+    long long out_cap;
+    unsigned long long *out_n, *tau_bits, *hist, *mark;
+    int *lock;
+    long long nkeep;
+    int fix_shift;
+    double *sumsq;
+    unsigned long long *n_live, *n_nonzero, *n_read;
+    unsigned *queue;
+    int *status;
+};
+bool gather_shape(const SysDev &d, GatherShape *p);  // false: the system is outside the gather's limits
+int gather_slots();
+int gather_slots_log2();
+cudaError_t launch_pair_integrals(const SysDev &d, double *W, cudaStream_t st);
+cudaError_t launch_row_pointers(const SysDev &d, const unsigned long long *rank, long long n, unsigned *rp,
+                                cudaStream_t st);
+// sources in run order, beta strings numbered (count in bid[cb]), runs in words[0]
+cudaError_t gather_sources(const SysDev &d, const GatherShape &p, const unsigned long long *rank, const double *coef,
+                           long long n, const GatherBufs &b, cudaStream_t st);
+// beta tables, substring lists, row plan (active rows in apos[ca], units in uoff[ca], list parts in poff[ca],
+// records in rec_off[ca], one-hop sources in ab_off[ca])
+cudaError_t gather_tables(const SysDev &d, const GatherShape &p, long long n, unsigned nd, const double *W,
+                          const unsigned *rp, const GatherBufs &b, const RowPlanArgs &ra, cudaStream_t st);
+cudaError_t gather_lists(const SysDev &d, const GatherShape &p, unsigned long long n_act, unsigned long long n_parts,
+                         const double *W, const unsigned *rp, const GatherBufs &b, const RowPlanArgs &ra,
+                         cudaStream_t st);
+cudaError_t launch_gather(const GatherArgs &A, cudaStream_t st);
 
 // sfci_select.cu
 size_t select_workspace_bytes(long long n_items, long long k);

@@ -249,6 +249,13 @@ struct sfci_lanczos {
     unsigned long long alpha_runs = 0;  // runs of inputs sharing alpha (last sigma's plan)
     double *dmin = nullptr;             // device word: min |kept|
     int n_passes = 0, nb_log2 = 0;
+    // sigma by target rows (sfci_gather.cu)
+    bool gather_ok = false;             // the system is within its limits
+    int64_t share = 0;                  // device bytes a batch leaves this solver (0: no batch)
+    GatherShape gs{};
+    Buf ga, gb, gc, vrp, seen;          // work arrays by the stage that sizes them; row pointers of each w_j;
+                                        // elements and distinct entries by row weight
+    std::vector<char> vrp_ok;           // row pointers of w_j are current
 };
 
 namespace {
@@ -262,7 +269,7 @@ void destroy_lz(sfci_lanczos *z) {
     for (auto *b : {&z->bcount, &z->belem, &z->bovf, &z->bovf_sorted, &z->tmp_counts, &z->ovf_off,
                     &z->probes, &z->pcount, &z->poff, &z->scan_ws, &z->sig_key, &z->sig_val,
                     &z->cand_key, &z->cand_val, &z->weights, &z->rowmap, &z->boff, &z->wpre, &z->ptl,
-                    &z->pth, &z->pbstart, &z->pcap, &z->pq, &z->start4})
+                    &z->pth, &z->pbstart, &z->pcap, &z->pq, &z->start4, &z->ga, &z->gb, &z->gc, &z->vrp, &z->seen})
         cudaFree(b->p);
     cudaFree(z->words);
     for (int j = 0; j < kMaxVec; ++j) cudaFree(z->sigw[j]);
@@ -517,6 +524,7 @@ sfci_status bucketed_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long
                             (double)z->bovf.bytes + (double)z->bovf_sorted.bytes;
         double avail = 0.85 * ((double)free_b + held);
         if (z->p.mem_budget > 0) avail = std::min(avail, (double)z->p.mem_budget);
+        if (z->share > 0) avail = std::min(avail, (double)z->share);
         const double sig_bytes = 1.1 * sig_need * 16.0;
         // for the element regions (a pass's region offsets are 32-bit counts of 4 slots)
         const double budget = std::min(avail - sig_bytes - 2.0 * ovf_cap * 16.0, 4.0 * 4294967295.0 * sizeof(Slot));
@@ -834,6 +842,266 @@ sfci_status bucketed_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long
     return SFCI_E_CAPACITY;
 }
 
+// Memory one buffer hands out in 256-byte pieces (first pass: sizes only)
+struct Arena {
+    char *base = nullptr;
+    size_t off = 0;
+    template <class T>
+    T *take(size_t n) {
+        T *p = base ? reinterpret_cast<T *>(base + off) : nullptr;
+        off += a256(n * sizeof(T));
+        return p;
+    }
+};
+
+void gather_arena_a(Arena &a, GatherBufs &b, const SysDev &d, const GatherShape &p, long long n) {
+    const size_t ca = size_t(d.ca), cb = size_t(d.cb);
+    b.words = a.take<unsigned long long>(8);
+    b.skey = a.take<unsigned long long>(n);
+    b.sc = a.take<double>(n);
+    b.sort_ws = a.take<char>(p.bb > gather_slots_log2() ? sort_pairs_bytes(n) : 0);
+    b.scan_ws = a.take<char>(scan_ws_bytes((long long)std::max({ca, cb, size_t(p.nk1), size_t(p.nk2)}) + 1));
+    b.bflag = a.take<unsigned>(cb);
+    b.bid = a.take<unsigned long long>(cb + 1);
+    b.s_pi = a.take<unsigned>(n);
+    b.s_b = a.take<unsigned>(n);
+    b.s_kb = a.take<unsigned>(n);
+    b.s_diag = a.take<double>(n);
+    b.cnt1 = a.take<unsigned>(size_t(p.nk1) + p.nk2);
+    b.cnt2 = b.cnt1 + p.nk1;
+    b.off1 = a.take<unsigned long long>(size_t(p.nk1) + 1);
+    b.off2 = a.take<unsigned long long>(size_t(p.nk2) + 1);
+    b.s1 = a.take<unsigned>(ca);
+    b.s2 = a.take<unsigned>(ca);
+    b.act = a.take<unsigned>(ca);
+    b.apos = a.take<unsigned long long>(ca + 1);
+    b.act_row = a.take<unsigned>(ca);
+    b.act_str = a.take<unsigned long long>(ca);
+    b.wpre = a.take<unsigned long long>(ca + 1);
+    b.aw = a.take<unsigned long long>(3 * ca);
+    b.nrec = reinterpret_cast<unsigned *>(b.aw + ca), b.nab = b.nrec + ca, b.np = b.nab + ca, b.nu = b.np + ca;
+    b.uoff = a.take<unsigned long long>(ca + 1);
+    b.poff = a.take<unsigned long long>(ca + 1);
+    b.rec_off = a.take<unsigned long long>(ca + 1);
+    b.ab_off = a.take<unsigned long long>(ca + 1);
+}
+
+void gather_arena_b(Arena &a, GatherBufs &b, const SysDev &d, const GatherShape &p, size_t nd, size_t n) {
+    b.bstr = a.take<unsigned long long>(nd);
+    b.t1 = a.take<uint2>(nd * d.sb);
+    b.idx1 = a.take<unsigned short>(nd * ((1 << p.kb1) + 1));
+    b.t2p = a.take<unsigned>(nd * p.nd2);
+    b.t2e = a.take<double>(nd * p.nd2);
+    b.idx2 = a.take<unsigned>(nd * ((1 << p.kb2) + 1));
+    b.ent1 = a.take<uint4>(n * d.na);
+    b.ent2 = a.take<uint4>(n * d.po_a);
+}
+
+// device bytes that sigma's buffers may take in all
+double sigma_budget(const sfci_lanczos *z, double held) {
+    size_t free_b = 0, tot_b = 0;
+    cudaMemGetInfo(&free_b, &tot_b);
+    const double avail = 0.85 * ((double)free_b + held);
+    return z->share > 0 ? std::min(avail, (double)z->share) : avail;
+}
+
+// Sigma by target rows is taken unless the caller shapes the bucketed path
+// (bucket size, memory budget, overflow limit, launch shape, stress flag) or
+// the system is outside its limits.
+bool gather_wanted(const sfci_lanczos *z) {
+    return z->gather_ok && z->p.bucket_elems == 0 && z->p.mem_budget == 0 && z->p.ovf_max_log2 == 0 &&
+           z->p.emit_warps == 0 && z->p.flags == 0;
+}
+
+// sigma_i = H w_i by target rows, with sigma recorded at every basis entry;
+// results as bucketed_sigma's.  *done = false: its tables do not fit in memory
+// (the caller takes the bucketed path).
+sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long long *n_out, unsigned long long *n_live,
+                         unsigned long long *n_nonzero, double *sumsq, bool *done) {
+    *done = false;
+    const SysDev &d = z->sys->d;
+    const GatherShape &gs = z->gs;
+    const long long n_in = z->wn[i];
+    const double E = (double)n_in * (double)(d.n_conn + 1);
+    const auto t_plan0 = std::chrono::steady_clock::now();
+    sfci_status r;
+    GatherBufs b{};
+    Arena size_a, a;
+    gather_arena_a(size_a, b, d, gs, n_in);
+    // (room for what every CTA streams before the first raise of a zero threshold can act)
+    double sig_need = std::min(std::max(16.0 * (double)z->nkeep, 8.0e6), E) + 2.0 * (double)z->nkeep + 1024.0;
+    const size_t vrp_bytes = size_t(z->NL) * (size_t(d.ca) + 1) * 4;
+    const double held = (double)z->ga.bytes + z->gb.bytes + z->gc.bytes + z->vrp.bytes + z->sig_key.bytes +
+                        z->sig_val.bytes + z->belem.bytes + z->bovf.bytes + z->bovf_sorted.bytes;
+    const double budget = sigma_budget(z, held);
+    double need = (double)size_a.off + (double)vrp_bytes + 16.0 * sig_need;
+    if (need > budget) return SFCI_OK;
+    SFCI_CUDA(cudaEventRecord(z->evp[0], z->st));
+    if ((r = ensure(z->ga, size_a.off, z->st, "row gather arrays", 1.25))) return r;
+    if (z->vrp.bytes < vrp_bytes) z->vrp_ok.assign(z->NL, 0);
+    if ((r = ensure(z->vrp, vrp_bytes, z->st, "row pointers"))) return r;
+    a.base = static_cast<char *>(z->ga.p);
+    gather_arena_a(a, b, d, gs, n_in);
+    auto *vrp = P<unsigned>(z->vrp);
+    for (int j = 0; j <= i; ++j)
+        if (!z->vrp_ok[j]) {
+            SFCI_CUDA(launch_row_pointers(d, z->wr[j], z->wn[j], vrp + size_t(j) * (size_t(d.ca) + 1), z->st));
+            z->vrp_ok[j] = 1;
+        }
+    const unsigned *rp = vrp + size_t(i) * (size_t(d.ca) + 1);
+    if (!z->seen.p) {
+        if ((r = ensure(z->seen, 2 * kSeenBins * 8, z->st, "row weight bins"))) return r;
+        SFCI_CUDA(cudaMemsetAsync(z->seen.p, 0, 2 * kSeenBins * 8, z->st));
+    }
+    b.seen = P<unsigned long long>(z->seen);
+    SFCI_CUDA(gather_sources(d, gs, z->wr[i], z->wc[i], n_in, b, z->st));
+    unsigned long long nd = 0, runs = 0;
+    SFCI_CUDA(cudaMemcpyAsync(&nd, b.bid + d.cb, 8, cudaMemcpyDeviceToHost, z->st));
+    SFCI_CUDA(cudaMemcpyAsync(&runs, b.words, 8, cudaMemcpyDeviceToHost, z->st));
+    SFCI_CUDA(cudaStreamSynchronize(z->st));
+    Arena size_b, ab;
+    gather_arena_b(size_b, b, d, gs, nd, (size_t)n_in);
+    // 32-bit positions in the singles' table and the lists, 25 bits for a beta string's number; memory
+    if (nd >= (1ull << 25) || (double)nd * std::max(d.sb, 1) >= 4294967296.0 || (double)n_in * std::max(d.po_a, d.na) >= 4294967296.0 ||
+        need + (double)size_b.off > budget)
+        return SFCI_OK;
+    if ((r = ensure(z->gb, size_b.off, z->st, "row gather tables", 1.1))) return r;
+    ab.base = static_cast<char *>(z->gb.p);
+    gather_arena_b(ab, b, d, gs, nd, (size_t)n_in);
+    RowPlanArgs ra{};
+    // light rows repeat entries about 1.45 times (1.3 to 2): a group fills about 0.55 of its table
+    ra.half = (unsigned long long)(0.55 * 1.45 * gather_slots());
+    ra.fill = 0.65 * gather_slots();
+    // at most 120 rows in a group (7 bits), and fewer than its key bits can number
+    ra.w_fixed = std::max(32u, (unsigned)(2 * ra.half / std::min(120, (1 << (32 - gs.bb)) - 2) + 1));
+    SFCI_CUDA(gather_tables(d, gs, n_in, (unsigned)nd, z->sys->pair_int, rp, b, ra, z->st));
+    unsigned long long n_act = 0, n_units = 0, n_parts = 0, n_rec = 0, n_ab = 0;
+    SFCI_CUDA(cudaMemcpyAsync(&n_act, b.apos + d.ca, 8, cudaMemcpyDeviceToHost, z->st));
+    SFCI_CUDA(cudaMemcpyAsync(&n_units, b.uoff + d.ca, 8, cudaMemcpyDeviceToHost, z->st));
+    SFCI_CUDA(cudaMemcpyAsync(&n_parts, b.poff + d.ca, 8, cudaMemcpyDeviceToHost, z->st));
+    SFCI_CUDA(cudaMemcpyAsync(&n_rec, b.rec_off + d.ca, 8, cudaMemcpyDeviceToHost, z->st));
+    SFCI_CUDA(cudaMemcpyAsync(&n_ab, b.ab_off + d.ca, 8, cudaMemcpyDeviceToHost, z->st));
+    SFCI_CUDA(cudaStreamSynchronize(z->st));
+    if (n_units >= (1ull << 31) || n_parts >= (1ull << 31) || n_ab >= (1ull << 32)) return SFCI_OK;
+    Arena size_c, ac;
+    auto arena_c = [&](Arena &m) {
+        b.units = m.take<GatherUnit>(n_units);
+        b.part_k = m.take<unsigned>(n_parts);
+        b.cursor = m.take<unsigned>(2 * n_act);
+        b.split = b.cursor + n_act;
+        b.split_rows = m.take<unsigned>(n_act);
+        b.rkey = m.take<unsigned>(n_rec);
+        b.rval = m.take<double>(n_rec);
+        const size_t n_ord = gs.bb > gather_slots_log2() ? n_rec : 0;
+        b.okey = m.take<unsigned>(n_ord);
+        b.oval = m.take<double>(n_ord);
+        b.ab = m.take<uint4>(n_ab);
+    };
+    arena_c(size_c);
+    if (need + (double)size_b.off + (double)size_c.off > budget) return SFCI_OK;
+    if ((r = ensure(z->gc, size_c.off, z->st, "row gather lists", 1.1))) return r;
+    ac.base = static_cast<char *>(z->gc.p);
+    arena_c(ac);
+    SFCI_CUDA(gather_lists(d, gs, n_act, n_parts, z->sys->pair_int, rp, b, ra, z->st));
+    for (int j = 0; j <= i; ++j) {
+        if (!z->sigw[j]) SFCI_CUDA(cudaMalloc(&z->sigw[j], size_t(z->nkeep) * 8));
+        if (z->wn[j] > 0) SFCI_CUDA(cudaMemsetAsync(z->sigw[j], 0, size_t(z->wn[j]) * 8, z->st));  // rows without elements
+    }
+    int fix_shift = (int)std::floor(125.0 - std::log2(std::max(1e-300, (double)(d.n_conn + 1) * d.hbound)));
+    fix_shift = std::max(-900, std::min(1000, fix_shift));
+    const double tau_start = *tau_io;
+    double tau = tau_start;
+    for (int attempt = 0; attempt < 8; ++attempt) {
+        const size_t want_sig = size_t(sig_need) * 8;
+        if ((r = ensure(z->sig_key, want_sig, z->st, "sigma keys", 1.1))) return r;
+        if ((r = ensure(z->sig_val, want_sig, z->st, "sigma values", 1.1))) return r;
+        z->sig_cap = (long long)(std::min(z->sig_key.bytes, z->sig_val.bytes) / 8);
+        const long long u_room = 2 * z->nkeep + 1024;
+        const long long out_cap = std::max<long long>(z->sig_cap - u_room, 0);
+        SFCI_CUDA(cudaMemsetAsync(z->words, 0, kHistBins * 8 + 1024, z->st));
+        unsigned long long tw[2];
+        std::memcpy(&tw[0], &tau, 8);
+        tw[1] = (unsigned long long)out_cap / 4;
+        SFCI_CUDA(cudaMemcpyAsync(z->tau_w, tw, 16, cudaMemcpyHostToDevice, z->st));
+        GatherArgs A{};
+        A.gs = gs, A.cb = d.cb, A.g = d.g, A.gf = d.gf;
+        A.sb = (unsigned)d.sb, A.nd2 = d.ss_any ? (unsigned)gs.nd2 : 0u;
+        A.units = b.units, A.n_units = (unsigned)n_units, A.act_row = b.act_row;
+        A.rkey = b.rkey, A.rval = b.rval, A.okey = b.okey, A.oval = b.oval, A.split = b.split, A.ab = b.ab;
+        A.rec_off = b.rec_off, A.ab_off = b.ab_off, A.rp = rp;
+        A.s_b = b.s_b, A.s_kb = b.s_kb, A.s_c = b.sc;
+        A.t1 = b.t1, A.idx1 = b.idx1, A.t2p = b.t2p, A.t2e = b.t2e, A.idx2 = b.idx2;
+        A.seen = b.seen;
+        const double eps_el = z->p.eps_element > 0.0 ? z->p.eps_element : 0.0;
+        std::memcpy(&A.min_bits, &eps_el, 8);
+        A.min_bits = std::max(A.min_bits, 1ull);
+        A.nvec = i + 1, A.ja = i, A.jb = i > 0 ? i - 1 : -1;
+        for (int j = 0; j <= i; ++j) {
+            A.vrp[j] = vrp + size_t(j) * (size_t(d.ca) + 1);
+            A.vrank[j] = z->wr[j];
+            A.sigw[j] = z->sigw[j];
+        }
+        A.eps = z->p.eps_screen > 0.0 ? z->p.eps_screen : 0.0;
+        A.out_key = P<unsigned long long>(z->sig_key), A.out_val = P<double>(z->sig_val);
+        A.out_cap = out_cap, A.out_n = z->outn;
+        A.tau_bits = z->tau_w, A.hist = z->hist, A.mark = z->mark_w, A.lock = z->lock_w;
+        A.nkeep = z->nkeep, A.fix_shift = fix_shift;
+        A.sumsq = z->msumsq, A.n_live = z->mlive, A.n_nonzero = z->nnz, A.n_read = z->nread_w;
+        A.queue = z->queue, A.status = z->mstatus;
+        if (attempt == 0) {
+            SFCI_CUDA(cudaEventRecord(z->evp[1], z->st));
+            z->ms_plan = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_plan0).count();
+        }
+        SFCI_CUDA(launch_gather(A, z->st));
+        SFCI_CUDA(cudaEventRecord(z->evp[2], z->st));
+        int hs = 0;
+        unsigned long long ho = 0, hl = 0, hz = 0, tb = 0, hr = 0;
+        double hq = 0.0;
+        SFCI_CUDA(cudaMemcpyAsync(&hs, z->mstatus, 4, cudaMemcpyDeviceToHost, z->st));
+        SFCI_CUDA(cudaMemcpyAsync(&ho, z->outn, 8, cudaMemcpyDeviceToHost, z->st));
+        SFCI_CUDA(cudaMemcpyAsync(&hl, z->mlive, 8, cudaMemcpyDeviceToHost, z->st));
+        SFCI_CUDA(cudaMemcpyAsync(&hz, z->nnz, 8, cudaMemcpyDeviceToHost, z->st));
+        SFCI_CUDA(cudaMemcpyAsync(&hq, z->msumsq, 8, cudaMemcpyDeviceToHost, z->st));
+        SFCI_CUDA(cudaMemcpyAsync(&tb, z->tau_w, 8, cudaMemcpyDeviceToHost, z->st));
+        SFCI_CUDA(cudaMemcpyAsync(&hr, z->nread_w, 8, cudaMemcpyDeviceToHost, z->st));
+        SFCI_CUDA(cudaStreamSynchronize(z->st));
+        std::memcpy(&tau, &tb, 8);
+        if (hs & 32) {  // an element beyond the fixed-point range (an input not normalised): coarser units
+            fix_shift -= 16;
+            tau = tau_start;
+            continue;
+        }
+        if (hs & 8) {  // the stream outgrew its buffer before the raises caught up
+            sig_need = std::max(sig_need * 2.0, (double)ho * 1.3 + 2.0 * z->nkeep);
+            continue;
+        }
+        *tau_io = tau;
+        *n_out = ho, *n_live = hl, *n_nonzero = hz, *sumsq = hq;
+        float te = 0.f, tm = 0.f;
+        cudaEventElapsedTime(&te, z->evp[0], z->evp[1]);
+        cudaEventElapsedTime(&tm, z->evp[1], z->evp[2]);
+        z->ms_emit = te, z->ms_merge = tm;
+        z->mult_prev = E / std::max(1.0, (double)hl);
+        z->n_emitted = (long long)hr;
+        z->stream_prev = ho;
+        z->ovf_used = 0;
+        z->elem_prev = E;
+        z->n_passes = 1;
+        z->n_split = 0;
+        z->alpha_runs = runs;
+        z->nb_log2 = 0;
+        while ((1ull << z->nb_log2) < n_units) ++z->nb_log2;
+        z->budget_gb = budget / 1e9;
+        z->free_gb = (budget - held) / 1e9, z->held_gb = held / 1e9;
+        z->regions_gb = E * sizeof(Slot) / 1e9;  // what the elements would take as records
+        z->ms_alloc = 0.0;
+        *done = true;
+        return SFCI_OK;
+    }
+    set_error("sigma's stream did not fit after 8 attempts");
+    return SFCI_E_CAPACITY;
+}
+
 // w_0 = normalise(top_{N_d}(trial vector)); a new cycle begins
 sfci_status load_vector(sfci_lanczos *z, const uint64_t *rank, const double *coef, long long n) {
     Items it{reinterpret_cast<const unsigned long long *>(rank), coef, 1, n};
@@ -845,6 +1113,7 @@ sfci_status load_vector(sfci_lanczos *z, const uint64_t *rank, const double *coe
     SFCI_CUDA(cudaMemcpyAsync(&hn, z->ndev, 8, cudaMemcpyDeviceToHost, z->st));
     SFCI_CUDA(cudaStreamSynchronize(z->st));
     z->wn[0] = (long long)std::min<unsigned long long>(hn, (unsigned long long)z->nkeep);
+    std::fill(z->vrp_ok.begin(), z->vrp_ok.end(), 0);
     z->idx = 0;
     z->have_prev = false;
     z->just_ended = false;
@@ -888,12 +1157,18 @@ sfci_status sfci_lanczos_set_input(sfci_lanczos *z, const uint64_t *rank, const 
     SFCI_CUDA(cudaMemcpyAsync(z->wc[i], coef, size_t(n) * 8, cudaMemcpyDeviceToDevice, z->st));
     SFCI_CUDA(cudaStreamSynchronize(z->st));
     z->wn[i] = n;
+    z->vrp_ok[i] = 0;
     return SFCI_OK;
 }
 
-sfci_status sfci_lanczos_create(sfci_lanczos **out, const sfci_system *sys,
-                                const sfci_params *params, const uint64_t *init_rank,
-                                const double *init_coef, int64_t n_init, void *stream) {
+}  // extern "C"
+
+namespace sfci {
+
+// sfci_lanczos_create; share > 0: the device bytes a batch leaves this solver's sigma
+sfci_status lanczos_create(sfci_lanczos **out, const sfci_system *sys, const sfci_params *params,
+                           const uint64_t *init_rank, const double *init_coef, int64_t n_init, void *stream,
+                           int64_t share) {
     if (!out || !sys || !params) {
         set_error("null argument");
         return SFCI_E_INVALID;
@@ -914,6 +1189,7 @@ sfci_status sfci_lanczos_create(sfci_lanczos **out, const sfci_system *sys,
     if (!z) return SFCI_E_NOMEM;
     z->sys = sys;
     z->p = *params;
+    z->share = share;
     z->st = static_cast<cudaStream_t>(stream);
     z->NL = params->n_lanczos;
     z->nkeep = params->n_keep;
@@ -922,6 +1198,8 @@ sfci_status sfci_lanczos_create(sfci_lanczos **out, const sfci_system *sys,
     z->wn.assign(z->NL, 0);
     z->T.assign(size_t(z->NL) * z->NL, 0.0);
     z->S.assign(size_t(z->NL) * z->NL, 0.0);
+    z->vrp_ok.assign(z->NL, 0);
+    z->gather_ok = gather_shape(sys->d, &z->gs) && z->nkeep < (1ll << 31);
     cudaError_t e = cudaSuccess;
     for (int j = 0; j < z->NL && e == cudaSuccess; ++j) {
         e = cudaMalloc(&z->wr[j], size_t(z->nkeep) * 8);
@@ -974,6 +1252,7 @@ sfci_status sfci_lanczos_create(sfci_lanczos **out, const sfci_system *sys,
     cudaMemGetInfo(&free_b, &total_b);
     double table_bytes = 0.8 * (double)free_b;
     if (params->mem_budget > 0) table_bytes = std::min(table_bytes, 0.5 * (double)params->mem_budget);
+    if (share > 0) table_bytes = std::min(table_bytes, 0.5 * (double)share);
     unsigned long long bud = (unsigned long long)table_bytes / sizeof(Slot);
     unsigned long long p2 = 1;
     while ((p2 << 1) <= bud) p2 <<= 1;
@@ -986,6 +1265,16 @@ sfci_status sfci_lanczos_create(sfci_lanczos **out, const sfci_system *sys,
     }
     *out = z;
     return SFCI_OK;
+}
+
+}  // namespace sfci
+
+extern "C" {
+
+sfci_status sfci_lanczos_create(sfci_lanczos **out, const sfci_system *sys,
+                                const sfci_params *params, const uint64_t *init_rank,
+                                const double *init_coef, int64_t n_init, void *stream) {
+    return lanczos_create(out, sys, params, init_rank, init_coef, n_init, stream, 0);
 }
 
 sfci_status sfci_lanczos_step(sfci_lanczos *z, sfci_step_info *info) {
@@ -1022,7 +1311,10 @@ sfci_status sfci_lanczos_step(sfci_lanczos *z, sfci_step_info *info) {
         double sq = 0.0;
         {
             NvtxRange nv("sigma (plan, emit, merge)");
-            const sfci_status rs = bucketed_sigma(z, i, &tau, &n_stream, &n_live, &n_nz, &sq);
+            bool gathered = false;
+            sfci_status rs = SFCI_OK;
+            if (gather_wanted(z)) rs = gather_sigma(z, i, &tau, &n_stream, &n_live, &n_nz, &sq, &gathered);
+            if (rs == SFCI_OK && !gathered) rs = bucketed_sigma(z, i, &tau, &n_stream, &n_live, &n_nz, &sq);
             if (rs != SFCI_OK) return rs;
         }
         info->ms_sigma = z->ms_emit + z->ms_merge;
@@ -1137,6 +1429,7 @@ sfci_status sfci_lanczos_step(sfci_lanczos *z, sfci_step_info *info) {
                              z->scratch + z->off_sort, z->st));
         SFCI_CUDA(normalize_vec(z->wc[i + 1], z->nkeep, z->ndev, z->scratch + z->off_norm, z->st));
         z->wn[i + 1] = (long long)kept;
+        z->vrp_ok[i + 1] = 0;
         SFCI_CUDA(cudaEventRecord(z->evp[0], z->st));
         SFCI_CUDA(cudaEventSynchronize(z->evp[0]));
         {
@@ -1188,6 +1481,7 @@ sfci_status sfci_lanczos_step(sfci_lanczos *z, sfci_step_info *info) {
         unsigned long long ptot = 0;
         rs = table_topk(z, pcap, 0, nullptr, &ptot);
         if (rs != SFCI_OK) return rs;
+        std::fill(z->vrp_ok.begin(), z->vrp_ok.end(), 0);
         info->n_psi = (long long)ptot;
         info->n_kept = z->wn[0];
         if (z->p.conv_tol > 0.0 && z->have_prev && z->e_prev - lam < z->p.conv_tol) info->converged = 1;

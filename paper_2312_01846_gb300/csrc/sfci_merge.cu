@@ -25,7 +25,7 @@
 // the previous step's truncation cut; the caller checks afterwards that the
 // N_d largest all cleared it, and otherwise redoes the step with tau = 0), so
 // the truncation reads a few N_d entries instead of all of sigma.
-#include "sfci_internal.cuh"
+#include "sfci_stream.cuh"
 
 namespace sfci {
 namespace {
@@ -49,10 +49,6 @@ __device__ __forceinline__ unsigned smem_slot(unsigned long long key, int log2B)
     key *= 0xD6E8FEB86659FD93ull;
     key ^= key >> 32;
     return (unsigned)key & (kSlots - 1);
-}
-
-__device__ __forceinline__ unsigned long long abs_bits(double v) {
-    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
 }
 
 // ------------------------------------------------------------- scan
@@ -227,54 +223,6 @@ __global__ void uniform_offsets_kernel(unsigned long long *boff, unsigned long l
 // registers (independent loads in flight together), then inserts them; slots
 // taken for the first time are listed, so clearing and streaming out touch only
 // the occupied slots.
-// Called by every thread of the CTA that holds A.lock: the highest histogram
-// bin b whose streamed entries at or above it number >= nkeep (counts read
-// while other CTAs still add, so they only undercount: the threshold is never
-// too high), then tau = max(tau, lower edge of b) and the next mark halfway
-// between out_n and out_cap; releases the lock.
-__device__ __noinline__ void raise_threshold(const MergeArgs &A, int tid, int *s_bin,
-                                             unsigned long long *part) {
-    constexpr int per = kHistBins / kMT;  // bins per thread, thread 0 owns the top ones
-    unsigned long long sum = 0;
-    const int top = kHistBins - 1 - tid * per;
-    for (int q = 0; q < per; ++q) sum += *(volatile unsigned long long *)&A.hist[top - q];
-    part[tid] = sum;
-    __syncthreads();
-    if (tid == 0) {  // exclusive prefix from the top (kMT values)
-        unsigned long long run = 0;
-        for (int t = 0; t < kMT; ++t) {
-            const unsigned long long v = part[t];
-            part[t] = run;
-            run += v;
-        }
-    }
-    __syncthreads();
-    const unsigned long long need = (unsigned long long)(A.nkeep > 0 ? A.nkeep : 1);
-    unsigned long long run = part[tid];
-    if (run < need && run + sum >= need) {
-        // re-read: counts only grow, so a bin found with fresher counts is still
-        // one with >= nkeep streamed entries at or above it
-        for (int q = 0; q < per; ++q) {
-            run += *(volatile unsigned long long *)&A.hist[top - q];
-            if (run >= need) {
-                *s_bin = top - q;
-                break;
-            }
-        }
-    }
-    __syncthreads();
-    if (tid == 0) {
-        const int b = *s_bin;
-        if (b > 0) atomicMax(A.tau_bits, (unsigned long long)b << kHistShift);
-        const unsigned long long on = *(volatile unsigned long long *)A.out_n;
-        const unsigned long long cap = (unsigned long long)(A.out_cap > 0 ? A.out_cap : 0);
-        *(volatile unsigned long long *)A.mark = on < cap ? on + (cap - on) / 2 : cap;
-        __threadfence();
-        atomicExch(A.lock, 0);
-    }
-    __syncthreads();
-}
-
 template <int kSlots>
 __global__ void __launch_bounds__(kMT, 4)
 merge_kernel(MergeArgs A) {
@@ -489,7 +437,7 @@ merge_kernel(MergeArgs A) {
         }
         __syncthreads();
         // (the bucket's occupied-slot list is spent: its shared memory holds the partial sums)
-        if (s_raise) raise_threshold(A, tid, &s_bin, reinterpret_cast<unsigned long long *>(occ));
+        if (s_raise) raise_threshold<kMT>(A, tid, &s_bin, reinterpret_cast<unsigned long long *>(occ));
         if (tid == 0) n_occ = 0, cur = atomicAdd(A.queue, 1u), s_tau = *(volatile unsigned long long *)A.tau_bits;
         __syncthreads();
     }

@@ -125,16 +125,16 @@ sfci_status sfci_scan_create(sfci_scan **out, int32_t count, const sfci_system *
     size_t free_b = 0, tot_b = 0;
     cudaMemGetInfo(&free_b, &tot_b);
     for (int i = 0; i < count; ++i) {
-        sfci_params p = params[i];
-        if (p.mem_budget == 0)  // a share of 80 % of what is free now
-            p.mem_budget = (int64_t)(0.8 * (double)free_b * work[i] / total);
+        // without a budget of its own: a share of 80 % of what is free now
+        const int64_t share =
+            params[i].mem_budget == 0 ? (int64_t)(0.8 * (double)free_b * work[i] / total) : 0;
         cudaError_t e = cudaStreamCreateWithFlags(&s->streams[i], cudaStreamNonBlocking);
         if (e != cudaSuccess) {
             destroy_scan(s);
             return cuda_fail(e, "sfci_scan_create");
         }
-        const sfci_status r = sfci_lanczos_create(&s->lz[i], systems[i], &p, init_rank[i], init_coef[i],
-                                                  n_init[i], s->streams[i]);
+        const sfci_status r = lanczos_create(&s->lz[i], systems[i], &params[i], init_rank[i], init_coef[i],
+                                             n_init[i], s->streams[i], share);
         if (r != SFCI_OK) {
             const std::string msg = "instance " + std::to_string(i) + ": " + sfci_last_error();
             destroy_scan(s);
