@@ -449,8 +449,8 @@ sfci_status sfci_truncate_topk(const uint64_t *rank, const double *coef, int64_t
     unsigned long long *ok = reinterpret_cast<unsigned long long *>(out_rank);
     SFCI_CUDA(select_topk(it, k, ok, out_coef, ndev, nullptr, nullptr, w + L.sel,
                           select_workspace_bytes(n, k), st));
-    SFCI_CUDA(sort_pairs(ok, out_coef, k, ndev, 64, w + L.sort, st));
-    if (normalize) SFCI_CUDA(normalize_vec(out_coef, k, ndev, w + L.norm, st));
+    if (normalize) SFCI_CUDA(sort_normalize(ok, out_coef, k, ndev, 64, w + L.sort, w + L.norm, st));
+    else SFCI_CUDA(sort_pairs(ok, out_coef, k, ndev, 64, w + L.sort, st));
     unsigned long long hn = 0;
     SFCI_CUDA(cudaMemcpyAsync(&hn, ndev, sizeof(hn), cudaMemcpyDeviceToHost, st));
     SFCI_CUDA(cudaStreamSynchronize(st));

@@ -730,7 +730,9 @@ struct Items {
 // receives sum val^2 over all valid items, and total_dev their number.
 cudaError_t select_topk(Items it, long long k, unsigned long long *out_key, double *out_val,
                         unsigned long long *n_out_dev, double *sumsq_dev,
-                        unsigned long long *total_dev, void *ws, size_t ws_bytes, cudaStream_t st);
+                        unsigned long long *total_dev, void *ws, size_t ws_bytes, cudaStream_t st,
+                        double *cut_dev = nullptr);  // cut_dev: smallest |val| kept
+bool select_is_small(const Items &it);  // one launch does the whole selection
 // Two-level top-k: one pass histograms the first digit (top 12 bits of the
 // composite key, 4096 bins), the bin holding the k-th item is picked, and one
 // more pass writes every item of a smaller bin to out and every item of the
@@ -751,6 +753,9 @@ size_t sort_workspace_bytes(long long n);
 size_t sort_pairs_bytes(long long cap);
 cudaError_t sort_pairs(unsigned long long *key, double *val, long long cap,
                        const unsigned long long *n_dev, int bits, void *ws, cudaStream_t st);
+// both of sort_pairs and normalize_vec
+cudaError_t sort_normalize(unsigned long long *key, double *val, long long cap, const unsigned long long *n_dev,
+                           int bits, void *sort_ws, void *norm_ws, cudaStream_t st);
 // c[i] /= sqrt(sum c^2) over n (device count) entries, deterministic order
 cudaError_t normalize_vec(double *val, long long cap, const unsigned long long *n_dev,
                           void *ws, cudaStream_t st);

@@ -315,9 +315,8 @@ sfci_status table_topk(sfci_lanczos *z, unsigned long long cap, int dst, double 
     Items it{&z->slots[0].key, &z->slots[0].val, 2, (long long)cap};
     SFCI_CUDA(select_topk(it, z->nkeep, z->wr[dst], z->wc[dst], z->ndev, z->sumsq, z->total,
                           z->scratch + z->off_sel, z->sel_bytes, z->st));
-    SFCI_CUDA(sort_pairs(z->wr[dst], z->wc[dst], z->nkeep, z->ndev, key_bits(z->sys->d.dim),
-                         z->scratch + z->off_sort, z->st));
-    SFCI_CUDA(normalize_vec(z->wc[dst], z->nkeep, z->ndev, z->scratch + z->off_norm, z->st));
+    SFCI_CUDA(sort_normalize(z->wr[dst], z->wc[dst], z->nkeep, z->ndev, key_bits(z->sys->d.dim),
+                             z->scratch + z->off_sort, z->scratch + z->off_norm, z->st));
     unsigned long long hn = 0;
     SFCI_CUDA(cudaMemcpyAsync(&hn, z->ndev, sizeof(hn), cudaMemcpyDeviceToHost, z->st));
     if (sumsq_host) SFCI_CUDA(cudaMemcpyAsync(sumsq_host, z->sumsq, 8, cudaMemcpyDeviceToHost, z->st));
@@ -1107,8 +1106,8 @@ sfci_status load_vector(sfci_lanczos *z, const uint64_t *rank, const double *coe
     Items it{reinterpret_cast<const unsigned long long *>(rank), coef, 1, n};
     SFCI_CUDA(select_topk(it, z->nkeep, z->wr[0], z->wc[0], z->ndev, nullptr, nullptr,
                           z->scratch + z->off_sel, z->sel_bytes, z->st));
-    SFCI_CUDA(sort_pairs(z->wr[0], z->wc[0], z->nkeep, z->ndev, 64, z->scratch + z->off_sort, z->st));
-    SFCI_CUDA(normalize_vec(z->wc[0], z->nkeep, z->ndev, z->scratch + z->off_norm, z->st));
+    SFCI_CUDA(sort_normalize(z->wr[0], z->wc[0], z->nkeep, z->ndev, 64, z->scratch + z->off_sort,
+                             z->scratch + z->off_norm, z->st));
     unsigned long long hn = 0;
     SFCI_CUDA(cudaMemcpyAsync(&hn, z->ndev, 8, cudaMemcpyDeviceToHost, z->st));
     SFCI_CUDA(cudaStreamSynchronize(z->st));
@@ -1425,9 +1424,8 @@ sfci_status sfci_lanczos_step(sfci_lanczos *z, sfci_step_info *info) {
         z->cut_at[i] = z->tau_prev;
         info->tau = tau;
         info->cut = z->tau_prev;
-        SFCI_CUDA(sort_pairs(z->wr[i + 1], z->wc[i + 1], z->nkeep, z->ndev, key_bits(d.dim),
-                             z->scratch + z->off_sort, z->st));
-        SFCI_CUDA(normalize_vec(z->wc[i + 1], z->nkeep, z->ndev, z->scratch + z->off_norm, z->st));
+        SFCI_CUDA(sort_normalize(z->wr[i + 1], z->wc[i + 1], z->nkeep, z->ndev, key_bits(d.dim),
+                                 z->scratch + z->off_sort, z->scratch + z->off_norm, z->st));
         z->wn[i + 1] = (long long)kept;
         z->vrp_ok[i + 1] = 0;
         SFCI_CUDA(cudaEventRecord(z->evp[0], z->st));

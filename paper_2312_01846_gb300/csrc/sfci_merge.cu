@@ -70,6 +70,36 @@ __global__ void scan_sums_kernel(const T *in, long long m, unsigned long long *b
     }
 }
 
+// up to kSmallScan entries: one CTA, one launch
+constexpr long long kSmallScan = 8192;
+template <typename T>
+__global__ void scan_small_kernel(const T *in, int m, unsigned long long *out) {
+    __shared__ unsigned long long w[32];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    unsigned long long carry = 0;
+    for (int b0 = 0; b0 < m; b0 += 1024) {
+        const int i = b0 + (int)threadIdx.x;
+        const unsigned long long v = i < m ? in[i] : 0;
+        unsigned long long x = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(kFull, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) w[wp] = x;
+        __syncthreads();
+        unsigned long long s = w[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(kFull, s, o);
+            if (lane >= o) s += y;
+        }
+        const unsigned long long before = wp > 0 ? __shfl_sync(kFull, s, wp - 1) : 0ull;
+        if (i < m) out[i] = carry + before + x - v;
+        carry += __shfl_sync(kFull, s, 31);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[m] = carry;
+}
+
 __global__ void scan_top_kernel(unsigned long long *bsum, long long nb) {
     // one block: exclusive scan of nb block sums in place
     __shared__ unsigned long long carry, w[32];
@@ -532,28 +562,26 @@ __global__ void aligned_dots_kernel(VecPackRef vp, SigPack sp, double *partial) 
 }
 
 __global__ void aligned_finish_kernel(const double *partial, int np, double *out) {
+    __shared__ double sh[kDotBlocks];  // (fetched together, then added in order)
+    for (int k = threadIdx.x; k < np; k += blockDim.x) sh[k] = partial[(size_t)blockIdx.x * np + k];
+    __syncthreads();
     if (threadIdx.x == 0) {
         double r = 0.0;
-        for (int k = 0; k < np; ++k) r += partial[(size_t)blockIdx.x * np + k];
+        for (int k = 0; k < np; ++k) r += sh[k];
         out[blockIdx.x] = r;
     }
 }
 
-__global__ void min_abs_kernel(const double *val, const unsigned long long *n_dev, long long cap,
-                               double *out) {
-    __shared__ double sh[32];
+__global__ void min_init_kernel(double *out) { *out = __longlong_as_double(0x7ff0000000000000ll); }  // +inf
+
+__global__ void min_abs_kernel(const double *val, const unsigned long long *n_dev, long long cap, double *out) {
     long long n = (long long)*n_dev;
     if (n > cap) n = cap;
-    double m = __longlong_as_double(0x7ff0000000000000ll);  // +inf
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) m = fmin(m, fabs(val[i]));
-    for (int o = 16; o > 0; o >>= 1) m = fmin(m, __shfl_xor_sync(kFull, m, o));
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double r = sh[0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = fmin(r, sh[w]);
-        *out = r;
-    }
+    unsigned long long m = 0x7ff0000000000000ull;  // non-negative doubles order as integers
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        m = min(m, abs_bits(val[i]));
+    for (int o = 16; o > 0; o >>= 1) m = min(m, __shfl_xor_sync(kFull, m, o));
+    if ((threadIdx.x & 31) == 0) atomicMin(reinterpret_cast<unsigned long long *>(out), m);
 }
 
 int sm_count() {
@@ -582,6 +610,11 @@ namespace {
 template <typename T>
 cudaError_t exclusive_scan_t(const T *in, long long m, unsigned long long *out, void *ws, cudaStream_t st) {
     if (m <= 0) return cudaMemsetAsync(out, 0, 8, st);
+    if (m <= kSmallScan) {
+        count_launch();
+        scan_small_kernel<<<1, 1024, 0, st>>>(in, (int)m, out);
+        return cudaGetLastError();
+    }
     const long long nb = (m + 1023) / 1024;
     unsigned long long *bsum = static_cast<unsigned long long *>(ws);
     count_launch();
@@ -689,7 +722,9 @@ cudaError_t launch_u_entries(VecRef wi, const double *sig_i, VecRef wm, const do
 cudaError_t min_abs(const double *val, const unsigned long long *n_dev, long long cap, double *out,
                     cudaStream_t st) {
     count_launch();
-    min_abs_kernel<<<1, 1024, 0, st>>>(val, n_dev, cap, out);
+    min_init_kernel<<<1, 1, 0, st>>>(out);
+    count_launch();
+    min_abs_kernel<<<grid_for(cap, 2), 256, 0, st>>>(val, n_dev, cap, out);
     return cudaGetLastError();
 }
 
@@ -705,7 +740,7 @@ cudaError_t aligned_dots(const VecRef *vecs, double *const *sig, int nvec, doubl
     count_launch();
     aligned_dots_kernel<<<dim3(kDotBlocks, nvec), 256, 0, st>>>(vp, sp, partial);
     count_launch();
-    aligned_finish_kernel<<<nvec, 32, 0, st>>>(partial, kDotBlocks, out_dev);
+    aligned_finish_kernel<<<nvec, 320, 0, st>>>(partial, kDotBlocks, out_dev);
     return cudaGetLastError();
 }
 

@@ -6,15 +6,25 @@
 // are the k smallest X (for non-negative doubles the bit pattern orders like
 // the value).  A radix select walks X from the top in 12-bit digits (the last
 // digit has 7 bits): each pass histograms the digit of the entries whose
-// higher digits equal the prefix found so far, and a one-block kernel picks
-// the bin that holds the k-th smallest.  All state stays on the device; a pass
-// that finds its bin exactly full ends the search early.  A last pass gathers
-// every entry whose prefix is <= the threshold prefix.
+// higher digits equal the prefix found so far, and the block that finishes its
+// part last picks the bin that holds the k-th smallest.  All state stays on the
+// device; a pass that finds its bin exactly full ends the search early.  A last
+// pass gathers every entry whose prefix is <= the threshold prefix.  Up to
+// kSmall items one CTA does all passes in shared memory.
 //
 // sort: stable LSD radix sort of (uint64 key, double val) pairs with 8-bit
-// digits over the significant key bits only (ceil(log2(dim)) bits): per tile
-// a digit histogram, one exclusive scan over (digit, tile), then a stable
-// scatter ranked per warp with __match_any_sync.
+// digits over the significant key bits only (ceil(log2(dim)) bits): one pass
+// counts every digit of every key (digits that all keys share are skipped),
+// then per digit a histogram per tile, one scan per digit value over the
+// tiles, and a stable scatter ranked per warp with __match_any_sync.  Up to
+// kSmall pairs one CTA sorts (and normalises) in shared memory.
+//
+// What bounds it: at 3e6 items (48 MB) launches and the chain of passes, not
+// bandwidth; the 2e5 largest of 3e6, sorted: 554 us with one-block scans over
+// all counters and a pick launch per pass, 379 us so.  Where the capacity is
+// far above the count, the kernels follow the count: an unsorted sigma of 3e7
+// entries 60.2 ms when sorting over the capacity, 27.3 ms so.  A step on the
+// whole 4900-determinant space: 1066 us with 30 launches a sort, 839 us so.
 #include "sfci_internal.cuh"
 
 namespace sfci {
@@ -24,6 +34,10 @@ constexpr int kT = 256;
 constexpr int kBins = 4096;
 constexpr int kPasses = 11;  // 10 x 12 bits + 7 bits = 127
 constexpr int kRedBlocks = 304;
+// one CTA's shared memory holds this many pairs and its counters; below it a launch
+// costs more than the work (10 to 30 launches of 2 to 5 us against one of 20 to 40 us)
+constexpr int kSmall = 8192;
+constexpr int kSmallT = 1024;
 
 __host__ __device__ inline int pass_width(int p) { return p < 10 ? 12 : 7; }
 __host__ __device__ inline int pass_low(int p) { return 127 - 12 * p - pass_width(p); }
@@ -31,7 +45,8 @@ __host__ __device__ inline int pass_low(int p) { return 127 - 12 * p - pass_widt
 struct SelState {
     unsigned long long pfx_hi, pfx_lo, mask_hi, mask_lo;
     unsigned long long need, total;
-    int done, all, pass, pad;
+    int done, all, pass;
+    unsigned ticket;  // blocks that have finished the pass's histogram
     double sumsq;
 };
 
@@ -74,16 +89,87 @@ __global__ void sel_init_kernel(SelState *s, unsigned long long k, unsigned long
         s->done = (k == 0);
         s->all = 0;
         s->pass = 0;
+        s->ticket = 0;
         s->sumsq = 0.0;
         *n_gather = 0;
     }
     for (int b = threadIdx.x; b < kBins; b += blockDim.x) hist[b] = 0;
 }
 
+// the prefix and mask extended by digit b of the pass
+__device__ __forceinline__ void sel_extend(SelState *s, unsigned b, int pass) {
+    const int w = pass_width(pass), p = pass_low(pass);
+    const unsigned long long dm = (1ull << w) - 1ull;
+    // set digit b at bits [p, p+w) of the composite prefix and mask
+    if (p >= 64) {
+        s->pfx_hi |= (unsigned long long)b << (p - 64);
+        s->mask_hi |= dm << (p - 64);
+    } else if (p + w <= 64) {
+        s->pfx_lo |= (unsigned long long)b << p;
+        s->mask_lo |= dm << p;
+    } else {
+        s->pfx_lo |= (unsigned long long)b << p;
+        s->mask_lo |= dm << p;
+        s->pfx_hi |= (unsigned long long)b >> (64 - p);
+        s->mask_hi |= dm >> (64 - p);
+    }
+}
+
+// One block: choose the bin holding the need-th smallest.  Each thread owns kBins / T
+// consecutive bins; a warp scan and a scan of the warps' sums find the thread.
+template <int T>
+__device__ void sel_pick(SelState *s, const unsigned long long *hist, int pass) {
+    __shared__ unsigned long long wsum[T / 32];
+    __shared__ int found_bin;
+    __shared__ unsigned long long found_before, found_count;
+    constexpr int per = kBins / T;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned long long need = s->need;
+    if (pass == 0 && __ldcg(&s->total) <= need) {
+        __syncthreads();
+        if (tid == 0) s->all = 1, s->done = 1;
+        return;
+    }
+    unsigned long long mine = 0;
+    for (int q = 0; q < per; ++q) mine += __ldcg(&hist[tid * per + q]);
+    unsigned long long x = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(kFull, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[warp] = x;
+    if (tid == 0) found_bin = -1;
+    __syncthreads();
+    unsigned long long before = x - mine;
+    for (int w = 0; w < warp; ++w) before += wsum[w];
+    if (before < need && before + mine >= need) {
+        unsigned long long run = before;
+        for (int q = 0; q < per; ++q) {
+            const unsigned long long c = __ldcg(&hist[tid * per + q]);
+            if (run + c >= need) {
+                found_bin = tid * per + q;
+                found_before = run;
+                found_count = c;
+                break;
+            }
+            run += c;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        // found_bin < 0 cannot happen for need <= total; stop instead of looping on
+        sel_extend(s, found_bin < 0 ? 0u : (unsigned)found_bin, pass);
+        s->need = need - (found_bin < 0 ? 0ull : found_before);
+        if (found_bin < 0 || found_count == s->need || pass == kPasses - 1) s->done = 1;
+        s->pass = pass + 1;
+    }
+}
+
 __global__ void sel_hist_kernel(Items it, SelState *s, unsigned long long *hist, int pass) {
     __shared__ unsigned sh[kBins];
     __shared__ double ssq[kT / 32];
     __shared__ unsigned long long scount[kT / 32];
+    __shared__ bool last;
     if (s->done) return;
     for (int b = threadIdx.x; b < kBins; b += blockDim.x) sh[b] = 0;
     __syncthreads();
@@ -93,16 +179,17 @@ __global__ void sel_hist_kernel(Items it, SelState *s, unsigned long long *hist,
     unsigned long long cnt = 0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < it.n;
          i += (long long)gridDim.x * blockDim.x) {
-        const unsigned long long key = it.key[(size_t)i * it.stride];
         const unsigned long long vb = (unsigned long long)__double_as_longlong(it.val[(size_t)i * it.stride]);
-        if (!item_valid(key, vb)) continue;
         const unsigned long long hi = 0x7fffffffffffffffull - (vb & 0x7fffffffffffffffull);
+        if (pass > 0 && (hi & mh) != ph) continue;  // (the key is read only where the value's prefix fits)
+        const unsigned long long key = it.key[(size_t)i * it.stride];
+        if (!item_valid(key, vb)) continue;
         if (pass == 0) {
             const double v = __longlong_as_double((long long)vb);
             sq += v * v;
             cnt += 1;
         }
-        if ((hi & mh) != ph || (key & ml) != pl) continue;
+        if ((key & ml) != pl) continue;
         atomicAdd(&sh[digit_of(hi, key, p, w)], 1u);
     }
     if (pass == 0) {
@@ -122,75 +209,137 @@ __global__ void sel_hist_kernel(Items it, SelState *s, unsigned long long *hist,
         atomicAdd(&s->sumsq, a);
         atomicAdd(&s->total, c);
     }
-}
-
-// one block of kT threads: choose the bin holding the need-th smallest
-__global__ void sel_pick_kernel(SelState *s, unsigned long long *hist, int pass) {
-    __shared__ unsigned long long tsum[kT];
-    __shared__ int found_bin;
-    __shared__ unsigned long long found_before;
-    if (s->done) return;
-    if (pass == 0 && s->total <= s->need) {
-        __syncthreads();
-        if (threadIdx.x == 0) s->all = 1, s->done = 1;
-        return;
-    }
-    constexpr int per = kBins / kT;
-    unsigned long long mine = 0;
-    for (int q = 0; q < per; ++q) mine += hist[threadIdx.x * per + q];
-    tsum[threadIdx.x] = mine;
+    // the last block to get here picks the bin and clears the histogram
+    __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) {
-        // exclusive scan (kT entries, sequential: tiny)
-        unsigned long long run = 0;
-        for (int t = 0; t < kT; ++t) {
-            unsigned long long c = tsum[t];
-            tsum[t] = run;
-            run += c;
-        }
-        found_bin = -1;
-    }
+    if (threadIdx.x == 0) last = atomicAdd(&s->ticket, 1u) == gridDim.x - 1;
     __syncthreads();
-    const unsigned long long need = s->need;
-    const unsigned long long before = tsum[threadIdx.x];
-    if (before < need && before + mine >= need) {
-        unsigned long long run = before;
-        for (int q = 0; q < per; ++q) {
-            const unsigned long long c = hist[threadIdx.x * per + q];
-            if (run + c >= need) {
-                found_bin = threadIdx.x * per + q;
-                found_before = run;
-                break;
-            }
-            run += c;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const int b = found_bin < 0 ? 0 : found_bin;
-        const unsigned long long cnt = hist[b];
-        const int w = pass_width(pass), p = pass_low(pass);
-        const unsigned long long dm = (1ull << w) - 1ull;
-        // set digit b at bits [p, p+w) of the composite prefix and mask
-        if (p >= 64) {
-            s->pfx_hi |= (unsigned long long)b << (p - 64);
-            s->mask_hi |= dm << (p - 64);
-        } else if (p + w <= 64) {
-            s->pfx_lo |= (unsigned long long)b << p;
-            s->mask_lo |= dm << p;
-        } else {
-            s->pfx_lo |= (unsigned long long)b << p;
-            s->mask_lo |= dm << p;
-            s->pfx_hi |= (unsigned long long)b >> (64 - p);
-            s->mask_hi |= dm >> (64 - p);
-        }
-        s->need = need - found_before;
-        // found_bin < 0 cannot happen for need <= total; stop instead of looping on
-        if (found_bin < 0 || cnt == s->need || pass == kPasses - 1) s->done = 1;
-        s->pass = pass + 1;
-    }
+    if (!last) return;
+    __threadfence();
+    sel_pick<kT>(s, hist, pass);
     __syncthreads();
     for (int q = threadIdx.x; q < kBins; q += blockDim.x) hist[q] = 0;
+    if (threadIdx.x == 0) s->ticket = 0;
+}
+
+// The whole selection of up to kSmall items by one CTA, the items in shared memory:
+// the passes over 12-bit digits, then the chosen ones in order.  *cut (may be null):
+// the smallest |val| chosen (+inf when none).
+__global__ void __launch_bounds__(kSmallT)
+sel_small_kernel(Items it, unsigned long long k, unsigned long long *out_key, double *out_val,
+                 unsigned long long *n_out, double *sumsq_out, unsigned long long *total_out, double *cut) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    unsigned long long *key = reinterpret_cast<unsigned long long *>(sm);
+    unsigned long long *vb = key + kSmall;
+    unsigned *hist = reinterpret_cast<unsigned *>(vb + kSmall);
+    __shared__ unsigned long long ph, pl, mh, ml, need;
+    __shared__ int done, all, found;
+    __shared__ unsigned wsum[kSmallT / 32], found_before;
+    __shared__ double ssq[kSmallT / 32], scut[kSmallT / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = (int)it.n;
+    double sq = 0.0;
+    unsigned cnt = 0;
+    for (int i = tid; i < n; i += kSmallT) {
+        const unsigned long long kk = it.key[(size_t)i * it.stride];
+        unsigned long long v = (unsigned long long)__double_as_longlong(it.val[(size_t)i * it.stride]);
+        if (!item_valid(kk, v)) v = 0ull;  // (a zero value marks an item that does not count)
+        else sq += __longlong_as_double((long long)v) * __longlong_as_double((long long)v), ++cnt;
+        key[i] = kk, vb[i] = v;
+    }
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(kFull, sq, o), cnt += __shfl_xor_sync(kFull, cnt, o);
+    if (lane == 0) ssq[warp] = sq, wsum[warp] = cnt;
+    __syncthreads();
+    if (tid == 0) {
+        double a = 0.0;
+        unsigned long long c = 0;
+        for (int w = 0; w < kSmallT / 32; ++w) a += ssq[w], c += wsum[w];
+        need = k, ph = pl = mh = ml = 0ull;
+        all = c <= k, done = all;
+        if (sumsq_out) *sumsq_out = a;
+        if (total_out) *total_out = c;
+    }
+    __syncthreads();
+    constexpr int per = kBins / kSmallT;
+    for (int pass = 0; pass < kPasses && !done; ++pass) {
+        const int w = pass_width(pass), p = pass_low(pass);
+        for (int q = 0; q < per; ++q) hist[tid * per + q] = 0u;
+        if (tid == 0) found = -1;
+        __syncthreads();
+        for (int i = tid; i < n; i += kSmallT) {
+            const unsigned long long v = vb[i], hi = 0x7fffffffffffffffull - (v & 0x7fffffffffffffffull);
+            if ((v << 1) != 0ull && (hi & mh) == ph && (key[i] & ml) == pl) atomicAdd(&hist[digit_of(hi, key[i], p, w)], 1u);
+        }
+        __syncthreads();
+        unsigned mine = 0;
+        for (int q = 0; q < per; ++q) mine += hist[tid * per + q];
+        unsigned x = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(kFull, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[warp] = x;
+        __syncthreads();
+        unsigned before = x - mine;
+        for (int q = 0; q < warp; ++q) before += wsum[q];
+        if (before < need && before + mine >= need) {
+            for (int q = 0; q < per; ++q) {
+                const unsigned c = hist[tid * per + q];
+                if (before + c >= need) {
+                    found = tid * per + q, found_before = before;
+                    break;
+                }
+                before += c;
+            }
+        }
+        __syncthreads();
+        if (tid == 0) {
+            SelState t{};
+            t.pfx_hi = ph, t.pfx_lo = pl, t.mask_hi = mh, t.mask_lo = ml;
+            sel_extend(&t, found < 0 ? 0u : (unsigned)found, pass);
+            ph = t.pfx_hi, pl = t.pfx_lo, mh = t.mask_hi, ml = t.mask_lo;
+            if (found >= 0) need -= found_before;
+            if (found < 0 || hist[found] == need || pass == kPasses - 1) done = 1;
+        }
+        __syncthreads();
+    }
+    // the chosen items, in their order
+    double least = __longlong_as_double(0x7ff0000000000000ll);  // +inf
+    unsigned base = 0;
+    for (int i0 = 0; i0 < n; i0 += kSmallT) {
+        const int i = i0 + tid;
+        bool ok = false;
+        unsigned long long v = 0ull;
+        if (i < n) {
+            v = vb[i];
+            const unsigned long long hi = (0x7fffffffffffffffull - (v & 0x7fffffffffffffffull)) & mh;
+            ok = (v << 1) != 0ull && (all || hi < ph || (hi == ph && (key[i] & ml) <= pl));
+        }
+        const unsigned bal = __ballot_sync(kFull, ok);
+        if (lane == 0) wsum[warp] = __popc(bal);
+        __syncthreads();
+        unsigned pos = base, tot = 0;
+        for (int q = 0; q < kSmallT / 32; ++q) {
+            if (q < warp) pos += wsum[q];
+            tot += wsum[q];
+        }
+        pos += __popc(bal & ((1u << lane) - 1u));
+        if (ok) {
+            if ((unsigned long long)pos < k) out_key[pos] = key[i], out_val[pos] = __longlong_as_double((long long)v);
+            least = fmin(least, fabs(__longlong_as_double((long long)v)));
+        }
+        base += tot;
+        __syncthreads();
+    }
+    for (int o = 16; o > 0; o >>= 1) least = fmin(least, __shfl_xor_sync(kFull, least, o));
+    if (lane == 0) scut[warp] = least;
+    __syncthreads();
+    if (tid == 0) {
+        *n_out = base;
+        if (cut) {
+            for (int q = 1; q < kSmallT / 32; ++q) scut[0] = fmin(scut[0], scut[q]);
+            *cut = scut[0];
+        }
+    }
 }
 
 __global__ void sel_gather_kernel(Items it, const SelState *s, unsigned long long *out_key,
@@ -325,113 +474,282 @@ constexpr int kSortItems = 8;
 constexpr int kTile = kT * kSortItems;  // 2048
 constexpr int kRadix = 256;
 
-__global__ void rs_hist_kernel(const unsigned long long *key, long long cap,
-                               const unsigned long long *n_dev, int shift, unsigned *counts,
-                               int ntiles) {
-    __shared__ unsigned h[kRadix];
-    for (int b = threadIdx.x; b < kRadix; b += blockDim.x) h[b] = 0;
-    __syncthreads();
-    long long n = (long long)*n_dev;
-    if (n > cap) n = cap;
-    const long long t0 = (long long)blockIdx.x * kTile;
-    for (int q = 0; q < kSortItems; ++q) {
-        const long long i = t0 + (long long)q * kT + threadIdx.x;
-        if (i < n) atomicAdd(&h[(key[i] >> shift) & 0xff], 1u);
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < kRadix; b += blockDim.x) counts[(size_t)b * ntiles + blockIdx.x] = h[b];
+constexpr int kDigits = 8;
+
+// shared by a sort's kernels: how often each digit value occurs, and one of the keys
+// (a digit whose value in that key is every key's needs no pass)
+struct SortState {
+    unsigned digit[kDigits][kRadix];
+    unsigned long long key0;
+};
+
+__device__ __forceinline__ bool rs_skip(const SortState *s, unsigned n, int p) {
+    return s->digit[p][(s->key0 >> (8 * p)) & 0xff] == n;
 }
 
-// exclusive scan of m unsigned counters in place, one block of 1024 threads
-__global__ void rs_scan_kernel(unsigned *c, long long m) {
-    __shared__ unsigned long long wsum[32];
-    __shared__ unsigned long long carry;
-    if (threadIdx.x == 0) carry = 0;
+// which of the two buffers holds the pairs before pass p
+__device__ __forceinline__ int rs_buffer(const SortState *s, unsigned n, int p) {
+    int c = 0;
+    for (int q = 0; q < p; ++q) c ^= !rs_skip(s, n, q);
+    return c;
+}
+
+__device__ __forceinline__ long long rs_count(const unsigned long long *n_dev, long long cap) {
+    const long long n = (long long)*n_dev;
+    return n < cap ? n : cap;
+}
+
+__global__ void rs_digits_kernel(const unsigned long long *key, long long cap, const unsigned long long *n_dev,
+                                 int passes, SortState *s) {
+    __shared__ unsigned h[kDigits][kRadix];
+    for (int b = threadIdx.x; b < kDigits * kRadix; b += blockDim.x) (&h[0][0])[b] = 0;
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (long long b0 = 0; b0 < m; b0 += blockDim.x) {
-        const long long i = b0 + threadIdx.x;
-        unsigned long long v = i < m ? c[i] : 0;
-        unsigned long long x = v;
+    const long long n = rs_count(n_dev, cap);
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const unsigned long long k = key[i];
+        for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(k >> (8 * p)) & 0xff], 1u);
+        if (i == 0) s->key0 = k;
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < passes * kRadix; b += blockDim.x)
+        if ((&h[0][0])[b]) atomicAdd(&(&s->digit[0][0])[b], (&h[0][0])[b]);
+}
+
+// per tile and digit value: the keys that have it; counts[value * tiles + tile]
+__global__ void rs_hist_kernel(const unsigned long long *ka, const unsigned long long *kb, long long cap,
+                               const unsigned long long *n_dev, int p, const SortState *s, unsigned *counts) {
+    __shared__ unsigned h[kRadix];
+    const long long n = rs_count(n_dev, cap);
+    if (rs_skip(s, (unsigned)n, p)) return;
+    const unsigned long long *key = rs_buffer(s, (unsigned)n, p) ? kb : ka;
+    const int tiles = (int)((n + kTile - 1) / kTile);
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        h[threadIdx.x] = 0;  // kT == kRadix
+        __syncthreads();
+        const long long t0 = (long long)t * kTile;
+        for (int q = 0; q < kSortItems; ++q) {
+            const long long i = t0 + (long long)q * kT + threadIdx.x;
+            if (i < n) atomicAdd(&h[(key[i] >> (8 * p)) & 0xff], 1u);
+        }
+        __syncthreads();
+        counts[(size_t)threadIdx.x * tiles + t] = h[threadIdx.x];
+        __syncthreads();
+    }
+}
+
+// block v: exclusive scan over the tiles of digit value v, from the keys of smaller values on
+__global__ void rs_scan_kernel(unsigned *counts, long long cap, const unsigned long long *n_dev, int p,
+                               const SortState *s) {
+    __shared__ unsigned wsum[32];
+    const long long n = rs_count(n_dev, cap);
+    if (rs_skip(s, (unsigned)n, p)) return;
+    const int tiles = (int)((n + kTile - 1) / kTile), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned *c = counts + (size_t)blockIdx.x * tiles;
+    unsigned carry = 0;
+    {
+        unsigned v = threadIdx.x < blockIdx.x ? s->digit[p][threadIdx.x] : 0u;  // (kRadix <= threads)
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+        if (lane == 0) wsum[warp] = v;
+        __syncthreads();
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) carry += wsum[w];
+        __syncthreads();
+    }
+    for (int b0 = 0; b0 < tiles; b0 += blockDim.x) {
+        const int i = b0 + threadIdx.x;
+        const unsigned v = i < tiles ? c[i] : 0u;
+        unsigned x = v;
         for (int o = 1; o < 32; o <<= 1) {
-            unsigned long long y = __shfl_up_sync(kFull, x, o);
+            const unsigned y = __shfl_up_sync(kFull, x, o);
             if (lane >= o) x += y;
         }
         if (lane == 31) wsum[warp] = x;
         __syncthreads();
-        if (warp == 0) {
-            unsigned long long s = wsum[lane];
-            unsigned long long t = s;
-            for (int o = 1; o < 32; o <<= 1) {
-                unsigned long long y = __shfl_up_sync(kFull, t, o);
-                if (lane >= o) t += y;
-            }
-            wsum[lane] = t - s;  // exclusive over warps
+        unsigned before = carry, tot = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+            if (w < warp) before += wsum[w];
+            tot += wsum[w];
         }
-        __syncthreads();
-        const unsigned long long excl = carry + wsum[warp] + x - v;
-        if (i < m) c[i] = (unsigned)excl;
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry = excl + v;
+        if (i < tiles) c[i] = before + x - v;
+        carry += tot;
         __syncthreads();
     }
 }
 
-__global__ void rs_scatter_kernel(const unsigned long long *kin, const double *vin,
-                                  unsigned long long *kout, double *vout, long long cap,
-                                  const unsigned long long *n_dev, int shift,
-                                  const unsigned *offsets, int ntiles) {
+__global__ void rs_scatter_kernel(unsigned long long *ka, double *va, unsigned long long *kb, double *vb,
+                                  long long cap, const unsigned long long *n_dev, int p, const SortState *s,
+                                  const unsigned *offsets) {
     __shared__ unsigned wc[kT / 32][kRadix];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int b = threadIdx.x; b < (kT / 32) * kRadix; b += blockDim.x) (&wc[0][0])[b] = 0;
-    __syncthreads();
-    long long n = (long long)*n_dev;
-    if (n > cap) n = cap;
-    const long long w0 = (long long)blockIdx.x * kTile + (long long)warp * (32 * kSortItems);
-    unsigned loc[kSortItems];
-    unsigned dig[kSortItems];
-    for (int q = 0; q < kSortItems; ++q) {
-        const long long i = w0 + (long long)q * 32 + lane;
-        const bool valid = i < n;
-        const unsigned d = valid ? (unsigned)((kin[i] >> shift) & 0xff) : (0x1000u | lane);
-        const unsigned peers = __match_any_sync(kFull, d);
-        const unsigned before = __popc(peers & ((1u << lane) - 1u));
-        unsigned base = valid ? wc[warp][d] : 0u;
-        __syncwarp();
-        if (valid && (peers >> lane) == 1u) wc[warp][d] = base + __popc(peers);  // highest peer
-        __syncwarp();
-        loc[q] = base + before;
-        dig[q] = d;
-    }
-    __syncthreads();
-    for (int d = threadIdx.x; d < kRadix; d += blockDim.x) {
-        unsigned run = 0;
-        for (int w = 0; w < kT / 32; ++w) {
-            unsigned c = wc[w][d];
-            wc[w][d] = run;
-            run += c;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, shift = 8 * p;
+    const long long n = rs_count(n_dev, cap);
+    if (rs_skip(s, (unsigned)n, p)) return;
+    const bool from_b = rs_buffer(s, (unsigned)n, p) != 0;
+    const unsigned long long *kin = from_b ? kb : ka;
+    const double *vin = from_b ? vb : va;
+    unsigned long long *kout = from_b ? ka : kb;
+    double *vout = from_b ? va : vb;
+    const int tiles = (int)((n + kTile - 1) / kTile);
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        for (int b = threadIdx.x; b < (kT / 32) * kRadix; b += blockDim.x) (&wc[0][0])[b] = 0;
+        __syncthreads();
+        const long long w0 = (long long)t * kTile + (long long)warp * (32 * kSortItems);
+        unsigned loc[kSortItems];
+        unsigned long long key[kSortItems];
+        for (int q = 0; q < kSortItems; ++q) {
+            const long long i = w0 + (long long)q * 32 + lane;
+            key[q] = i < n ? kin[i] : 0ull;
         }
-    }
-    __syncthreads();
-    for (int q = 0; q < kSortItems; ++q) {
-        const long long i = w0 + (long long)q * 32 + lane;
-        if (i < n) {
-            const unsigned d = dig[q];
-            const unsigned long long pos =
-                (unsigned long long)offsets[(size_t)d * ntiles + blockIdx.x] + wc[warp][d] + loc[q];
-            kout[pos] = kin[i];
-            vout[pos] = vin[i];
+        for (int q = 0; q < kSortItems; ++q) {
+            const long long i = w0 + (long long)q * 32 + lane;
+            const bool valid = i < n;
+            const unsigned d = valid ? (unsigned)((key[q] >> shift) & 0xff) : (0x1000u | lane);
+            const unsigned peers = __match_any_sync(kFull, d);
+            const unsigned before = __popc(peers & ((1u << lane) - 1u));
+            const unsigned base = valid ? wc[warp][d] : 0u;
+            __syncwarp();
+            if (valid && (peers >> lane) == 1u) wc[warp][d] = base + __popc(peers);  // highest peer
+            __syncwarp();
+            loc[q] = base + before;
         }
+        __syncthreads();
+        {
+            unsigned run = offsets[(size_t)threadIdx.x * tiles + t];  // kT == kRadix
+            for (int w = 0; w < kT / 32; ++w) {
+                const unsigned c = wc[w][threadIdx.x];
+                wc[w][threadIdx.x] = run;
+                run += c;
+            }
+        }
+        __syncthreads();
+        for (int q = 0; q < kSortItems; ++q) {
+            const long long i = w0 + (long long)q * 32 + lane;
+            if (i < n) {
+                const unsigned pos = wc[warp][(key[q] >> shift) & 0xff] + loc[q];
+                kout[pos] = key[q];
+                vout[pos] = vin[i];
+            }
+        }
+        __syncthreads();
     }
 }
 
-__global__ void copy_pairs_kernel(const unsigned long long *ks, const double *vs,
-                                  unsigned long long *kd, double *vd, long long cap,
-                                  const unsigned long long *n_dev) {
-    long long n = (long long)*n_dev;
-    if (n > cap) n = cap;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
+// The sum over the kRedBlocks partial sums, in order (thread 0's value; every thread of
+// a block of at least 32 calls it): the partials are fetched together, then added.
+__device__ __forceinline__ double ordered_sum(const double *partial, int np, double *sh) {
+    for (int k = threadIdx.x; k < np; k += blockDim.x) sh[k] = partial[k];
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x == 0)
+        for (int k = 0; k < np; ++k) s += sh[k];
+    return s;
+}
+
+// Up to kSmall pairs sorted by one CTA in shared memory and, with `normalize`, divided
+// by their 2-norm (summed in the order of sumsq_kernel and scale_kernel).
+__global__ void __launch_bounds__(kSmallT)
+small_sort_kernel(unsigned long long *key, double *val, long long cap, const unsigned long long *n_dev, int bits,
+                  int normalize) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    unsigned long long *sk = reinterpret_cast<unsigned long long *>(sm);
+    double *sv = reinterpret_cast<double *>(sk + kSmall);
+    unsigned *wc = reinterpret_cast<unsigned *>(sv + kSmall);  // [warps][kRadix]
+    __shared__ unsigned dsum[kRadix / 32];
+    __shared__ double part[kSmallT / 256][8], norm;
+    constexpr int W = kSmallT / 32, kItems = kSmall / kSmallT;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n = (int)rs_count(n_dev, cap), per = (n + kSmallT - 1) / kSmallT;  // rounds of 32 per warp
+    unsigned long long k[kItems];
+    double v[kItems];
+    const int w0 = warp * 32 * per + lane;
+#pragma unroll
+    for (int q = 0; q < kItems; ++q) {
+        const int i = w0 + q * 32;
+        k[q] = 0ull, v[q] = 0.0;
+        if (q < per && i < n) k[q] = key[i], v[q] = val[i];
+    }
+    for (int shift = 0; shift < bits; shift += 8) {
+        for (int b = tid; b < W * kRadix; b += kSmallT) wc[b] = 0u;
+        __syncthreads();
+        unsigned loc[kItems];
+#pragma unroll
+        for (int q = 0; q < kItems; ++q) {
+            loc[q] = 0u;
+            if (q >= per) continue;
+            const bool valid = w0 + q * 32 < n;
+            const unsigned d = valid ? (unsigned)((k[q] >> shift) & 0xff) : (0x1000u | lane);
+            const unsigned peers = __match_any_sync(kFull, d);
+            const unsigned base = valid ? wc[warp * kRadix + d] : 0u;
+            __syncwarp();
+            if (valid && (peers >> lane) == 1u) wc[warp * kRadix + d] = base + __popc(peers);  // highest peer
+            __syncwarp();
+            loc[q] = base + __popc(peers & ((1u << lane) - 1u));
+        }
+        __syncthreads();
+        unsigned tot = 0, x = 0;
+        if (tid < kRadix) {
+            for (int w = 0; w < W; ++w) tot += wc[w * kRadix + tid];
+            x = tot;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(kFull, x, o);
+                if (lane >= o) x += y;
+            }
+            if (lane == 31) dsum[warp] = x;
+        }
+        __syncthreads();
+        if (tid < kRadix) {
+            unsigned run = x - tot;
+            for (int w = 0; w < warp; ++w) run += dsum[w];
+            for (int w = 0; w < W; ++w) {
+                const unsigned c = wc[w * kRadix + tid];
+                wc[w * kRadix + tid] = run;
+                run += c;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kItems; ++q)
+            if (q < per && w0 + q * 32 < n) {
+                const unsigned pos = wc[warp * kRadix + ((k[q] >> shift) & 0xff)] + loc[q];
+                sk[pos] = k[q], sv[pos] = v[q];
+            }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kItems; ++q)
+            if (q < per && w0 + q * 32 < n) k[q] = sk[w0 + q * 32], v[q] = sv[w0 + q * 32];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kItems; ++q)
+        if (q < per && w0 + q * 32 < n) key[w0 + q * 32] = k[q], sv[w0 + q * 32] = v[q];
+    __syncthreads();
+    if (normalize) {
+        double s = 0.0;  // (thread 0) over the blocks of 256 in order
+        for (int b0 = 0; b0 < n; b0 += kSmallT) {
+            const int i = b0 + tid;
+            double a = i < n ? __fma_rn(sv[i], sv[i], 0.0) : 0.0;
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(kFull, a, o);
+            if (lane == 0) part[warp >> 3][warp & 7] = a;
+            __syncthreads();
+            if (tid == 0)
+                for (int b = 0; b < kSmallT / 256; ++b) {
+                    double r = 0.0;
+                    for (int w = 0; w < 8; ++w) r += part[b][w];
+                    s += r;
+                }
+            __syncthreads();
+        }
+        if (tid == 0) norm = sqrt(s);
+        __syncthreads();
+    }
+    const double d = normalize ? norm : 1.0;
+    for (int i = tid; i < n; i += kSmallT) val[i] = normalize && d > 0.0 ? __ddiv_rn(sv[i], d) : sv[i];
+}
+
+// back into the caller's arrays when an odd number of passes ran
+__global__ void copy_pairs_kernel(const unsigned long long *ks, const double *vs, unsigned long long *kd, double *vd,
+                                  long long cap, const unsigned long long *n_dev, int passes, const SortState *s) {
+    const long long n = rs_count(n_dev, cap);
+    if (!rs_buffer(s, (unsigned)n, passes)) return;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         kd[i] = ks[i];
         vd[i] = vs[i];
     }
@@ -460,12 +778,9 @@ __global__ void sumsq_kernel(const double *v, long long cap, const unsigned long
 
 __global__ void scale_kernel(double *v, long long cap, const unsigned long long *n_dev,
                              const double *partial, int nparts) {
-    __shared__ double norm;
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int k = 0; k < nparts; ++k) s += partial[k];
-        norm = sqrt(s);
-    }
+    __shared__ double norm, sh[kRedBlocks];
+    const double s = ordered_sum(partial, nparts, sh);
+    if (threadIdx.x == 0) norm = sqrt(s);
     __syncthreads();
     long long n = (long long)*n_dev;
     if (n > cap) n = cap;
@@ -480,11 +795,22 @@ __global__ void scale_kernel(double *v, long long cap, const unsigned long long 
 
 size_t select_workspace_bytes(long long, long long) { return sel_layout().bytes; }
 
+bool select_is_small(const Items &it) { return it.n <= kSmall; }
+
 cudaError_t select_topk(Items it, long long k, unsigned long long *out_key, double *out_val,
                         unsigned long long *n_out_dev, double *sumsq_dev,
-                        unsigned long long *total_dev, void *ws, size_t ws_bytes, cudaStream_t st) {
+                        unsigned long long *total_dev, void *ws, size_t ws_bytes, cudaStream_t st, double *cut_dev) {
     const SelLayout L = sel_layout();
     if (ws_bytes < L.bytes) return cudaErrorInvalidValue;
+    if (select_is_small(it)) {
+        const size_t smem = size_t(kSmall) * 16 + kBins * 4;
+        cudaError_t e = allow_max_smem(sel_small_kernel, smem);
+        if (e != cudaSuccess) return e;
+        count_launch();
+        sel_small_kernel<<<1, kSmallT, smem, st>>>(it, (unsigned long long)(k < 0 ? 0 : k), out_key, out_val, n_out_dev,
+                                                   sumsq_dev, total_dev, cut_dev);
+        return cudaGetLastError();
+    }
     char *base = static_cast<char *>(ws);
     SelState *s = reinterpret_cast<SelState *>(base + L.state);
     unsigned long long *hist = reinterpret_cast<unsigned long long *>(base + L.hist);
@@ -494,8 +820,6 @@ cudaError_t select_topk(Items it, long long k, unsigned long long *out_key, doub
     for (int p = 0; p < kPasses; ++p) {
         count_launch();
         sel_hist_kernel<<<g, kT, 0, st>>>(it, s, hist, p);
-        count_launch();
-        sel_pick_kernel<<<1, kT, 0, st>>>(s, hist, p);
     }
     count_launch();
     sel_gather_kernel<<<grid_for(it.n, 8), kT, 0, st>>>(it, s, out_key, out_val, k, n_out_dev);
@@ -503,6 +827,7 @@ cudaError_t select_topk(Items it, long long k, unsigned long long *out_key, doub
         count_launch();
         sel_stats_kernel<<<1, 32, 0, st>>>(s, sumsq_dev, total_dev);
     }
+    if (cut_dev) return min_abs(out_val, n_out_dev, k, cut_dev, st);
     return cudaGetLastError();
 }
 
@@ -524,8 +849,6 @@ cudaError_t select_split(Items it, long long k,
     count_launch();
     sel_hist_kernel<<<grid_for(it.n, 4), kT, 0, st>>>(it, s, hist, 0);
     count_launch();
-    sel_pick_kernel<<<1, kT, 0, st>>>(s, hist, 0);
-    count_launch();
     sel_split_kernel<<<grid_for(it.n, 8), kT, 0, st>>>(it, s, out_key, out_val, k, n_out_dev,
                                                        cand_key, cand_val, cand_cap, cand_n);
     count_launch();
@@ -537,40 +860,58 @@ cudaError_t select_split(Items it, long long k,
 
 size_t sort_pairs_bytes(long long cap) {
     const long long ntiles = (cap + kTile - 1) / kTile;
-    return a256(size_t(cap) * 8) * 2 + a256(size_t(ntiles > 0 ? ntiles : 1) * kRadix * 4);
+    return a256(size_t(cap) * 8) * 2 + a256(size_t(ntiles > 0 ? ntiles : 1) * kRadix * 4) + a256(sizeof(SortState));
 }
 
 size_t sort_workspace_bytes(long long n) { return sort_pairs_bytes(n); }
 
+namespace {
+cudaError_t small_sort(unsigned long long *key, double *val, long long cap, const unsigned long long *n_dev, int bits,
+                       int normalize, cudaStream_t st) {
+    const size_t smem = size_t(kSmall) * 16 + size_t(kSmallT / 32) * kRadix * 4;
+    cudaError_t e = allow_max_smem(small_sort_kernel, smem);
+    if (e != cudaSuccess) return e;
+    count_launch();
+    small_sort_kernel<<<1, kSmallT, smem, st>>>(key, val, cap, n_dev, bits, normalize);
+    return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t sort_pairs(unsigned long long *key, double *val, long long cap,
                        const unsigned long long *n_dev, int bits, void *ws, cudaStream_t st) {
     if (cap <= 0) return cudaSuccess;
-    const int ntiles = (int)((cap + kTile - 1) / kTile);
+    if (cap <= kSmall) return small_sort(key, val, cap, n_dev, bits, 0, st);
+    const long long ntiles = (cap + kTile - 1) / kTile;
     char *b = static_cast<char *>(ws);
     unsigned long long *k2 = reinterpret_cast<unsigned long long *>(b);
     double *v2 = reinterpret_cast<double *>(b + a256(size_t(cap) * 8));
     unsigned *counts = reinterpret_cast<unsigned *>(b + 2 * a256(size_t(cap) * 8));
-    unsigned long long *ka = key, *kb = k2;
-    double *va = val, *vb = v2;
-    int passes = 0;
-    for (int shift = 0; shift < bits; shift += 8) {
+    SortState *s = reinterpret_cast<SortState *>(b + 2 * a256(size_t(cap) * 8) + a256(size_t(ntiles) * kRadix * 4));
+    const int passes = (bits + 7) / 8;
+    cudaError_t e = cudaMemsetAsync(s, 0, sizeof(SortState), st);
+    if (e != cudaSuccess) return e;
+    count_launch();
+    rs_digits_kernel<<<grid_for(cap, 4), kT, 0, st>>>(key, cap, n_dev, passes, s);
+    const unsigned g = (unsigned)(ntiles < (long long)sms() * 8 ? ntiles : (long long)sms() * 8);
+    for (int p = 0; p < passes; ++p) {
         count_launch();
-        rs_hist_kernel<<<ntiles, kT, 0, st>>>(ka, cap, n_dev, shift, counts, ntiles);
+        rs_hist_kernel<<<g, kT, 0, st>>>(key, k2, cap, n_dev, p, s, counts);
         count_launch();
-        rs_scan_kernel<<<1, 1024, 0, st>>>(counts, (long long)ntiles * kRadix);
+        rs_scan_kernel<<<kRadix, ntiles > 2048 ? 1024 : 256, 0, st>>>(counts, cap, n_dev, p, s);
         count_launch();
-        rs_scatter_kernel<<<ntiles, kT, 0, st>>>(ka, va, kb, vb, cap, n_dev, shift, counts, ntiles);
-        unsigned long long *tk = ka;
-        ka = kb, kb = tk;
-        double *tv = va;
-        va = vb, vb = tv;
-        ++passes;
+        rs_scatter_kernel<<<g, kT, 0, st>>>(key, val, k2, v2, cap, n_dev, p, s, counts);
     }
-    if (passes & 1) {
-        count_launch();
-        copy_pairs_kernel<<<grid_for(cap, 8), kT, 0, st>>>(ka, va, key, val, cap, n_dev);
-    }
+    count_launch();
+    copy_pairs_kernel<<<grid_for(cap, 8), kT, 0, st>>>(k2, v2, key, val, cap, n_dev, passes, s);
     return cudaGetLastError();
+}
+
+cudaError_t sort_normalize(unsigned long long *key, double *val, long long cap, const unsigned long long *n_dev,
+                           int bits, void *sort_ws, void *norm_ws, cudaStream_t st) {
+    if (cap <= 0) return cudaSuccess;
+    if (cap <= kSmall) return small_sort(key, val, cap, n_dev, bits, 1, st);
+    const cudaError_t e = sort_pairs(key, val, cap, n_dev, bits, sort_ws, st);
+    return e == cudaSuccess ? normalize_vec(val, cap, n_dev, norm_ws, st) : e;
 }
 
 size_t normalize_ws_bytes(long long) { return a256(sizeof(double) * kRedBlocks); }
