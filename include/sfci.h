@@ -112,7 +112,8 @@ sfci_status sfci_unrank(const sfci_system *sys, const uint64_t *rank, uint64_t *
 /* Workspace (bytes, device) that sfci_sigma needs for n_in input entries and
  * room for out_cap output entries.  It holds an open-addressing table of
  * 2^ceil(log2(2 out_cap)) slots (at least 1024; 32 bytes each with the exact
- * sums) plus sort buffers. */
+ * sums) plus sort buffers.  Where the lists of the sum by target rows fit in
+ * the table's space, sfci_sigma keeps those there instead of the table. */
 sfci_status sfci_sigma_workspace_bytes(const sfci_system *sys, int64_t n_in, int64_t out_cap,
                                        size_t *bytes);
 
@@ -126,7 +127,7 @@ sfci_status sfci_sigma_workspace_bytes(const sfci_system *sys, int64_t n_in, int
  * their count to *n_out (host).
  * in_rank/in_coef: device, n_in entries, ranks strictly ascending and < dim.
  * Returns SFCI_E_CAPACITY if more than out_cap entries result: then *n_out is
- * the exact count when it is at most the table's slot count, otherwise a lower
+ * the exact count, or, when the table was used and has too few slots, a lower
  * bound (retry with a larger out_cap).  SFCI_E_CAPACITY also when ws_bytes is
  * below sfci_sigma_workspace_bytes.  No allocation; synchronises the stream.
  * Each entry is summed exactly (128-bit fixed point in units of 2^-S, S set

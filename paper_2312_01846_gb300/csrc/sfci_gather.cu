@@ -1247,7 +1247,7 @@ gather_kernel(const __grid_constant__ GatherArgs A) {
                             ++n_nonzero;
                             sq = __fma_rn(v, v, sq);
                         }
-                        w = nz && !(ab < tau_bits);
+                        w = A.all ? live : nz && !(ab < tau_bits);
                         keys[h] = kNoKey;
                         limb[h] = limb[h + kGSlots] = limb[h + 2 * kGSlots] = limb[h + 3 * kGSlots] = 0u;
                         if (w) hb = (unsigned)(ab >> kHistShift);
@@ -1255,8 +1255,10 @@ gather_kernel(const __grid_constant__ GatherArgs A) {
                     const unsigned bal = __ballot_sync(kFull, w);
                     if (bal) {
                         // histogram of the streamed entries (lanes sharing a bin add once)
-                        const unsigned peers = __match_any_sync(kFull, hb);
-                        if (w && (peers & lt) == 0) atomicAdd(&A.hist[hb], (unsigned long long)__popc(peers));
+                        if (!A.all) {
+                            const unsigned peers = __match_any_sync(kFull, hb);
+                            if (w && (peers & lt) == 0) atomicAdd(&A.hist[hb], (unsigned long long)__popc(peers));
+                        }
                         unsigned long long base = 0;
                         if (lane == 0) base = atomicAdd(A.out_n, (unsigned long long)__popc(bal));
                         base = __shfl_sync(kFull, base, 0);
@@ -1357,8 +1359,121 @@ bool gather_shape(const SysDev &d, GatherShape *p) {
     return d.sb < 65536;
 }
 
-int gather_slots() { return kGSlots; }
-int gather_slots_log2() { return kGLog; }
+// Memory one buffer hands out in 256-byte pieces (no base: sizes only)
+namespace {
+struct Arena {
+    char *base = nullptr;
+    size_t off = 0;
+    template <class T>
+    T *take(size_t n) {
+        T *p = base ? reinterpret_cast<T *>(base + off) : nullptr;
+        off += (n * sizeof(T) + 255) & ~size_t(255);
+        return p;
+    }
+};
+}  // namespace
+
+size_t gather_place_sources(char *base, GatherBufs &b, const SysDev &d, const GatherShape &p, long long n) {
+    Arena a{base};
+    const size_t ca = size_t(d.ca), cb = size_t(d.cb);
+    b.words = a.take<unsigned long long>(8);
+    b.skey = a.take<unsigned long long>(n);
+    b.sc = a.take<double>(n);
+    b.sort_ws = a.take<char>(p.bb > kGLog ? sort_pairs_bytes(n) : 0);
+    b.scan_ws = a.take<char>(scan_ws_bytes((long long)std::max({ca, cb, size_t(p.nk1), size_t(p.nk2)}) + 1));
+    b.bflag = a.take<unsigned>(cb);
+    b.bid = a.take<unsigned long long>(cb + 1);
+    b.s_pi = a.take<unsigned>(n);
+    b.s_b = a.take<unsigned>(n);
+    b.s_kb = a.take<unsigned>(n);
+    b.s_diag = a.take<double>(n);
+    b.cnt1 = a.take<unsigned>(size_t(p.nk1) + p.nk2);
+    b.cnt2 = b.cnt1 + p.nk1;
+    b.off1 = a.take<unsigned long long>(size_t(p.nk1) + 1);
+    b.off2 = a.take<unsigned long long>(size_t(p.nk2) + 1);
+    b.s1 = a.take<unsigned>(ca);
+    b.s2 = a.take<unsigned>(ca);
+    b.act = a.take<unsigned>(ca);
+    b.apos = a.take<unsigned long long>(ca + 1);
+    b.act_row = a.take<unsigned>(ca);
+    b.act_str = a.take<unsigned long long>(ca);
+    b.wpre = a.take<unsigned long long>(ca + 1);
+    b.aw = a.take<unsigned long long>(3 * ca);
+    b.nrec = reinterpret_cast<unsigned *>(b.aw + ca), b.nab = b.nrec + ca, b.np = b.nab + ca, b.nu = b.np + ca;
+    b.uoff = a.take<unsigned long long>(ca + 1);
+    b.poff = a.take<unsigned long long>(ca + 1);
+    b.rec_off = a.take<unsigned long long>(ca + 1);
+    b.ab_off = a.take<unsigned long long>(ca + 1);
+    return a.off;
+}
+
+size_t gather_place_tables(char *base, GatherBufs &b, const SysDev &d, const GatherShape &p, size_t nd, long long n) {
+    Arena a{base};
+    b.bstr = a.take<unsigned long long>(nd);
+    b.t1 = a.take<uint2>(nd * d.sb);
+    b.idx1 = a.take<unsigned short>(nd * ((1 << p.kb1) + 1));
+    b.t2p = a.take<unsigned>(nd * p.nd2);
+    b.t2e = a.take<double>(nd * p.nd2);
+    b.idx2 = a.take<unsigned>(nd * ((1 << p.kb2) + 1));
+    b.ent1 = a.take<uint4>(size_t(n) * d.na);
+    b.ent2 = a.take<uint4>(size_t(n) * d.po_a);
+    return a.off;
+}
+
+size_t gather_place_lists(char *base, GatherBufs &b, const GatherShape &p, const GatherCounts &n) {
+    Arena a{base};
+    b.units = a.take<GatherUnit>(n.units);
+    b.part_k = a.take<unsigned>(n.parts);
+    b.cursor = a.take<unsigned>(2 * n.act);
+    b.split = b.cursor + n.act;
+    b.split_rows = a.take<unsigned>(n.act);
+    b.rkey = a.take<unsigned>(n.rec);
+    b.rval = a.take<double>(n.rec);
+    const size_t n_ord = p.bb > kGLog ? n.rec : 0;
+    b.okey = a.take<unsigned>(n_ord);
+    b.oval = a.take<double>(n_ord);
+    b.ab = a.take<uint4>(n.ab);
+    return a.off;
+}
+
+// 32-bit positions in the singles' table and the lists, 25 bits for a beta string's number
+bool gather_numbers(const SysDev &d, long long n, unsigned long long nd) {
+    return nd < (1ull << 25) && (double)nd * std::max(d.sb, 1) < 4294967296.0 &&
+           (double)n * std::max(d.po_a, d.na) < 4294967296.0;
+}
+
+RowPlanArgs row_plan_args(const GatherShape &p) {
+    RowPlanArgs ra{};
+    // light rows repeat entries about 1.45 times (1.3 to 2): a group fills about 0.55 of its table
+    ra.half = (unsigned long long)(0.55 * 1.45 * kGSlots);
+    ra.fill = 0.65 * kGSlots;
+    // at most 120 rows in a group (7 bits), and fewer than its key bits can number
+    ra.w_fixed = std::max(32u, (unsigned)(2 * ra.half / std::min(120, (1 << (32 - p.bb)) - 2) + 1));
+    return ra;
+}
+
+cudaError_t gather_counts(const SysDev &d, const GatherBufs &b, GatherCounts *n, cudaStream_t st) {
+    const unsigned long long *src[5] = {b.apos + d.ca, b.uoff + d.ca, b.poff + d.ca, b.rec_off + d.ca, b.ab_off + d.ca};
+    unsigned long long *dst[5] = {&n->act, &n->units, &n->parts, &n->rec, &n->ab};
+    for (int k = 0; k < 5; ++k) {
+        const cudaError_t e = cudaMemcpyAsync(dst[k], src[k], 8, cudaMemcpyDeviceToHost, st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaStreamSynchronize(st);
+}
+
+void gather_inputs(GatherArgs &A, const SysDev &d, const GatherShape &p, const GatherBufs &b, const GatherCounts &n,
+                   const unsigned *rp) {
+    A.gs = p, A.cb = d.cb, A.g = d.g, A.gf = d.gf;
+    A.sb = (unsigned)d.sb, A.nd2 = d.ss_any ? (unsigned)p.nd2 : 0u;
+    A.units = b.units, A.n_units = (unsigned)n.units, A.act_row = b.act_row;
+    A.rkey = b.rkey, A.rval = b.rval, A.okey = b.okey, A.oval = b.oval, A.split = b.split, A.ab = b.ab;
+    A.rec_off = b.rec_off, A.ab_off = b.ab_off, A.rp = rp;
+    A.s_b = b.s_b, A.s_kb = b.s_kb, A.s_c = b.sc;
+    A.t1 = b.t1, A.idx1 = b.idx1, A.t2p = b.t2p, A.t2e = b.t2e, A.idx2 = b.idx2;
+    A.seen = b.seen;
+    A.min_bits = 1ull;
+}
 
 cudaError_t launch_pair_integrals(const SysDev &d, double *W, cudaStream_t st) {
     const int np = d.n * (d.n - 1) / 2;

@@ -633,6 +633,10 @@ struct GatherBufs {
     double *rval, *oval;
     uint4 *ab;                  // one-hop sources
 };
+struct GatherCounts {  // as planned: rows with elements, units, list parts, records, one-hop sources
+    unsigned long long act, units, parts, rec, ab;
+    bool fit() const { return units < (1ull << 31) && parts < (1ull << 31) && ab < (1ull << 32); }
+};
 struct ListArgs {
     SysDev d;
     GatherShape gs;
@@ -680,6 +684,7 @@ struct GatherArgs {
     const unsigned *idx2;
     unsigned long long *seen;
     unsigned long long min_bits;  // smallest |element * c| generated, as bits (at least 1: zeros are dropped)
+    int all;             // every entry leaves (a zero sum too): tau_bits, hist, mark, lock stay as they are
     int nvec, ja, jb;
     const unsigned *vrp[kMaxVec];
     const unsigned long long *vrank[kMaxVec];
@@ -698,8 +703,16 @@ struct GatherArgs {
     int *status;
 };
 bool gather_shape(const SysDev &d, GatherShape *p);  // false: the system is outside the gather's limits
-int gather_slots();
-int gather_slots_log2();
+// its buffers in three parts, each placed when the counts it depends on are known: bytes
+// taken, pointers from base on (base null: sizes only)
+size_t gather_place_sources(char *base, GatherBufs &b, const SysDev &d, const GatherShape &p, long long n);
+size_t gather_place_tables(char *base, GatherBufs &b, const SysDev &d, const GatherShape &p, size_t nd, long long n);
+size_t gather_place_lists(char *base, GatherBufs &b, const GatherShape &p, const GatherCounts &n);
+bool gather_numbers(const SysDev &d, long long n, unsigned long long nd);  // false: positions outgrow their fields
+RowPlanArgs row_plan_args(const GatherShape &p);
+cudaError_t gather_counts(const SysDev &d, const GatherBufs &b, GatherCounts *n, cudaStream_t st);  // synchronises
+void gather_inputs(GatherArgs &A, const SysDev &d, const GatherShape &p, const GatherBufs &b, const GatherCounts &n,
+                   const unsigned *rp);
 cudaError_t launch_pair_integrals(const SysDev &d, double *W, cudaStream_t st);
 cudaError_t launch_row_pointers(const SysDev &d, const unsigned long long *rank, long long n, unsigned *rp,
                                 cudaStream_t st);

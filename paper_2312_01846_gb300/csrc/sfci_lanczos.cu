@@ -841,61 +841,6 @@ sfci_status bucketed_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long
     return SFCI_E_CAPACITY;
 }
 
-// Memory one buffer hands out in 256-byte pieces (first pass: sizes only)
-struct Arena {
-    char *base = nullptr;
-    size_t off = 0;
-    template <class T>
-    T *take(size_t n) {
-        T *p = base ? reinterpret_cast<T *>(base + off) : nullptr;
-        off += a256(n * sizeof(T));
-        return p;
-    }
-};
-
-void gather_arena_a(Arena &a, GatherBufs &b, const SysDev &d, const GatherShape &p, long long n) {
-    const size_t ca = size_t(d.ca), cb = size_t(d.cb);
-    b.words = a.take<unsigned long long>(8);
-    b.skey = a.take<unsigned long long>(n);
-    b.sc = a.take<double>(n);
-    b.sort_ws = a.take<char>(p.bb > gather_slots_log2() ? sort_pairs_bytes(n) : 0);
-    b.scan_ws = a.take<char>(scan_ws_bytes((long long)std::max({ca, cb, size_t(p.nk1), size_t(p.nk2)}) + 1));
-    b.bflag = a.take<unsigned>(cb);
-    b.bid = a.take<unsigned long long>(cb + 1);
-    b.s_pi = a.take<unsigned>(n);
-    b.s_b = a.take<unsigned>(n);
-    b.s_kb = a.take<unsigned>(n);
-    b.s_diag = a.take<double>(n);
-    b.cnt1 = a.take<unsigned>(size_t(p.nk1) + p.nk2);
-    b.cnt2 = b.cnt1 + p.nk1;
-    b.off1 = a.take<unsigned long long>(size_t(p.nk1) + 1);
-    b.off2 = a.take<unsigned long long>(size_t(p.nk2) + 1);
-    b.s1 = a.take<unsigned>(ca);
-    b.s2 = a.take<unsigned>(ca);
-    b.act = a.take<unsigned>(ca);
-    b.apos = a.take<unsigned long long>(ca + 1);
-    b.act_row = a.take<unsigned>(ca);
-    b.act_str = a.take<unsigned long long>(ca);
-    b.wpre = a.take<unsigned long long>(ca + 1);
-    b.aw = a.take<unsigned long long>(3 * ca);
-    b.nrec = reinterpret_cast<unsigned *>(b.aw + ca), b.nab = b.nrec + ca, b.np = b.nab + ca, b.nu = b.np + ca;
-    b.uoff = a.take<unsigned long long>(ca + 1);
-    b.poff = a.take<unsigned long long>(ca + 1);
-    b.rec_off = a.take<unsigned long long>(ca + 1);
-    b.ab_off = a.take<unsigned long long>(ca + 1);
-}
-
-void gather_arena_b(Arena &a, GatherBufs &b, const SysDev &d, const GatherShape &p, size_t nd, size_t n) {
-    b.bstr = a.take<unsigned long long>(nd);
-    b.t1 = a.take<uint2>(nd * d.sb);
-    b.idx1 = a.take<unsigned short>(nd * ((1 << p.kb1) + 1));
-    b.t2p = a.take<unsigned>(nd * p.nd2);
-    b.t2e = a.take<double>(nd * p.nd2);
-    b.idx2 = a.take<unsigned>(nd * ((1 << p.kb2) + 1));
-    b.ent1 = a.take<uint4>(n * d.na);
-    b.ent2 = a.take<uint4>(n * d.po_a);
-}
-
 // device bytes that sigma's buffers may take in all
 double sigma_budget(const sfci_lanczos *z, double held) {
     size_t free_b = 0, tot_b = 0;
@@ -925,22 +870,20 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     const auto t_plan0 = std::chrono::steady_clock::now();
     sfci_status r;
     GatherBufs b{};
-    Arena size_a, a;
-    gather_arena_a(size_a, b, d, gs, n_in);
+    const size_t size_a = gather_place_sources(nullptr, b, d, gs, n_in);
     // (room for what every CTA streams before the first raise of a zero threshold can act)
     double sig_need = std::min(std::max(16.0 * (double)z->nkeep, 8.0e6), E) + 2.0 * (double)z->nkeep + 1024.0;
     const size_t vrp_bytes = size_t(z->NL) * (size_t(d.ca) + 1) * 4;
     const double held = (double)z->ga.bytes + z->gb.bytes + z->gc.bytes + z->vrp.bytes + z->sig_key.bytes +
                         z->sig_val.bytes + z->belem.bytes + z->bovf.bytes + z->bovf_sorted.bytes;
     const double budget = sigma_budget(z, held);
-    double need = (double)size_a.off + (double)vrp_bytes + 16.0 * sig_need;
+    double need = (double)size_a + (double)vrp_bytes + 16.0 * sig_need;
     if (need > budget) return SFCI_OK;
     SFCI_CUDA(cudaEventRecord(z->evp[0], z->st));
-    if ((r = ensure(z->ga, size_a.off, z->st, "row gather arrays", 1.25))) return r;
+    if ((r = ensure(z->ga, size_a, z->st, "row gather arrays", 1.25))) return r;
     if (z->vrp.bytes < vrp_bytes) z->vrp_ok.assign(z->NL, 0);
     if ((r = ensure(z->vrp, vrp_bytes, z->st, "row pointers"))) return r;
-    a.base = static_cast<char *>(z->ga.p);
-    gather_arena_a(a, b, d, gs, n_in);
+    gather_place_sources(static_cast<char *>(z->ga.p), b, d, gs, n_in);
     auto *vrp = P<unsigned>(z->vrp);
     for (int j = 0; j <= i; ++j)
         if (!z->vrp_ok[j]) {
@@ -958,50 +901,20 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     SFCI_CUDA(cudaMemcpyAsync(&nd, b.bid + d.cb, 8, cudaMemcpyDeviceToHost, z->st));
     SFCI_CUDA(cudaMemcpyAsync(&runs, b.words, 8, cudaMemcpyDeviceToHost, z->st));
     SFCI_CUDA(cudaStreamSynchronize(z->st));
-    Arena size_b, ab;
-    gather_arena_b(size_b, b, d, gs, nd, (size_t)n_in);
-    // 32-bit positions in the singles' table and the lists, 25 bits for a beta string's number; memory
-    if (nd >= (1ull << 25) || (double)nd * std::max(d.sb, 1) >= 4294967296.0 || (double)n_in * std::max(d.po_a, d.na) >= 4294967296.0 ||
-        need + (double)size_b.off > budget)
-        return SFCI_OK;
-    if ((r = ensure(z->gb, size_b.off, z->st, "row gather tables", 1.1))) return r;
-    ab.base = static_cast<char *>(z->gb.p);
-    gather_arena_b(ab, b, d, gs, nd, (size_t)n_in);
-    RowPlanArgs ra{};
-    // light rows repeat entries about 1.45 times (1.3 to 2): a group fills about 0.55 of its table
-    ra.half = (unsigned long long)(0.55 * 1.45 * gather_slots());
-    ra.fill = 0.65 * gather_slots();
-    // at most 120 rows in a group (7 bits), and fewer than its key bits can number
-    ra.w_fixed = std::max(32u, (unsigned)(2 * ra.half / std::min(120, (1 << (32 - gs.bb)) - 2) + 1));
+    const size_t size_b = gather_place_tables(nullptr, b, d, gs, nd, n_in);
+    if (!gather_numbers(d, n_in, nd) || need + (double)size_b > budget) return SFCI_OK;
+    if ((r = ensure(z->gb, size_b, z->st, "row gather tables", 1.1))) return r;
+    gather_place_tables(static_cast<char *>(z->gb.p), b, d, gs, nd, n_in);
+    const RowPlanArgs ra = row_plan_args(gs);
     SFCI_CUDA(gather_tables(d, gs, n_in, (unsigned)nd, z->sys->pair_int, rp, b, ra, z->st));
-    unsigned long long n_act = 0, n_units = 0, n_parts = 0, n_rec = 0, n_ab = 0;
-    SFCI_CUDA(cudaMemcpyAsync(&n_act, b.apos + d.ca, 8, cudaMemcpyDeviceToHost, z->st));
-    SFCI_CUDA(cudaMemcpyAsync(&n_units, b.uoff + d.ca, 8, cudaMemcpyDeviceToHost, z->st));
-    SFCI_CUDA(cudaMemcpyAsync(&n_parts, b.poff + d.ca, 8, cudaMemcpyDeviceToHost, z->st));
-    SFCI_CUDA(cudaMemcpyAsync(&n_rec, b.rec_off + d.ca, 8, cudaMemcpyDeviceToHost, z->st));
-    SFCI_CUDA(cudaMemcpyAsync(&n_ab, b.ab_off + d.ca, 8, cudaMemcpyDeviceToHost, z->st));
-    SFCI_CUDA(cudaStreamSynchronize(z->st));
-    if (n_units >= (1ull << 31) || n_parts >= (1ull << 31) || n_ab >= (1ull << 32)) return SFCI_OK;
-    Arena size_c, ac;
-    auto arena_c = [&](Arena &m) {
-        b.units = m.take<GatherUnit>(n_units);
-        b.part_k = m.take<unsigned>(n_parts);
-        b.cursor = m.take<unsigned>(2 * n_act);
-        b.split = b.cursor + n_act;
-        b.split_rows = m.take<unsigned>(n_act);
-        b.rkey = m.take<unsigned>(n_rec);
-        b.rval = m.take<double>(n_rec);
-        const size_t n_ord = gs.bb > gather_slots_log2() ? n_rec : 0;
-        b.okey = m.take<unsigned>(n_ord);
-        b.oval = m.take<double>(n_ord);
-        b.ab = m.take<uint4>(n_ab);
-    };
-    arena_c(size_c);
-    if (need + (double)size_b.off + (double)size_c.off > budget) return SFCI_OK;
-    if ((r = ensure(z->gc, size_c.off, z->st, "row gather lists", 1.1))) return r;
-    ac.base = static_cast<char *>(z->gc.p);
-    arena_c(ac);
-    SFCI_CUDA(gather_lists(d, gs, n_act, n_parts, z->sys->pair_int, rp, b, ra, z->st));
+    GatherCounts gn{};
+    SFCI_CUDA(gather_counts(d, b, &gn, z->st));
+    if (!gn.fit()) return SFCI_OK;
+    const size_t size_c = gather_place_lists(nullptr, b, gs, gn);
+    if (need + (double)size_b + (double)size_c > budget) return SFCI_OK;
+    if ((r = ensure(z->gc, size_c, z->st, "row gather lists", 1.1))) return r;
+    gather_place_lists(static_cast<char *>(z->gc.p), b, gs, gn);
+    SFCI_CUDA(gather_lists(d, gs, gn.act, gn.parts, z->sys->pair_int, rp, b, ra, z->st));
     for (int j = 0; j <= i; ++j) {
         if (!z->sigw[j]) SFCI_CUDA(cudaMalloc(&z->sigw[j], size_t(z->nkeep) * 8));
         if (z->wn[j] > 0) SFCI_CUDA(cudaMemsetAsync(z->sigw[j], 0, size_t(z->wn[j]) * 8, z->st));  // rows without elements
@@ -1023,14 +936,7 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
         tw[1] = (unsigned long long)out_cap / 4;
         SFCI_CUDA(cudaMemcpyAsync(z->tau_w, tw, 16, cudaMemcpyHostToDevice, z->st));
         GatherArgs A{};
-        A.gs = gs, A.cb = d.cb, A.g = d.g, A.gf = d.gf;
-        A.sb = (unsigned)d.sb, A.nd2 = d.ss_any ? (unsigned)gs.nd2 : 0u;
-        A.units = b.units, A.n_units = (unsigned)n_units, A.act_row = b.act_row;
-        A.rkey = b.rkey, A.rval = b.rval, A.okey = b.okey, A.oval = b.oval, A.split = b.split, A.ab = b.ab;
-        A.rec_off = b.rec_off, A.ab_off = b.ab_off, A.rp = rp;
-        A.s_b = b.s_b, A.s_kb = b.s_kb, A.s_c = b.sc;
-        A.t1 = b.t1, A.idx1 = b.idx1, A.t2p = b.t2p, A.t2e = b.t2e, A.idx2 = b.idx2;
-        A.seen = b.seen;
+        gather_inputs(A, d, gs, b, gn, rp);
         const double eps_el = z->p.eps_element > 0.0 ? z->p.eps_element : 0.0;
         std::memcpy(&A.min_bits, &eps_el, 8);
         A.min_bits = std::max(A.min_bits, 1ull);
@@ -1089,7 +995,7 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
         z->n_split = 0;
         z->alpha_runs = runs;
         z->nb_log2 = 0;
-        while ((1ull << z->nb_log2) < n_units) ++z->nb_log2;
+        while ((1ull << z->nb_log2) < gn.units) ++z->nb_log2;
         z->budget_gb = budget / 1e9;
         z->free_gb = (budget - held) / 1e9, z->held_gb = held / 1e9;
         z->regions_gb = E * sizeof(Slot) / 1e9;  // what the elements would take as records
