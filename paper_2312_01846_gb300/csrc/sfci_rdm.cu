@@ -17,6 +17,16 @@
 // E = e_core <psi|psi> + sum h gamma + 1/2 sum (pq|rs) Gamma = <psi|H|psi>,
 // so dE/dh = gamma / <psi|psi> and dE/d(pq|rs) = Gamma / (2 <psi|psi>) for a
 // fixed psi.
+//
+// Two ways to find the pairs (D, D') that are both in psi:
+//  * by rows (rdm_rows_kernel; a row: the determinants of one alpha string).
+//    Each unordered pair is met once and adds to one of its images; a last pass
+//    sums Gamma over the images (p,q,r,s), (r,s,p,q), (q,p,s,r), (s,r,q,p).
+//  * by lookups (rdm_kernel): every excitation of every determinant, in a global
+//    hash table; for vectors and systems outside the limits of the former.
+#include <algorithm>
+#include <type_traits>
+
 #include "sfci_internal.cuh"
 
 namespace sfci {
@@ -197,20 +207,28 @@ __global__ void norm2_kernel(const double *c, long long m, double *partial) {
     }
 }
 
+// the sum of np partial sums, by one warp
+__device__ __forceinline__ double warp_total(const double *partial, int np) {
+    double t = 0.0;
+    for (int k = threadIdx.x; k < np; k += 32) t += partial[k];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+    return t;
+}
+
 __global__ void norm2_finish(const double *partial, int np, double *out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double t = 0.0;
-        for (int k = 0; k < np; ++k) t += partial[k];
-        *out = t;
-    }
+    const double t = warp_total(partial, np);
+    if (threadIdx.x == 0) *out = t;
 }
 
 constexpr int kNormBlocks = 152;
 
-// partial[b] = sum over block b's share of k of x[k] y[k] (x, y of length m),
-// fixed grid and order; two launches (h.gamma, then g.Gamma) write disjoint halves
-__global__ void contract_kernel(const double *x, const double *y, long long m, double *partial) {
+// partial[b] = sum over block b's share of k of x[k] y[k], fixed grid and order:
+// h.gamma (blockIdx.y 0), g.Gamma (1)
+__global__ void contract_kernel(const double *h, const double *g1, long long n2, const double *g, const double *g2,
+                                long long n4, double *partial) {
     __shared__ double sh[kWarps];
+    const double *x = blockIdx.y ? g : h, *y = blockIdx.y ? g2 : g1;
+    const long long m = blockIdx.y ? n4 : n2;
     double a = 0.0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m;
          i += (long long)gridDim.x * blockDim.x)
@@ -221,19 +239,457 @@ __global__ void contract_kernel(const double *x, const double *y, long long m, d
     if (threadIdx.x == 0) {
         double t = 0.0;
         for (int w = 0; w < kWarps; ++w) t += sh[w];
-        partial[blockIdx.x] = t;
+        partial[blockIdx.y * gridDim.x + blockIdx.x] = t;
     }
 }
 
 // E = e_core + (sum h gamma + 1/2 sum g Gamma) / norm2 from the two halves of partial
 __global__ void energy_finish(const double *partial, int np, double e_core, double norm2, double *out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double one = 0.0, two = 0.0;
-        for (int k = 0; k < np; ++k) one += partial[k];
-        for (int k = 0; k < np; ++k) two += partial[np + k];
+    const double one = warp_total(partial, np), two = warp_total(partial + np, np);
+    if (threadIdx.x == 0) {
         out[0] = e_core + (one + 0.5 * two) / norm2;
         out[1] = one;
         out[2] = two;
+    }
+}
+
+// ------------------------------------------------------------- pairs by rows
+//
+// The lookups of rdm_kernel (7876 a determinant at 20 orbitals, 1e9 at 3e5
+// determinants counted once per pair) are bound by the L2 sectors of the hash
+// table: 30 ms.  Here a CTA holds a row A' in a shared-memory table (beta index ->
+// position) and looks up
+//   opposite spin: the beta hops (tabulated once per beta string) of the
+//       determinants of the rows one alpha hop away,
+//   alpha singles and alpha-alpha doubles: the determinants of the rows one and
+//       two hops away themselves,
+// of each pair of rows the longer one in the table, so the shorter one is walked.
+// Pairs within a row (beta singles, beta-beta doubles) come from comparing all its
+// strings: m / 2 comparisons a determinant against sb + C(nb,2) C(vb,2) lookups.
+
+constexpr int kT = 256;
+constexpr unsigned kChunk = 4096;       // determinants of a row in the table at once
+constexpr unsigned kSlots = 8192;
+constexpr unsigned kNone = 0xffffffffu;
+constexpr unsigned kGrab = 4;           // units taken from the queue at a time
+
+struct RowArgs {
+    SysDev d;
+    const unsigned long long *rank;
+    const double *coef;
+    unsigned n;
+    const int *flag;        // set: the ranks are not valid, nothing runs
+    unsigned *first;        // [n] 1: starts a row
+    unsigned long long *run_of;   // [n + 1] rows before
+    unsigned *run_off;      // [n + 1] first determinant
+    unsigned *run_row;      // [n]
+    unsigned long long *run_str;  // [n] alpha string
+    unsigned long long *units, *uoff;  // [n], [n + 1]
+    unsigned *row_run;      // [ca] row -> run
+    unsigned *b_seen;       // [cb]
+    unsigned long long *b_id;     // [cb + 1]
+    unsigned *s_b, *s_id;   // [n] beta index, number of the beta string
+    unsigned *id_b;         // [distinct] its beta index
+    unsigned long long *bstr;     // [distinct]
+    uint2 *hops;            // [distinct * sb] beta index of the hop, b n + j | sign << 31
+    unsigned long long *queue;
+    double *g1, *g2;
+};
+
+struct RowUnits {  // of a row of m determinants
+    unsigned long long n1, n2, n3;
+    unsigned p1, p2, nb1, nb2, nf;
+};
+
+__device__ __forceinline__ RowUnits row_units(const SysDev &d, unsigned m) {
+    RowUnits u;
+    const unsigned nt = (m + kChunk - 1) / kChunk, tiles = (m + kT - 1) / kT;
+    u.nb1 = d.sb > 0 ? (d.sa + kT - 1) / kT : 0u;
+    u.nb2 = (d.sa + d.po_a * d.pv_a + kT - 1) / kT;
+    u.p1 = (m + 31) / 32, u.p2 = (m + kT - 1) / kT;
+    u.nf = (tiles + 3) / 4;
+    u.n1 = (unsigned long long)u.nb1 * u.p1 * nt;
+    u.n2 = (unsigned long long)u.nb2 * u.p2 * nt;
+    u.n3 = (unsigned long long)tiles * u.nf;
+    return u;
+}
+
+__global__ void rows_mark_kernel(RowArgs A) {
+    if (*A.flag) return;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n; i += gridDim.x * blockDim.x) {
+        const unsigned long long r = A.rank[i], row = r / A.d.cb;
+        const unsigned b = (unsigned)(r - row * A.d.cb);
+        A.first[i] = i == 0 || A.rank[i - 1] / A.d.cb != row;
+        A.s_b[i] = b;
+        A.b_seen[b] = 1u;
+    }
+}
+
+__global__ void rows_place_kernel(RowArgs A) {
+    if (*A.flag) return;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n; i += gridDim.x * blockDim.x) {
+        const unsigned b = A.s_b[i], id = (unsigned)A.b_id[b];
+        A.s_id[i] = id;
+        A.id_b[id] = b;
+        A.units[i] = 0ull;
+        if (A.first[i]) {
+            const unsigned run = (unsigned)A.run_of[i], row = (unsigned)(A.rank[i] / A.d.cb);
+            A.run_off[run] = i;
+            A.run_row[run] = row;
+            A.row_run[row] = run;
+        }
+        if (i == A.n - 1) A.run_off[A.run_of[A.n]] = A.n;
+    }
+}
+
+// a warp per distinct beta string: the string and its hops; then per row: its string, its units
+__global__ void __launch_bounds__(kT) rows_strings_kernel(RowArgs A) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    if (*A.flag) return;
+    const SysDev &d = A.d;
+    unsigned long long *bt = reinterpret_cast<unsigned long long *>(sm);
+    for (int i = threadIdx.x; i < (d.n + 1) * d.ks; i += blockDim.x) bt[i] = d.binom[i];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const unsigned nd = (unsigned)A.b_id[d.cb], runs = (unsigned)A.run_of[A.n];
+    for (unsigned w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nd + runs; w += (gridDim.x * blockDim.x) >> 5) {
+        if (w >= nd) {
+            const unsigned run = w - nd;
+            const unsigned long long str = string_unrank_warp(A.run_row[run], d.n, d.na, bt, d.ks);
+            if (lane == 0) {
+                const RowUnits u = row_units(d, A.run_off[run + 1] - A.run_off[run]);
+                A.run_str[run] = str;
+                A.units[run] = u.n1 + u.n2 + u.n3;
+            }
+            continue;
+        }
+        const unsigned long long str = string_unrank_warp(A.id_b[w], d.n, d.nb, bt, d.ks);
+        if (lane == 0) A.bstr[w] = str;
+        // lane p: whether orbital p is occupied; a hop per (occupied, empty) pair, by their positions
+        int x = 0;
+        for (unsigned long long o = str; o; o &= o - 1ull) {
+            const int j = __ffsll((long long)o) - 1;
+            int y = 0;
+            for (int b = 0; b < d.n; ++b) {
+                if ((str >> b) & 1ull) continue;
+                if (((x * d.vb + y) & 31) == lane) {
+                    const unsigned sg = parity64(str & between_mask(j, b));
+                    A.hops[(size_t)w * d.sb + x * d.vb + y] =
+                        make_uint2((unsigned)string_rank(str ^ (1ull << j) ^ (1ull << b), bt, d.ks), (unsigned)(b * d.n + j) | sg << 31);
+                }
+                ++y;
+            }
+            ++x;
+        }
+    }
+}
+
+// D (string `from`) and D' (`to`) differ in this spin by one or two electrons, the other
+// spin's string is `other`; v = c_D c_D' without the sign
+__device__ __noinline__ void same_spin_pair(double *g1, double *g2, int n, unsigned long long from, unsigned long long to,
+                                            unsigned long long other, double v) {
+    const size_t N1 = size_t(n), N2 = N1 * n, N3 = N2 * n;
+    unsigned long long out = from & ~to, in = to & ~from;
+    const int i = __ffsll((long long)out) - 1, a = __ffsll((long long)in) - 1;
+    int s = parity64(from & between_mask(i, a));
+    out &= out - 1ull, in &= in - 1ull;
+    if (out) {
+        const int j = __ffsll((long long)out) - 1, b = __ffsll((long long)in) - 1;
+        s ^= parity64((from ^ (1ull << i) ^ (1ull << a)) & between_mask(j, b));
+        if (s) v = -v;
+        acc(g2, a * N3 + i * N2 + b * N1 + j, v);
+        acc(g2, a * N3 + j * N2 + b * N1 + i, -v);
+        return;
+    }
+    if (s) v = -v;
+    acc(g1, size_t(a) * n + i, v);
+    for (unsigned long long k = from & to; k; k &= k - 1ull) {
+        const int p = __ffsll((long long)k) - 1;
+        acc(g2, a * N3 + i * N2 + p * N1 + p, v);
+        acc(g2, a * N3 + p * N2 + p * N1 + i, -v);
+    }
+    for (unsigned long long k = other; k; k &= k - 1ull) {
+        const int p = __ffsll((long long)k) - 1;
+        acc(g2, a * N3 + i * N2 + p * N1 + p, v);
+    }
+}
+
+struct RowShared {
+    unsigned keys[kSlots];
+    unsigned short pos[kSlots];  // (pairs within a row: strings and coefficients in place of both)
+    unsigned start[kT + 1], off[kT], hop[kT];
+    unsigned wsum[kT / 32];
+    unsigned char occ[64], vir[64];
+    unsigned long long u0;
+    unsigned run;
+};
+constexpr unsigned kTileF = 4 * kT;  // strings compared with a tile of 256 at a time
+static_assert(kTileF * 16 <= kSlots * 4 && kT * 16 <= kSlots * 2, "a row's strings lie in the table's memory");
+
+__device__ __forceinline__ int row_find(const unsigned *keys, unsigned mask, int shift, unsigned key) {
+    unsigned h = (key * 0x9E3779B1u) >> shift;
+    for (;;) {  // (at most half of the slots are taken)
+        const unsigned k = keys[h];
+        if (k == key) return (int)h;
+        if (k == kNone) return -1;
+        h = (h + 1u) & mask;
+    }
+}
+
+__global__ void __launch_bounds__(kT, 3) rdm_rows_kernel(const __grid_constant__ RowArgs A) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    if (*A.flag) return;
+    RowShared &S = *reinterpret_cast<RowShared *>(sm);
+    unsigned long long *bt = reinterpret_cast<unsigned long long *>(sm + al16(sizeof(RowShared)));
+    const SysDev &d = A.d;
+    const int n = d.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const size_t N1 = size_t(n), N2 = N1 * n, N3 = N2 * n;
+    for (int i = tid; i < (n + 1) * d.ks; i += kT) bt[i] = d.binom[i];
+    const unsigned runs = (unsigned)A.run_of[A.n];
+    const unsigned long long total = A.uoff[A.n];
+    unsigned have_run = kNone, have_t = 0u;  // what the table holds
+    unsigned mask = 0u;
+    int shift = 0;
+    for (;;) {
+        __syncthreads();
+        if (warp == 0) {
+            unsigned long long u = 0ull;
+            if (lane == 0) u = atomicAdd(A.queue, (unsigned long long)kGrab);
+            u = __shfl_sync(kFull, u, 0);
+            unsigned lo = 0, hi = runs;  // the last run whose units start at or before u
+            while (u < total && hi - lo > 1u) {
+                const unsigned step = (hi - lo + 31u) / 32u, at = lo + (lane + 1u) * step;
+                const unsigned k = __popc(__ballot_sync(kFull, at < hi && __ldg(&A.uoff[at]) <= u));
+                lo += k * step;
+                hi = min(hi, lo + step);
+            }
+            if (lane == 0) S.u0 = u, S.run = lo;
+        }
+        __syncthreads();
+        const unsigned long long u0 = S.u0, u1 = u0 + kGrab < total ? u0 + kGrab : total;
+        if (u0 >= total) break;
+        unsigned run = S.run;
+        for (unsigned long long u = u0; u < u1; ++u) {
+            while (u >= __ldg(&A.uoff[run + 1])) ++run;
+            const unsigned base = __ldg(&A.run_off[run]), m = __ldg(&A.run_off[run + 1]) - base;
+            const unsigned long long str = __ldg(&A.run_str[run]);
+            const RowUnits U = row_units(d, m);
+            unsigned long long q = u - __ldg(&A.uoff[run]);
+            __syncthreads();  // (the unit before is done with the shared memory)
+            if (q >= U.n1 + U.n2) {
+                // ---- pairs within the row: tile e against the strings f < e of four tiles
+                q -= U.n1 + U.n2;
+                const unsigned te = (unsigned)(q / U.nf), f0 = (unsigned)(q % U.nf) * kTileF;
+                if (f0 > te * kT) continue;
+                have_run = kNone;
+                unsigned long long *fs = reinterpret_cast<unsigned long long *>(S.keys);
+                double *fc = reinterpret_cast<double *>(fs + kTileF);
+                unsigned long long *es = reinterpret_cast<unsigned long long *>(S.pos);
+                double *ec = reinterpret_cast<double *>(es + kT);
+                const unsigned e = te * kT + tid, nf = min(kTileF, m - f0), ne = min((unsigned)kT, m - te * kT);
+                for (unsigned f = tid; f < nf; f += kT) {
+                    fs[f] = __ldg(&A.bstr[__ldg(&A.s_id[base + f0 + f])]);
+                    fc[f] = __ldg(&A.coef[base + f0 + f]);
+                }
+                if (e < m) {
+                    es[tid] = __ldg(&A.bstr[__ldg(&A.s_id[base + e])]);
+                    ec[tid] = __ldg(&A.coef[base + e]);
+                }
+                __syncthreads();
+                if (e < m) {
+                    const unsigned long long be = es[tid];
+                    const double ce = ec[tid];
+                    const unsigned fe = min(nf, e > f0 ? e - f0 : 0u);
+                    for (unsigned f = 0; f < fe; ++f) {
+                        const unsigned long long bf = fs[f];
+                        if (__popcll(be ^ bf) > 4) continue;
+                        const double cf = fc[f];
+                        if (ce != 0.0 && cf != 0.0) same_spin_pair(A.g1, A.g2, n, be, bf, str, ce * cf);
+                    }
+                }
+                if (f0 == 0u) {
+                    // D' = D: a thread per pair of beta orbitals (p < q: both occupied; p = q:
+                    // one) and one for the row's weight, along the tile
+                    for (int x = tid; x <= n * n; x += kT) {
+                        const int p = x / n, r = x - p * n;
+                        if (x < n * n && r < p) continue;
+                        const unsigned long long both = x < n * n ? (1ull << p | 1ull << r) : 0ull;
+                        double w = 0.0;
+                        for (unsigned f = 0; f < ne; ++f)
+                            if ((es[f] & both) == both && ec[f] != 0.0) w = __fma_rn(ec[f], ec[f], w);
+                        if (w == 0.0) continue;
+                        if (x == n * n) {
+                            for (unsigned long long k = str; k; k &= k - 1ull) {
+                                const int i = __ffsll((long long)k) - 1;
+                                acc(A.g1, size_t(i) * n + i, w);
+                                for (unsigned long long l = k & (k - 1ull); l; l &= l - 1ull) {
+                                    const int j = __ffsll((long long)l) - 1;
+                                    acc(A.g2, i * N3 + i * N2 + j * N1 + j, 0.5 * w);
+                                    acc(A.g2, i * N3 + j * N2 + j * N1 + i, -0.5 * w);
+                                }
+                            }
+                        } else if (p == r) {
+                            acc(A.g1, size_t(p) * n + p, w);
+                            for (unsigned long long k = str; k; k &= k - 1ull) {
+                                const int i = __ffsll((long long)k) - 1;
+                                acc(A.g2, i * N3 + i * N2 + p * N1 + p, 0.5 * w);
+                            }
+                        } else {
+                            acc(A.g2, p * N3 + p * N2 + r * N1 + r, 0.5 * w);
+                            acc(A.g2, p * N3 + r * N2 + r * N1 + p, -0.5 * w);
+                        }
+                    }
+                }
+                continue;
+            }
+            const bool opposite = q < U.n1;
+            if (!opposite) q -= U.n1;
+            const unsigned parts = opposite ? U.p1 : U.p2, nbat = opposite ? U.nb1 : U.nb2;
+            const unsigned t = (unsigned)(q / ((unsigned long long)parts * nbat));
+            const unsigned rem = (unsigned)(q - (unsigned long long)t * parts * nbat), batch = rem / parts, part = rem % parts;
+            const unsigned t0 = t * kChunk, mc = min(kChunk, m - t0);
+            // ---- the row's table and orbital lists
+            if (have_run != run || have_t != t) {
+                have_run = run, have_t = t;
+                unsigned size = 256u;
+                while (size < 4u * mc && size < kSlots) size *= 2u;
+                mask = size - 1u;
+                shift = 33 - __ffs((int)size);
+                for (unsigned h = tid; h < size; h += kT) S.keys[h] = kNone;
+                if (tid < n) {
+                    const int below = __popcll(str & ((1ull << tid) - 1ull));
+                    if ((str >> tid) & 1ull) S.occ[below] = (unsigned char)tid;
+                    else S.vir[tid - below] = (unsigned char)tid;
+                }
+                __syncthreads();
+                for (unsigned f = tid; f < mc; f += kT) {
+                    const unsigned key = __ldg(&A.s_b[base + t0 + f]);
+                    unsigned h = (key * 0x9E3779B1u) >> shift;
+                    while (atomicCAS(&S.keys[h], kNone, key) != kNone) h = (h + 1u) & mask;
+                    S.pos[h] = (unsigned short)f;
+                }
+            }
+            // ---- a batch of rows one or two hops away: hop from them to this row
+            const unsigned x = batch * kT + tid, n_hops = opposite ? d.sa : d.sa + d.po_a * d.pv_a;
+            unsigned cnt = 0, off = 0, hop = 0;
+            unsigned long long from = 0ull;
+            if (x < n_hops) {
+                int i1, a1, i2 = 0, a2 = 0;
+                const bool one = x < (unsigned)d.sa;
+                if (one) {
+                    a1 = S.occ[x / d.va], i1 = S.vir[x % d.va];
+                    from = str ^ (1ull << a1) ^ (1ull << i1);
+                } else {
+                    const unsigned y = x - d.sa;
+                    const unsigned char *po = d.pairs + 2 * (d.pair_off[0] + y / d.pv_a), *pv = d.pairs + 2 * (d.pair_off[1] + y % d.pv_a);
+                    a1 = S.occ[po[0]], a2 = S.occ[po[1]], i1 = S.vir[pv[0]], i2 = S.vir[pv[1]];
+                    from = str ^ (1ull << a1) ^ (1ull << i1) ^ (1ull << a2) ^ (1ull << i2);
+                }
+                const unsigned o = __ldg(&A.row_run[string_rank(from, bt, d.ks)]);
+                if (o != kNone) {
+                    off = __ldg(&A.run_off[o]);
+                    const unsigned mo = __ldg(&A.run_off[o + 1]) - off;
+                    if (mo < m || (mo == m && o < run)) cnt = mo;
+                }
+                hop = (unsigned)(a1 * n + i1) | (unsigned)parity64(from & between_mask(i1, a1)) << 31;
+            }
+            unsigned inc = cnt;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(kFull, inc, o);
+                if (lane >= o) inc += y;
+            }
+            if (lane == 31) S.wsum[warp] = inc;
+            __syncthreads();
+            for (int w = 0; w < warp; ++w) inc += S.wsum[w];
+            S.start[tid] = inc - cnt;
+            S.off[tid] = off - (inc - cnt);
+            S.hop[tid] = opposite ? hop : x;
+            if (tid == kT - 1) S.start[kT] = inc;
+            __syncthreads();
+            const unsigned tot = S.start[kT];
+            const unsigned lo = (unsigned)((unsigned long long)tot * part / parts), hi = (unsigned)((unsigned long long)tot * (part + 1) / parts);
+            if (lo == hi) continue;
+            auto segment = [&](unsigned at) {
+                unsigned o = 0;
+                for (unsigned step = kT / 2; step; step >>= 1)
+                    if (S.start[o + step] <= at) o += step;
+                return o;
+            };
+            if (opposite) {
+                // a warp takes up to 32 determinants and runs through their hops end to end
+                const unsigned per = min(32u, (hi - lo + kT / 32 - 1u) / (kT / 32));
+                for (unsigned p0 = lo + warp * per; p0 < hi; p0 += per * (kT / 32)) {
+                    const unsigned k = min(per, hi - p0);
+                    unsigned id = 0, hp = 0;
+                    double c = 0.0;
+                    if ((unsigned)lane < k) {
+                        const unsigned o = segment(p0 + lane), s = S.off[o] + p0 + lane;
+                        id = __ldg(&A.s_id[s]) * (unsigned)d.sb, hp = S.hop[o];
+                        c = __ldg(&A.coef[s]);
+                    }
+                    unsigned l = (unsigned)lane / d.sb, y = (unsigned)lane % d.sb;
+                    const unsigned dl = 32u / d.sb, dy = 32u % d.sb;
+                    for (unsigned r = 0; r < k * d.sb; r += 32u) {
+                        const bool in = l < k;
+                        const unsigned src = in ? l : 0u;
+                        const unsigned id1 = __shfl_sync(kFull, id, src), hp1 = __shfl_sync(kFull, hp, src);
+                        const double c1 = __shfl_sync(kFull, c, src);
+                        if (in) {
+                            const uint2 e = __ldg(&A.hops[(size_t)id1 + y]);
+                            const int f = row_find(S.keys, mask, shift, e.x);
+                            if (f >= 0) {
+                                const double c2 = __ldg(&A.coef[base + t0 + S.pos[f]]);
+                                if (c1 != 0.0 && c2 != 0.0) {
+                                    const double v = c1 * c2;
+                                    acc(A.g2, size_t(hp1 & 0x7fffffffu) * N2 + (e.y & 0x7fffffffu), (hp1 ^ e.y) >> 31 ? -v : v);
+                                }
+                            }
+                        }
+                        l += dl, y += dy;
+                        if (y >= (unsigned)d.sb) y -= d.sb, ++l;
+                    }
+                }
+            } else {
+                for (unsigned it = lo + tid; it < hi; it += kT) {
+                    const unsigned o = segment(it), s = S.off[o] + it;
+                    const int f = row_find(S.keys, mask, shift, __ldg(&A.s_b[s]));
+                    if (f < 0) continue;
+                    const double c1 = __ldg(&A.coef[s]), c2 = __ldg(&A.coef[base + t0 + S.pos[f]]);
+                    if (c1 == 0.0 || c2 == 0.0) continue;
+                    const unsigned y = S.hop[o];
+                    unsigned long long a = str;
+                    if (y < (unsigned)d.sa) {
+                        a ^= (1ull << S.occ[y / d.va]) ^ (1ull << S.vir[y % d.va]);
+                    } else {
+                        const unsigned z = y - d.sa;
+                        const unsigned char *po = d.pairs + 2 * (d.pair_off[0] + z / d.pv_a), *pv = d.pairs + 2 * (d.pair_off[1] + z % d.pv_a);
+                        a ^= (1ull << S.occ[po[0]]) ^ (1ull << S.occ[po[1]]) ^ (1ull << S.vir[pv[0]]) ^ (1ull << S.vir[pv[1]]);
+                    }
+                    same_spin_pair(A.g1, A.g2, n, a, str, __ldg(&A.bstr[__ldg(&A.s_id[s])]), c1 * c2);
+                }
+            }
+        }
+    }
+}
+
+// each pair added to one image of its elements: the others, in place (an orbit per thread)
+__global__ void rows_images_kernel(int n, const int *flag, double *g1, double *g2) {
+    if (*flag) return;
+    const unsigned n2 = n * n, n4 = n2 * n2;
+    for (unsigned x = blockIdx.x * blockDim.x + threadIdx.x; x < n4; x += gridDim.x * blockDim.x) {
+        const unsigned pq = x / n2, rs = x - pq * n2;
+        const unsigned qp = pq % n * n + pq / n, sr = rs % n * n + rs / n;
+        const unsigned x1 = rs * n2 + pq, x2 = qp * n2 + sr, x3 = sr * n2 + qp;
+        if (x > x1 || x > x2 || x > x3) continue;
+        const double v = (g2[x] + g2[x1]) + (g2[x2] + g2[x3]);
+        g2[x] = g2[x1] = g2[x2] = g2[x3] = v;
+    }
+    for (unsigned x = blockIdx.x * blockDim.x + threadIdx.x; x < n2; x += gridDim.x * blockDim.x) {
+        const unsigned p = x / n, q = x - p * n;
+        if (p < q) {
+            const double v = g1[x] + g1[q * n + p];
+            g1[x] = g1[q * n + p] = v;
+        }
     }
 }
 
@@ -263,6 +719,46 @@ RdmLayout rdm_layout(long long m) {
     return L;
 }
 
+// the row path's buffers in the workspace (base null: sizes only)
+size_t rows_place(char *base, RowArgs &A, size_t &scan_ws, size_t &partial, const SysDev &d, long long n) {
+    size_t o = 0;
+    auto take = [&](auto *&p, size_t count) {
+        p = base ? reinterpret_cast<std::remove_reference_t<decltype(p)>>(base + o) : nullptr;
+        o = a256(o + count * sizeof(*p));
+    };
+    const size_t nn = size_t(n), ca = size_t(d.ca), cb = size_t(d.cb), nd = std::min(nn, cb);
+    take(A.queue, 1);        // (the queue and b_seen are cleared together)
+    take(A.b_seen, cb);
+    take(A.row_run, ca);
+    take(A.b_id, cb + 1);
+    take(A.first, nn);
+    take(A.run_of, nn + 1);
+    take(A.run_off, nn + 1);
+    take(A.run_row, nn);
+    take(A.run_str, nn);
+    take(A.units, nn);
+    take(A.uoff, nn + 1);
+    take(A.s_b, nn);
+    take(A.s_id, nn);
+    take(A.id_b, nd);
+    take(A.bstr, nd);
+    take(A.hops, nd * size_t(d.sb));
+    scan_ws = o, o = a256(o + scan_ws_bytes((long long)std::max(nn, cb) + 1));
+    partial = o, o = a256(o + 8 * (kNormBlocks + 1));
+    return o;
+}
+
+// Pairs by rows: strings are numbered in 26 bits, their hops in 32; the comparisons
+// within a row stay cheaper than lookups: at most min(cb, n) / 2 of 0.15 ps a
+// determinant (issue), against 12.5 ps for each of the beta excitations (measured).
+bool rows_taken(const SysDev &d, long long n) {
+    const double exc = (double)d.sb + (double)d.po_b * d.pv_b;
+    return n > 0 && n < (1ll << 31) && d.ca <= (1ull << 26) && d.cb <= (1ull << 26) &&
+           std::min((double)n, (double)d.cb) * std::max(d.sb, 1) < 4294967296.0 &&
+           (double)d.sa + (double)d.po_a * d.pv_a < 2147483648.0 &&
+           std::min((double)n, (double)d.cb) <= 4096.0 + 128.0 * exc;
+}
+
 int sms() {
     int dev = 0, n = 0;
     cudaGetDevice(&dev);
@@ -283,6 +779,11 @@ sfci_status sfci_rdm12_workspace_bytes(const sfci_system *s, int64_t n, size_t *
         return SFCI_E_INVALID;
     }
     *bytes = rdm_layout(n).bytes;
+    if (rows_taken(s->d, n)) {
+        RowArgs A{};
+        size_t scan_ws, partial;
+        *bytes = std::max(*bytes, rows_place(nullptr, A, scan_ws, partial, s->d, n));
+    }
     return SFCI_OK;
 }
 
@@ -304,38 +805,74 @@ sfci_status sfci_rdm12(const sfci_system *s, const uint64_t *rank, const double 
     char *w = static_cast<char *>(workspace);
     SFCI_CUDA(cudaMemsetAsync(rdm1, 0, n2 * 8, st));
     SFCI_CUDA(cudaMemsetAsync(rdm2, 0, n2 * n2 * 8, st));
-    Table t;
-    t.slots = reinterpret_cast<Slot *>(w + L.table);
-    t.mask = L.slots - 1;
-    t.shift = 64 - __builtin_ctzll(L.slots);
-    t.status = reinterpret_cast<int *>(w + L.status);
-    t.count = reinterpret_cast<unsigned long long *>(w + L.count);
     const unsigned long long *r = reinterpret_cast<const unsigned long long *>(rank);
     int *flag = s->dev_status;
     SFCI_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), st));
     SFCI_CUDA(validate_sorted(r, n, d.dim, flag, st));
-    SFCI_CUDA(table_clear(t, st));
-    SFCI_CUDA(table_axpy(t, r, coef, n, nullptr, 1.0, 1.0, st));
-    double *partial = reinterpret_cast<double *>(w + L.partial);
-    double *nrm = reinterpret_cast<double *>(w + L.norm);
+    RowArgs A{};
+    size_t scan_ws = 0, part_at = L.partial;
+    const bool by_rows = rows_taken(d, n) && rows_place(nullptr, A, scan_ws, part_at, d, n) <= ws_bytes;
+    if (!by_rows) part_at = L.partial;
+    double *partial = reinterpret_cast<double *>(w + part_at);
+    double *nrm = by_rows ? partial + kNormBlocks : reinterpret_cast<double *>(w + L.norm);
     count_launch();
     norm2_kernel<<<kNormBlocks, kThreads, 0, st>>>(coef, n, partial);
     count_launch();
     norm2_finish<<<1, 32, 0, st>>>(partial, kNormBlocks, nrm);
-    if (n > 0) {
-        const size_t smem = rdm_block_smem(d) + kWarps * rdm_warp_smem(d);
-        SFCI_CUDA(allow_max_smem(rdm_kernel, smem));
+    if (by_rows) {
+        size_t ignore;
+        rows_place(w, A, ignore, ignore, d, n);
+        A.d = d, A.rank = r, A.coef = coef, A.n = (unsigned)n, A.flag = flag, A.g1 = rdm1, A.g2 = rdm2;
+        SFCI_CUDA(cudaMemsetAsync(A.queue, 0, size_t((char *)A.row_run - (char *)A.queue), st));
+        SFCI_CUDA(cudaMemsetAsync(A.row_run, 0xff, size_t(d.ca) * 4, st));
+        const unsigned g = (unsigned)std::min<long long>((n + kT - 1) / kT, sms() * 8ll);
+        count_launch();
+        rows_mark_kernel<<<g, kT, 0, st>>>(A);
+        SFCI_CUDA(exclusive_scan(A.first, n, A.run_of, w + scan_ws, st));
+        SFCI_CUDA(exclusive_scan(A.b_seen, (long long)d.cb, A.b_id, w + scan_ws, st));
+        count_launch();
+        rows_place_kernel<<<g, kT, 0, st>>>(A);
+        const size_t bts = size_t(d.n + 1) * d.ks * 8;
+        count_launch();
+        rows_strings_kernel<<<(unsigned)std::min<long long>((n + kT / 64 - 1) / (kT / 64), sms() * 8ll), kT, bts, st>>>(A);
+        SFCI_CUDA(exclusive_scan(A.units, n, A.uoff, w + scan_ws, st));
+        const size_t smem = al16(sizeof(RowShared)) + bts;
+        SFCI_CUDA(allow_max_smem(rdm_rows_kernel, smem));
         int per_sm = 0;
-        SFCI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdm_kernel, kThreads, smem));
+        SFCI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdm_rows_kernel, kT, smem));
         if (per_sm < 1) {
             set_error("rdm kernel does not fit on an SM for this system");
             return SFCI_E_CAPACITY;
         }
-        long long grid = (long long)sms() * per_sm, want = (n + kWarps - 1) / kWarps;
-        if (want < grid) grid = want;
         count_launch();
-        rdm_kernel<<<(unsigned)grid, kThreads, smem, st>>>(d, r, coef, n, t, rdm1, rdm2);
+        rdm_rows_kernel<<<sms() * per_sm, kT, smem, st>>>(A);
+        count_launch();
+        rows_images_kernel<<<(unsigned)std::min<size_t>((n2 * n2 + kT - 1) / kT, size_t(sms()) * 8), kT, 0, st>>>(d.n, flag, rdm1, rdm2);
         SFCI_CUDA(cudaGetLastError());
+    } else {
+        Table t;
+        t.slots = reinterpret_cast<Slot *>(w + L.table);
+        t.mask = L.slots - 1;
+        t.shift = 64 - __builtin_ctzll(L.slots);
+        t.status = reinterpret_cast<int *>(w + L.status);
+        t.count = reinterpret_cast<unsigned long long *>(w + L.count);
+        SFCI_CUDA(table_clear(t, st));
+        SFCI_CUDA(table_axpy(t, r, coef, n, nullptr, 1.0, 1.0, st));
+        if (n > 0) {
+            const size_t smem = rdm_block_smem(d) + kWarps * rdm_warp_smem(d);
+            SFCI_CUDA(allow_max_smem(rdm_kernel, smem));
+            int per_sm = 0;
+            SFCI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdm_kernel, kThreads, smem));
+            if (per_sm < 1) {
+                set_error("rdm kernel does not fit on an SM for this system");
+                return SFCI_E_CAPACITY;
+            }
+            long long grid = (long long)sms() * per_sm, want = (n + kWarps - 1) / kWarps;
+            if (want < grid) grid = want;
+            count_launch();
+            rdm_kernel<<<(unsigned)grid, kThreads, smem, st>>>(d, r, coef, n, t, rdm1, rdm2);
+            SFCI_CUDA(cudaGetLastError());
+        }
     }
     int hflag = 0;
     double hn = 0.0;
@@ -366,9 +903,7 @@ sfci_status sfci_rdm_energy(int n_orb, const double *rdm1, const double *rdm2, d
     double *out = partial + 2 * kNormBlocks;
     const long long n2 = (long long)n_orb * n_orb;
     count_launch();
-    contract_kernel<<<kNormBlocks, kThreads, 0, st>>>(h, rdm1, n2, partial);
-    count_launch();
-    contract_kernel<<<kNormBlocks, kThreads, 0, st>>>(g, rdm2, n2 * n2, partial + kNormBlocks);
+    contract_kernel<<<dim3(kNormBlocks, 2), kThreads, 0, st>>>(h, rdm1, n2, g, rdm2, n2 * n2, partial);
     count_launch();
     energy_finish<<<1, 32, 0, st>>>(partial, kNormBlocks, e_core, norm2, out);
     SFCI_CUDA(cudaGetLastError());
