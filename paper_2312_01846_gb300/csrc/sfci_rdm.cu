@@ -268,10 +268,10 @@ __global__ void energy_finish(const double *partial, int np, double e_core, doub
 // strings: m / 2 comparisons a determinant against sb + C(nb,2) C(vb,2) lookups.
 
 constexpr int kT = 256;
-constexpr unsigned kChunk = 4096;       // determinants of a row in the table at once
-constexpr unsigned kSlots = 8192;
+constexpr unsigned kChunk = 2048;       // determinants of a row in the table at once
+constexpr unsigned kSlots = 4096;
 constexpr unsigned kNone = 0xffffffffu;
-constexpr unsigned kGrab = 4;           // units taken from the queue at a time
+constexpr unsigned kGrab = 1;  // units taken from the queue at a time (4: 0.7 ms more at 3e5 determinants)
 
 struct RowArgs {
     SysDev d;
@@ -436,7 +436,7 @@ __device__ __forceinline__ int row_find(const unsigned *keys, unsigned mask, int
     }
 }
 
-__global__ void __launch_bounds__(kT, 3) rdm_rows_kernel(const __grid_constant__ RowArgs A) {
+__global__ void __launch_bounds__(kT, 5) rdm_rows_kernel(const __grid_constant__ RowArgs A) {
     extern __shared__ __align__(16) unsigned char sm[];
     if (*A.flag) return;
     RowShared &S = *reinterpret_cast<RowShared *>(sm);
