@@ -9,7 +9,7 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,na,nb", [(1, 1, 0), (5, 0, 5), (28, 7, 7), (35, 16, 3), (36, 18, 18), (64, 1, 63), (64, 7, 6)])
+@pytest.mark.parametrize("n,na,nb", [(1, 1, 0), (5, 0, 5), (28, 7, 7), (35, 16, 3), (36, 18, 3), (64, 1, 63), (64, 7, 6)])
 def test_unrank_edges(n, na, nb):
     torch = pytest.importorskip("torch")
     import paper_2312_01846_gb300 as sf
