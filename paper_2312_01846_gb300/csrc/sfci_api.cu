@@ -219,6 +219,10 @@ sfci_status sfci_system_create(sfci_system **out, int n, int na, int nb, const d
         const size_t np = size_t(n) * (n - 1) / 2;
         o = a256(o + np * np * 8);
     }
+    const size_t off_sg = o;
+    o = a256(o + 2 * nh * n * 8);
+    const size_t off_sgf = o;
+    if (fp32) o = a256(o + 2 * nh * n * 4);
     std::vector<float> hf, gf;
     if (fp32) {
         hf.resize(nh), gf.resize(ng);
@@ -276,7 +280,11 @@ sfci_status sfci_system_create(sfci_system **out, int n, int na, int nb, const d
     s->d = d;
     s->dev_block = blk;
     s->pair_int = reinterpret_cast<double *>(blk + off_pi);
+    double *sg = reinterpret_cast<double *>(blk + off_sg);
+    float *sgf = fp32 ? reinterpret_cast<float *>(blk + off_sgf) : nullptr;
+    s->d.sg = sg, s->d.sgf = sgf;
     e = launch_pair_integrals(d, s->pair_int, nullptr);
+    if (e == cudaSuccess) e = launch_hop_integrals(d, sg, sgf, nullptr);
     if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) {
         cudaFree(blk);
@@ -399,7 +407,7 @@ sfci_status sigma_rows(const sfci_system *s, const unsigned long long *rank, con
     if (!gather_numbers(d, n, nd) || at + size_b > room) return SFCI_OK;
     gather_place_tables(w + at, b, d, gs, nd, n);
     at += size_b;
-    const RowPlanArgs ra = row_plan_args(gs);
+    const RowPlanArgs ra = row_plan_args(d, gs, n);
     SFCI_CUDA(gather_tables(d, gs, n, (unsigned)nd, s->pair_int, rp, b, ra, st));
     GatherCounts gn{};
     SFCI_CUDA(gather_counts(d, b, &gn, st));

@@ -51,7 +51,6 @@ constexpr int kGSlots = 1 << kGLog;
 constexpr unsigned kNoKey = 0xffffffffu;
 constexpr int kMaxE = kGatherMaxElectrons;
 constexpr int kLT = 256;          // list CTA threads
-constexpr unsigned kPartWork = 1024;  // list items per part of a row
 constexpr unsigned kMaxParts = 512;
 constexpr int kMaxClassLog = 11;  // log2 of the most classes a row is planned in
 
@@ -77,16 +76,14 @@ __device__ __forceinline__ double flip_d(double x, unsigned s) {
     return __longlong_as_double(__double_as_longlong(x) ^ ((long long)s << 63));
 }
 
-// greedy inverse of Eq. 12, one thread
+// inverse of Eq. 12, one thread: orbital c is occupied when C(c, i) <= r with i electrons
+// left (the lanes of a warp walk the orbitals together)
 __device__ unsigned long long unrank_one(unsigned long long r, int n, int m, const unsigned long long *bt, int ks) {
     unsigned long long s = 0;
-    int top = n - 1;
-    for (int i = m; i >= 1; --i) {
-        int c = top;
-        while (c > 0 && bt[c * ks + i] > r) --c;
-        s |= 1ull << c;
-        r -= bt[c * ks + i];
-        top = c - 1;
+    int i = m;
+    for (int c = n - 1; c >= 0; --c) {
+        const unsigned long long x = bt[c * ks + i];
+        if (i && x <= r) r -= x, s |= 1ull << c, --i;
     }
     return s;
 }
@@ -105,26 +102,20 @@ __device__ __forceinline__ unsigned long long next_string(unsigned long long x) 
 __device__ __noinline__ double single_of(const SysDev &d, int i, int a, unsigned long long alpha,
                                          unsigned long long beta, unsigned long long same) {
     const int n = d.n;
-    const size_t n2 = size_t(n) * n;
+    const size_t at = size_t(a * n + i) * 2 * n;
     if (d.gf) {
-        const float *gai = d.gf + size_t(a * n + i) * n2;
+        const float *gai = d.sgf + at;
         float v = __ldg(&d.hf[a * n + i]);
-        for (unsigned long long s = alpha; s; s &= s - 1ull) v = __fadd_rn(v, __ldg(&gai[(__ffsll((long long)s) - 1) * (n + 1)]));
-        for (unsigned long long s = beta; s; s &= s - 1ull) v = __fadd_rn(v, __ldg(&gai[(__ffsll((long long)s) - 1) * (n + 1)]));
-        for (unsigned long long s = same; s; s &= s - 1ull) {
-            const int o = __ffsll((long long)s) - 1;
-            v = __fsub_rn(v, __ldg(&d.gf[(size_t(a * n + o) * n + o) * n + i]));
-        }
+        for (unsigned long long s = alpha; s; s &= s - 1ull) v = __fadd_rn(v, __ldg(&gai[__ffsll((long long)s) - 1]));
+        for (unsigned long long s = beta; s; s &= s - 1ull) v = __fadd_rn(v, __ldg(&gai[__ffsll((long long)s) - 1]));
+        for (unsigned long long s = same; s; s &= s - 1ull) v = __fsub_rn(v, __ldg(&gai[n + __ffsll((long long)s) - 1]));
         return (double)v;
     }
-    const double *gai = d.g + size_t(a * n + i) * n2;
+    const double *gai = d.sg + at;
     double v = __ldg(&d.h[a * n + i]);
-    for (unsigned long long s = alpha; s; s &= s - 1ull) v = __dadd_rn(v, __ldg(&gai[(__ffsll((long long)s) - 1) * (n + 1)]));
-    for (unsigned long long s = beta; s; s &= s - 1ull) v = __dadd_rn(v, __ldg(&gai[(__ffsll((long long)s) - 1) * (n + 1)]));
-    for (unsigned long long s = same; s; s &= s - 1ull) {
-        const int o = __ffsll((long long)s) - 1;
-        v = __dsub_rn(v, __ldg(&d.g[(size_t(a * n + o) * n + o) * n + i]));
-    }
+    for (unsigned long long s = alpha; s; s &= s - 1ull) v = __dadd_rn(v, __ldg(&gai[__ffsll((long long)s) - 1]));
+    for (unsigned long long s = beta; s; s &= s - 1ull) v = __dadd_rn(v, __ldg(&gai[__ffsll((long long)s) - 1]));
+    for (unsigned long long s = same; s; s &= s - 1ull) v = __dsub_rn(v, __ldg(&gai[n + __ffsll((long long)s) - 1]));
     return v;
 }
 
@@ -139,18 +130,17 @@ __device__ double diagonal_of(const SysDev &d, unsigned long long alpha, unsigne
     for (int s = 0; s < 2; ++s)
         for (unsigned long long x = str[s]; x; x &= x - 1ull) {
             const int p = __ffsll((long long)x) - 1;
-            const double *gpp = d.g + size_t(p * n + p) * n * n;
+            const double *gpp = d.sg + size_t(p * n + p) * 2 * n;
             for (int t = 0; t < 2; ++t)
                 for (unsigned long long y = str[t]; y; y &= y - 1ull)
-                    coul = __dadd_rn(coul, __ldg(&gpp[(__ffsll((long long)y) - 1) * (n + 1)]));
+                    coul = __dadd_rn(coul, __ldg(&gpp[__ffsll((long long)y) - 1]));
         }
     for (int s = 0; s < 2; ++s)
         for (unsigned long long x = str[s]; x; x &= x - 1ull) {
             const int p = __ffsll((long long)x) - 1;
-            for (unsigned long long y = str[s]; y; y &= y - 1ull) {
-                const int q = __ffsll((long long)y) - 1;
-                exch = __dadd_rn(exch, __ldg(&d.g[(size_t(p * n + q) * n + q) * n + p]));
-            }
+            const double *gpq = d.sg + (size_t(p * n + p) * 2 + 1) * n;
+            for (unsigned long long y = str[s]; y; y &= y - 1ull)
+                exch = __dadd_rn(exch, __ldg(&gpq[__ffsll((long long)y) - 1]));
         }
     return __dsub_rn(__dadd_rn(__dadd_rn(d.e_core, one), __dmul_rn(0.5, coul)), __dmul_rn(0.5, exch));
 }
@@ -175,6 +165,17 @@ __global__ void pair_integrals_kernel(const SysDev d, int np, double *W) {
         const size_t x1 = (size_t(a * n + i) * n + b) * n + j, x2 = (size_t(a * n + j) * n + b) * n + i;
         W[t] = a == i || a == j || b == i || b == j ? 0.0
                : d.gf ? (double)__fsub_rn(d.gf[x1], d.gf[x2]) : __dsub_rn(d.g[x1], d.g[x2]);
+    }
+}
+
+__global__ void hop_integrals_kernel(const SysDev d, double *sg, float *sgf) {
+    const int n = d.n;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n * n * n; t += gridDim.x * blockDim.x) {
+        const int ai = t / n, k = t - ai * n, a = ai / n, i = ai - a * n;
+        const size_t x = size_t(ai) * n * n + size_t(k) * (n + 1), y = (size_t(a * n + k) * n + k) * n + i;
+        const size_t o = size_t(ai) * 2 * n + k;
+        sg[o] = d.g[x], sg[o + n] = d.g[y];
+        if (sgf) sgf[o] = d.gf[x], sgf[o + n] = d.gf[y];
     }
 }
 
@@ -402,37 +403,51 @@ __device__ __forceinline__ void string_prefix(unsigned long long s, const unsign
 // entry holds what a row needs of it, so that reading a list is one coalesced stream:
 //   ent1 {pi(beta), beta string's number | i << 25 | s_K(i) << 31, c}
 //   ent2 {pi(beta), pair (i, j) | s_K(i, j) << 31, c}
-// with i (i, j) the orbitals the substring lacks.
+// with i (i, j) the orbitals the substring lacks.  Bound by the counters' atomics: sources
+// lie by alpha string, so whole warps meet at the same substrings, and one lane counts for
+// all that share a string; blockIdx.y is the first electron taken out (2e4 sources of 924
+// strings: 161 us for both passes with an atomic per source and substring).
 __global__ void substring_lists_kernel(const SysDev d, const GatherShape p, const unsigned long long *skey,
                                        const double *sc, const unsigned *sb, long long n, unsigned *cnt1, unsigned *cnt2,
                                        const unsigned long long *off1, const unsigned long long *off2, uint4 *ent1,
                                        uint4 *ent2) {
     extern __shared__ unsigned long long bt[];
     load_binom(d, bt);
-    const int m = d.na;
+    const int m = d.na, x = blockIdx.y, lane = threadIdx.x & 31;
     unsigned P0[kMaxE + 1], P1[kMaxE + 1], P2[kMaxE + 1];
     unsigned char e[kMaxE];
-    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
-        const unsigned long long key = skey[s];
-        string_prefix(unrank_one(key >> p.bb, d.n, m, bt, d.ks), bt, d.ks, P0, P1, P2, e);
-        const unsigned pi = (unsigned)key & p.bmask, id = ent2 ? sb[s] : 0u;
-        const double c = sc[s];
+    for (long long s0 = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); s0 < n; s0 += (long long)gridDim.x * blockDim.x) {
+        const long long s = s0 + lane;
+        const bool in = s < n;
+        const unsigned long long key = skey[in ? s : n - 1];
+        const unsigned row = (unsigned)(key >> p.bb);
+        string_prefix(unrank_one(row, d.n, m, bt, d.ks), bt, d.ks, P0, P1, P2, e);
+        const unsigned pi = (unsigned)key & p.bmask, id = ent2 && in ? sb[s] : 0u;
+        const double c = in ? sc[s] : 0.0;
         const unsigned clo = (unsigned)__double2loint(c), chi = (unsigned)__double2hiint(c);
-        for (int x = 0; x < m; ++x) {
-            const unsigned K = rank_without(P0, P1, P2, m, x, m);
-            if (!ent2) atomicAdd(&cnt1[K], 1u);
-            else
-                ent1[off1[K] + atomicSub(&cnt1[K], 1u) - 1u] =
-                    make_uint4(pi, id | (unsigned)e[x] << 25 | (unsigned)(x & 1) << 31, clo, chi);
-        }
-        for (int x = 0; x < m; ++x)
-            for (int y = x + 1; y < m; ++y) {
-                const unsigned K = rank_without(P0, P1, P2, m, x, y);
-                if (!ent2) atomicAdd(&cnt2[K], 1u);
-                else
-                    ent2[off2[K] + atomicSub(&cnt2[K], 1u) - 1u] = make_uint4(
-                        pi, (unsigned)(e[y] * (e[y] - 1) / 2 + e[x]) | (unsigned)((x + y - 1) & 1) << 31, clo, chi);
+        // the lanes of one alpha string take their places together
+        const unsigned peers = __match_any_sync(kFull, in ? row : kNoKey);
+        const int lead = __ffs((int)peers) - 1;
+        const unsigned many = __popc(peers), mine = __popc(peers & ((1u << lane) - 1u));
+        auto place = [&](unsigned *cnt, unsigned K) {
+            unsigned base = 0u;
+            if (in && lane == lead) {
+                if (!ent2) atomicAdd(&cnt[K], many);
+                else base = atomicSub(&cnt[K], many) - many;
             }
+            return ent2 ? __shfl_sync(kFull, base, lead) + mine : 0u;
+        };
+        {
+            const unsigned K = rank_without(P0, P1, P2, m, x, m), at = place(cnt1, K);
+            if (ent2 && in)
+                ent1[off1[K] + at] = make_uint4(pi, id | (unsigned)e[x] << 25 | (unsigned)(x & 1) << 31, clo, chi);
+        }
+        for (int y = x + 1; y < m; ++y) {
+            const unsigned K = rank_without(P0, P1, P2, m, x, y), at = place(cnt2, K);
+            if (ent2 && in)
+                ent2[off2[K] + at] = make_uint4(
+                    pi, (unsigned)(e[y] * (e[y] - 1) / 2 + e[x]) | (unsigned)((x + y - 1) & 1) << 31, clo, chi);
+        }
     }
 }
 
@@ -478,7 +493,7 @@ __global__ void row_sources_kernel(const SysDev d, const unsigned *rp, const uns
 // sources, weight (elements and the fixed cost of a row), parts of its lists
 __global__ void active_rows_kernel(const SysDev d, const GatherShape p, const unsigned *rp, const unsigned *s1,
                                    const unsigned *s2, const unsigned *act, const unsigned long long *pos,
-                                   unsigned w_fixed, unsigned *row, unsigned long long *str, unsigned long long *aw,
+                                   unsigned w_fixed, unsigned part_work, unsigned *row, unsigned long long *str, unsigned long long *aw,
                                    unsigned *nrec, unsigned *nab, unsigned *np) {
     extern __shared__ unsigned long long bt[];
     load_binom(d, bt);
@@ -496,7 +511,7 @@ __global__ void active_rows_kernel(const SysDev d, const GatherShape p, const un
                 nrec[k] = rec;
                 nab[k] = ab;
                 aw[k] = rec + (unsigned long long)ab * d.sb + (unsigned long long)L * (d.ss_any ? p.nd2 : 0) + w_fixed;
-                np[k] = min((rec + ab + kPartWork - 1) / kPartWork + (rec + ab == 0u), kMaxParts);
+                np[k] = min((rec + ab + part_work - 1) / part_work + (rec + ab == 0u), kMaxParts);
             }
     }
 }
@@ -1380,7 +1395,7 @@ size_t gather_place_sources(char *base, GatherBufs &b, const SysDev &d, const Ga
     b.skey = a.take<unsigned long long>(n);
     b.sc = a.take<double>(n);
     b.sort_ws = a.take<char>(p.bb > kGLog ? sort_pairs_bytes(n) : 0);
-    b.scan_ws = a.take<char>(scan_ws_bytes((long long)std::max({ca, cb, size_t(p.nk1), size_t(p.nk2)}) + 1));
+    b.scan_ws = a.take<char>(4 * scan_ws_bytes((long long)std::max({ca, cb, size_t(p.nk1), size_t(p.nk2)}) + 1));
     b.bflag = a.take<unsigned>(cb);
     b.bid = a.take<unsigned long long>(cb + 1);
     b.s_pi = a.take<unsigned>(n);
@@ -1442,8 +1457,11 @@ bool gather_numbers(const SysDev &d, long long n, unsigned long long nd) {
            (double)n * std::max(d.po_a, d.na) < 4294967296.0;
 }
 
-RowPlanArgs row_plan_args(const GatherShape &p) {
+RowPlanArgs row_plan_args(const SysDev &d, const GatherShape &p, long long n) {
     RowPlanArgs ra{};
+    // a warp makes 128 to 1024 list items: as many warps as the chip holds twice, where there are enough
+    const double items = (double)n * (1.0 + d.sb + 2.0 * d.sa + (d.ss_any ? (double)d.po_a * (d.pv_a + d.sa + d.po_a) : 0.0));
+    ra.part_work = std::min(1024u, std::max(128u, (unsigned)std::min(items / 10000.0, 4096.0) & ~31u));
     // light rows repeat entries about 1.45 times (1.3 to 2): a group fills about 0.55 of its table
     ra.half = (unsigned long long)(0.55 * 1.45 * kGSlots);
     ra.fill = 0.65 * kGSlots;
@@ -1480,6 +1498,12 @@ cudaError_t launch_pair_integrals(const SysDev &d, double *W, cudaStream_t st) {
     if (np <= 0) return cudaSuccess;
     count_launch();
     pair_integrals_kernel<<<grid_for((unsigned long long)np * np, 256), 256, 0, st>>>(d, np, W);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_hop_integrals(const SysDev &d, double *sg, float *sgf, cudaStream_t st) {
+    count_launch();
+    hop_integrals_kernel<<<grid_for((long long)d.n * d.n * d.n, 256), 256, 0, st>>>(d, sg, sgf);
     return cudaGetLastError();
 }
 
@@ -1522,14 +1546,13 @@ cudaError_t gather_tables(const SysDev &d, const GatherShape &p, long long n, un
     tables<<<std::min(nd, 152u * 64u), 256, smem, st>>>(d, p, b.bstr, nd, W, b.t1, b.idx1, b.t2p, b.t2e, b.idx2);
     e = cudaMemsetAsync(b.cnt1, 0, (size_t(p.nk1) + p.nk2) * 4, st);  // cnt1 | cnt2
     if (e != cudaSuccess) return e;
-    count_launch();
-    substring_lists_kernel<<<grid_for(n, 128), 128, bts, st>>>(d, p, b.skey, b.sc, b.s_b, n, b.cnt1, b.cnt2, nullptr,
+    const dim3 sub_grid(grid_for(n, 128), (unsigned)d.na);
+    if (d.na) count_launch(), substring_lists_kernel<<<sub_grid, 128, bts, st>>>(d, p, b.skey, b.sc, b.s_b, n, b.cnt1, b.cnt2, nullptr,
                                                               nullptr, nullptr, nullptr);
     e = exclusive_scan(static_cast<const unsigned *>(b.cnt1), p.nk1, b.off1, b.scan_ws, st);
     if (e == cudaSuccess) e = exclusive_scan(static_cast<const unsigned *>(b.cnt2), p.nk2, b.off2, b.scan_ws, st);
     if (e != cudaSuccess) return e;
-    count_launch();
-    substring_lists_kernel<<<grid_for(n, 128), 128, bts, st>>>(d, p, b.skey, b.sc, b.s_b, n, b.cnt1, b.cnt2, b.off1,
+    if (d.na) count_launch(), substring_lists_kernel<<<sub_grid, 128, bts, st>>>(d, p, b.skey, b.sc, b.s_b, n, b.cnt1, b.cnt2, b.off1,
                                                               b.off2, b.ent1, b.ent2);
     const unsigned long long chunks = (d.ca + kRowChunk - 1) / kRowChunk;
     count_launch();
@@ -1539,17 +1562,14 @@ cudaError_t gather_tables(const SysDev &d, const GatherShape &p, long long n, un
     if (e == cudaSuccess) e = cudaMemsetAsync(b.aw, 0, size_t(d.ca) * 24, st);  // aw | nrec | nab | np | nu
     if (e != cudaSuccess) return e;
     count_launch();
-    active_rows_kernel<<<grid_for(chunks, 128), 128, bts, st>>>(d, p, rp, b.s1, b.s2, b.act, b.apos, ra.w_fixed,
+    active_rows_kernel<<<grid_for(chunks, 128), 128, bts, st>>>(d, p, rp, b.s1, b.s2, b.act, b.apos, ra.w_fixed, ra.part_work,
                                                                b.act_row, b.act_str, b.aw, b.nrec, b.nab, b.np);
     e = exclusive_scan(static_cast<const unsigned long long *>(b.aw), (long long)d.ca, b.wpre, b.scan_ws, st);
     if (e != cudaSuccess) return e;
     count_launch();
     row_units_kernel<<<grid_for(d.ca, 256), 256, 0, st>>>(row_plan(d, p, b, ra), b.aw, b.wpre, b.apos + d.ca, b.nu);
-    e = exclusive_scan(static_cast<const unsigned *>(b.nu), (long long)d.ca, b.uoff, b.scan_ws, st);
-    if (e == cudaSuccess) e = exclusive_scan(static_cast<const unsigned *>(b.np), (long long)d.ca, b.poff, b.scan_ws, st);
-    if (e == cudaSuccess) e = exclusive_scan(static_cast<const unsigned *>(b.nrec), (long long)d.ca, b.rec_off, b.scan_ws, st);
-    if (e == cudaSuccess) e = exclusive_scan(static_cast<const unsigned *>(b.nab), (long long)d.ca, b.ab_off, b.scan_ws, st);
-    return e;
+    unsigned long long *const out[4] = {b.rec_off, b.ab_off, b.poff, b.uoff};  // nrec | nab | np | nu
+    return exclusive_scan4(b.nrec, (long long)d.ca, out, b.scan_ws, st);
 }
 
 cudaError_t gather_lists(const SysDev &d, const GatherShape &p, unsigned long long n_act, unsigned long long n_parts,

@@ -139,6 +139,11 @@ struct SysDev {
     // for every (b, j); bound_ss[i*n+j] >= |(ai|bj) - (aj|bi)| for every (a, b)
     const double *bound_ab;
     const double *bound_ss;
+    // the integrals of a hop i -> a and of the diagonal, over the other orbital k, side by
+    // side: sg[((a n + i) 2 + 0) n + k] = (ai|kk), [.. + 1 ..] = (ak|ki) (a list's single
+    // touches a few lines of L2 instead of one per electron)
+    const double *sg;
+    const float *sgf;    // float32 copy (SFCI_FP32_ELEMENTS), else null
     int ab_any;          // 1: some (ai|bj) with a != i is non-zero (else every opposite-spin double is zero)
     int ss_any;          // 1: some bound_ss entry is non-zero (else every same-spin double is zero)
     double hbound;       // |<D'|H|D>| <= hbound for every pair of determinants
@@ -542,6 +547,9 @@ cudaError_t exclusive_scan(const unsigned *in, long long m, unsigned long long *
                            cudaStream_t st);
 cudaError_t exclusive_scan(const unsigned long long *in, long long m, unsigned long long *out, void *ws,
                            cudaStream_t st);
+// four arrays of m counts, one behind the other, in the same launches (ws: 4 scan_ws_bytes(m))
+cudaError_t exclusive_scan4(const unsigned *in, long long m, unsigned long long *const out[4], void *ws,
+                            cudaStream_t st);
 cudaError_t sort_overflow(const Buckets &bk, const unsigned *count, unsigned lo, unsigned nb,
                           const Slot *ovf, const unsigned long long *ovf_n, long long ovf_cap,
                           unsigned *tmp_counts, unsigned long long *off, void *scan_ws, Slot *out,
@@ -584,6 +592,7 @@ struct GatherShape {
 struct RowPlanArgs {
     unsigned long long half;  // a row of more weight is heavy (units of its own); a group weighs at most 2 half
     double fill;              // distinct entries a class should hold
+    unsigned part_work;       // items of a row's lists that one warp makes
     unsigned w_fixed;         // weight of a row besides its elements (a group holds at most 2 half / w_fixed rows)
 };
 // a group of light rows or one class of a heavy row, as ranges of its lists
@@ -709,11 +718,12 @@ size_t gather_place_sources(char *base, GatherBufs &b, const SysDev &d, const Ga
 size_t gather_place_tables(char *base, GatherBufs &b, const SysDev &d, const GatherShape &p, size_t nd, long long n);
 size_t gather_place_lists(char *base, GatherBufs &b, const GatherShape &p, const GatherCounts &n);
 bool gather_numbers(const SysDev &d, long long n, unsigned long long nd);  // false: positions outgrow their fields
-RowPlanArgs row_plan_args(const GatherShape &p);
+RowPlanArgs row_plan_args(const SysDev &d, const GatherShape &p, long long n);
 cudaError_t gather_counts(const SysDev &d, const GatherBufs &b, GatherCounts *n, cudaStream_t st);  // synchronises
 void gather_inputs(GatherArgs &A, const SysDev &d, const GatherShape &p, const GatherBufs &b, const GatherCounts &n,
                    const unsigned *rp);
 cudaError_t launch_pair_integrals(const SysDev &d, double *W, cudaStream_t st);
+cudaError_t launch_hop_integrals(const SysDev &d, double *sg, float *sgf, cudaStream_t st);
 cudaError_t launch_row_pointers(const SysDev &d, const unsigned long long *rank, long long n, unsigned *rp,
                                 cudaStream_t st);
 // sources in run order, beta strings numbered (count in bid[cb]), runs in words[0]

@@ -905,7 +905,7 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     if (!gather_numbers(d, n_in, nd) || need + (double)size_b > budget) return SFCI_OK;
     if ((r = ensure(z->gb, size_b, z->st, "row gather tables", 1.1))) return r;
     gather_place_tables(static_cast<char *>(z->gb.p), b, d, gs, nd, n_in);
-    const RowPlanArgs ra = row_plan_args(gs);
+    const RowPlanArgs ra = row_plan_args(d, gs, n_in);
     SFCI_CUDA(gather_tables(d, gs, n_in, (unsigned)nd, z->sys->pair_int, rp, b, ra, z->st));
     GatherCounts gn{};
     SFCI_CUDA(gather_counts(d, b, &gn, z->st));

@@ -54,10 +54,16 @@ __device__ __forceinline__ unsigned smem_slot(unsigned long long key, int log2B)
 // ------------------------------------------------------------- scan
 
 // exclusive scan of unsigned 32- or 64-bit counts into 64-bit offsets, m
-// entries, out[m] = total; three kernels (block sums, scan of sums, block scans)
+// entries, out[m] = total; three kernels (block sums, scan of sums, block scans).
+// blockIdx.y: which of up to four arrays, in one behind the other.
+struct ScanOut {
+    unsigned long long *p[4];
+};
+
 template <typename T>
 __global__ void scan_sums_kernel(const T *in, long long m, unsigned long long *bsum) {
     __shared__ unsigned long long w[32];
+    in += blockIdx.y * m, bsum += blockIdx.y * (long long)gridDim.x;
     const long long i = (long long)blockIdx.x * 1024 + threadIdx.x;
     unsigned long long v = i < m ? in[i] : 0;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
@@ -73,8 +79,10 @@ __global__ void scan_sums_kernel(const T *in, long long m, unsigned long long *b
 // up to kSmallScan entries: one CTA, one launch
 constexpr long long kSmallScan = 8192;
 template <typename T>
-__global__ void scan_small_kernel(const T *in, int m, unsigned long long *out) {
+__global__ void scan_small_kernel(const T *in, int m, ScanOut outs) {
     __shared__ unsigned long long w[32];
+    unsigned long long *out = outs.p[blockIdx.y];
+    in += blockIdx.y * (long long)m;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     unsigned long long carry = 0;
     for (int b0 = 0; b0 < m; b0 += 1024) {
@@ -103,6 +111,7 @@ __global__ void scan_small_kernel(const T *in, int m, unsigned long long *out) {
 __global__ void scan_top_kernel(unsigned long long *bsum, long long nb) {
     // one block: exclusive scan of nb block sums in place
     __shared__ unsigned long long carry, w[32];
+    bsum += blockIdx.y * nb;
     if (threadIdx.x == 0) carry = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -136,8 +145,10 @@ __global__ void scan_top_kernel(unsigned long long *bsum, long long nb) {
 
 template <typename T>
 __global__ void scan_block_kernel(const T *in, long long m, const unsigned long long *bsum,
-                                  unsigned long long *out) {
+                                  ScanOut outs) {
     __shared__ unsigned long long w[32];
+    unsigned long long *out = outs.p[blockIdx.y];
+    in += blockIdx.y * m, bsum += blockIdx.y * (long long)gridDim.x;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const long long i = (long long)blockIdx.x * 1024 + threadIdx.x;
     const unsigned long long v = i < m ? in[i] : 0;
@@ -608,33 +619,44 @@ size_t scan_ws_bytes(long long m) {
 
 namespace {
 template <typename T>
-cudaError_t exclusive_scan_t(const T *in, long long m, unsigned long long *out, void *ws, cudaStream_t st) {
-    if (m <= 0) return cudaMemsetAsync(out, 0, 8, st);
+cudaError_t exclusive_scan_t(const T *in, long long m, ScanOut out, unsigned k, void *ws, cudaStream_t st) {
+    if (m <= 0) {
+        for (unsigned q = 0; q < k; ++q) {
+            const cudaError_t e = cudaMemsetAsync(out.p[q], 0, 8, st);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
     if (m <= kSmallScan) {
         count_launch();
-        scan_small_kernel<<<1, 1024, 0, st>>>(in, (int)m, out);
+        scan_small_kernel<<<dim3(1, k), 1024, 0, st>>>(in, (int)m, out);
         return cudaGetLastError();
     }
     const long long nb = (m + 1023) / 1024;
     unsigned long long *bsum = static_cast<unsigned long long *>(ws);
     count_launch();
-    scan_sums_kernel<<<(unsigned)nb, 1024, 0, st>>>(in, m, bsum);
+    scan_sums_kernel<<<dim3((unsigned)nb, k), 1024, 0, st>>>(in, m, bsum);
     count_launch();
-    scan_top_kernel<<<1, 1024, 0, st>>>(bsum, nb);
+    scan_top_kernel<<<dim3(1, k), 1024, 0, st>>>(bsum, nb);
     count_launch();
-    scan_block_kernel<<<(unsigned)nb, 1024, 0, st>>>(in, m, bsum, out);
+    scan_block_kernel<<<dim3((unsigned)nb, k), 1024, 0, st>>>(in, m, bsum, out);
     return cudaGetLastError();
 }
 }  // namespace
 
 cudaError_t exclusive_scan(const unsigned *in, long long m, unsigned long long *out, void *ws,
                            cudaStream_t st) {
-    return exclusive_scan_t(in, m, out, ws, st);
+    return exclusive_scan_t(in, m, ScanOut{{out}}, 1, ws, st);
 }
 
 cudaError_t exclusive_scan(const unsigned long long *in, long long m, unsigned long long *out, void *ws,
                            cudaStream_t st) {
-    return exclusive_scan_t(in, m, out, ws, st);
+    return exclusive_scan_t(in, m, ScanOut{{out}}, 1, ws, st);
+}
+
+cudaError_t exclusive_scan4(const unsigned *in, long long m, unsigned long long *const out[4], void *ws,
+                            cudaStream_t st) {
+    return exclusive_scan_t(in, m, ScanOut{{out[0], out[1], out[2], out[3]}}, 4, ws, st);
 }
 
 cudaError_t sort_overflow(const Buckets &bk, const unsigned *count, unsigned lo, unsigned nb,

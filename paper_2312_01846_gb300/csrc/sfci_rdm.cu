@@ -350,7 +350,9 @@ __global__ void __launch_bounds__(kT) rows_strings_kernel(RowArgs A) {
     unsigned long long *bt = reinterpret_cast<unsigned long long *>(sm);
     for (int i = threadIdx.x; i < (d.n + 1) * d.ks; i += blockDim.x) bt[i] = d.binom[i];
     __syncthreads();
+    __shared__ unsigned char lists[kT / 32][128];
     const int lane = threadIdx.x & 31;
+    unsigned char *occ = lists[threadIdx.x >> 5], *vir = occ + 64;
     const unsigned nd = (unsigned)A.b_id[d.cb], runs = (unsigned)A.run_of[A.n];
     for (unsigned w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nd + runs; w += (gridDim.x * blockDim.x) >> 5) {
         if (w >= nd) {
@@ -365,21 +367,18 @@ __global__ void __launch_bounds__(kT) rows_strings_kernel(RowArgs A) {
         }
         const unsigned long long str = string_unrank_warp(A.id_b[w], d.n, d.nb, bt, d.ks);
         if (lane == 0) A.bstr[w] = str;
-        // lane p: whether orbital p is occupied; a hop per (occupied, empty) pair, by their positions
-        int x = 0;
-        for (unsigned long long o = str; o; o &= o - 1ull) {
-            const int j = __ffsll((long long)o) - 1;
-            int y = 0;
-            for (int b = 0; b < d.n; ++b) {
-                if ((str >> b) & 1ull) continue;
-                if (((x * d.vb + y) & 31) == lane) {
-                    const unsigned sg = parity64(str & between_mask(j, b));
-                    A.hops[(size_t)w * d.sb + x * d.vb + y] =
-                        make_uint2((unsigned)string_rank(str ^ (1ull << j) ^ (1ull << b), bt, d.ks), (unsigned)(b * d.n + j) | sg << 31);
-                }
-                ++y;
-            }
-            ++x;
+        __syncwarp();
+        for (int p = lane; p < d.n; p += 32) {
+            const int below = __popcll(str & ((1ull << p) - 1ull));
+            if ((str >> p) & 1ull) occ[below] = (unsigned char)p;
+            else vir[p - below] = (unsigned char)p;
+        }
+        __syncwarp();
+        for (int x = lane; x < d.sb; x += 32) {
+            const int j = occ[x / d.vb], b = vir[x % d.vb];
+            const unsigned sg = parity64(str & between_mask(j, b));
+            A.hops[(size_t)w * d.sb + x] =
+                make_uint2((unsigned)string_rank(str ^ (1ull << j) ^ (1ull << b), bt, d.ks), (unsigned)(b * d.n + j) | sg << 31);
         }
     }
 }
