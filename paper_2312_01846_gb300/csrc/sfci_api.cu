@@ -364,7 +364,8 @@ namespace sfci {
 namespace {
 
 // sigma by target rows in the bytes [w, w + room) of the workspace, for a validated
-// input; unsorted entries leave to out_rank / out_coef, their number to *n_out and L.ndev.
+// input; unsorted entries leave to out_rank / out_coef, their number to *n_out (on the device
+// at *n_dev).
 // *done = false: its lists do not fit there (or the system is outside its limits).
 //
 // The table path keeps every entry in a global hash table (32 bytes a slot, two to four
@@ -373,7 +374,7 @@ namespace {
 // 2.82 ms; by rows 5.99 ms and 1.10 ms, of which sorting the entries is the largest part.
 sfci_status sigma_rows(const sfci_system *s, const unsigned long long *rank, const double *coef, long long n, double eps,
                        int fix_shift, unsigned long long *out_rank, double *out_coef, long long out_cap, char *w,
-                       size_t room, unsigned long long *ndev, unsigned long long *n_out, bool *done, cudaStream_t st) {
+                       size_t room, const unsigned long long **n_dev, unsigned long long *n_out, bool *done, cudaStream_t st) {
     *done = false;
     const SysDev &d = s->d;
     GatherShape gs{};
@@ -385,7 +386,7 @@ sfci_status sigma_rows(const sfci_system *s, const unsigned long long *rank, con
     if (at > room) return SFCI_OK;
     // head: counters of the gather kernel (zeroed), rows' weights seen so far (none)
     struct Words {
-        unsigned long long tau, mark, live, nonzero, read;
+        unsigned long long out, tau, mark, live, nonzero, read;
         double sumsq;
         unsigned queue;
         int lock, status;
@@ -397,7 +398,6 @@ sfci_status sigma_rows(const sfci_system *s, const unsigned long long *rank, con
     gather_place_sources(w + head + rps, b, d, gs, n);
     SFCI_CUDA(cudaMemsetAsync(w, 0, head, st));
     SFCI_CUDA(cudaMemsetAsync(&words->mark, 0xff, 8, st));
-    SFCI_CUDA(cudaMemsetAsync(ndev, 0, 8, st));
     SFCI_CUDA(launch_row_pointers(d, rank, n, rp, st));
     SFCI_CUDA(gather_sources(d, gs, rank, coef, n, b, st));
     unsigned long long nd = 0;
@@ -419,18 +419,19 @@ sfci_status sigma_rows(const sfci_system *s, const unsigned long long *rank, con
     A.all = 1;
     A.ja = A.jb = -1;
     A.eps = eps;
-    A.out_key = out_rank, A.out_val = out_coef, A.out_cap = out_cap, A.out_n = ndev;
+    A.out_key = out_rank, A.out_val = out_coef, A.out_cap = out_cap, A.out_n = &words->out;
     A.tau_bits = &words->tau, A.mark = &words->mark, A.lock = &words->lock;
     A.fix_shift = fix_shift;
     A.sumsq = &words->sumsq, A.n_live = &words->live, A.n_nonzero = &words->nonzero, A.n_read = &words->read;
     A.queue = &words->queue, A.status = &words->status;
     SFCI_CUDA(launch_gather(A, st));
-    int hs = 0;
-    SFCI_CUDA(cudaMemcpyAsync(&hs, &words->status, 4, cudaMemcpyDeviceToHost, st));
-    SFCI_CUDA(cudaMemcpyAsync(n_out, ndev, 8, cudaMemcpyDeviceToHost, st));
+    Words hw{};
+    SFCI_CUDA(cudaMemcpyAsync(&hw, words, sizeof(hw), cudaMemcpyDeviceToHost, st));
     SFCI_CUDA(cudaStreamSynchronize(st));
     *done = true;
-    if (hs & 32) {
+    *n_out = hw.out;
+    *n_dev = &words->out;
+    if (hw.status & 32) {
         *n_out = 0;
         return invalid("an element fell outside the fixed-point range of the exact sums");
     }
@@ -472,10 +473,15 @@ sfci_status sfci_sigma(const sfci_system *s, const uint64_t *in_rank, const doub
     // exact sums: units 2^-S with no entry beyond (n_conn + 1) hbound max|c| < 2^125 units
     unsigned long long mbits = 0;
     SFCI_CUDA(max_abs_bits(in_coef, n_in, reinterpret_cast<unsigned long long *>(w + L.maxabs), st));
-    SFCI_CUDA(cudaMemcpyAsync(&mbits, w + L.maxabs, 8, cudaMemcpyDeviceToHost, st));
-    int hflag = 0;
-    SFCI_CUDA(cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
+    // (flag and maxabs lie two pieces of the layout apart: one copy reads both)
+    char head[1024];
+    const size_t span = L.maxabs + 8 - L.flag;
+    if (L.maxabs < L.flag || span > sizeof(head)) return invalid("workspace layout");
+    SFCI_CUDA(cudaMemcpyAsync(head, flag, span, cudaMemcpyDeviceToHost, st));
     SFCI_CUDA(cudaStreamSynchronize(st));
+    int hflag = 0;
+    std::memcpy(&hflag, head, sizeof(int));
+    std::memcpy(&mbits, head + (L.maxabs - L.flag), 8);
     double cmax = 0.0;
     std::memcpy(&cmax, &mbits, 8);
     if (!std::isfinite(cmax)) return invalid("non-finite input coefficients");
@@ -490,9 +496,10 @@ sfci_status sfci_sigma(const sfci_system *s, const uint64_t *in_rank, const doub
     const double eps = eps_screen > 0.0 ? eps_screen : 0.0;
     unsigned long long hn = 0, hcount = 0;
     bool by_rows = false;
+    const unsigned long long *n_rows = nullptr;
     if (n_in > 0) {
         const sfci_status r = sigma_rows(s, ir, in_coef, n_in, eps, t.fix_shift, reinterpret_cast<unsigned long long *>(out_rank),
-                                         out_coef, out_cap, w, L.status, ndev, &hn, &by_rows, st);
+                                         out_coef, out_cap, w, L.status, &n_rows, &hn, &by_rows, st);
         if (r != SFCI_OK) {
             *n_out = 0;
             return r;
@@ -504,7 +511,7 @@ sfci_status sfci_sigma(const sfci_system *s, const uint64_t *in_rank, const doub
             set_error("sigma has more entries than out_cap");
             return SFCI_E_CAPACITY;
         }
-        SFCI_CUDA(sort_pairs(reinterpret_cast<unsigned long long *>(out_rank), out_coef, (long long)hn, ndev,
+        SFCI_CUDA(sort_pairs(reinterpret_cast<unsigned long long *>(out_rank), out_coef, (long long)hn, n_rows,
                              key_bits(s->d.dim), w + L.sortws, st));
         SFCI_CUDA(cudaStreamSynchronize(st));
         return SFCI_OK;

@@ -548,6 +548,8 @@ cudaError_t exclusive_scan(const unsigned *in, long long m, unsigned long long *
 cudaError_t exclusive_scan(const unsigned long long *in, long long m, unsigned long long *out, void *ws,
                            cudaStream_t st);
 // four arrays of m counts, one behind the other, in the same launches (ws: 4 scan_ws_bytes(m))
+// sig[j][0..n[j]) = 0
+cudaError_t zero_vectors(double *const *sig, const long long *n, int nvec, cudaStream_t st);
 cudaError_t exclusive_scan4(const unsigned *in, long long m, unsigned long long *const out[4], void *ws,
                             cudaStream_t st);
 cudaError_t sort_overflow(const Buckets &bk, const unsigned *count, unsigned lo, unsigned nb,
@@ -608,7 +610,7 @@ struct GatherUnit {
 static_assert(sizeof(GatherUnit) == 64, "read as four 16-byte words");
 constexpr int kSeenBins = 128;
 struct GatherBufs {
-    unsigned long long *words;  // [8]: runs, n
+    unsigned long long *words;  // [8]: runs, n, rows summed in classes, GatherCounts
     unsigned long long *skey;   // [n] row << bb | pi(beta), runs in the order of pi
     double *sc;                 // [n]
     void *sort_ws, *scan_ws;

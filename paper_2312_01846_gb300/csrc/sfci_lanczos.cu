@@ -179,7 +179,19 @@ void log_step(const sfci_step_info &s) {
 
 using namespace sfci;
 
+// What the host reads back of a step.  Page-locked: a copy into it takes 3 us of the
+// stream, one into ordinary memory 11 us of the host's, and a step reads some twenty words.
+struct StepWords {
+    unsigned long long w[12];            // the words at sfci_lanczos::outn
+    double TS[2 * sfci::kMaxVec];
+    sfci::SplitResult split;
+    sfci::GatherCounts counts;
+    unsigned long long nd, runs, n, total;
+    double sumsq;
+};
+
 struct sfci_lanczos {
+    StepWords *host = nullptr;
     const sfci_system *sys = nullptr;
     sfci_params p{};
     cudaStream_t st = nullptr;
@@ -272,6 +284,7 @@ void destroy_lz(sfci_lanczos *z) {
                     &z->pth, &z->pbstart, &z->pcap, &z->pq, &z->start4, &z->ga, &z->gb, &z->gc, &z->vrp, &z->seen})
         cudaFree(b->p);
     cudaFree(z->words);
+    cudaFreeHost(z->host);
     for (int j = 0; j < kMaxVec; ++j) cudaFree(z->sigw[j]);
     for (auto &e : z->ev)
         if (e) cudaEventDestroy(e);
@@ -317,12 +330,13 @@ sfci_status table_topk(sfci_lanczos *z, unsigned long long cap, int dst, double 
                           z->scratch + z->off_sel, z->sel_bytes, z->st));
     SFCI_CUDA(sort_normalize(z->wr[dst], z->wc[dst], z->nkeep, z->ndev, key_bits(z->sys->d.dim),
                              z->scratch + z->off_sort, z->scratch + z->off_norm, z->st));
-    unsigned long long hn = 0;
-    SFCI_CUDA(cudaMemcpyAsync(&hn, z->ndev, sizeof(hn), cudaMemcpyDeviceToHost, z->st));
-    if (sumsq_host) SFCI_CUDA(cudaMemcpyAsync(sumsq_host, z->sumsq, 8, cudaMemcpyDeviceToHost, z->st));
-    if (total_host) SFCI_CUDA(cudaMemcpyAsync(total_host, z->total, 8, cudaMemcpyDeviceToHost, z->st));
+    SFCI_CUDA(cudaMemcpyAsync(&z->host->n, z->ndev, 8, cudaMemcpyDeviceToHost, z->st));
+    if (sumsq_host) SFCI_CUDA(cudaMemcpyAsync(&z->host->sumsq, z->sumsq, 8, cudaMemcpyDeviceToHost, z->st));
+    if (total_host) SFCI_CUDA(cudaMemcpyAsync(&z->host->total, z->total, 8, cudaMemcpyDeviceToHost, z->st));
     SFCI_CUDA(cudaStreamSynchronize(z->st));
-    z->wn[dst] = (long long)std::min<unsigned long long>(hn, (unsigned long long)z->nkeep);
+    if (sumsq_host) *sumsq_host = z->host->sumsq;
+    if (total_host) *total_host = z->host->total;
+    z->wn[dst] = (long long)std::min<unsigned long long>(z->host->n, (unsigned long long)z->nkeep);
     return SFCI_OK;
 }
 
@@ -876,9 +890,17 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     const size_t vrp_bytes = size_t(z->NL) * (size_t(d.ca) + 1) * 4;
     const double held = (double)z->ga.bytes + z->gb.bytes + z->gc.bytes + z->vrp.bytes + z->sig_key.bytes +
                         z->sig_val.bytes + z->belem.bytes + z->bovf.bytes + z->bovf_sorted.bytes;
-    const double budget = sigma_budget(z, held);
+    // (the driver is asked for the free memory only when a buffer has to grow)
+    double budget = -1.0;
+    const auto fits = [&](bool have, double bytes) {
+        if (have) return true;
+        if (budget < 0.0) budget = sigma_budget(z, held);
+        return bytes <= budget;
+    };
+    const bool have_a = z->ga.bytes >= size_a && z->vrp.bytes >= vrp_bytes &&
+                        (double)std::min(z->sig_key.bytes, z->sig_val.bytes) >= 8.0 * sig_need;
     double need = (double)size_a + (double)vrp_bytes + 16.0 * sig_need;
-    if (need > budget) return SFCI_OK;
+    if (!fits(have_a, need)) return SFCI_OK;
     SFCI_CUDA(cudaEventRecord(z->evp[0], z->st));
     if ((r = ensure(z->ga, size_a, z->st, "row gather arrays", 1.25))) return r;
     if (z->vrp.bytes < vrp_bytes) z->vrp_ok.assign(z->NL, 0);
@@ -897,28 +919,28 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     }
     b.seen = P<unsigned long long>(z->seen);
     SFCI_CUDA(gather_sources(d, gs, z->wr[i], z->wc[i], n_in, b, z->st));
-    unsigned long long nd = 0, runs = 0;
-    SFCI_CUDA(cudaMemcpyAsync(&nd, b.bid + d.cb, 8, cudaMemcpyDeviceToHost, z->st));
-    SFCI_CUDA(cudaMemcpyAsync(&runs, b.words, 8, cudaMemcpyDeviceToHost, z->st));
+    SFCI_CUDA(cudaMemcpyAsync(&z->host->nd, b.bid + d.cb, 8, cudaMemcpyDeviceToHost, z->st));
+    SFCI_CUDA(cudaMemcpyAsync(&z->host->runs, b.words, 8, cudaMemcpyDeviceToHost, z->st));
     SFCI_CUDA(cudaStreamSynchronize(z->st));
+    const unsigned long long nd = z->host->nd, runs = z->host->runs;
     const size_t size_b = gather_place_tables(nullptr, b, d, gs, nd, n_in);
-    if (!gather_numbers(d, n_in, nd) || need + (double)size_b > budget) return SFCI_OK;
+    const bool have_b = have_a && z->gb.bytes >= size_b;
+    if (!gather_numbers(d, n_in, nd) || !fits(have_b, need + (double)size_b)) return SFCI_OK;
     if ((r = ensure(z->gb, size_b, z->st, "row gather tables", 1.1))) return r;
     gather_place_tables(static_cast<char *>(z->gb.p), b, d, gs, nd, n_in);
     const RowPlanArgs ra = row_plan_args(d, gs, n_in);
     SFCI_CUDA(gather_tables(d, gs, n_in, (unsigned)nd, z->sys->pair_int, rp, b, ra, z->st));
-    GatherCounts gn{};
-    SFCI_CUDA(gather_counts(d, b, &gn, z->st));
+    SFCI_CUDA(gather_counts(d, b, &z->host->counts, z->st));
+    const GatherCounts gn = z->host->counts;
     if (!gn.fit()) return SFCI_OK;
     const size_t size_c = gather_place_lists(nullptr, b, gs, gn);
-    if (need + (double)size_b + (double)size_c > budget) return SFCI_OK;
+    if (!fits(have_b && z->gc.bytes >= size_c, need + (double)size_b + (double)size_c)) return SFCI_OK;
     if ((r = ensure(z->gc, size_c, z->st, "row gather lists", 1.1))) return r;
     gather_place_lists(static_cast<char *>(z->gc.p), b, gs, gn);
     SFCI_CUDA(gather_lists(d, gs, gn.act, gn.parts, z->sys->pair_int, rp, b, ra, z->st));
-    for (int j = 0; j <= i; ++j) {
+    for (int j = 0; j <= i; ++j)
         if (!z->sigw[j]) SFCI_CUDA(cudaMalloc(&z->sigw[j], size_t(z->nkeep) * 8));
-        if (z->wn[j] > 0) SFCI_CUDA(cudaMemsetAsync(z->sigw[j], 0, size_t(z->wn[j]) * 8, z->st));  // rows without elements
-    }
+    SFCI_CUDA(zero_vectors(z->sigw, z->wn.data(), i + 1, z->st));  // rows without elements
     int fix_shift = (int)std::floor(125.0 - std::log2(std::max(1e-300, (double)(d.n_conn + 1) * d.hbound)));
     fix_shift = std::max(-900, std::min(1000, fix_shift));
     const double tau_start = *tau_io;
@@ -959,17 +981,15 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
         }
         SFCI_CUDA(launch_gather(A, z->st));
         SFCI_CUDA(cudaEventRecord(z->evp[2], z->st));
-        int hs = 0;
-        unsigned long long ho = 0, hl = 0, hz = 0, tb = 0, hr = 0;
-        double hq = 0.0;
-        SFCI_CUDA(cudaMemcpyAsync(&hs, z->mstatus, 4, cudaMemcpyDeviceToHost, z->st));
-        SFCI_CUDA(cudaMemcpyAsync(&ho, z->outn, 8, cudaMemcpyDeviceToHost, z->st));
-        SFCI_CUDA(cudaMemcpyAsync(&hl, z->mlive, 8, cudaMemcpyDeviceToHost, z->st));
-        SFCI_CUDA(cudaMemcpyAsync(&hz, z->nnz, 8, cudaMemcpyDeviceToHost, z->st));
-        SFCI_CUDA(cudaMemcpyAsync(&hq, z->msumsq, 8, cudaMemcpyDeviceToHost, z->st));
-        SFCI_CUDA(cudaMemcpyAsync(&tb, z->tau_w, 8, cudaMemcpyDeviceToHost, z->st));
-        SFCI_CUDA(cudaMemcpyAsync(&hr, z->nread_w, 8, cudaMemcpyDeviceToHost, z->st));
+        SFCI_CUDA(cudaMemcpyAsync(z->host->w, z->outn, sizeof(z->host->w), cudaMemcpyDeviceToHost, z->st));
         SFCI_CUDA(cudaStreamSynchronize(z->st));
+        // (a word's place in the block is its distance from outn)
+        const auto word = [&](const void *p) { return z->host->w[(static_cast<const char *>(p) - reinterpret_cast<char *>(z->outn)) / 8]; };
+        const int hs = (int)(word(z->queue) >> 32);  // mstatus, behind the queue's 32 bits
+        const unsigned long long ho = word(z->outn), hl = word(z->mlive), hz = word(z->nnz), hr = word(z->nread_w);
+        const unsigned long long tb = word(z->tau_w), qb = word(z->msumsq);
+        double hq = 0.0;
+        std::memcpy(&hq, &qb, 8);
         std::memcpy(&tau, &tb, 8);
         if (hs & 32) {  // an element beyond the fixed-point range (an input not normalised): coarser units
             fix_shift -= 16;
@@ -996,8 +1016,7 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
         z->alpha_runs = runs;
         z->nb_log2 = 0;
         while ((1ull << z->nb_log2) < gn.units) ++z->nb_log2;
-        z->budget_gb = budget / 1e9;
-        z->free_gb = (budget - held) / 1e9, z->held_gb = held / 1e9;
+        if (budget >= 0.0) z->budget_gb = budget / 1e9, z->free_gb = (budget - held) / 1e9, z->held_gb = held / 1e9;
         z->regions_gb = E * sizeof(Slot) / 1e9;  // what the elements would take as records
         z->ms_alloc = 0.0;
         *done = true;
@@ -1014,10 +1033,9 @@ sfci_status load_vector(sfci_lanczos *z, const uint64_t *rank, const double *coe
                           z->scratch + z->off_sel, z->sel_bytes, z->st));
     SFCI_CUDA(sort_normalize(z->wr[0], z->wc[0], z->nkeep, z->ndev, 64, z->scratch + z->off_sort,
                              z->scratch + z->off_norm, z->st));
-    unsigned long long hn = 0;
-    SFCI_CUDA(cudaMemcpyAsync(&hn, z->ndev, 8, cudaMemcpyDeviceToHost, z->st));
+    SFCI_CUDA(cudaMemcpyAsync(&z->host->n, z->ndev, 8, cudaMemcpyDeviceToHost, z->st));
     SFCI_CUDA(cudaStreamSynchronize(z->st));
-    z->wn[0] = (long long)std::min<unsigned long long>(hn, (unsigned long long)z->nkeep);
+    z->wn[0] = (long long)std::min<unsigned long long>(z->host->n, (unsigned long long)z->nkeep);
     std::fill(z->vrp_ok.begin(), z->vrp_ok.end(), 0);
     z->idx = 0;
     z->have_prev = false;
@@ -1122,6 +1140,7 @@ sfci_status lanczos_create(sfci_lanczos **out, const sfci_system *sys, const sfc
     for (int k = 0; k < 4 && e == cudaSuccess; ++k) e = cudaEventCreate(&z->ev[k]);
     for (int k = 0; k < 4 && e == cudaSuccess; ++k) e = cudaEventCreate(&z->evp[k]);
     if (e == cudaSuccess) e = cudaMalloc(&z->words, kHistBins * 8 + 1024);
+    if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void **>(&z->host), sizeof(StepWords));
     if (e == cudaSuccess) {
         z->hist = reinterpret_cast<unsigned long long *>(z->words);
         char *w = z->words + kHistBins * 8;
@@ -1210,6 +1229,7 @@ sfci_status sfci_lanczos_step(sfci_lanczos *z, sfci_step_info *info) {
     }
     std::vector<VecRef> vr(i + 1);
     for (int j = 0; j <= i; ++j) vr[j] = VecRef{z->wr[j], z->wc[j], z->wn[j]};
+    bool truncated = false;
     for (int attempt = 0;; ++attempt) {
         // ---- sigma_i = H w_i, bucketed merge with the probes of w_0..w_i
         unsigned long long n_stream = 0, n_live = 0, n_nz = 0;
@@ -1245,9 +1265,10 @@ sfci_status sfci_lanczos_step(sfci_lanczos *z, sfci_step_info *info) {
         SFCI_CUDA(aligned_dots(vr.data(), z->sigw, i + 1, z->dT, z->scratch + z->off_dots, z->st));
         SFCI_CUDA(vec_overlaps(vr.data(), i + 1, vr[i], z->dS, z->scratch + z->off_dots, z->st));
         std::vector<double> tcol(i + 1), scol(i + 1);
-        SFCI_CUDA(cudaMemcpyAsync(tcol.data(), z->dT, 8 * (i + 1), cudaMemcpyDeviceToHost, z->st));
-        SFCI_CUDA(cudaMemcpyAsync(scol.data(), z->dS, 8 * (i + 1), cudaMemcpyDeviceToHost, z->st));
+        SFCI_CUDA(cudaMemcpyAsync(z->host->TS, z->dT, sizeof(z->host->TS), cudaMemcpyDeviceToHost, z->st));
         SFCI_CUDA(cudaStreamSynchronize(z->st));
+        std::copy(z->host->TS, z->host->TS + i + 1, tcol.begin());
+        std::copy(z->host->TS + kMaxVec, z->host->TS + kMaxVec + i + 1, scol.begin());
         for (int j = 0; j <= i; ++j) {
             z->T[size_t(j) * NL + i] = tcol[j];
             z->S[size_t(j) * NL + i] = scol[j];
@@ -1276,14 +1297,13 @@ sfci_status sfci_lanczos_step(sfci_lanczos *z, sfci_step_info *info) {
         if ((rs = ensure(z->cand_val, size_t(cand_cap) * 8, z->st, "candidates"))) return rs;
         z->cand_cap = cand_cap;
         Items it{skey, sval, 1, n_items};
-        SplitResult res{};
         SFCI_CUDA(select_split(it, z->nkeep, z->wr[i + 1], z->wc[i + 1], z->ndev,
                                static_cast<unsigned long long *>(z->cand_key.p),
                                static_cast<double *>(z->cand_val.p), cand_cap, z->cand_n,
-                               z->scratch + z->off_sel, z->sel_bytes, &res, z->st));
+                               z->scratch + z->off_sel, z->sel_bytes, &z->host->split, z->st));
+        const SplitResult res = z->host->split;
         unsigned long long kept = std::min<unsigned long long>(res.n_out, (unsigned long long)z->nkeep);
         if (!res.done && !res.all) {
-            unsigned long long n2 = 0;
             if ((long long)res.n_cand > cand_cap) {  // the picked bin is too crowded: exact select over all
                 SFCI_CUDA(select_topk(it, z->nkeep, z->wr[i + 1], z->wc[i + 1], z->total, nullptr, nullptr,
                                       z->scratch + z->off_sel, z->sel_bytes, z->st));
@@ -1295,18 +1315,20 @@ sfci_status sfci_lanczos_step(sfci_lanczos *z, sfci_step_info *info) {
                                       z->total, nullptr, nullptr, z->scratch + z->off_sel, z->sel_bytes,
                                       z->st));
             }
-            SFCI_CUDA(cudaMemcpyAsync(&n2, z->total, 8, cudaMemcpyDeviceToHost, z->st));
+            SFCI_CUDA(cudaMemcpyAsync(&z->host->n, z->total, 8, cudaMemcpyDeviceToHost, z->st));
             SFCI_CUDA(cudaStreamSynchronize(z->st));
-            kept = std::min<unsigned long long>(kept + n2, (unsigned long long)z->nkeep);
+            kept = std::min<unsigned long long>(kept + z->host->n, (unsigned long long)z->nkeep);
         }
         double usq = 0.0, cut = 0.0;
-        int hs = 0;
         SFCI_CUDA(cudaMemcpyAsync(z->ndev, &kept, 8, cudaMemcpyHostToDevice, z->st));
         SFCI_CUDA(min_abs(z->wc[i + 1], z->ndev, z->nkeep, z->dmin, z->st));
-        SFCI_CUDA(cudaMemcpyAsync(&cut, z->dmin, 8, cudaMemcpyDeviceToHost, z->st));
-        SFCI_CUDA(cudaMemcpyAsync(&usq, z->msumsq, 8, cudaMemcpyDeviceToHost, z->st));
-        SFCI_CUDA(cudaMemcpyAsync(&hs, z->mstatus, 4, cudaMemcpyDeviceToHost, z->st));
+        SFCI_CUDA(cudaMemcpyAsync(z->host->w, z->outn, sizeof(z->host->w), cudaMemcpyDeviceToHost, z->st));
         SFCI_CUDA(cudaStreamSynchronize(z->st));
+        const char *hw = reinterpret_cast<const char *>(z->host->w), *dw = reinterpret_cast<const char *>(z->outn);
+        int hs = 0;
+        std::memcpy(&cut, hw + (reinterpret_cast<const char *>(z->dmin) - dw), 8);
+        std::memcpy(&usq, hw + (reinterpret_cast<const char *>(z->msumsq) - dw), 8);
+        std::memcpy(&hs, hw + (reinterpret_cast<const char *>(z->mstatus) - dw), 4);
         if (hs & 8) {
             set_error("sigma output buffer overflowed while appending u");
             return SFCI_E_CAPACITY;
@@ -1335,12 +1357,7 @@ sfci_status sfci_lanczos_step(sfci_lanczos *z, sfci_step_info *info) {
         z->wn[i + 1] = (long long)kept;
         z->vrp_ok[i + 1] = 0;
         SFCI_CUDA(cudaEventRecord(z->evp[0], z->st));
-        SFCI_CUDA(cudaEventSynchronize(z->evp[0]));
-        {
-            float tk = 0.f;
-            cudaEventElapsedTime(&tk, z->evp[3], z->evp[0]);
-            info->ms_topk = tk;
-        }
+        truncated = true;
         const double unorm = std::sqrt(usq);
         info->u_norm = unorm;
         if (unorm < 1e-14 * std::fabs(a) || res.total == 0) {
@@ -1401,7 +1418,9 @@ sfci_status sfci_lanczos_step(sfci_lanczos *z, sfci_step_info *info) {
     }
     SFCI_CUDA(cudaEventRecord(z->ev[3], z->st));
     SFCI_CUDA(cudaEventSynchronize(z->ev[3]));
-    float ms = 0.f;
+    float ms = 0.f, tk = 0.f;
+    if (truncated) cudaEventElapsedTime(&tk, z->evp[3], z->evp[0]);
+    info->ms_topk = tk;
     cudaEventElapsedTime(&ms, z->ev[0], z->ev[3]);
     info->ms_step = ms;
     log_step(*info);

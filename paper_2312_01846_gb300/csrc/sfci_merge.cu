@@ -583,6 +583,17 @@ __global__ void aligned_finish_kernel(const double *partial, int np, double *out
     }
 }
 
+struct ZeroPack {
+    double *p[kMaxVec];
+    long long n[kMaxVec];
+};
+
+__global__ void zero_vectors_kernel(const __grid_constant__ ZeroPack z) {
+    double *p = z.p[blockIdx.y];
+    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < z.n[blockIdx.y]; k += (long long)gridDim.x * blockDim.x)
+        p[k] = 0.0;
+}
+
 __global__ void min_init_kernel(double *out) { *out = __longlong_as_double(0x7ff0000000000000ll); }  // +inf
 
 __global__ void min_abs_kernel(const double *val, const unsigned long long *n_dev, long long cap, double *out) {
@@ -751,6 +762,15 @@ cudaError_t min_abs(const double *val, const unsigned long long *n_dev, long lon
 }
 
 size_t aligned_dots_ws_bytes(int nvec) { return size_t(nvec > 0 ? nvec : 1) * kDotBlocks * 8; }
+
+cudaError_t zero_vectors(double *const *sig, const long long *n, int nvec, cudaStream_t st) {
+    ZeroPack z{};
+    long long most = 1;
+    for (int j = 0; j < nvec; ++j) z.p[j] = sig[j], z.n[j] = n[j], most = most > n[j] ? most : n[j];
+    count_launch();
+    zero_vectors_kernel<<<dim3(grid_for(most, 2), nvec), 256, 0, st>>>(z);
+    return cudaGetLastError();
+}
 
 cudaError_t aligned_dots(const VecRef *vecs, double *const *sig, int nvec, double *out_dev, void *ws,
                          cudaStream_t st) {
