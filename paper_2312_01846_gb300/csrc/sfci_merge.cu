@@ -572,13 +572,17 @@ __global__ void aligned_dots_kernel(VecPackRef vp, SigPack sp, double *partial) 
     }
 }
 
+// a fixed tree over the partial sums of each vector
 __global__ void aligned_finish_kernel(const double *partial, int np, double *out) {
-    __shared__ double sh[kDotBlocks];  // (fetched together, then added in order)
-    for (int k = threadIdx.x; k < np; k += blockDim.x) sh[k] = partial[(size_t)blockIdx.x * np + k];
+    __shared__ double sh[32];
+    double r = 0.0;
+    for (int k = threadIdx.x; k < np; k += blockDim.x) r += partial[(size_t)blockIdx.x * np + k];
+    for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = r;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double r = 0.0;
-        for (int k = 0; k < np; ++k) r += sh[k];
+        r = 0.0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += sh[w];
         out[blockIdx.x] = r;
     }
 }

@@ -17,7 +17,7 @@
 // counts every digit of every key (digits that all keys share are skipped),
 // then per digit a histogram per tile, one scan per digit value over the
 // tiles, and a stable scatter ranked per warp with __match_any_sync.  Up to
-// kSmall pairs one CTA sorts (and normalises) in shared memory.
+// kSmall pairs one CTA sorts in shared memory.
 //
 // What bounds it: at 3e6 items (48 MB) launches and the chain of passes, not
 // bandwidth; the 2e5 largest of 3e6, sorted: 554 us with one-block scans over
@@ -25,6 +25,8 @@
 // far above the count, the kernels follow the count: an unsorted sigma of 3e7
 // entries 60.2 ms when sorting over the capacity, 27.3 ms so.  A step on the
 // whole 4900-determinant space: 1066 us with 30 launches a sort, 839 us so.
+// With a pass of up to 256 tiles in one launch and the partial sums added by a
+// tree: 379 -> 319 us, that step 599 -> 534 us.
 #include "sfci_internal.cuh"
 
 namespace sfci {
@@ -515,6 +517,115 @@ __global__ void rs_digits_kernel(const unsigned long long *key, long long cap, c
         if ((&h[0][0])[b]) atomicAdd(&(&s->digit[0][0])[b], (&h[0][0])[b]);
 }
 
+// Up to kFusedTiles tiles a pass is one launch: each tile's block adds up the counts of the
+// tiles before it, and while it places its pairs it counts, for the tile each one lands in,
+// the digit of the next pass that is not skipped.  counts: three buffers of [tile][value],
+// taken in turn (read, filled, cleared).  Three launches a pass took 20 us each pass at
+// 2e4 to 2e5 pairs, mostly launch gaps; above kFusedTiles the scan over all tiles is shared.
+constexpr int kFusedTiles = 256;
+
+__device__ __forceinline__ int rs_next(const SortState *s, unsigned n, int p, int passes) {
+    while (++p < passes && rs_skip(s, n, p)) {}
+    return p;
+}
+
+__device__ __forceinline__ int rs_done(const SortState *s, unsigned n, int p) {  // passes run before p
+    int c = 0;
+    for (int q = 0; q < p; ++q) c += !rs_skip(s, n, q);
+    return c;
+}
+
+__global__ void rs_first_kernel(const unsigned long long *key, long long cap, const unsigned long long *n_dev, int passes,
+                                const SortState *s, unsigned *counts) {
+    __shared__ unsigned h[kRadix];
+    const long long n = rs_count(n_dev, cap), t0 = (long long)blockIdx.x * kTile;
+    const int p = rs_next(s, (unsigned)n, -1, passes);
+    if (p >= passes || t0 >= n) return;
+    h[threadIdx.x] = 0;  // kT == kRadix
+    __syncthreads();
+    for (int q = 0; q < kSortItems; ++q) {
+        const long long i = t0 + (long long)q * kT + threadIdx.x;
+        if (i < n) atomicAdd(&h[(key[i] >> (8 * p)) & 0xff], 1u);
+    }
+    __syncthreads();
+    counts[(size_t)blockIdx.x * kRadix + threadIdx.x] = h[threadIdx.x];
+}
+
+// the pairs of a tile (kSortItems rounds of each warp's 32): their places among the pairs of
+// their digit value in the tile; wc[warp][value]: the warp's count
+__device__ __forceinline__ void rs_rank(const unsigned long long *key, long long w0, long long n, int shift, int warp,
+                                        int lane, unsigned (*wc)[kRadix], unsigned *loc) {
+#pragma unroll
+    for (int q = 0; q < kSortItems; ++q) {
+        const bool valid = w0 + (long long)q * 32 + lane < n;
+        const unsigned d = valid ? (unsigned)((key[q] >> shift) & 0xff) : (0x1000u | lane);
+        const unsigned peers = __match_any_sync(kFull, d);
+        const unsigned before = __popc(peers & ((1u << lane) - 1u));
+        const unsigned base = valid ? wc[warp][d] : 0u;
+        __syncwarp();
+        if (valid && (peers >> lane) == 1u) wc[warp][d] = base + __popc(peers);  // highest peer
+        __syncwarp();
+        loc[q] = base + before;
+    }
+}
+
+__global__ void rs_pass_kernel(unsigned long long *ka, double *va, unsigned long long *kb, double *vb, long long cap,
+                               const unsigned long long *n_dev, int p, int passes, const SortState *s, unsigned *counts,
+                               size_t stride) {
+    __shared__ unsigned wc[kT / 32][kRadix], wsum[kT / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, shift = 8 * p;
+    const long long n = rs_count(n_dev, cap), t0 = (long long)blockIdx.x * kTile;
+    if (t0 >= n || rs_skip(s, (unsigned)n, p)) return;
+    const int done = rs_done(s, (unsigned)n, p), next = rs_next(s, (unsigned)n, p, passes);
+    const unsigned *now = counts + (size_t)(done % 3) * stride;
+    unsigned *then = counts + (size_t)((done + 1) % 3) * stride;
+    counts[(size_t)((done + 2) % 3) * stride + (size_t)blockIdx.x * kRadix + tid] = 0u;
+    const unsigned long long *kin = done & 1 ? kb : ka;
+    const double *vin = done & 1 ? vb : va;
+    unsigned long long *kout = done & 1 ? ka : kb;
+    double *vout = done & 1 ? va : vb;
+    const long long w0 = t0 + (long long)warp * (32 * kSortItems);
+    unsigned long long key[kSortItems];
+    double val[kSortItems];
+#pragma unroll
+    for (int q = 0; q < kSortItems; ++q) {
+        const long long i = w0 + (long long)q * 32 + lane;
+        key[q] = 0ull, val[q] = 0.0;
+        if (i < n) key[q] = kin[i], val[q] = vin[i];
+    }
+    // where this tile's pairs of digit value tid begin
+    unsigned before = 0, total = s->digit[p][tid], x = total;
+    for (unsigned t = 0; t < blockIdx.x; ++t) before += now[(size_t)t * kRadix + tid];
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(kFull, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[warp] = x;
+    for (int b = tid; b < (kT / 32) * kRadix; b += kT) (&wc[0][0])[b] = 0;
+    __syncthreads();
+    before += x - total;
+    for (int w = 0; w < warp; ++w) before += wsum[w];
+    unsigned loc[kSortItems];
+    rs_rank(key, w0, n, shift, warp, lane, wc, loc);
+    __syncthreads();
+    for (int w = 0; w < kT / 32; ++w) {
+        const unsigned c = wc[w][tid];
+        wc[w][tid] = before;
+        before += c;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kSortItems; ++q) {
+        const long long i = w0 + (long long)q * 32 + lane;
+        if (i < n) {
+            const unsigned pos = wc[warp][(key[q] >> shift) & 0xff] + loc[q];
+            kout[pos] = key[q];
+            vout[pos] = val[q];
+            if (next < passes) atomicAdd(&then[(size_t)(pos / kTile) * kRadix + ((key[q] >> (8 * next)) & 0xff)], 1u);
+        }
+    }
+}
+
 // per tile and digit value: the keys that have it; counts[value * tiles + tile]
 __global__ void rs_hist_kernel(const unsigned long long *ka, const unsigned long long *kb, long long cap,
                                const unsigned long long *n_dev, int p, const SortState *s, unsigned *counts) {
@@ -598,18 +709,7 @@ __global__ void rs_scatter_kernel(unsigned long long *ka, double *va, unsigned l
             const long long i = w0 + (long long)q * 32 + lane;
             key[q] = i < n ? kin[i] : 0ull;
         }
-        for (int q = 0; q < kSortItems; ++q) {
-            const long long i = w0 + (long long)q * 32 + lane;
-            const bool valid = i < n;
-            const unsigned d = valid ? (unsigned)((key[q] >> shift) & 0xff) : (0x1000u | lane);
-            const unsigned peers = __match_any_sync(kFull, d);
-            const unsigned before = __popc(peers & ((1u << lane) - 1u));
-            const unsigned base = valid ? wc[warp][d] : 0u;
-            __syncwarp();
-            if (valid && (peers >> lane) == 1u) wc[warp][d] = base + __popc(peers);  // highest peer
-            __syncwarp();
-            loc[q] = base + before;
-        }
+        rs_rank(key, w0, n, shift, warp, lane, wc, loc);
         __syncthreads();
         {
             unsigned run = offsets[(size_t)threadIdx.x * tiles + t];  // kT == kRadix
@@ -632,41 +732,55 @@ __global__ void rs_scatter_kernel(unsigned long long *ka, double *va, unsigned l
     }
 }
 
-// The sum over the kRedBlocks partial sums, in order (thread 0's value; every thread of
-// a block of at least 32 calls it): the partials are fetched together, then added.
-__device__ __forceinline__ double ordered_sum(const double *partial, int np, double *sh) {
-    for (int k = threadIdx.x; k < np; k += blockDim.x) sh[k] = partial[k];
-    __syncthreads();
+// The sum over the partial sums (thread 0's value; all kT threads call it): a fixed tree,
+// so the same on every run (one thread adding 304 of them in order took 12 us).
+__device__ __forceinline__ double partial_total(const double *partial, int np, double *sh) {
     double s = 0.0;
+    for (int k = threadIdx.x; k < np; k += kT) s += partial[k];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    s = 0.0;
     if (threadIdx.x == 0)
-        for (int k = 0; k < np; ++k) s += sh[k];
+        for (int w = 0; w < kT / 32; ++w) s += sh[w];
     return s;
 }
 
-// Up to kSmall pairs sorted by one CTA in shared memory and, with `normalize`, divided
-// by their 2-norm (summed in the order of sumsq_kernel and scale_kernel).
+// Up to kSmall pairs sorted by one CTA in shared memory; digits that all keys share are
+// skipped.  (Dividing by the norm here too was slower than its two launches: one SM's
+// float64 units take 25 us for 4900 entries.)
 __global__ void __launch_bounds__(kSmallT)
-small_sort_kernel(unsigned long long *key, double *val, long long cap, const unsigned long long *n_dev, int bits,
-                  int normalize) {
+small_sort_kernel(unsigned long long *key, double *val, long long cap, const unsigned long long *n_dev, int bits) {
     extern __shared__ __align__(16) unsigned char sm[];
     unsigned long long *sk = reinterpret_cast<unsigned long long *>(sm);
     double *sv = reinterpret_cast<double *>(sk + kSmall);
     unsigned *wc = reinterpret_cast<unsigned *>(sv + kSmall);  // [warps][kRadix]
     __shared__ unsigned dsum[kRadix / 32];
-    __shared__ double part[kSmallT / 256][8], norm;
+    __shared__ unsigned differ[2];  // bits in which some key differs from the first
     constexpr int W = kSmallT / 32, kItems = kSmall / kSmallT;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = (int)rs_count(n_dev, cap), per = (n + kSmallT - 1) / kSmallT;  // rounds of 32 per warp
     unsigned long long k[kItems];
     double v[kItems];
     const int w0 = warp * 32 * per + lane;
+    const unsigned long long key0 = n > 0 ? key[0] : 0ull;
+    unsigned long long diff = 0ull;
+    if (tid < 2) differ[tid] = 0u;
+    __syncthreads();
 #pragma unroll
     for (int q = 0; q < kItems; ++q) {
         const int i = w0 + q * 32;
         k[q] = 0ull, v[q] = 0.0;
-        if (q < per && i < n) k[q] = key[i], v[q] = val[i];
+        if (q < per && i < n) k[q] = key[i], v[q] = val[i], diff |= k[q] ^ key0;
     }
+    {
+        const unsigned lo = __reduce_or_sync(kFull, (unsigned)diff), hi = __reduce_or_sync(kFull, (unsigned)(diff >> 32));
+        if (lane == 0) atomicOr(&differ[0], lo), atomicOr(&differ[1], hi);
+    }
+    __syncthreads();
+    diff = differ[0] | (unsigned long long)differ[1] << 32;
     for (int shift = 0; shift < bits; shift += 8) {
+        if (((diff >> shift) & 0xffull) == 0ull) continue;
         for (int b = tid; b < W * kRadix; b += kSmallT) wc[b] = 0u;
         __syncthreads();
         unsigned loc[kItems];
@@ -716,32 +830,9 @@ small_sort_kernel(unsigned long long *key, double *val, long long cap, const uns
         for (int q = 0; q < kItems; ++q)
             if (q < per && w0 + q * 32 < n) k[q] = sk[w0 + q * 32], v[q] = sv[w0 + q * 32];
     }
-    __syncthreads();
 #pragma unroll
     for (int q = 0; q < kItems; ++q)
-        if (q < per && w0 + q * 32 < n) key[w0 + q * 32] = k[q], sv[w0 + q * 32] = v[q];
-    __syncthreads();
-    if (normalize) {
-        double s = 0.0;  // (thread 0) over the blocks of 256 in order
-        for (int b0 = 0; b0 < n; b0 += kSmallT) {
-            const int i = b0 + tid;
-            double a = i < n ? __fma_rn(sv[i], sv[i], 0.0) : 0.0;
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(kFull, a, o);
-            if (lane == 0) part[warp >> 3][warp & 7] = a;
-            __syncthreads();
-            if (tid == 0)
-                for (int b = 0; b < kSmallT / 256; ++b) {
-                    double r = 0.0;
-                    for (int w = 0; w < 8; ++w) r += part[b][w];
-                    s += r;
-                }
-            __syncthreads();
-        }
-        if (tid == 0) norm = sqrt(s);
-        __syncthreads();
-    }
-    const double d = normalize ? norm : 1.0;
-    for (int i = tid; i < n; i += kSmallT) val[i] = normalize && d > 0.0 ? __ddiv_rn(sv[i], d) : sv[i];
+        if (q < per && w0 + q * 32 < n) key[w0 + q * 32] = k[q], val[w0 + q * 32] = v[q];
 }
 
 // back into the caller's arrays when an odd number of passes ran
@@ -778,8 +869,8 @@ __global__ void sumsq_kernel(const double *v, long long cap, const unsigned long
 
 __global__ void scale_kernel(double *v, long long cap, const unsigned long long *n_dev,
                              const double *partial, int nparts) {
-    __shared__ double norm, sh[kRedBlocks];
-    const double s = ordered_sum(partial, nparts, sh);
+    __shared__ double norm, sh[kT / 32];
+    const double s = partial_total(partial, nparts, sh);
     if (threadIdx.x == 0) norm = sqrt(s);
     __syncthreads();
     long long n = (long long)*n_dev;
@@ -858,21 +949,27 @@ cudaError_t select_split(Items it, long long k,
     return cudaStreamSynchronize(st);
 }
 
+namespace {
+size_t sort_counts_bytes(long long ntiles) {
+    return a256(size_t(ntiles > 0 ? ntiles : 1) * kRadix * 4 * (ntiles <= kFusedTiles ? 3 : 1));
+}
+}  // namespace
+
 size_t sort_pairs_bytes(long long cap) {
     const long long ntiles = (cap + kTile - 1) / kTile;
-    return a256(size_t(cap) * 8) * 2 + a256(size_t(ntiles > 0 ? ntiles : 1) * kRadix * 4) + a256(sizeof(SortState));
+    return a256(size_t(cap) * 8) * 2 + sort_counts_bytes(ntiles) + a256(sizeof(SortState));
 }
 
 size_t sort_workspace_bytes(long long n) { return sort_pairs_bytes(n); }
 
 namespace {
 cudaError_t small_sort(unsigned long long *key, double *val, long long cap, const unsigned long long *n_dev, int bits,
-                       int normalize, cudaStream_t st) {
+                       cudaStream_t st) {
     const size_t smem = size_t(kSmall) * 16 + size_t(kSmallT / 32) * kRadix * 4;
     cudaError_t e = allow_max_smem(small_sort_kernel, smem);
     if (e != cudaSuccess) return e;
     count_launch();
-    small_sort_kernel<<<1, kSmallT, smem, st>>>(key, val, cap, n_dev, bits, normalize);
+    small_sort_kernel<<<1, kSmallT, smem, st>>>(key, val, cap, n_dev, bits);
     return cudaGetLastError();
 }
 }  // namespace
@@ -880,18 +977,32 @@ cudaError_t small_sort(unsigned long long *key, double *val, long long cap, cons
 cudaError_t sort_pairs(unsigned long long *key, double *val, long long cap,
                        const unsigned long long *n_dev, int bits, void *ws, cudaStream_t st) {
     if (cap <= 0) return cudaSuccess;
-    if (cap <= kSmall) return small_sort(key, val, cap, n_dev, bits, 0, st);
+    if (cap <= kSmall) return small_sort(key, val, cap, n_dev, bits, st);
     const long long ntiles = (cap + kTile - 1) / kTile;
     char *b = static_cast<char *>(ws);
     unsigned long long *k2 = reinterpret_cast<unsigned long long *>(b);
     double *v2 = reinterpret_cast<double *>(b + a256(size_t(cap) * 8));
     unsigned *counts = reinterpret_cast<unsigned *>(b + 2 * a256(size_t(cap) * 8));
-    SortState *s = reinterpret_cast<SortState *>(b + 2 * a256(size_t(cap) * 8) + a256(size_t(ntiles) * kRadix * 4));
+    SortState *s = reinterpret_cast<SortState *>(b + 2 * a256(size_t(cap) * 8) + sort_counts_bytes(ntiles));
     const int passes = (bits + 7) / 8;
     cudaError_t e = cudaMemsetAsync(s, 0, sizeof(SortState), st);
     if (e != cudaSuccess) return e;
     count_launch();
     rs_digits_kernel<<<grid_for(cap, 4), kT, 0, st>>>(key, cap, n_dev, passes, s);
+    if (ntiles <= kFusedTiles) {
+        const size_t stride = size_t(ntiles) * kRadix;
+        e = cudaMemsetAsync(counts, 0, stride * 12, st);
+        if (e != cudaSuccess) return e;
+        count_launch();
+        rs_first_kernel<<<(unsigned)ntiles, kT, 0, st>>>(key, cap, n_dev, passes, s, counts);
+        for (int p = 0; p < passes; ++p) {
+            count_launch();
+            rs_pass_kernel<<<(unsigned)ntiles, kT, 0, st>>>(key, val, k2, v2, cap, n_dev, p, passes, s, counts, stride);
+        }
+        count_launch();
+        copy_pairs_kernel<<<grid_for(cap, 8), kT, 0, st>>>(k2, v2, key, val, cap, n_dev, passes, s);
+        return cudaGetLastError();
+    }
     const unsigned g = (unsigned)(ntiles < (long long)sms() * 8 ? ntiles : (long long)sms() * 8);
     for (int p = 0; p < passes; ++p) {
         count_launch();
@@ -908,8 +1019,6 @@ cudaError_t sort_pairs(unsigned long long *key, double *val, long long cap,
 
 cudaError_t sort_normalize(unsigned long long *key, double *val, long long cap, const unsigned long long *n_dev,
                            int bits, void *sort_ws, void *norm_ws, cudaStream_t st) {
-    if (cap <= 0) return cudaSuccess;
-    if (cap <= kSmall) return small_sort(key, val, cap, n_dev, bits, 1, st);
     const cudaError_t e = sort_pairs(key, val, cap, n_dev, bits, sort_ws, st);
     return e == cudaSuccess ? normalize_vec(val, cap, n_dev, norm_ws, st) : e;
 }
