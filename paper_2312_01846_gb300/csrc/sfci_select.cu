@@ -256,7 +256,7 @@ sel_small_kernel(Items it, unsigned long long k, unsigned long long *out_key, do
         unsigned long long c = 0;
         for (int w = 0; w < kSmallT / 32; ++w) a += ssq[w], c += wsum[w];
         need = k, ph = pl = mh = ml = 0ull;
-        all = c <= k, done = all;
+        all = c <= k, done = all || k == 0;
         if (sumsq_out) *sumsq_out = a;
         if (total_out) *total_out = c;
     }
@@ -307,6 +307,7 @@ sel_small_kernel(Items it, unsigned long long k, unsigned long long *out_key, do
     // the chosen items, in their order
     double least = __longlong_as_double(0x7ff0000000000000ll);  // +inf
     unsigned base = 0;
+    const bool none = k == 0 && !all;
     for (int i0 = 0; i0 < n; i0 += kSmallT) {
         const int i = i0 + tid;
         bool ok = false;
@@ -314,7 +315,7 @@ sel_small_kernel(Items it, unsigned long long k, unsigned long long *out_key, do
         if (i < n) {
             v = vb[i];
             const unsigned long long hi = (0x7fffffffffffffffull - (v & 0x7fffffffffffffffull)) & mh;
-            ok = (v << 1) != 0ull && (all || hi < ph || (hi == ph && (key[i] & ml) <= pl));
+            ok = (v << 1) != 0ull && !none && (all || hi < ph || (hi == ph && (key[i] & ml) <= pl));
         }
         const unsigned bal = __ballot_sync(kFull, ok);
         if (lane == 0) wsum[warp] = __popc(bal);

@@ -41,3 +41,13 @@ def test_truncate_exact(n, share, values):
     if norm > 0:
         # a norm of non-negative terms summed in any order: relative error <= n * 2^-53
         np.testing.assert_allclose(gv.cpu().numpy(), coef[order] / norm, rtol=(n + 4) * 2.0 ** -52, atol=1e-320)
+
+
+@pytest.mark.parametrize("n", [5, SMALL, SMALL + 1])
+def test_nothing_asked_for(n):
+    """k = 0 keeps nothing, whatever the values."""
+    torch = pytest.importorskip("torch")
+    import paper_2312_01846_gb300 as sf
+    c = torch.full((n,), float("inf"), dtype=torch.float64, device="cuda")
+    r, v = sf.sfci_truncate_topk(torch.arange(n, device="cuda"), c, 0, normalize=False)
+    assert r.numel() == 0 and v.numel() == 0
