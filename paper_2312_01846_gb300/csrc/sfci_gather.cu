@@ -120,27 +120,29 @@ __device__ __noinline__ double single_of(const SysDev &d, int i, int a, unsigned
 }
 
 // <D|H|D>, the emit kernel's term order
-__device__ double diagonal_of(const SysDev &d, unsigned long long alpha, unsigned long long beta) {
+// (J + p stride: (pp|kk) over k, then (pk|kp); hd: the diagonal of h, hstride apart)
+__device__ double diagonal_of(const SysDev &d, const double *J, int stride, const double *hd, int hstride,
+                              unsigned long long alpha, unsigned long long beta) {
     const int n = d.n;
     double one = 0.0, coul = 0.0, exch = 0.0;
     unsigned long long str[2] = {alpha, beta};
     for (int s = 0; s < 2; ++s)
         for (unsigned long long x = str[s]; x; x &= x - 1ull)
-            one = __dadd_rn(one, __ldg(&d.h[(__ffsll((long long)x) - 1) * (n + 1)]));
+            one = __dadd_rn(one, hd[(__ffsll((long long)x) - 1) * hstride]);
     for (int s = 0; s < 2; ++s)
         for (unsigned long long x = str[s]; x; x &= x - 1ull) {
             const int p = __ffsll((long long)x) - 1;
-            const double *gpp = d.sg + size_t(p * n + p) * 2 * n;
+            const double *gpp = J + size_t(p) * stride;
             for (int t = 0; t < 2; ++t)
                 for (unsigned long long y = str[t]; y; y &= y - 1ull)
-                    coul = __dadd_rn(coul, __ldg(&gpp[__ffsll((long long)y) - 1]));
+                    coul = __dadd_rn(coul, gpp[__ffsll((long long)y) - 1]);
         }
     for (int s = 0; s < 2; ++s)
         for (unsigned long long x = str[s]; x; x &= x - 1ull) {
             const int p = __ffsll((long long)x) - 1;
-            const double *gpq = d.sg + (size_t(p * n + p) * 2 + 1) * n;
+            const double *gpq = J + size_t(p) * stride + n;
             for (unsigned long long y = str[s]; y; y &= y - 1ull)
-                exch = __dadd_rn(exch, __ldg(&gpq[__ffsll((long long)y) - 1]));
+                exch = __dadd_rn(exch, gpq[__ffsll((long long)y) - 1]);
         }
     return __dsub_rn(__dadd_rn(__dadd_rn(d.e_core, one), __dmul_rn(0.5, coul)), __dmul_rn(0.5, exch));
 }
@@ -214,11 +216,23 @@ __global__ void sources_kernel(const GatherShape p, const unsigned long long *ra
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(runs, (unsigned long long)c);
 }
 
-// per source (in run order): pi(beta), number of its beta string, <D|H|D>
+// per source (in run order): pi(beta), number of its beta string, <D|H|D>.  The diagonal is a
+// chain of some hundred adds: its integrals are staged in shared memory (up to kStageN
+// orbitals), since the first thread to need one waits for L2 (45 us for 2e4 sources).
+constexpr int kStageN = 48;
 __global__ void source_fields_kernel(const SysDev d, const GatherShape p, const unsigned long long *skey, long long n,
                                      const unsigned long long *bid, unsigned *spi, unsigned *sb, double *diag,
                                      unsigned long long *bstr) {
     extern __shared__ unsigned long long bt[];
+    const int no = d.n;
+    const double *J = d.sg, *hd = d.h;
+    int stride = (no + 1) * 2 * no, hstride = no + 1;
+    if (no <= kStageN) {
+        double *sj = reinterpret_cast<double *>(bt + (no + 1) * d.ks), *sh = sj + 2 * no * no;
+        for (int i = threadIdx.x; i < 2 * no * no; i += blockDim.x) sj[i] = __ldg(&d.sg[size_t(i / (2 * no)) * stride + i % (2 * no)]);
+        for (int i = threadIdx.x; i < no; i += blockDim.x) sh[i] = __ldg(&d.h[i * hstride]);
+        J = sj, hd = sh, stride = 2 * no, hstride = 1;
+    }
     load_binom(d, bt);
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
         const unsigned long long k = skey[s];
@@ -228,7 +242,7 @@ __global__ void source_fields_kernel(const SysDev d, const GatherShape p, const 
         spi[s] = pi;
         sb[s] = id;
         bstr[id] = beta;  // every source of this beta string writes the same
-        diag[s] = diagonal_of(d, alpha, beta);
+        diag[s] = diagonal_of(d, J, stride, hd, hstride, alpha, beta);
     }
 }
 
@@ -1543,7 +1557,8 @@ cudaError_t gather_tables(const SysDev &d, const GatherShape &p, long long n, un
                           const unsigned *rp, const GatherBufs &b, const RowPlanArgs &ra, cudaStream_t st) {
     const size_t bts = size_t(d.n + 1) * d.ks * 8;
     count_launch();
-    source_fields_kernel<<<grid_for(n, 128), 128, bts, st>>>(d, p, b.skey, n, b.bid, b.s_pi, b.s_b, b.s_diag, b.bstr);
+    const size_t fields_smem = bts + (d.n <= kStageN ? size_t(2 * d.n + 1) * d.n * 8 : 0);
+    source_fields_kernel<<<grid_for(n, 128), 128, fields_smem, st>>>(d, p, b.skey, n, b.bid, b.s_pi, b.s_b, b.s_diag, b.bstr);
     const bool keep = beta_smem(d, true) <= 100 * 1024;
     const size_t smem = beta_smem(d, keep);
     auto tables = keep ? beta_tables_kernel<true> : beta_tables_kernel<false>;
