@@ -1065,7 +1065,7 @@ __global__ void rank_kernel(const SysDev d, const unsigned long long *a, const u
         const unsigned long long x = a[k], y = b[k];
         if (__popcll(x) != d.na || __popcll(y) != d.nb || (x & high) || (y & high)) {
             r[k] = ~0ull;
-            atomicOr(status, 1);
+            *(volatile int *)status = 1;
             continue;
         }
         r[k] = string_rank(x, bt_s, d.ks) * d.cb + string_rank(y, bt_s, d.ks);
@@ -1092,7 +1092,7 @@ __global__ void unrank_kernel(const SysDev d, const unsigned long long *r, unsig
         const unsigned long long x = r[k];
         if (x >= d.dim) {
             a[k] = 0, b[k] = 0;
-            atomicOr(status, 1);
+            *(volatile int *)status = 1;
             continue;
         }
         const unsigned long long ha = x / d.cb, hb = x - ha * d.cb;

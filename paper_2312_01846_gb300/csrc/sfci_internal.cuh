@@ -10,6 +10,8 @@
 //    in the 129 MB L2) and are read through the read-only path.
 #pragma once
 
+#include <atomic>
+
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -151,10 +153,12 @@ struct SysDev {
 
 }  // namespace sfci
 
+constexpr unsigned kStatusWords = 64;
 struct sfci_system {
     sfci::SysDev d;
     void *dev_block;  // one allocation holding h, g, binom, pairs
-    int *dev_status;  // scratch status words for rank/unrank
+    int *host_status; // page-locked status words that rank/unrank kernels write (kStatusWords)
+    std::atomic<unsigned> next_status{0};  // calls at the same time take words of their own
     double *pair_int; // (ai|bj) - (aj|bi) over orbital pairs (a < b), (i < j)
     int device;
 };

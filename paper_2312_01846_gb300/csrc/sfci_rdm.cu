@@ -743,7 +743,7 @@ size_t rows_place(char *base, RowArgs &A, size_t &scan_ws, size_t &partial, cons
     take(A.bstr, nd);
     take(A.hops, nd * size_t(d.sb));
     scan_ws = o, o = a256(o + scan_ws_bytes((long long)std::max(nn, cb) + 1));
-    partial = o, o = a256(o + 8 * (kNormBlocks + 1));
+    partial = o, o = a256(o + 8 * (kNormBlocks + 2));
     return o;
 }
 
@@ -805,15 +805,16 @@ sfci_status sfci_rdm12(const sfci_system *s, const uint64_t *rank, const double 
     SFCI_CUDA(cudaMemsetAsync(rdm1, 0, n2 * 8, st));
     SFCI_CUDA(cudaMemsetAsync(rdm2, 0, n2 * n2 * 8, st));
     const unsigned long long *r = reinterpret_cast<const unsigned long long *>(rank);
-    int *flag = s->dev_status;
-    SFCI_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), st));
-    SFCI_CUDA(validate_sorted(r, n, d.dim, flag, st));
     RowArgs A{};
     size_t scan_ws = 0, part_at = L.partial;
     const bool by_rows = rows_taken(d, n) && rows_place(nullptr, A, scan_ws, part_at, d, n) <= ws_bytes;
     if (!by_rows) part_at = L.partial;
     double *partial = reinterpret_cast<double *>(w + part_at);
+    // the norm and, behind it, the flag of invalid ranks: read back together
     double *nrm = by_rows ? partial + kNormBlocks : reinterpret_cast<double *>(w + L.norm);
+    int *flag = reinterpret_cast<int *>(nrm + 1);
+    SFCI_CUDA(cudaMemsetAsync(nrm, 0, 16, st));
+    SFCI_CUDA(validate_sorted(r, n, d.dim, flag, st));
     count_launch();
     norm2_kernel<<<kNormBlocks, kThreads, 0, st>>>(coef, n, partial);
     count_launch();
@@ -873,16 +874,17 @@ sfci_status sfci_rdm12(const sfci_system *s, const uint64_t *rank, const double 
             SFCI_CUDA(cudaGetLastError());
         }
     }
-    int hflag = 0;
-    double hn = 0.0;
-    SFCI_CUDA(cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
-    SFCI_CUDA(cudaMemcpyAsync(&hn, nrm, 8, cudaMemcpyDeviceToHost, st));
+    struct {
+        double norm;
+        int flag, pad;
+    } host{};
+    SFCI_CUDA(cudaMemcpyAsync(&host, nrm, 16, cudaMemcpyDeviceToHost, st));
     SFCI_CUDA(cudaStreamSynchronize(st));
-    if (hflag) {
+    if (host.flag) {
         set_error("input ranks must be strictly ascending and below dim");
         return SFCI_E_INVALID;
     }
-    if (norm2) *norm2 = hn;
+    if (norm2) *norm2 = host.norm;
     return SFCI_OK;
 }
 

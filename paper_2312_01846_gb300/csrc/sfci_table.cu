@@ -53,7 +53,7 @@ __global__ void validate_kernel(const unsigned long long *r, long long n, unsign
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         const unsigned long long x = r[i];
-        if (x >= dim || (i + 1 < n && r[i + 1] <= x)) atomicOr(flag, 1);
+        if (x >= dim || (i + 1 < n && r[i + 1] <= x)) *(volatile int *)flag = 1;
     }
 }
 
