@@ -211,14 +211,19 @@ def sigma_workspace_bytes(sys: System, n_in, out_cap):
 
 def sfci_sigma(sys: System, rank, coef, eps_screen=0.0, out_cap=None, stream=None):
     """sigma = H psi; returns (rank, coef) ascending by rank.  If out_cap is not
-    given it starts from min(n_in * (n_conn + 1), 2^24) and grows on
-    SFCI_E_CAPACITY."""
+    given it starts from min(n_in * (n_conn + 1), 2^25) (3 GB with the workspace; 2^24 with
+    more than 12 electrons of a spin) and grows on SFCI_E_CAPACITY."""
     r = _dev(rank, torch.int64)
     c = _dev(coef, torch.float64)
     if out_cap is not None:
         cap = int(out_cap)
     else:
-        cap = max(1024, min(r.numel() * (sys.n_conn + 1), 1 << 24))
+        # sigma by target rows touches only what it writes: room that is not used costs memory
+        # alone, and a second call because of a capacity that was too small is a whole sigma
+        # (3e7 entries: 5.1 ms so, 3.2 ms in one call); the hash table, which takes over beyond
+        # 12 electrons of a spin, is cleared and read throughout
+        room = 1 << (25 if max(sys.na, sys.nb) <= 12 else 24)
+        cap = max(1024, min(r.numel() * (sys.n_conn + 1), room))
     for _ in range(16):
         ws = torch.empty(sigma_workspace_bytes(sys, r.numel(), cap), dtype=torch.uint8, device="cuda")
         orank = torch.empty(max(cap, 1), dtype=torch.int64, device="cuda")
