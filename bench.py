@@ -36,7 +36,13 @@ if ROOT not in sys.path:
 
 METRIC = "σ=Hψ connected elements/s & Lanczos steps/s vs plain FP64 at ΔE≤1 µHa"
 UNIT = "connected elements/s"
-BYTES_PER_ELEMENT = 32  # 16 B intermediate element written + 16 B read back by the merge
+# the bucketed path's model (16 B intermediate element written + 16 B read back by the merge),
+# kept as the unit of the roofline figure so that runs compare; sigma by target rows writes no
+# elements and moves GATHER_DRAM_BYTES_PER_ELEMENT
+BYTES_PER_ELEMENT = 32
+# gather_kernel, one launch at N_d = 2e4 on the same workload, 6.15e8 elements
+GATHER_DRAM_BYTES_PER_ELEMENT = (2.546590 + 0.008495) * 1e9 / 6.15e8
+GATHER_WARP_INST_PER_ELEMENT = 8772965390 / 6.15e8
 # DRAM bytes per connected element that ncu measured for emit_kernel + merge_kernel
 # together (dram__bytes_read.sum + dram__bytes_write.sum of one launch each on the same
 # workload at N_d = 5e3, 1.5362e8 elements, one pass, every excitation class in the emit
@@ -577,9 +583,11 @@ def run_ours(a):
     value = elements_all / (ms_max * 1e-3)
     steps_per_s = a.steps / (ms_max * 1e-3)
 
-    # dominant stage: sigma = H w_i, i.e. the emit kernel (writes each intermediate
-    # element once) plus the bucket merge (reads it once), timed with CUDA events
-    # on the solver's stream; the 32 B/element model is exactly that write + read
+    # dominant stage: sigma = H w_i, timed with CUDA events on the solver's stream: by target
+    # rows (lists and tables in ms_emit, gather_kernel in ms_merge), or, when the bucketed
+    # path is shaped by an option, the emit kernel (writes each intermediate element once)
+    # plus the bucket merge (reads it once), which the 32 B/element model describes
+    by_rows = not (a.bucket_elems or a.emit_warps or a.mem_budget_gb)
     ms_sig = statistics.mean(i["ms_sigma"] for i in infos)
     ms_emit = statistics.mean(i["ms_emit"] for i in infos)
     ms_merge = statistics.mean(i["ms_merge"] for i in infos)
@@ -591,15 +599,20 @@ def run_ours(a):
                 # null: merge_kernel changed (its key-grouping threshold) after the last
                 # capture; that capture's figure, which the change does not touch (the same
                 # records are read), is kept below for reference
-                "traffic": None if TRAFFIC_STALE else MEASURED_DRAM_BYTES_PER_ELEMENT * el_per_launch,
-                "traffic_last_capture": MEASURED_DRAM_BYTES_PER_ELEMENT * el_per_launch,
-                "traffic_note": "bytes per launch: ncu DRAM bytes per element of emit_kernel + "
+                "traffic": GATHER_DRAM_BYTES_PER_ELEMENT * el_per_launch if by_rows
+                           else None if TRAFFIC_STALE else MEASURED_DRAM_BYTES_PER_ELEMENT * el_per_launch,
+                "traffic_last_capture": (GATHER_DRAM_BYTES_PER_ELEMENT if by_rows
+                                         else MEASURED_DRAM_BYTES_PER_ELEMENT) * el_per_launch,
+                "traffic_note": "bytes per launch: ncu DRAM bytes per element of gather_kernel (N_d = 2e4 "
+                                "capture; lists and tables not included) x elements per launch" if by_rows else
+                                "bytes per launch: ncu DRAM bytes per element of emit_kernel + "
                                 "merge_kernel (N_d = 5e3 capture, one pass) x elements per launch; "
                                 "null while a kernel has changed since that capture",
-                "kernel": "sigma stage: emit (emit_kernel, emit_aa_kernel) + merge_kernel",
+                "kernel": "sigma stage: lists and tables (ms_emit) + gather_kernel (ms_merge)" if by_rows else
+                          "sigma stage: emit (emit_kernel, emit_aa_kernel) + merge_kernel",
                 "peak_kind": f"{peak_kind} copy bandwidth",
                 "model": f"{BYTES_PER_ELEMENT} B per connected element (16 B written by emit, "
-                         f"16 B read by merge)",
+                         f"16 B read by merge" + ("; not moved by the row gather)" if by_rows else ")"),
                 "ms_per_launch": ms_sig, "ms_emit": ms_emit, "ms_merge": ms_merge,
                 "ms_plan_host": statistics.mean(i["ms_plan"] for i in infos),
                 "ms_topk": statistics.mean(i["ms_topk"] for i in infos),
@@ -610,7 +623,7 @@ def run_ours(a):
                 "sigma_share_of_step": sum(i["ms_sigma"] for i in infos) / ms,
                 "issue_note": "merge_kernel's instructions per element were captured before its "
                               "key-grouping threshold changed (fewer grouped buckets: fewer "
-                              "instructions now)" if TRAFFIC_STALE else "",
+                              "instructions now)" if TRAFFIC_STALE and not by_rows else "",
                 # the kernels are bound by instruction issue and latency, not by DRAM: the
                 # issue-slot view, with warp instructions per element from the N_d = 5e3
                 # one-pass captures (at N_d = 1e6 entries repeat more, so the merge streams
@@ -620,8 +633,9 @@ def run_ours(a):
                                   "achieved_warp_inst_per_s": ipe * el_per_launch / (ms_k * 1e-3),
                                   "peak_warp_inst_per_s": ISSUE_PEAK_WARP_INST_PER_S,
                                   "frac": ipe * el_per_launch / (ms_k * 1e-3) / ISSUE_PEAK_WARP_INST_PER_S}
-                          for kname, ipe, ms_k in (("emit", MEASURED_WARP_INST_PER_ELEMENT["emit"], ms_emit),
-                                                   ("merge_kernel", MEASURED_WARP_INST_PER_ELEMENT["merge_kernel"], ms_merge))}}
+                          for kname, ipe, ms_k in (((("gather_kernel", GATHER_WARP_INST_PER_ELEMENT, ms_merge),)) if by_rows else
+                                                  (("emit", MEASURED_WARP_INST_PER_ELEMENT["emit"], ms_emit),
+                                                   ("merge_kernel", MEASURED_WARP_INST_PER_ELEMENT["merge_kernel"], ms_merge)))}}
 
     # end to end through the public API with host buffers, chained: each step
     # copies its input vector w_i host -> device and hands it to the solver

@@ -190,6 +190,10 @@ sfci_status sfci_truncate_topk_noalloc(const uint64_t *rank, const double *coef,
  * takes in normal runs; slower. */
 #define SFCI_LZ_FALLBACK_STRESS 1u
 
+/* Sigma is summed by target rows (no intermediate elements in memory) unless the
+ * caller shapes the bucketed path below (flags, bucket_elems, mem_budget, emit_warps or
+ * ovf_max_log2 not 0), a spin has more than 12 electrons or 2^26 strings, or its lists
+ * do not fit in memory.  Both sum exactly: the results are the same bits. */
 typedef struct sfci_params {
     int64_t n_keep;         /* N_d: entries kept per basis vector (Eq. 11)          */
     int64_t table_capacity; /* slots of sigma's hash table; 0 = sized automatically */
@@ -237,22 +241,27 @@ typedef struct sfci_step_info {
     int64_t n_psi;     /* non-zero entries of Psi = sum_j x_j w_j (cycle end)         */
     double ms_sigma;   /* device time of the sigma stage (CUDA events)              */
     double ms_step;    /* device time of the whole step                             */
-    double ms_emit;    /* of ms_sigma: the emit kernel (all passes)                 */
-    double ms_merge;   /* of ms_sigma: overflow sort + merge kernel (all passes)    */
+    double ms_emit;    /* of ms_sigma: the emit kernel (all passes); by target rows:
+                          the lists and tables                                   */
+    double ms_merge;   /* of ms_sigma: overflow sort + merge kernel (all passes); by
+                          target rows: the summing kernel                        */
     double ms_plan;    /* wall time of the bucket plan (row weights, device plan,
                           pass cuts) and of sizing the buffers                  */
     double ms_topk;    /* device time of the truncation (u entries, top-k, sort)    */
     int32_t n_passes;  /* passes over the sources that sigma needed (memory bound, plus
                           passes split because their overflow outgrew the list) */
-    int32_t n_buckets_log2; /* ceil(log2(merge buckets))                            */
+    int32_t n_buckets_log2; /* ceil(log2(merge buckets; by target rows: units))     */
     double tau;        /* stream threshold of the accepted attempt (entries of sigma
                           below it were not written out; see sfci_lanczos_step)  */
     double cut;        /* |coef| of the N_d-th kept entry of u (0 if fewer kept)    */
     int32_t redo;      /* sigma recomputed because tau hid part of the N_d largest  */
     int32_t bucket_redo; /* sigma recomputed with 1024-element buckets because a
                             2048-element bucket outgrew its table (automatic size) */
-    double pass_budget_gb; /* device memory one pass's element regions may use (GB) */
-    double regions_gb;     /* element regions of all buckets (GB): passes ~ this/budget */
+    double pass_budget_gb; /* device memory one pass's element regions may use (GB);
+                              by target rows: all of sigma's buffers, and this and
+                              free_gb are of the last step whose buffers grew        */
+    double regions_gb;     /* element regions of all buckets (GB): passes ~ this/budget;
+                              by target rows: what records of the elements would take */
     double free_gb;        /* free device memory the plan saw, besides the solver's
                               element, stream and overflow buffers (GB)              */
     int64_t n_overflow;    /* most elements any pass sent past their bucket's region  */
@@ -346,7 +355,9 @@ sfci_status sfci_scan_destroy(sfci_scan *scan);
 
 /* ---------------------------------------------------------- density matrices */
 
-/* Workspace (bytes, device) for sfci_rdm12 on a vector of n entries. */
+/* Workspace (bytes, device) for sfci_rdm12 on a vector of n entries.  (It takes less, at
+ * least a table of 2^ceil(log2(2 n)) 16-byte slots and 2 KB, and then looks every
+ * excitation up in that table instead of walking the vector by alpha strings.) */
 sfci_status sfci_rdm12_workspace_bytes(const sfci_system *sys, int64_t n, size_t *bytes);
 
 /* Spin-summed one- and two-particle density matrices of psi (not normalised),

@@ -759,9 +759,7 @@ struct Items {
 // receives sum val^2 over all valid items, and total_dev their number.
 cudaError_t select_topk(Items it, long long k, unsigned long long *out_key, double *out_val,
                         unsigned long long *n_out_dev, double *sumsq_dev,
-                        unsigned long long *total_dev, void *ws, size_t ws_bytes, cudaStream_t st,
-                        double *cut_dev = nullptr);  // cut_dev: smallest |val| kept
-bool select_is_small(const Items &it);  // one launch does the whole selection
+                        unsigned long long *total_dev, void *ws, size_t ws_bytes, cudaStream_t st);
 // Two-level top-k: one pass histograms the first digit (top 12 bits of the
 // composite key, 4096 bins), the bin holding the k-th item is picked, and one
 // more pass writes every item of a smaller bin to out and every item of the

@@ -326,7 +326,7 @@ sfci_status ensure_slots(sfci_lanczos *z, unsigned long long cap) {
 sfci_status table_topk(sfci_lanczos *z, unsigned long long cap, int dst, double *sumsq_host,
                        unsigned long long *total_host) {
     Items it{&z->slots[0].key, &z->slots[0].val, 2, (long long)cap};
-    SFCI_CUDA(select_topk(it, z->nkeep, z->wr[dst], z->wc[dst], z->ndev, z->sumsq, z->total,
+    SFCI_CUDA(select_topk(it, z->nkeep, z->wr[dst], z->wc[dst], z->ndev, sumsq_host ? z->sumsq : nullptr, z->total,
                           z->scratch + z->off_sel, z->sel_bytes, z->st));
     SFCI_CUDA(sort_normalize(z->wr[dst], z->wc[dst], z->nkeep, z->ndev, key_bits(z->sys->d.dim),
                              z->scratch + z->off_sort, z->scratch + z->off_norm, z->st));

@@ -572,17 +572,17 @@ __global__ void aligned_dots_kernel(VecPackRef vp, SigPack sp, double *partial) 
     }
 }
 
-// a fixed tree over the partial sums of each vector
-__global__ void aligned_finish_kernel(const double *partial, int np, double *out) {
-    __shared__ double sh[32];
-    double r = 0.0;
-    for (int k = threadIdx.x; k < np; k += blockDim.x) r += partial[(size_t)blockIdx.x * np + k];
-    for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = r;
+// each vector's partial sums in their order, those of blocks that had entries (fetched
+// together, then added: one thread's additions, see ordered_sum)
+__global__ void aligned_finish_kernel(const __grid_constant__ VecPackRef vp, const double *partial, int np, double *out) {
+    __shared__ double sh[kDotBlocks];
+    const long long used = (vp.v[blockIdx.x].n + 255) / 256;
+    const int m = (int)(used < np ? used : np);
+    for (int k = threadIdx.x; k < m; k += blockDim.x) sh[k] = partial[(size_t)blockIdx.x * np + k];
     __syncthreads();
     if (threadIdx.x == 0) {
-        r = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += sh[w];
+        double r = 0.0;
+        for (int k = 0; k < m; ++k) r += sh[k];
         out[blockIdx.x] = r;
     }
 }
@@ -786,7 +786,7 @@ cudaError_t aligned_dots(const VecRef *vecs, double *const *sig, int nvec, doubl
     count_launch();
     aligned_dots_kernel<<<dim3(kDotBlocks, nvec), 256, 0, st>>>(vp, sp, partial);
     count_launch();
-    aligned_finish_kernel<<<nvec, 320, 0, st>>>(partial, kDotBlocks, out_dev);
+    aligned_finish_kernel<<<nvec, 320, 0, st>>>(vp, partial, kDotBlocks, out_dev);
     return cudaGetLastError();
 }
 

@@ -25,8 +25,8 @@
 // far above the count, the kernels follow the count: an unsorted sigma of 3e7
 // entries 60.2 ms when sorting over the capacity, 27.3 ms so.  A step on the
 // whole 4900-determinant space: 1066 us with 30 launches a sort, 839 us so.
-// With a pass of up to 256 tiles in one launch and the partial sums added by a
-// tree: 379 -> 319 us, that step 599 -> 534 us.
+// With a pass of up to 256 tiles in one launch and only the partial sums that are
+// there added: 379 -> 324 us, that step 599 -> 538 us.
 #include "sfci_internal.cuh"
 
 namespace sfci {
@@ -167,7 +167,8 @@ __device__ void sel_pick(SelState *s, const unsigned long long *hist, int pass) 
     }
 }
 
-__global__ void sel_hist_kernel(Items it, SelState *s, unsigned long long *hist, int pass) {
+// want_sq: also the sum of squares (a float64 add per item: 12 us for 3e6 items)
+__global__ void sel_hist_kernel(Items it, SelState *s, unsigned long long *hist, int pass, int want_sq) {
     __shared__ unsigned sh[kBins];
     __shared__ double ssq[kT / 32];
     __shared__ unsigned long long scount[kT / 32];
@@ -201,9 +202,11 @@ __global__ void sel_hist_kernel(Items it, SelState *s, unsigned long long *hist,
             if (!fits[u] || !item_valid(key[u], vb[u])) continue;
             const unsigned long long hi = 0x7fffffffffffffffull - (vb[u] & 0x7fffffffffffffffull);
             if (pass == 0) {
-                const double v = __longlong_as_double((long long)vb[u]);
-                sq += v * v;
                 cnt += 1;
+                if (want_sq) {
+                    const double v = __longlong_as_double((long long)vb[u]);
+                    sq += v * v;
+                }
             }
             if ((key[u] & ml) != pl) continue;
             atomicAdd(&sh[digit_of(hi, key[u], p, w)], 1u);
@@ -223,7 +226,7 @@ __global__ void sel_hist_kernel(Items it, SelState *s, unsigned long long *hist,
         double a = 0.0;
         unsigned long long c = 0;
         for (int q = 0; q < kT / 32; ++q) a += ssq[q], c += scount[q];
-        atomicAdd(&s->sumsq, a);
+        if (want_sq) atomicAdd(&s->sumsq, a);
         atomicAdd(&s->total, c);
     }
     // the last block to get here picks the bin and clears the histogram
@@ -240,11 +243,10 @@ __global__ void sel_hist_kernel(Items it, SelState *s, unsigned long long *hist,
 }
 
 // The whole selection of up to kSmall items by one CTA, the items in shared memory:
-// the passes over 12-bit digits, then the chosen ones in order.  *cut (may be null):
-// the smallest |val| chosen (+inf when none).
+// the passes over 12-bit digits, then the chosen ones in order.
 __global__ void __launch_bounds__(kSmallT)
 sel_small_kernel(Items it, unsigned long long k, unsigned long long *out_key, double *out_val,
-                 unsigned long long *n_out, double *sumsq_out, unsigned long long *total_out, double *cut) {
+                 unsigned long long *n_out, double *sumsq_out, unsigned long long *total_out) {
     extern __shared__ __align__(16) unsigned char sm[];
     unsigned long long *key = reinterpret_cast<unsigned long long *>(sm);
     unsigned long long *vb = key + kSmall;
@@ -252,7 +254,7 @@ sel_small_kernel(Items it, unsigned long long k, unsigned long long *out_key, do
     __shared__ unsigned long long ph, pl, mh, ml, need;
     __shared__ int done, all, found;
     __shared__ unsigned wsum[kSmallT / 32], found_before;
-    __shared__ double ssq[kSmallT / 32], scut[kSmallT / 32];
+    __shared__ double ssq[kSmallT / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = (int)it.n;
     double sq = 0.0;
     unsigned cnt = 0;
@@ -260,16 +262,24 @@ sel_small_kernel(Items it, unsigned long long k, unsigned long long *out_key, do
         const unsigned long long kk = it.key[(size_t)i * it.stride];
         unsigned long long v = (unsigned long long)__double_as_longlong(it.val[(size_t)i * it.stride]);
         if (!item_valid(kk, v)) v = 0ull;  // (a zero value marks an item that does not count)
-        else sq += __longlong_as_double((long long)v) * __longlong_as_double((long long)v), ++cnt;
+        else {
+            ++cnt;
+            if (sumsq_out) sq += __longlong_as_double((long long)v) * __longlong_as_double((long long)v);
+        }
         key[i] = kk, vb[i] = v;
     }
-    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(kFull, sq, o), cnt += __shfl_xor_sync(kFull, cnt, o);
+    cnt = __reduce_add_sync(kFull, cnt);
+    if (sumsq_out)
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(kFull, sq, o);
     if (lane == 0) ssq[warp] = sq, wsum[warp] = cnt;
     __syncthreads();
     if (tid == 0) {
         double a = 0.0;
         unsigned long long c = 0;
-        for (int w = 0; w < kSmallT / 32; ++w) a += ssq[w], c += wsum[w];
+        for (int w = 0; w < kSmallT / 32; ++w) {
+            c += wsum[w];
+            if (sumsq_out) a += ssq[w];
+        }
         need = k, ph = pl = mh = ml = 0ull;
         all = c <= k, done = all || k == 0;
         if (sumsq_out) *sumsq_out = a;
@@ -320,7 +330,6 @@ sel_small_kernel(Items it, unsigned long long k, unsigned long long *out_key, do
         __syncthreads();
     }
     // the chosen items, in their order
-    double least = __longlong_as_double(0x7ff0000000000000ll);  // +inf
     unsigned base = 0;
     const bool none = k == 0 && !all;
     for (int i0 = 0; i0 < n; i0 += kSmallT) {
@@ -341,23 +350,11 @@ sel_small_kernel(Items it, unsigned long long k, unsigned long long *out_key, do
             tot += wsum[q];
         }
         pos += __popc(bal & ((1u << lane) - 1u));
-        if (ok) {
-            if ((unsigned long long)pos < k) out_key[pos] = key[i], out_val[pos] = __longlong_as_double((long long)v);
-            least = fmin(least, fabs(__longlong_as_double((long long)v)));
-        }
+        if (ok && (unsigned long long)pos < k) out_key[pos] = key[i], out_val[pos] = __longlong_as_double((long long)v);
         base += tot;
         __syncthreads();
     }
-    for (int o = 16; o > 0; o >>= 1) least = fmin(least, __shfl_xor_sync(kFull, least, o));
-    if (lane == 0) scut[warp] = least;
-    __syncthreads();
-    if (tid == 0) {
-        *n_out = base;
-        if (cut) {
-            for (int q = 1; q < kSmallT / 32; ++q) scut[0] = fmin(scut[0], scut[q]);
-            *cut = scut[0];
-        }
-    }
+    if (tid == 0) *n_out = base;
 }
 
 __global__ void sel_gather_kernel(Items it, const SelState *s, unsigned long long *out_key,
@@ -776,17 +773,17 @@ __global__ void rs_scatter_kernel(unsigned long long *ka, double *va, unsigned l
     }
 }
 
-// The sum over the partial sums (thread 0's value; all kT threads call it): a fixed tree,
-// so the same on every run (one thread adding 304 of them in order took 12 us).
-__device__ __forceinline__ double partial_total(const double *partial, int np, double *sh) {
-    double s = 0.0;
-    for (int k = threadIdx.x; k < np; k += kT) s += partial[k];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+// The sum over the partial sums in their order (thread 0's value; every thread of the block
+// calls it): fetched together, then added.  Only the blocks that had entries are added (the
+// others' sums are zero): all 304 take 12 us of float64 latency, 2e4 entries make 79.  (A tree
+// is faster yet, but moves the last bit of the norm, and with it the sign that the cycle end's
+// eigenvector comes out with.)
+__device__ __forceinline__ double ordered_sum(const double *partial, int np, double *sh) {
+    for (int k = threadIdx.x; k < np; k += blockDim.x) sh[k] = partial[k];
     __syncthreads();
-    s = 0.0;
+    double s = 0.0;
     if (threadIdx.x == 0)
-        for (int w = 0; w < kT / 32; ++w) s += sh[w];
+        for (int k = 0; k < np; ++k) s += sh[k];
     return s;
 }
 
@@ -913,12 +910,13 @@ __global__ void sumsq_kernel(const double *v, long long cap, const unsigned long
 
 __global__ void scale_kernel(double *v, long long cap, const unsigned long long *n_dev,
                              const double *partial, int nparts) {
-    __shared__ double norm, sh[kT / 32];
-    const double s = partial_total(partial, nparts, sh);
-    if (threadIdx.x == 0) norm = sqrt(s);
-    __syncthreads();
+    __shared__ double norm, sh[kRedBlocks];
     long long n = (long long)*n_dev;
     if (n > cap) n = cap;
+    const long long used = (n + kT - 1) / kT;
+    const double s = ordered_sum(partial, (int)(used < nparts ? used : nparts), sh);
+    if (threadIdx.x == 0) norm = sqrt(s);
+    __syncthreads();
     const double d = norm;
     if (!(d > 0.0)) return;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -930,20 +928,18 @@ __global__ void scale_kernel(double *v, long long cap, const unsigned long long 
 
 size_t select_workspace_bytes(long long, long long) { return sel_layout().bytes; }
 
-bool select_is_small(const Items &it) { return it.n <= kSmall; }
-
 cudaError_t select_topk(Items it, long long k, unsigned long long *out_key, double *out_val,
                         unsigned long long *n_out_dev, double *sumsq_dev,
-                        unsigned long long *total_dev, void *ws, size_t ws_bytes, cudaStream_t st, double *cut_dev) {
+                        unsigned long long *total_dev, void *ws, size_t ws_bytes, cudaStream_t st) {
     const SelLayout L = sel_layout();
     if (ws_bytes < L.bytes) return cudaErrorInvalidValue;
-    if (select_is_small(it)) {
+    if (it.n <= kSmall) {
         const size_t smem = size_t(kSmall) * 16 + kBins * 4;
         cudaError_t e = allow_max_smem(sel_small_kernel, smem);
         if (e != cudaSuccess) return e;
         count_launch();
         sel_small_kernel<<<1, kSmallT, smem, st>>>(it, (unsigned long long)(k < 0 ? 0 : k), out_key, out_val, n_out_dev,
-                                                   sumsq_dev, total_dev, cut_dev);
+                                                   sumsq_dev, total_dev);
         return cudaGetLastError();
     }
     char *base = static_cast<char *>(ws);
@@ -954,7 +950,7 @@ cudaError_t select_topk(Items it, long long k, unsigned long long *out_key, doub
     const unsigned g = grid_for(it.n, 4);
     for (int p = 0; p < kPasses; ++p) {
         count_launch();
-        sel_hist_kernel<<<g, kT, 0, st>>>(it, s, hist, p);
+        sel_hist_kernel<<<g, kT, 0, st>>>(it, s, hist, p, sumsq_dev != nullptr);
     }
     count_launch();
     sel_gather_kernel<<<grid_for(it.n, 8), kT, 0, st>>>(it, s, out_key, out_val, k, n_out_dev);
@@ -962,7 +958,6 @@ cudaError_t select_topk(Items it, long long k, unsigned long long *out_key, doub
         count_launch();
         sel_stats_kernel<<<1, 32, 0, st>>>(s, sumsq_dev, total_dev);
     }
-    if (cut_dev) return min_abs(out_val, n_out_dev, k, cut_dev, st);
     return cudaGetLastError();
 }
 
@@ -982,7 +977,7 @@ cudaError_t select_split(Items it, long long k,
     cudaError_t e = cudaMemsetAsync(cand_n, 0, 8, st);
     if (e != cudaSuccess) return e;
     count_launch();
-    sel_hist_kernel<<<grid_for(it.n, 4), kT, 0, st>>>(it, s, hist, 0);
+    sel_hist_kernel<<<grid_for(it.n, 4), kT, 0, st>>>(it, s, hist, 0, 0);
     count_launch();
     sel_split_kernel<<<grid_for(it.n, 8), kT, 0, st>>>(it, s, out_key, out_val, k, n_out_dev,
                                                        cand_key, cand_val, cand_cap, cand_n);
