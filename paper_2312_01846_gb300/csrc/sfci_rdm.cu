@@ -268,8 +268,9 @@ __global__ void energy_finish(const double *partial, int np, double e_core, doub
 // strings: m / 2 comparisons a determinant against sb + C(nb,2) C(vb,2) lookups.
 // Pairs found wait in a queue per warp until 32 are there, and the diagonal's sums stay
 // with the CTA: 3e5 determinants of 20 orbitals 30.4 ms by lookups, 5.9 ms with each pair
-// worked on where it was found, 4.5 ms so (opposite spin 2.3, alpha 0.8, within rows 0.5);
-// 128 threads a CTA 5.9 ms, four CTAs an SM instead of five 4.7 ms.
+// worked on where it was found, 4.5 ms so (opposite spin 2.3, alpha 0.8, within rows 0.5),
+// 3.3 ms with short rows compared string by string (up to 64 determinants 3.9, 256 3.3);
+// 128 threads a CTA and four CTAs an SM instead of five were slower.
 
 constexpr int kT = 256;
 constexpr unsigned kChunk = 2048;       // determinants of a row in the table at once
@@ -417,12 +418,18 @@ __device__ __noinline__ void same_spin_pair(double *g1, double *g2, int n, unsig
     }
 }
 
+// Opposite spin: a row of up to so many determinants is compared string by string (16 warp
+// instructions per 32 pairs) instead of looking up every hop of the other row's (sb of them,
+// 25 per 32 lookups); most rows of a sparse vector hold a few determinants.
+constexpr unsigned kFew = 128;
+
 struct RowShared {
     unsigned keys[kSlots];
     unsigned short pos[kSlots];  // (pairs within a row: strings and coefficients in place of both)
     unsigned start[kT + 1], off[kT], hop[kT];
     unsigned wsum[kT / 32];
     unsigned long long queue[kT / 32][64];  // pairs found, each warp's
+    unsigned long long str[kFew];           // the strings of a row that is compared, not looked up in
     unsigned char occ[64], vir[64];
     unsigned long long u0;
     unsigned run;
@@ -617,6 +624,7 @@ __global__ void __launch_bounds__(kT, 5) rdm_rows_kernel(const __grid_constant__
                     unsigned h = (key * 0x9E3779B1u) >> shift;
                     while (atomicCAS(&S.keys[h], kNone, key) != kNone) h = (h + 1u) & mask;
                     S.pos[h] = (unsigned short)f;
+                    if (m <= kFew) S.str[f] = __ldg(&A.bstr[__ldg(&A.s_id[base + f])]);
                 }
             }
             // ---- a batch of rows one or two hops away: hop from them to this row
@@ -665,7 +673,40 @@ __global__ void __launch_bounds__(kT, 5) rdm_rows_kernel(const __grid_constant__
                     if (S.start[o + step] <= at) o += step;
                 return o;
             };
-            if (opposite) {
+            if (opposite && m <= kFew && m < 2u * d.sb) {
+                auto pair = [&](unsigned long long x) {
+                    const unsigned s = (unsigned)(x >> 32), hp = S.hop[(unsigned)x >> 16 & 0xffffu], f = (unsigned)x & 0xffffu;
+                    const double c1 = __ldg(&A.coef[s]), c2 = __ldg(&A.coef[base + f]);
+                    if (c1 == 0.0 || c2 == 0.0) return;
+                    const unsigned long long b1 = __ldg(&A.bstr[__ldg(&A.s_id[s])]), b2 = S.str[f];
+                    const int j = __ffsll((long long)(b1 & ~b2)) - 1, b = __ffsll((long long)(b2 & ~b1)) - 1;
+                    const double v = c1 * c2;
+                    acc(A.g2, size_t(hp & 0x7fffffffu) * N2 + b * n + j,
+                        (hp >> 31 ^ (unsigned)parity64(b1 & between_mask(j, b))) ? -v : v);
+                };
+                // a warp takes up to 32 determinants and runs through the row for each, end to end
+                const unsigned per = min(32u, (hi - lo + kT / 32 - 1u) / (kT / 32));
+                for (unsigned p0 = lo + warp * per; p0 < hi; p0 += per * (kT / 32)) {
+                    const unsigned k = min(per, hi - p0);
+                    unsigned o = 0, s = 0;
+                    unsigned long long bs = 0ull;
+                    if ((unsigned)lane < k) {
+                        o = segment(p0 + lane), s = S.off[o] + p0 + lane;
+                        bs = __ldg(&A.bstr[__ldg(&A.s_id[s])]);
+                    }
+                    unsigned l = (unsigned)lane / m, y = (unsigned)lane % m;
+                    const unsigned dl = 32u / m, dy = 32u % m;
+                    for (unsigned r = 0; r < k * m; r += 32u) {
+                        const unsigned src = l < k ? l : 0u;
+                        const unsigned long long b1 = __shfl_sync(kFull, bs, src);
+                        const unsigned s1 = __shfl_sync(kFull, s, src), o1 = __shfl_sync(kFull, o, src);
+                        push(l < k && __popcll(b1 ^ S.str[y]) == 2, (unsigned long long)s1 << 32 | o1 << 16 | y, pair);
+                        l += dl, y += dy;
+                        if (y >= m) y -= m, ++l;
+                    }
+                }
+                finish(pair);
+            } else if (opposite) {
                 // a warp takes up to 32 determinants and runs through their hops end to end
                 const unsigned per = min(32u, (hi - lo + kT / 32 - 1u) / (kT / 32));
                 for (unsigned p0 = lo + warp * per; p0 < hi; p0 += per * (kT / 32)) {
