@@ -27,6 +27,8 @@
 // whole 4900-determinant space: 1066 us with 30 launches a sort, 839 us so.
 // With a pass of up to 256 tiles in one launch and only the partial sums that are
 // there added: 379 -> 324 us, that step 599 -> 538 us.
+#include <algorithm>
+
 #include "sfci_internal.cuh"
 
 namespace sfci {
@@ -989,11 +991,16 @@ cudaError_t select_split(Items it, long long k,
 }
 
 namespace {
+// Counters of up to ntiles tiles: three buffers for a pass of up to kFusedTiles tiles in one
+// launch, one beyond.  Never less for more tiles: a caller may sort fewer pairs than its
+// workspace was sized for, and 257 tiles alone need a third of what 256 do.
 size_t sort_counts_bytes(long long ntiles) {
-    return a256(size_t(ntiles > 0 ? ntiles : 1) * kRadix * 4 * (ntiles <= kFusedTiles ? 3 : 1));
+    const long long fused = std::min<long long>(std::max<long long>(ntiles, 1), kFusedTiles);
+    return a256(size_t(std::max(3 * fused, ntiles)) * kRadix * 4);
 }
 }  // namespace
 
+// (grows with cap: sfci_sigma sizes it for out_cap and sorts the entries it found)
 size_t sort_pairs_bytes(long long cap) {
     const long long ntiles = (cap + kTile - 1) / kTile;
     return a256(size_t(cap) * 8) * 2 + sort_counts_bytes(ntiles) + a256(sizeof(SortState));
