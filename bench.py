@@ -565,6 +565,7 @@ def run_ours(a):
         warm.append(brief(lz.step()))
     barrier()
     launches0 = sf.kernel_launches()
+    rows0 = sf.row_sigmas()
     ev0 = torch.cuda.Event(enable_timing=True)
     ev1 = torch.cuda.Event(enable_timing=True)
     infos = []
@@ -577,6 +578,7 @@ def run_ours(a):
         ev1.record(stream)
         barrier()
     launches = sf.kernel_launches() - launches0
+    by_rows = sf.row_sigmas() - rows0 >= a.steps
     ms = ev0.elapsed_time(ev1)
     elements = sum(i["n_elements"] for i in infos)
     ms_max, elements_all = reduce_over_ranks(ms, elements, dist, "cuda")
@@ -584,10 +586,9 @@ def run_ours(a):
     steps_per_s = a.steps / (ms_max * 1e-3)
 
     # dominant stage: sigma = H w_i, timed with CUDA events on the solver's stream: by target
-    # rows (lists and tables in ms_emit, gather_kernel in ms_merge), or, when the bucketed
-    # path is shaped by an option, the emit kernel (writes each intermediate element once)
-    # plus the bucket merge (reads it once), which the 32 B/element model describes
-    by_rows = not (a.bucket_elems or a.emit_warps or a.mem_budget_gb)
+    # rows (lists and tables in ms_emit, gather_kernel in ms_merge), or, when some step took the
+    # bucketed path (an option shapes it, or memory), the emit kernel (writes each intermediate
+    # element once) plus the bucket merge (reads it once), which the 32 B/element model describes
     ms_sig = statistics.mean(i["ms_sigma"] for i in infos)
     ms_emit = statistics.mean(i["ms_emit"] for i in infos)
     ms_merge = statistics.mean(i["ms_merge"] for i in infos)

@@ -64,6 +64,10 @@ int sfci_version(void);
 /* Number of CUDA kernels the library has launched in this process so far
  * (a diagnostic: the difference across a region counts its launches). */
 int64_t sfci_kernel_launches(void);
+/* Number of sigmas (sfci_sigma, sfci_lanczos_step, sfci_scan_step) that were
+ * summed by target rows in this process so far; the others took the hash table
+ * or the buckets (a diagnostic: which path a call took). */
+int64_t sfci_row_sigmas(void);
 
 /* ------------------------------------------------------------- system */
 
@@ -400,6 +404,15 @@ sfci_status sfci_rdm_energy(int n_orb, const double *rdm1, const double *rdm2, d
 sfci_status sfci_debug_excitations(const sfci_system *sys, const uint64_t *rank, int64_t n,
                                    int64_t *src, uint64_t *tgt, double *elem, int64_t cap,
                                    int64_t *n_out, void *stream);
+
+/* Diagnostic of a solver's memory: *held (host, may be null) = device bytes of the
+ * buffers that sigma's two paths size from free memory (stream, target-row lists
+ * and tables, element regions, overflow lists).  share >= 0 replaces the device
+ * bytes that sigma may take (0: 85 % of what is free); alloc_limit >= 0: a
+ * target-row buffer above so many bytes counts as out of memory (0: none does).
+ * Negative values leave the setting as it is.  For tests of the fallbacks. */
+sfci_status sfci_debug_lanczos_memory(sfci_lanczos *lz, int64_t share, int64_t alloc_limit,
+                                      int64_t *held);
 
 /* Diagnostic: the rate (lane operations per second) of one SM pipe operation
  * that bounds the sigma kernels, measured alone on the current device with

@@ -77,6 +77,7 @@ def lib():
         "sfci_last_error": (C.c_char_p, []),
         "sfci_version": (_i32, []),
         "sfci_kernel_launches": (_i64, []),
+        "sfci_row_sigmas": (_i64, []),
         "sfci_lanczos_load": (_i32, [_vp, _vp, _vp, _i64]),
         "sfci_lanczos_set_input": (_i32, [_vp, _vp, _vp, _i64]),
         "sfci_system_create": (_i32, [C.POINTER(_vp), _i32, _i32, _i32, _vp, _vp, _f64, C.c_uint32]),
@@ -104,6 +105,7 @@ def lib():
                                    _vp]),
         "sfci_debug_pipe_rate": (_i32, [_i32, _i64, _vp, C.POINTER(_f64), _vp]),
         "sfci_debug_excitations": (_i32, [_vp, _vp, _i64, _vp, _vp, _vp, _i64, C.POINTER(_i64), _vp]),
+        "sfci_debug_lanczos_memory": (_i32, [_vp, _i64, _i64, C.POINTER(_i64)]),
         "sfci_scan_create": (_i32, [C.POINTER(_vp), _i32, C.POINTER(_vp), C.POINTER(Params),
                                     C.POINTER(_vp), C.POINTER(_vp), C.POINTER(_i64), _i32]),
         "sfci_scan_step": (_i32, [_vp, C.POINTER(StepInfo)]),
@@ -393,6 +395,13 @@ class Lanczos:
                "sfci_lanczos_vector")
         return r[: n.value], c[: n.value]
 
+    def debug_memory(self, share=-1, alloc_limit=-1):
+        """Bytes of sigma's large buffers; sets the solver's limits (sfci_debug_lanczos_memory)."""
+        held = C.c_int64()
+        _check(lib().sfci_debug_lanczos_memory(self.handle, int(share), int(alloc_limit), C.byref(held)),
+               "sfci_debug_lanczos_memory")
+        return held.value
+
     def matrices(self):
         import numpy as np
         NL = int(self.params.n_lanczos)
@@ -495,6 +504,11 @@ def pipe_rate(kind, iters=1 << 14, stream=None):
 def kernel_launches():
     """Kernels libsfci.so has launched in this process so far."""
     return int(lib().sfci_kernel_launches())
+
+
+def row_sigmas():
+    """Sigmas summed by target rows in this process so far (sfci_row_sigmas)."""
+    return int(lib().sfci_row_sigmas())
 
 
 def to_u64(t):

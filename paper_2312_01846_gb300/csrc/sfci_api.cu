@@ -14,11 +14,12 @@ namespace sfci {
 
 namespace {
 thread_local std::string g_last_error;
-std::atomic<long long> g_launches{0};
+std::atomic<long long> g_launches{0}, g_row_sigmas{0};
 }
 
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 long long launch_count() { return g_launches.load(std::memory_order_relaxed); }
+void count_row_sigma() { g_row_sigmas.fetch_add(1, std::memory_order_relaxed); }
 
 void set_error(const std::string &msg) { g_last_error = msg; }
 
@@ -125,6 +126,8 @@ const char *sfci_last_error(void) { return g_last_error.c_str(); }
 int sfci_version(void) { return 100; }
 
 int64_t sfci_kernel_launches(void) { return launch_count(); }
+
+int64_t sfci_row_sigmas(void) { return g_row_sigmas.load(std::memory_order_relaxed); }
 
 sfci_status sfci_system_create(sfci_system **out, int n, int na, int nb, const double *h_host,
                                const double *g_host, double e_core, uint32_t flags) {
@@ -433,6 +436,7 @@ sfci_status sigma_rows(const sfci_system *s, const unsigned long long *rank, con
     SFCI_CUDA(cudaMemcpyAsync(&hw, words, sizeof(hw), cudaMemcpyDeviceToHost, st));
     SFCI_CUDA(cudaStreamSynchronize(st));
     *done = true;
+    count_row_sigma();
     *n_out = hw.out;
     *n_dev = &words->out;
     if (hw.status & 32) {

@@ -169,6 +169,7 @@ namespace sfci {
 // every kernel launch of the library increments this host counter
 void count_launch();
 long long launch_count();
+void count_row_sigma();
 
 // ------------------------------------------------------------- shared memory
 // Let `func` use up to the device's opt-in shared memory per block, less its

@@ -264,6 +264,7 @@ struct sfci_lanczos {
     // sigma by target rows (sfci_gather.cu)
     bool gather_ok = false;             // the system is within its limits
     int64_t share = 0;                  // device bytes a batch leaves this solver (0: no batch)
+    int64_t alloc_limit = 0;            // a row gather buffer above it counts as out of memory (tests; 0: off)
     GatherShape gs{};
     Buf ga, gb, gc, vrp, seen;          // work arrays by the stage that sizes them; row pointers of each w_j;
                                         // elements and distinct entries by row weight
@@ -902,9 +903,16 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     double need = (double)size_a + (double)vrp_bytes + 16.0 * sig_need;
     if (!fits(have_a, need)) return SFCI_OK;
     SFCI_CUDA(cudaEventRecord(z->evp[0], z->st));
-    if ((r = ensure(z->ga, size_a, z->st, "row gather arrays", 1.25))) return r;
+    const auto grow = [&](sfci_lanczos::Buf &buf, size_t want, const char *what, double headroom) {
+        if (z->alloc_limit > 0 && want > (size_t)z->alloc_limit && buf.bytes < want) {
+            set_error(std::string(what) + ": above the allocation limit");
+            return SFCI_E_NOMEM;
+        }
+        return ensure(buf, want, z->st, what, headroom);
+    };
+    if ((r = grow(z->ga, size_a, "row gather arrays", 1.25))) return r;
     if (z->vrp.bytes < vrp_bytes) z->vrp_ok.assign(z->NL, 0);
-    if ((r = ensure(z->vrp, vrp_bytes, z->st, "row pointers"))) return r;
+    if ((r = grow(z->vrp, vrp_bytes, "row pointers", 1.0))) return r;
     gather_place_sources(static_cast<char *>(z->ga.p), b, d, gs, n_in);
     auto *vrp = P<unsigned>(z->vrp);
     for (int j = 0; j <= i; ++j)
@@ -926,7 +934,7 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     const size_t size_b = gather_place_tables(nullptr, b, d, gs, nd, n_in);
     const bool have_b = have_a && z->gb.bytes >= size_b;
     if (!gather_numbers(d, n_in, nd) || !fits(have_b, need + (double)size_b)) return SFCI_OK;
-    if ((r = ensure(z->gb, size_b, z->st, "row gather tables", 1.1))) return r;
+    if ((r = grow(z->gb, size_b, "row gather tables", 1.1))) return r;
     gather_place_tables(static_cast<char *>(z->gb.p), b, d, gs, nd, n_in);
     const RowPlanArgs ra = row_plan_args(d, gs, n_in);
     SFCI_CUDA(gather_tables(d, gs, n_in, (unsigned)nd, z->sys->pair_int, rp, b, ra, z->st));
@@ -935,7 +943,7 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     if (!gn.fit()) return SFCI_OK;
     const size_t size_c = gather_place_lists(nullptr, b, gs, gn);
     if (!fits(have_b && z->gc.bytes >= size_c, need + (double)size_b + (double)size_c)) return SFCI_OK;
-    if ((r = ensure(z->gc, size_c, z->st, "row gather lists", 1.1))) return r;
+    if ((r = grow(z->gc, size_c, "row gather lists", 1.1))) return r;
     gather_place_lists(static_cast<char *>(z->gc.p), b, gs, gn);
     SFCI_CUDA(gather_lists(d, gs, gn.act, gn.parts, z->sys->pair_int, rp, b, ra, z->st));
     for (int j = 0; j <= i; ++j)
@@ -947,8 +955,8 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     double tau = tau_start;
     for (int attempt = 0; attempt < 8; ++attempt) {
         const size_t want_sig = size_t(sig_need) * 8;
-        if ((r = ensure(z->sig_key, want_sig, z->st, "sigma keys", 1.1))) return r;
-        if ((r = ensure(z->sig_val, want_sig, z->st, "sigma values", 1.1))) return r;
+        if ((r = grow(z->sig_key, want_sig, "sigma keys", 1.1))) return r;
+        if ((r = grow(z->sig_val, want_sig, "sigma values", 1.1))) return r;
         z->sig_cap = (long long)(std::min(z->sig_key.bytes, z->sig_val.bytes) / 8);
         const long long u_room = 2 * z->nkeep + 1024;
         const long long out_cap = std::max<long long>(z->sig_cap - u_room, 0);
@@ -1020,6 +1028,7 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
         z->regions_gb = E * sizeof(Slot) / 1e9;  // what the elements would take as records
         z->ms_alloc = 0.0;
         *done = true;
+        count_row_sigma();
         return SFCI_OK;
     }
     set_error("sigma's stream did not fit after 8 attempts");
@@ -1060,6 +1069,18 @@ sfci_status sfci_lanczos_load(sfci_lanczos *z, const uint64_t *rank, const doubl
         return SFCI_E_INVALID;
     }
     return load_vector(z, rank, coef, n);
+}
+
+sfci_status sfci_debug_lanczos_memory(sfci_lanczos *z, int64_t share, int64_t alloc_limit, int64_t *held) {
+    if (!z) {
+        set_error("null argument");
+        return SFCI_E_INVALID;
+    }
+    if (share >= 0) z->share = share;
+    if (alloc_limit >= 0) z->alloc_limit = alloc_limit;
+    if (held) *held = (int64_t)(z->ga.bytes + z->gb.bytes + z->gc.bytes + z->vrp.bytes + z->sig_key.bytes +
+                                z->sig_val.bytes + z->belem.bytes + z->bovf.bytes + z->bovf_sorted.bytes);
+    return SFCI_OK;
 }
 
 sfci_status sfci_lanczos_set_input(sfci_lanczos *z, const uint64_t *rank, const double *coef, int64_t n) {
