@@ -19,6 +19,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <limits>
 #include <mutex>
 #include <string>
@@ -366,6 +367,33 @@ sfci_status ensure(sfci_lanczos::Buf &b, size_t want, cudaStream_t st, const cha
     return SFCI_OK;
 }
 
+// The large buffers that only one of sigma's two paths uses: each counts the other's as
+// room and frees them before it grows.
+double row_bytes(const sfci_lanczos *z) {
+    return (double)z->ga.bytes + (double)z->gb.bytes + (double)z->gc.bytes + (double)z->vrp.bytes;
+}
+double bucket_bytes(const sfci_lanczos *z) {
+    return (double)z->belem.bytes + (double)z->bovf.bytes + (double)z->bovf_sorted.bytes;
+}
+
+sfci_status free_buffers(sfci_lanczos *z, std::initializer_list<sfci_lanczos::Buf *> bufs) {
+    bool any = false;
+    for (auto *b : bufs) any |= b->p != nullptr;
+    if (!any) return SFCI_OK;
+    SFCI_CUDA(cudaStreamSynchronize(z->st));
+    for (auto *b : bufs) {
+        cudaFree(b->p);
+        b->p = nullptr;
+        b->bytes = 0;
+    }
+    return SFCI_OK;
+}
+sfci_status free_row_buffers(sfci_lanczos *z) {
+    if (z->vrp.p) z->vrp_ok.assign(z->NL, 0);
+    return free_buffers(z, {&z->ga, &z->gb, &z->gc, &z->vrp});
+}
+sfci_status free_bucket_buffers(sfci_lanczos *z) { return free_buffers(z, {&z->belem, &z->bovf, &z->bovf_sorted}); }
+
 template <class T>
 T *P(const sfci_lanczos::Buf &b) {
     return static_cast<T *>(b.p);
@@ -534,8 +562,7 @@ sfci_status bucketed_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long
         size_t free_b = 0, tot_b = 0;
         SFCI_CUDA(cudaMemGetInfo(&free_b, &tot_b));
         // memory the element regions may use: what is free plus what the big buffers hold
-        const double held = (double)z->belem.bytes + (double)z->sig_key.bytes + (double)z->sig_val.bytes +
-                            (double)z->bovf.bytes + (double)z->bovf_sorted.bytes;
+        const double held = row_bytes(z) + bucket_bytes(z) + (double)z->sig_key.bytes + (double)z->sig_val.bytes;
         double avail = 0.85 * ((double)free_b + held);
         if (z->p.mem_budget > 0) avail = std::min(avail, (double)z->p.mem_budget);
         if (z->share > 0) avail = std::min(avail, (double)z->share);
@@ -584,12 +611,8 @@ sfci_status bucketed_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long
             // from one budget: free them all; the element regions get 5 % headroom,
             // the stream 10 %, and the overflow lists what is left (a longer list
             // saves splitting passes), up to a fifth of the elements each
-            SFCI_CUDA(cudaStreamSynchronize(z->st));
-            for (auto *bb : {&z->belem, &z->sig_key, &z->sig_val, &z->bovf, &z->bovf_sorted}) {
-                cudaFree(bb->p);
-                bb->p = nullptr;
-                bb->bytes = 0;
-            }
+            if ((r = free_buffers(z, {&z->belem, &z->sig_key, &z->sig_val, &z->bovf, &z->bovf_sorted}))) return r;
+            if ((r = free_row_buffers(z))) return r;
             want_sig = size_t(1.1 * sig_need) * 8;
             const size_t want_elem = size_t(std::min((double)need_elem * 1.05, budget));
             const double left = avail - sig_bytes - (double)want_elem;
@@ -856,11 +879,12 @@ sfci_status bucketed_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long
     return SFCI_E_CAPACITY;
 }
 
-// device bytes that sigma's buffers may take in all
-double sigma_budget(const sfci_lanczos *z, double held) {
+// device bytes that sigma's buffers may take in all: of what is free and what both paths hold
+double sigma_budget(const sfci_lanczos *z) {
     size_t free_b = 0, tot_b = 0;
     cudaMemGetInfo(&free_b, &tot_b);
-    const double avail = 0.85 * ((double)free_b + held);
+    const double avail = 0.85 * ((double)free_b + row_bytes(z) + bucket_bytes(z) + (double)z->sig_key.bytes +
+                                 (double)z->sig_val.bytes);
     return z->share > 0 ? std::min(avail, (double)z->share) : avail;
 }
 
@@ -873,9 +897,9 @@ bool gather_wanted(const sfci_lanczos *z) {
 }
 
 // sigma_i = H w_i by target rows, with sigma recorded at every basis entry;
-// results as bucketed_sigma's.  *done = false: its tables do not fit in memory
-// (the caller takes the bucketed path).
-sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long long *n_out, unsigned long long *n_live,
+// results as bucketed_sigma's.  *done = false: its tables do not fit in memory (also
+// SFCI_E_NOMEM then: an allocation failed).
+sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long *n_out, unsigned long long *n_live,
                          unsigned long long *n_nonzero, double *sumsq, bool *done) {
     *done = false;
     const SysDev &d = z->sys->d;
@@ -889,26 +913,27 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     // (room for what every CTA streams before the first raise of a zero threshold can act)
     double sig_need = std::min(std::max(16.0 * (double)z->nkeep, 8.0e6), E) + 2.0 * (double)z->nkeep + 1024.0;
     const size_t vrp_bytes = size_t(z->NL) * (size_t(d.ca) + 1) * 4;
-    const double held = (double)z->ga.bytes + z->gb.bytes + z->gc.bytes + z->vrp.bytes + z->sig_key.bytes +
-                        z->sig_val.bytes + z->belem.bytes + z->bovf.bytes + z->bovf_sorted.bytes;
+    const double held = row_bytes(z) + bucket_bytes(z) + (double)z->sig_key.bytes + (double)z->sig_val.bytes;
     // (the driver is asked for the free memory only when a buffer has to grow)
     double budget = -1.0;
     const auto fits = [&](bool have, double bytes) {
         if (have) return true;
-        if (budget < 0.0) budget = sigma_budget(z, held);
+        if (budget < 0.0) budget = sigma_budget(z);
         return bytes <= budget;
     };
     const bool have_a = z->ga.bytes >= size_a && z->vrp.bytes >= vrp_bytes &&
                         (double)std::min(z->sig_key.bytes, z->sig_val.bytes) >= 8.0 * sig_need;
-    double need = (double)size_a + (double)vrp_bytes + 16.0 * sig_need;
+    double need = 1.25 * (double)size_a + (double)vrp_bytes + 1.1 * 16.0 * sig_need;  // (as grown below)
     if (!fits(have_a, need)) return SFCI_OK;
     SFCI_CUDA(cudaEventRecord(z->evp[0], z->st));
     const auto grow = [&](sfci_lanczos::Buf &buf, size_t want, const char *what, double headroom) {
-        if (z->alloc_limit > 0 && want > (size_t)z->alloc_limit && buf.bytes < want) {
+        if (buf.p && buf.bytes >= want) return SFCI_OK;
+        if (z->alloc_limit > 0 && want > (size_t)z->alloc_limit) {
             set_error(std::string(what) + ": above the allocation limit");
             return SFCI_E_NOMEM;
         }
-        return ensure(buf, want, z->st, what, headroom);
+        const sfci_status f = free_bucket_buffers(z);  // (counted as room by the budget)
+        return f == SFCI_OK ? ensure(buf, want, z->st, what, headroom) : f;
     };
     if ((r = grow(z->ga, size_a, "row gather arrays", 1.25))) return r;
     if (z->vrp.bytes < vrp_bytes) z->vrp_ok.assign(z->NL, 0);
@@ -933,7 +958,7 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     const unsigned long long nd = z->host->nd, runs = z->host->runs;
     const size_t size_b = gather_place_tables(nullptr, b, d, gs, nd, n_in);
     const bool have_b = have_a && z->gb.bytes >= size_b;
-    if (!gather_numbers(d, n_in, nd) || !fits(have_b, need + (double)size_b)) return SFCI_OK;
+    if (!gather_numbers(d, n_in, nd) || !fits(have_b, need += 1.1 * (double)size_b)) return SFCI_OK;
     if ((r = grow(z->gb, size_b, "row gather tables", 1.1))) return r;
     gather_place_tables(static_cast<char *>(z->gb.p), b, d, gs, nd, n_in);
     const RowPlanArgs ra = row_plan_args(d, gs, n_in);
@@ -942,12 +967,16 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     const GatherCounts gn = z->host->counts;
     if (!gn.fit()) return SFCI_OK;
     const size_t size_c = gather_place_lists(nullptr, b, gs, gn);
-    if (!fits(have_b && z->gc.bytes >= size_c, need + (double)size_b + (double)size_c)) return SFCI_OK;
+    if (!fits(have_b && z->gc.bytes >= size_c, need + 1.1 * (double)size_c)) return SFCI_OK;
     if ((r = grow(z->gc, size_c, "row gather lists", 1.1))) return r;
     gather_place_lists(static_cast<char *>(z->gc.p), b, gs, gn);
     SFCI_CUDA(gather_lists(d, gs, gn.act, gn.parts, z->sys->pair_int, rp, b, ra, z->st));
     for (int j = 0; j <= i; ++j)
-        if (!z->sigw[j]) SFCI_CUDA(cudaMalloc(&z->sigw[j], size_t(z->nkeep) * 8));
+        if (!z->sigw[j] && cudaMalloc(&z->sigw[j], size_t(z->nkeep) * 8) != cudaSuccess) {
+            z->sigw[j] = nullptr;
+            set_error("cudaMalloc sigma at a basis vector's entries: out of memory");
+            return SFCI_E_NOMEM;
+        }
     SFCI_CUDA(zero_vectors(z->sigw, z->wn.data(), i + 1, z->st));  // rows without elements
     int fix_shift = (int)std::floor(125.0 - std::log2(std::max(1e-300, (double)(d.n_conn + 1) * d.hbound)));
     fix_shift = std::max(-900, std::min(1000, fix_shift));
@@ -1033,6 +1062,15 @@ sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long l
     }
     set_error("sigma's stream did not fit after 8 attempts");
     return SFCI_E_CAPACITY;
+}
+
+// sum_rows, where a lack of memory is no error: the bucketed path works in whatever there is
+sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long long *n_out, unsigned long long *n_live,
+                         unsigned long long *n_nonzero, double *sumsq, bool *done) {
+    const sfci_status r = sum_rows(z, i, tau_io, n_out, n_live, n_nonzero, sumsq, done);
+    if (r != SFCI_E_NOMEM) return r;
+    cudaGetLastError();  // (the failed allocation's, which a launch check would report)
+    return SFCI_OK;
 }
 
 // w_0 = normalise(top_{N_d}(trial vector)); a new cycle begins
