@@ -270,6 +270,8 @@ struct sfci_lanczos {
     Buf ga, gb, gc, vrp, seen;          // work arrays by the stage that sizes them; row pointers of each w_j;
                                         // elements and distinct entries by row weight
     std::vector<char> vrp_ok;           // row pointers of w_j are current
+    long long no_rows_n = 0;            // the last input whose lists did not fit (0: none yet),
+    double no_rows_budget = 0.0;        // in so many bytes
 };
 
 namespace {
@@ -1064,12 +1066,20 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
     return SFCI_E_CAPACITY;
 }
 
-// sum_rows, where a lack of memory is no error: the bucketed path works in whatever there is
+// sum_rows, where a lack of memory is no error: the bucketed path works in whatever there is,
+// so the row path leaves no buffer behind.  Vectors as long are not prepared again for nothing
+// while there is no more memory than there was.
 sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long long *n_out, unsigned long long *n_live,
                          unsigned long long *n_nonzero, double *sumsq, bool *done) {
+    *done = false;
+    if (z->no_rows_n > 0 && z->wn[i] >= z->no_rows_n && sigma_budget(z) <= 1.1 * z->no_rows_budget) return SFCI_OK;
     const sfci_status r = sum_rows(z, i, tau_io, n_out, n_live, n_nonzero, sumsq, done);
-    if (r != SFCI_E_NOMEM) return r;
-    cudaGetLastError();  // (the failed allocation's, which a launch check would report)
+    if (*done || (r != SFCI_OK && r != SFCI_E_NOMEM)) return r;
+    if (r == SFCI_E_NOMEM) cudaGetLastError();  // (the failed allocation's, which a launch check would report)
+    const sfci_status f = free_row_buffers(z);
+    if (f != SFCI_OK) return f;
+    z->no_rows_budget = sigma_budget(z);
+    z->no_rows_n = z->wn[i];
     return SFCI_OK;
 }
 

@@ -71,6 +71,22 @@ def test_out_of_memory(sf, inputs, alloc_limit):
     ref.close()
 
 
+def test_declined_late(sf, inputs):
+    _, vecs = inputs
+    lz, ref = _solver(sf, inputs, share=SHARE), _solver(sf, inputs, share=SHARE, emit_warps=8)
+    want = [_step(sf, ref, vecs[KEEP]) for _ in range(2)]
+    got = _step(sf, lz, vecs[KEEP])
+    assert got[0] == 0 and _same(got, want[0])
+    assert lz.debug_memory() <= SHARE  # nothing of the rows is left beside the buckets
+    again = _step(sf, lz, vecs[KEEP])
+    assert again[0] == 0 and _same(again, want[1])
+    assert again[1] == want[1][1]  # no preparation that is thrown away
+    lz.debug_memory(share=0)  # memory came back
+    assert _step(sf, lz, vecs[KEEP])[0] == 1
+    lz.close()
+    ref.close()
+
+
 def test_short_after_long(sf, inputs):
     """A vector whose lists fit, after one whose lists did not: the buckets' regions make room."""
     _, vecs = inputs
