@@ -196,8 +196,10 @@ sfci_status sfci_truncate_topk_noalloc(const uint64_t *rank, const double *coef,
 
 /* Sigma is summed by target rows (no intermediate elements in memory) unless the
  * caller shapes the bucketed path below (flags, bucket_elems, mem_budget, emit_warps or
- * ovf_max_log2 not 0), a spin has more than 12 electrons or 2^26 strings, or its lists
- * do not fit in memory.  Both sum exactly: the results are the same bits. */
+ * ovf_max_log2 not 0), a spin has more than 12 electrons or 2^26 strings, its lists do
+ * not fit in memory, or the buckets are faster: a short vector in a space of many alpha
+ * strings, or most of its entries on few alpha strings of a large space.  Both sum
+ * exactly: the results are the same bits. */
 typedef struct sfci_params {
     int64_t n_keep;         /* N_d: entries kept per basis vector (Eq. 11)          */
     int64_t table_capacity; /* slots of sigma's hash table; 0 = sized automatically */

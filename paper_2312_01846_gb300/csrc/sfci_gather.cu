@@ -53,6 +53,7 @@ constexpr int kMaxE = kGatherMaxElectrons;
 constexpr int kLT = 256;          // list CTA threads
 constexpr unsigned kMaxParts = 512;
 constexpr int kMaxClassLog = 11;  // log2 of the most classes a row is planned in
+constexpr unsigned long long kSeenEnough = 1000;  // entries from which a weight's statistics count
 
 // ------------------------------------------------------------- helpers
 
@@ -543,6 +544,11 @@ __device__ __forceinline__ int weight_bin(unsigned long long w) {  // half octav
     return 2 * l + (l > 0 ? (int)((w >> (l - 1)) & 1ull) : 0);
 }
 
+__device__ __forceinline__ unsigned class_count(const RowPlan &r, double entries) {
+    const unsigned n = (unsigned)ceil(entries / r.fill), most = r.bb > kGLog ? 1u << min(r.bb - kGLog, kMaxClassLog) : 1u;
+    return n < 1u ? 1u : n < most ? n : most;
+}
+
 // Classes of a heavy row, from the distinct entries expected of it: elements over 1.6
 // (w / 1024)^(1/4), moved towards what the rows of its weight had in the last sigmas (what truncated Lanczos vectors of 28 orbitals show: 1.6 at
 // 1e3 elements, 3.6 at 1.6e4, 6.5 at 3e5, 16 at 4e6).  Only a plan: a class that
@@ -551,27 +557,40 @@ __device__ __forceinline__ unsigned row_classes(const RowPlan &r, unsigned long 
     const int b = weight_bin(w);
     const unsigned long long e = r.seen[2 * b], x = r.seen[2 * b + 1];
     double est = (double)w / (1.6 * sqrt(sqrt((double)w / 1024.0)));
-    if (x > 1000ull) {
+    if (x > kSeenEnough) {
         const double was = (double)w * ((double)x / (double)e);
         est = was > est ? was : sqrt(was * est);
     }
-    if (est > r.cb) est = r.cb;
-    const unsigned n = (unsigned)ceil(est / r.fill), most = r.bb > kGLog ? 1u << min(r.bb - kGLog, kMaxClassLog) : 1u;
-    return n < 1u ? 1u : n < most ? n : most;
+    return class_count(r, est > r.cb ? r.cb : est);
 }
 
 // per active row: units it opens (a heavy row one per class, a light row one if
 // it is the first of its group: the light rows whose weight prefix starts in
 // one window of half a group)
+// visits: sources that its classes read, summed over the heavy rows; own ones count four
+// times (their segments are longer).  A row of a weight that no sigma has shown yet counts
+// 23 / 32 of the classes it would have if its elements were scattered over all strings: the
+// first plan's guess is for vectors like Lanczos', and scattered ones split each class again
+// and again.
 __global__ void row_units_kernel(RowPlan rp, const unsigned long long *aw, const unsigned long long *wpre,
-                                 const unsigned long long *n_act, unsigned *nu) {
+                                 const unsigned long long *n_act, const unsigned *nab, const unsigned *row,
+                                 const unsigned *src, unsigned *nu, unsigned long long *visits) {
     const unsigned long long A = *n_act;
+    unsigned long long sum = 0ull;
     for (unsigned long long k = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; k < A;
          k += (unsigned long long)gridDim.x * blockDim.x) {
         const unsigned long long w = aw[k];
-        if (w > rp.half) nu[k] = row_classes(rp, w);
-        else nu[k] = k == 0 || aw[k - 1] > rp.half || wpre[k - 1] / rp.half != wpre[k] / rp.half;
+        if (w > rp.half) {
+            const unsigned n = row_classes(rp, w);
+            nu[k] = n;
+            const unsigned long long v = nab[k] + 4ull * (src[row[k] + 1] - src[row[k]]);
+            const bool seen = rp.seen[2 * weight_bin(w) + 1] > kSeenEnough;
+            const unsigned m = seen ? n : class_count(rp, -rp.cb * expm1(-(double)w / rp.cb));
+            if (m > 1u) sum += seen ? m * v : m * v * 23ull / 32ull;
+        } else nu[k] = k == 0 || aw[k - 1] > rp.half || wpre[k - 1] / rp.half != wpre[k] / rp.half;
     }
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+    if ((threadIdx.x & 31) == 0 && sum) atomicAdd(visits, sum);
 }
 
 __global__ void write_units_kernel(RowPlan rp, const unsigned long long *aw, const unsigned long long *wpre,
@@ -1414,7 +1433,7 @@ struct Arena {
 size_t gather_place_sources(char *base, GatherBufs &b, const SysDev &d, const GatherShape &p, long long n) {
     Arena a{base};
     const size_t ca = size_t(d.ca), cb = size_t(d.cb);
-    b.words = a.take<unsigned long long>(8);
+    b.words = a.take<unsigned long long>(16);
     b.skey = a.take<unsigned long long>(n);
     b.sc = a.take<double>(n);
     b.sort_ws = a.take<char>(p.bb > kGLog ? sort_pairs_bytes(n) : 0);
@@ -1480,6 +1499,34 @@ bool gather_numbers(const SysDev &d, long long n, unsigned long long nd) {
            (double)n * std::max(d.po_a, d.na) < 4294967296.0;
 }
 
+// Sigma by target rows against the buckets (330 systems of 8 to 64 orbitals with random and with
+// level-like vectors, 10 to 3e5 determinants, both ways timed).  Besides its elements, 16 ps each
+// against 31 to 39, the row path pays for
+//  * every row of the space, 70 + 3.65 ps per substring of its string (the buckets: 62), and 0.25 ns
+//    per row that a source reaches; it saves about 1.2 ms of the buckets' launches and read-backs.
+//    28 orbitals with 12 + 12 electrons (3e7 rows): 30 determinants 11.9 ms by rows, 3.9 by buckets,
+//    1e4 35 and 24, 1e5 100 and 98; with 7 + 7 (1.2e6 rows) rows win from one determinant on (0.8 and 1.9).
+//    Without opposite-spin elements (no singles of one spin) all are records or own doubles, and
+//    the buckets win from 1e7 elements on (28 orbitals, 7 electrons: 1.70 ms and 2.58).
+bool gather_pays(const SysDev &d, long long n) {
+    const double ca = (double)d.ca, subs = d.na + d.po_a, hops = 1.0 + d.sa + (double)d.po_a * d.pv_a;
+    const double elements = (double)n * (double)(d.n_conn + 1);
+    if ((d.sa == 0 || d.sb == 0) && elements > 1e7) return false;
+    return ca * (8.0 + 3.65 * subs) + 250.0 * std::min(ca, n * hops) <= 1.2e9 + 4.0 * elements;
+}
+
+//  * every class of a heavy row that a source is read for, 12 to 44 ps: where few rows hold most
+//    sources, classes outnumber the excitations of a string and most visits find nothing.  Up to
+//    0.65 visits per element (truncated Lanczos vectors of 28 orbitals: 0.01 to 0.42, rows 815 ms
+//    and buckets 973 at 0.42; ten rows of 2500 sources of 29 orbitals, 1 + 10 electrons: 4.4,
+//    105 ms and 14).
+//  * a chip that a few units leave idle: 3.5 ns per element of a unit (30 rows of 9e5 elements:
+//    3.8 ms, buckets 3.1).
+bool gather_pays(const SysDev &d, long long n, const GatherCounts &c) {
+    const double elements = (double)n * (double)(d.n_conn + 1);
+    return (double)c.visits <= 0.65 * elements && (c.units >= 152 || elements <= 5e5 * (double)c.units);
+}
+
 RowPlanArgs row_plan_args(const SysDev &d, const GatherShape &p, long long n) {
     RowPlanArgs ra{};
     // a warp makes 128 to 1024 list items: as many warps as the chip holds twice, where there are enough
@@ -1494,7 +1541,7 @@ RowPlanArgs row_plan_args(const SysDev &d, const GatherShape &p, long long n) {
 }
 
 cudaError_t gather_counts(const SysDev &d, const GatherBufs &b, GatherCounts *n, cudaStream_t st) {
-    static_assert(sizeof(GatherCounts) == 40, "five words behind words[3]");
+    static_assert(sizeof(GatherCounts) == 48, "five words behind words[3], then the visits");
     count_launch();
     pack_counts_kernel<<<1, 32, 0, st>>>(b.apos + d.ca, b.uoff + d.ca, b.poff + d.ca, b.rec_off + d.ca, b.ab_off + d.ca,
                                          b.words + 3);
@@ -1539,7 +1586,7 @@ cudaError_t launch_row_pointers(const SysDev &d, const unsigned long long *rank,
 cudaError_t gather_sources(const SysDev &d, const GatherShape &p, const unsigned long long *rank, const double *coef,
                            long long n, const GatherBufs &b, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(b.bflag, 0, size_t(d.cb) * 4, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b.words, 0, 64, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b.words, 0, 128, st);
     if (e != cudaSuccess) return e;
     count_launch();
     sources_kernel<<<grid_for(n, 256), 256, 0, st>>>(p, rank, coef, n, d.cb, b.skey, b.sc, b.bflag, b.words, b.seen);
@@ -1590,7 +1637,8 @@ cudaError_t gather_tables(const SysDev &d, const GatherShape &p, long long n, un
     e = exclusive_scan(static_cast<const unsigned long long *>(b.aw), (long long)d.ca, b.wpre, b.scan_ws, st);
     if (e != cudaSuccess) return e;
     count_launch();
-    row_units_kernel<<<grid_for(d.ca, 256), 256, 0, st>>>(row_plan(d, p, b, ra), b.aw, b.wpre, b.apos + d.ca, b.nu);
+    row_units_kernel<<<grid_for(d.ca, 256), 256, 0, st>>>(row_plan(d, p, b, ra), b.aw, b.wpre, b.apos + d.ca, b.nab,
+                                                          b.act_row, rp, b.nu, b.words + 8);
     unsigned long long *const out[4] = {b.rec_off, b.ab_off, b.poff, b.uoff};  // nrec | nab | np | nu
     return exclusive_scan4(b.nrec, (long long)d.ca, out, b.scan_ws, st);
 }

@@ -615,7 +615,7 @@ struct GatherUnit {
 static_assert(sizeof(GatherUnit) == 64, "read as four 16-byte words");
 constexpr int kSeenBins = 128;
 struct GatherBufs {
-    unsigned long long *words;  // [8]: runs, n, rows summed in classes, GatherCounts
+    unsigned long long *words;  // [16]: runs, n, rows summed in classes, GatherCounts
     unsigned long long *skey;   // [n] row << bb | pi(beta), runs in the order of pi
     double *sc;                 // [n]
     void *sort_ws, *scan_ws;
@@ -651,6 +651,7 @@ struct GatherBufs {
 };
 struct GatherCounts {  // as planned: rows with elements, units, list parts, records, one-hop sources
     unsigned long long act, units, parts, rec, ab;
+    unsigned long long visits;  // see gather_pays
     bool fit() const { return units < (1ull << 31) && parts < (1ull << 31) && ab < (1ull << 32); }
 };
 struct ListArgs {
@@ -719,6 +720,9 @@ struct GatherArgs {
     int *status;
 };
 bool gather_shape(const SysDev &d, GatherShape *p);  // false: the system is outside the gather's limits
+// whether sigma by target rows is faster than the buckets: before anything is prepared, and as planned
+bool gather_pays(const SysDev &d, long long n);
+bool gather_pays(const SysDev &d, long long n, const GatherCounts &c);
 // its buffers in three parts, each placed when the counts it depends on are known: bytes
 // taken, pointers from base on (base null: sizes only)
 size_t gather_place_sources(char *base, GatherBufs &b, const SysDev &d, const GatherShape &p, long long n);

@@ -272,6 +272,8 @@ struct sfci_lanczos {
     std::vector<char> vrp_ok;           // row pointers of w_j are current
     long long no_rows_n = 0;            // the last input whose lists did not fit (0: none yet),
     double no_rows_budget = 0.0;        // in so many bytes
+    int rows_skip = 0, rows_wait = 0;   // sigmas that still go to the buckets without a plan by rows; after the next
+                                        // plan that does not pay
 };
 
 namespace {
@@ -614,13 +616,14 @@ sfci_status bucketed_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long
             // the stream 10 %, and the overflow lists what is left (a longer list
             // saves splitting passes), up to a fifth of the elements each
             if ((r = free_buffers(z, {&z->belem, &z->sig_key, &z->sig_val, &z->bovf, &z->bovf_sorted}))) return r;
-            if ((r = free_row_buffers(z))) return r;
             want_sig = size_t(1.1 * sig_need) * 8;
             const size_t want_elem = size_t(std::min((double)need_elem * 1.05, budget));
             const double left = avail - sig_bytes - (double)want_elem;
             const double ovf_room = std::min({left / (2.0 * sizeof(Slot)), 0.2 * E + (double)(1 << 22),
                                               (double)ovf_lim});
             const size_t want_ovf = size_t(std::max((double)ovf_cap, ovf_room)) * sizeof(Slot);
+            if (sig_bytes + (double)want_elem + 2.0 * (double)want_ovf + row_bytes(z) > avail && (r = free_row_buffers(z)))
+                return r;
             if ((r = ensure(z->sig_key, want_sig, z->st, "sigma keys"))) return r;
             if ((r = ensure(z->sig_val, want_sig, z->st, "sigma values"))) return r;
             if ((r = ensure(z->bovf, want_ovf, z->st, "overflow list"))) return r;
@@ -892,18 +895,18 @@ double sigma_budget(const sfci_lanczos *z) {
 
 // Sigma by target rows is taken unless the caller shapes the bucketed path
 // (bucket size, memory budget, overflow limit, launch shape, stress flag) or
-// the system is outside its limits.
+// the system is outside its limits, or the space too large for so short a vector.
 bool gather_wanted(const sfci_lanczos *z) {
     return z->gather_ok && z->p.bucket_elems == 0 && z->p.mem_budget == 0 && z->p.ovf_max_log2 == 0 &&
-           z->p.emit_warps == 0 && z->p.flags == 0;
+           z->p.emit_warps == 0 && z->p.flags == 0 && gather_pays(z->sys->d, z->wn[z->idx]);
 }
 
 // sigma_i = H w_i by target rows, with sigma recorded at every basis entry;
 // results as bucketed_sigma's.  *done = false: its tables do not fit in memory (also
-// SFCI_E_NOMEM then: an allocation failed).
+// SFCI_E_NOMEM then: an allocation failed), or *slow = true: the buckets are faster.
 sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long *n_out, unsigned long long *n_live,
-                         unsigned long long *n_nonzero, double *sumsq, bool *done) {
-    *done = false;
+                     unsigned long long *n_nonzero, double *sumsq, bool *done, bool *slow) {
+    *done = *slow = false;
     const SysDev &d = z->sys->d;
     const GatherShape &gs = z->gs;
     const long long n_in = z->wn[i];
@@ -934,8 +937,15 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
             set_error(std::string(what) + ": above the allocation limit");
             return SFCI_E_NOMEM;
         }
-        const sfci_status f = free_bucket_buffers(z);  // (counted as room by the budget)
-        return f == SFCI_OK ? ensure(buf, want, z->st, what, headroom) : f;
+        fits(false, 0.0);  // (budget)
+        sfci_status f = need + bucket_bytes(z) > budget ? free_bucket_buffers(z) : SFCI_OK;
+        if (f == SFCI_OK) f = ensure(buf, want, z->st, what, headroom);
+        if (f == SFCI_E_NOMEM && bucket_bytes(z) > 0.0) {
+            cudaGetLastError();
+            f = free_bucket_buffers(z);
+            if (f == SFCI_OK) f = ensure(buf, want, z->st, what, headroom);
+        }
+        return f;
     };
     if ((r = grow(z->ga, size_a, "row gather arrays", 1.25))) return r;
     if (z->vrp.bytes < vrp_bytes) z->vrp_ok.assign(z->NL, 0);
@@ -968,8 +978,12 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
     SFCI_CUDA(gather_counts(d, b, &z->host->counts, z->st));
     const GatherCounts gn = z->host->counts;
     if (!gn.fit()) return SFCI_OK;
+    if (!gather_pays(d, n_in, gn)) {
+        *slow = true;
+        return SFCI_OK;
+    }
     const size_t size_c = gather_place_lists(nullptr, b, gs, gn);
-    if (!fits(have_b && z->gc.bytes >= size_c, need + 1.1 * (double)size_c)) return SFCI_OK;
+    if (!fits(have_b && z->gc.bytes >= size_c, need += 1.1 * (double)size_c)) return SFCI_OK;
     if ((r = grow(z->gc, size_c, "row gather lists", 1.1))) return r;
     gather_place_lists(static_cast<char *>(z->gc.p), b, gs, gn);
     SFCI_CUDA(gather_lists(d, gs, gn.act, gn.parts, z->sys->pair_int, rp, b, ra, z->st));
@@ -1072,9 +1086,19 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
 sfci_status gather_sigma(sfci_lanczos *z, int i, double *tau_io, unsigned long long *n_out, unsigned long long *n_live,
                          unsigned long long *n_nonzero, double *sumsq, bool *done) {
     *done = false;
+    if (z->rows_skip > 0) {
+        --z->rows_skip;
+        return SFCI_OK;
+    }
     if (z->no_rows_n > 0 && z->wn[i] >= z->no_rows_n && sigma_budget(z) <= 1.1 * z->no_rows_budget) return SFCI_OK;
-    const sfci_status r = sum_rows(z, i, tau_io, n_out, n_live, n_nonzero, sumsq, done);
+    bool slow = false;
+    const sfci_status r = sum_rows(z, i, tau_io, n_out, n_live, n_nonzero, sumsq, done, &slow);
+    if (*done) z->rows_wait = 0;
     if (*done || (r != SFCI_OK && r != SFCI_E_NOMEM)) return r;
+    if (slow) {  // vectors change slowly: planned again after 4, 8, 16 and then every 32 sigmas
+        z->rows_skip = z->rows_wait = std::min(32, std::max(4, 2 * z->rows_wait));
+        return SFCI_OK;
+    }
     if (r == SFCI_E_NOMEM) cudaGetLastError();  // (the failed allocation's, which a launch check would report)
     const sfci_status f = free_row_buffers(z);
     if (f != SFCI_OK) return f;

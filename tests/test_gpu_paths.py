@@ -3,6 +3,8 @@
 The tests that compare the paths mean something only while each side takes the
 path it is meant to take (sfci_row_sigmas counts those summed by rows).
 """
+import math
+
 import numpy as np
 import pytest
 
@@ -40,6 +42,58 @@ def test_solver(sf, name):
 def test_solver_past_the_limit(sf):
     d = single._molecule(16, 13, 2)
     assert _by_rows(sf, lambda: solver._run(sf, d, 900, 3, solver.AUFBAU))[0] == 0
+
+
+def _restarts(sf, d, init, count, **kw):
+    """Rows taken and launches of `count` restarts from one vector, and the last step's vector."""
+    s = sf.System.from_dict(d)
+    lz = sf.Lanczos(s, *init, max(len(init[0]), 100), n_lanczos=3, **kw)
+    rows, launches = [], []
+    for _ in range(count):
+        lz.load(*init)
+        n0, l0 = sf.row_sigmas(), sf.kernel_launches()
+        info = lz.step()
+        rows.append(sf.row_sigmas() - n0)
+        launches.append(sf.kernel_launches() - l0)
+    r, c = lz.vector()
+    lz.close()
+    s.close()
+    return rows, launches, (info["a"], sf.to_u64(r), c.cpu().numpy().view(np.uint64))
+
+
+def _rows_vector(d, rows, n, seed=4):
+    """n determinants spread over `rows` alpha strings."""
+    ca, cb = math.comb(d["n"], d["na"]), math.comb(d["n"], d["nb"])
+    rng = np.random.default_rng(seed)
+    a = rng.choice(ca, rows, replace=False)
+    r = np.unique(rng.choice(a, 2 * n).astype(np.uint64) * np.uint64(cb) + rng.integers(0, cb, 2 * n).astype(np.uint64))
+    r = np.sort(rng.choice(r, n, replace=False))
+    return r, rng.normal(size=n)
+
+
+# what pays by rows and what does not: a space of many rows takes a long vector, and heavy rows
+# may not outnumber the excitations of a string by their classes
+@pytest.mark.parametrize("n,na,nb,rows,dets,by_rows", [
+    (28, 12, 2, 5, 30, 0),        # 3e7 rows for 30 determinants
+    (26, 10, 3, 100, 300, 0),     # 5e6 rows, few elements
+    (28, 1, 9, 8, 20000, 0),      # 2500 determinants to a row, 2000 classes
+    (24, 0, 12, 1, 34000, 0),     # one row
+    (28, 7, 0, 6000, 3000, 0),    # no opposite-spin elements
+    (30, 1, 3, 7, 8000, 0),       # 30 rows, one class each
+    (20, 5, 5, 500, 1000, 1),
+    (28, 7, 7, 20, 30, 1),        # 1e6 rows
+    (24, 1, 7, 6, 20000, 1),      # heavy rows of few classes
+])
+def test_solver_takes_the_faster_path(sf, n, na, nb, rows, dets, by_rows):
+    d = single._molecule(n, na, nb)
+    init = _rows_vector(d, rows, dets)
+    got, launches, out = _restarts(sf, d, init, 3)
+    _, want_launches, want = _restarts(sf, d, init, 3, emit_warps=8)
+    assert got == [by_rows] * 3
+    if not by_rows:  # and nothing is prepared again for a plan that did not pay (the plan's longer
+        # stream may save the buckets an attempt)
+        assert all(a <= b for a, b in zip(launches[1:], want_launches[1:]))
+    assert out[0] == want[0] and np.array_equal(out[1], want[1]) and np.array_equal(out[2], want[2])
 
 
 # (classes: by 20000 determinants its lists fit even then; test_sigma_classes has a longer vector)
