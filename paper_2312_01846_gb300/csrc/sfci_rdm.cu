@@ -297,7 +297,8 @@ struct RowArgs {
     unsigned *id_b;         // [distinct] its beta index
     unsigned long long *bstr;     // [distinct]
     uint2 *hops;            // [distinct * sb] beta index of the hop, b n + j | sign << 31
-    unsigned long long *queue;
+    unsigned long long *queue;    // and behind it the pairs of determinants that share a row
+    int count_pairs;
     double *g1, *g2;
 };
 
@@ -364,7 +365,9 @@ __global__ void __launch_bounds__(kT) rows_strings_kernel(RowArgs A) {
             const unsigned run = w - nd;
             const unsigned long long str = string_unrank_warp(A.run_row[run], d.n, d.na, bt, d.ks);
             if (lane == 0) {
-                const RowUnits u = row_units(d, A.run_off[run + 1] - A.run_off[run]);
+                const unsigned m = A.run_off[run + 1] - A.run_off[run];
+                const RowUnits u = row_units(d, m);
+                if (A.count_pairs && m > 1u) atomicAdd(A.queue + 1, (unsigned long long)m * (m - 1u) / 2ull);
                 A.run_str[run] = str;
                 A.units[run] = u.n1 + u.n2 + u.n3;
             }
@@ -838,7 +841,7 @@ size_t rows_place(char *base, RowArgs &A, size_t &scan_ws, size_t &partial, cons
         o = a256(o + count * sizeof(*p));
     };
     const size_t nn = size_t(n), ca = size_t(d.ca), cb = size_t(d.cb), nd = std::min(nn, cb);
-    take(A.queue, 1);        // (the queue and b_seen are cleared together)
+    take(A.queue, 2);        // (the queue, the pairs and b_seen are cleared together)
     take(A.b_seen, cb);
     take(A.row_run, ca);
     take(A.b_id, cb + 1);
@@ -859,15 +862,27 @@ size_t rows_place(char *base, RowArgs &A, size_t &scan_ws, size_t &partial, cons
     return o;
 }
 
-// Pairs by rows: strings are numbered in 26 bits, their hops in 32; the comparisons
-// within a row stay cheaper than lookups: at most min(cb, n) / 2 of 0.15 ps a
-// determinant (issue), against 12.5 ps for each of the beta excitations (measured).
+// Pairs by rows: strings are numbered in 26 bits, their hops in 32.  A determinant is compared
+// with all of its row, 0.6 to 1.2 ps a pair, where the lookups take 7 to 16 ps for each of its
+// excitations (28 orbitals, 7 + 7 electrons, level-like vectors: 3e5 determinants 20.5 ms and
+// 78 by lookups, 5.8e5 34 and 145; up to 587 000 strings by the last line).
 bool rows_taken(const SysDev &d, long long n) {
     const double exc = (double)d.sb + (double)d.po_b * d.pv_b;
     return n > 0 && n < (1ll << 31) && d.ca <= (1ull << 26) && d.cb <= (1ull << 26) &&
            std::min((double)n, (double)d.cb) * std::max(d.sb, 1) < 4294967296.0 &&
            (double)d.sa + (double)d.po_a * d.pv_a < 2147483648.0 &&
            std::min((double)n, (double)d.cb) <= 4096.0 + 128.0 * exc;
+}
+
+// Up to so many pairs within rows, and whether n determinants may have more: 26 per beta excitation
+// of each determinant is where one row of 28 orbitals breaks even.  28 orbitals, 7 beta electrons:
+// 5.8e5 determinants on one row 106 ms by rows and 43 by lookups, on four rows (with 7 alpha
+// electrons) 57 and 143, on 1e5 rows 21 and 140; 1e5 on one row 3.8 and 9.4.
+double row_pairs_limit(const SysDev &d, long long n) {
+    return (2048.0 + 26.0 * ((double)d.sb + (double)d.po_b * d.pv_b)) * (double)n;
+}
+bool row_pairs_may_exceed(const SysDev &d, long long n) {
+    return 0.5 * std::min((double)n, (double)d.cb) * (double)n > row_pairs_limit(d, n);
 }
 
 int sms() {
@@ -919,22 +934,30 @@ sfci_status sfci_rdm12(const sfci_system *s, const uint64_t *rank, const double 
     const unsigned long long *r = reinterpret_cast<const unsigned long long *>(rank);
     RowArgs A{};
     size_t scan_ws = 0, part_at = L.partial;
-    const bool by_rows = rows_taken(d, n) && rows_place(nullptr, A, scan_ws, part_at, d, n) <= ws_bytes;
-    if (!by_rows) part_at = L.partial;
-    double *partial = reinterpret_cast<double *>(w + part_at);
-    // the norm and, behind it, the flag of invalid ranks: read back together
-    double *nrm = by_rows ? partial + kNormBlocks : reinterpret_cast<double *>(w + L.norm);
-    int *flag = reinterpret_cast<int *>(nrm + 1);
-    SFCI_CUDA(cudaMemsetAsync(nrm, 0, 16, st));
-    SFCI_CUDA(validate_sorted(r, n, d.dim, flag, st));
-    count_launch();
-    norm2_kernel<<<kNormBlocks, kThreads, 0, st>>>(coef, n, partial);
-    count_launch();
-    norm2_finish<<<1, 32, 0, st>>>(partial, kNormBlocks, nrm);
+    bool by_rows = rows_taken(d, n) && rows_place(nullptr, A, scan_ws, part_at, d, n) <= ws_bytes;
+    double *nrm = nullptr;
+    int *flag = nullptr;
+    const auto norm_and_check = [&]() -> sfci_status {
+        double *partial = reinterpret_cast<double *>(w + (by_rows ? part_at : L.partial));
+        // the norm and, behind it, the flag of invalid ranks: read back together
+        nrm = by_rows ? partial + kNormBlocks : reinterpret_cast<double *>(w + L.norm);
+        flag = reinterpret_cast<int *>(nrm + 1);
+        SFCI_CUDA(cudaMemsetAsync(nrm, 0, 16, st));
+        SFCI_CUDA(validate_sorted(r, n, d.dim, flag, st));
+        count_launch();
+        norm2_kernel<<<kNormBlocks, kThreads, 0, st>>>(coef, n, partial);
+        count_launch();
+        norm2_finish<<<1, 32, 0, st>>>(partial, kNormBlocks, nrm);
+        SFCI_CUDA(cudaGetLastError());
+        return SFCI_OK;
+    };
+    sfci_status e = norm_and_check();
+    if (e != SFCI_OK) return e;
     if (by_rows) {
         size_t ignore;
         rows_place(w, A, ignore, ignore, d, n);
         A.d = d, A.rank = r, A.coef = coef, A.n = (unsigned)n, A.flag = flag, A.g1 = rdm1, A.g2 = rdm2;
+        A.count_pairs = row_pairs_may_exceed(d, n);
         SFCI_CUDA(cudaMemsetAsync(A.queue, 0, size_t((char *)A.row_run - (char *)A.queue), st));
         SFCI_CUDA(cudaMemsetAsync(A.row_run, 0xff, size_t(d.ca) * 4, st));
         const unsigned g = (unsigned)std::min<long long>((n + kT - 1) / kT, sms() * 8ll);
@@ -947,6 +970,18 @@ sfci_status sfci_rdm12(const sfci_system *s, const uint64_t *rank, const double 
         const size_t bts = size_t(d.n + 1) * d.ks * 8;
         count_launch();
         rows_strings_kernel<<<(unsigned)std::min<long long>((n + kT / 64 - 1) / (kT / 64), sms() * 8ll), kT, bts, st>>>(A);
+        if (A.count_pairs) {
+            unsigned long long pairs = 0;
+            SFCI_CUDA(cudaMemcpyAsync(&pairs, A.queue + 1, 8, cudaMemcpyDeviceToHost, st));
+            SFCI_CUDA(cudaStreamSynchronize(st));
+            if ((double)pairs > row_pairs_limit(d, n)) {  // (the table takes the rows' place in the workspace)
+                by_rows = false;
+                if ((e = norm_and_check()) != SFCI_OK) return e;
+            }
+        }
+    }
+    if (by_rows) {
+        const size_t bts = size_t(d.n + 1) * d.ks * 8;
         SFCI_CUDA(exclusive_scan(A.units, n, A.uoff, w + scan_ws, st));
         const size_t smem = al16(sizeof(RowShared)) + bts + (d.n <= kDiagN ? size_t(3) * d.n * d.n * 8 : 0);
         SFCI_CUDA(allow_max_smem(rdm_rows_kernel, smem));
