@@ -11,6 +11,7 @@ bit pattern of the library's uint64 ranks, coefficients in float64.
 from __future__ import annotations
 
 import ctypes as C
+import math
 import os
 
 import torch
@@ -211,25 +212,41 @@ def sigma_workspace_bytes(sys: System, n_in, out_cap):
     return int(nb.value)
 
 
+# first capacities of sfci_sigma: by target rows, room that is not used costs memory alone, and a
+# capacity that was too small a second sigma (2.2e7 entries of 20 orbitals: 5.1 ms in two calls, 3.2 in
+# one); the hash table, which takes over beyond the rows' limits (12 electrons and 2^26 strings of a
+# spin), is cleared and read throughout
+_SIGMA_ROOM, _SIGMA_ROOM_TABLE = 1 << 25, 1 << 24
+
+
+def _rows_possible(sys: System):
+    return all(m <= 12 and math.comb(sys.n, m) <= 1 << 26 for m in (sys.na, sys.nb))
+
+
 def sfci_sigma(sys: System, rank, coef, eps_screen=0.0, out_cap=None, stream=None):
     """sigma = H psi; returns (rank, coef) ascending by rank.  If out_cap is not
-    given it starts from min(n_in * (n_conn + 1), 2^25) (3 GB with the workspace; 2^24 with
-    more than 12 electrons of a spin) and grows on SFCI_E_CAPACITY."""
+    given it starts from min(n_in * (n_conn + 1), 2^25) (3 GB with the workspace while the call
+    runs; 2^24 beyond the limits of the sum by target rows, or where 3 GB are not free) and grows
+    on SFCI_E_CAPACITY; results of up to 2^24 entries come in buffers of their own size then."""
     r = _dev(rank, torch.int64)
     c = _dev(coef, torch.float64)
     if out_cap is not None:
         cap = int(out_cap)
     else:
-        # sigma by target rows touches only what it writes: room that is not used costs memory
-        # alone, and a second call because of a capacity that was too small is a whole sigma
-        # (3e7 entries: 5.1 ms so, 3.2 ms in one call); the hash table, which takes over beyond
-        # 12 electrons of a spin, is cleared and read throughout
-        room = 1 << (25 if max(sys.na, sys.nb) <= 12 else 24)
+        room = _SIGMA_ROOM if _rows_possible(sys) else _SIGMA_ROOM_TABLE
         cap = max(1024, min(r.numel() * (sys.n_conn + 1), room))
+    first = True
     for _ in range(16):
-        ws = torch.empty(sigma_workspace_bytes(sys, r.numel(), cap), dtype=torch.uint8, device="cuda")
-        orank = torch.empty(max(cap, 1), dtype=torch.int64, device="cuda")
-        ocoef = torch.empty(max(cap, 1), dtype=torch.float64, device="cuda")
+        try:
+            ws = torch.empty(sigma_workspace_bytes(sys, r.numel(), cap), dtype=torch.uint8, device="cuda")
+            orank = torch.empty(max(cap, 1), dtype=torch.int64, device="cuda")
+            ocoef = torch.empty(max(cap, 1), dtype=torch.float64, device="cuda")
+        except torch.OutOfMemoryError:
+            if out_cap is not None or not first or cap <= _SIGMA_ROOM_TABLE:
+                raise
+            ws = orank = ocoef = None
+            cap = _SIGMA_ROOM_TABLE
+            continue
         n = C.c_int64()
         st = lib().sfci_sigma(sys.handle, _ptr(r), _ptr(c), r.numel(), float(eps_screen),
                               _ptr(orank), _ptr(ocoef), cap, C.byref(n), _ptr(ws), ws.numel(),
@@ -237,9 +254,14 @@ def sfci_sigma(sys: System, rank, coef, eps_screen=0.0, out_cap=None, stream=Non
         if st == SFCI_E_CAPACITY and n.value > cap:
             del ws, orank, ocoef
             cap = max(int(n.value * 1.25) + 1024, 4 * cap)
+            first = False
             continue
         _check(st, "sfci_sigma")
-        return orank[: n.value], ocoef[: n.value]
+        orank, ocoef = orank[: n.value], ocoef[: n.value]
+        if out_cap is None and first and cap > _SIGMA_ROOM_TABLE and n.value <= _SIGMA_ROOM_TABLE:
+            orank, ocoef = orank.clone(), ocoef.clone()  # (a slice holds its whole buffer: 537 MB)
+            torch.cuda.current_stream().synchronize()  # (complete on return, whatever stream reads it)
+        return orank, ocoef
     raise SfciError(SFCI_E_CAPACITY, "sfci_sigma: output keeps growing")
 
 
