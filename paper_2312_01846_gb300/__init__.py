@@ -318,13 +318,21 @@ def sfci_debug_excitations(sys: System, rank, stream=None):
 
 
 def sfci_rdm12(sys: System, rank, coef, stream=None):
-    """Spin-summed 1- and 2-RDMs of psi (not normalised) and <psi|psi>."""
+    """Spin-summed 1- and 2-RDMs of psi (not normalised) and <psi|psi>.  Where the workspace of the
+    pairs by rows (0.6 GB at 5e5 determinants of 28 orbitals) is not free, a table of the
+    vector (16 MB) does: slower."""
     r = _dev(rank, torch.int64)
     c = _dev(coef, torch.float64)
     nb = C.c_size_t()
     _check(lib().sfci_rdm12_workspace_bytes(sys.handle, r.numel(), C.byref(nb)),
            "sfci_rdm12_workspace_bytes")
-    ws = torch.empty(int(nb.value), dtype=torch.uint8, device="cuda")
+    least = 2048 + 16 * max(1024, 1 << (2 * max(r.numel(), 1) - 1).bit_length())
+    try:
+        ws = torch.empty(int(nb.value), dtype=torch.uint8, device="cuda")
+    except torch.OutOfMemoryError:
+        if least >= nb.value:
+            raise
+        ws = torch.empty(least, dtype=torch.uint8, device="cuda")
     n = sys.n
     g1 = torch.empty((n, n), dtype=torch.float64, device="cuda")
     g2 = torch.empty((n, n, n, n), dtype=torch.float64, device="cuda")
