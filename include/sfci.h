@@ -271,7 +271,8 @@ typedef struct sfci_step_info {
     double free_gb;        /* free device memory the plan saw, besides the solver's
                               element, stream and overflow buffers (GB)              */
     int64_t n_overflow;    /* most elements any pass sent past their bucket's region  */
-    double ms_alloc;       /* of ms_plan: device buffer (re)allocation               */
+    double ms_alloc;       /* of ms_plan: device buffer (re)allocation; by target rows also
+                              what a longer stream took in a repeated attempt        */
     int64_t n_emitted;     /* intermediate elements generated for sigma_i and merged:
                               the non-zero products of n_elements                */
     int64_t n_alpha_runs;  /* runs of consecutive entries of w_i that share alpha

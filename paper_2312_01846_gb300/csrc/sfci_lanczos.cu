@@ -931,8 +931,10 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
     double need = 1.25 * (double)size_a + (double)vrp_bytes + 1.1 * 16.0 * sig_need;  // (as grown below)
     if (!fits(have_a, need)) return SFCI_OK;
     SFCI_CUDA(cudaEventRecord(z->evp[0], z->st));
+    z->ms_alloc = 0.0;
     const auto grow = [&](sfci_lanczos::Buf &buf, size_t want, const char *what, double headroom) {
         if (buf.p && buf.bytes >= want) return SFCI_OK;
+        const auto t0 = std::chrono::steady_clock::now();
         if (z->alloc_limit > 0 && want > (size_t)z->alloc_limit) {
             set_error(std::string(what) + ": above the allocation limit");
             return SFCI_E_NOMEM;
@@ -945,6 +947,7 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
             f = free_bucket_buffers(z);
             if (f == SFCI_OK) f = ensure(buf, want, z->st, what, headroom);
         }
+        z->ms_alloc += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         return f;
     };
     if ((r = grow(z->ga, size_a, "row gather arrays", 1.25))) return r;
@@ -1071,7 +1074,6 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
         while ((1ull << z->nb_log2) < gn.units) ++z->nb_log2;
         if (budget >= 0.0) z->budget_gb = budget / 1e9, z->free_gb = (budget - held) / 1e9, z->held_gb = held / 1e9;
         z->regions_gb = E * sizeof(Slot) / 1e9;  // what the elements would take as records
-        z->ms_alloc = 0.0;
         *done = true;
         count_row_sigma();
         return SFCI_OK;

@@ -98,3 +98,18 @@ def test_short_after_long(sf, inputs):
     assert lz.debug_memory() <= SHARE
     lz.close()
     ref.close()
+
+
+def test_allocation_time(sf, inputs):
+    """ms_alloc: what a step by rows spends on growing its buffers, and nothing once they have grown."""
+    _, vecs = inputs
+    lz = _solver(sf, inputs)
+    infos = []
+    for _ in range(2):
+        lz.load(*vecs[KEEP])
+        n0 = sf.row_sigmas()
+        infos.append(lz.step())
+        assert sf.row_sigmas() == n0 + 1
+    lz.close()
+    assert 0.0 < infos[0]["ms_alloc"] <= infos[0]["ms_plan"]
+    assert infos[1]["ms_alloc"] == 0.0
