@@ -1493,10 +1493,14 @@ size_t gather_place_lists(char *base, GatherBufs &b, const GatherShape &p, const
     return a.off;
 }
 
-// 32-bit positions in the singles' table and the lists, 25 bits for a beta string's number
+// 32-bit positions in the singles' table, the lists and one row's records (the sources listed
+// under its substrings, those one hop away, the diagonal and beta singles of its own, which are
+// as many as there are beta strings at most), 25 bits for a beta string's number
 bool gather_numbers(const SysDev &d, long long n, unsigned long long nd) {
-    return nd < (1ull << 25) && (double)nd * std::max(d.sb, 1) < 4294967296.0 &&
-           (double)n * std::max(d.po_a, d.na) < 4294967296.0;
+    constexpr double k32 = 4294967296.0;
+    return n < (1ll << 31) && nd < (1ull << 25) && (double)nd * std::max(d.sb, 1) < k32 &&
+           (double)n * std::max(d.po_a, d.na) < k32 &&
+           (double)n * (d.po_a + 1.0) + std::min((double)n, (double)nd) * (d.sb + 1.0) < k32;
 }
 
 // Sigma by target rows against the buckets (330 systems of 8 to 64 orbitals with random and with
