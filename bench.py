@@ -12,6 +12,9 @@ and two near-degenerate orbital clusters, N_d = 1e6 determinants per basis
 vector, N_L = 10.  The solver starts from the aufbau determinant; the warm-up
 steps grow the vector to N_d; the timed steps then run at full size.
 
+One JSON line on standard output; every step's record and the studies' figures in
+full go to standard error.
+
 value = connected elements enumerated per second over the timed steps
 (elements = sum over input determinants of 1 + the number of single and
 double excitations).  Multi-GPU: one independent replica per rank (the
@@ -363,6 +366,41 @@ def scan_study(sf, cap_scale, n_lanczos, warmup, steps, workers=0, bucket_elems=
     return out
 
 
+# what the printed line keeps of its longer parts; the rest goes to the detail line
+LINE_KEYS = {
+    "roofline": ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel", "peak_kind", "ms_per_launch"),
+    "cpu_baseline": ("value", "unit", "cores", "kind", "sample"),
+    "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps"),
+}
+ROW_KEYS = ("ms_per_step", "ms_per_pass", "elements_per_s", "value")
+DETAIL_KEYS = ("pipe_rates", "precision", "heat_bath_screen", "detail", "launch_shape", "autotune")
+
+
+def short_line(line):
+    """The benchmark's one line: every headline key, and of the studies one figure or two each.  It
+    stays below 2600 bytes, so that whoever keeps only the end of the output keeps all of it."""
+    def short(x):
+        return float(f"{x:.6g}") if isinstance(x, float) else x
+
+    out = {k: v for k, v in line.items() if k not in DETAIL_KEYS}
+    for part, keys in LINE_KEYS.items():
+        if isinstance(out.get(part), dict):
+            out[part] = {k: out[part][k] for k in keys if k in out[part]}
+    if isinstance(out.get("workloads"), dict):
+        rows = {k: v.get("batched", v) for k, v in out["workloads"].items()}
+        out["workloads"] = {k: {q: short(v[q]) for q in ROW_KEYS if q in v} for k, v in rows.items()}
+    if isinstance(line.get("precision"), dict):
+        out["precision"] = {k: short(line["precision"][k]) for k in ("speedup", "max_abs_delta_e_comparable")
+                            if k in line["precision"]}
+    return out
+
+
+def print_line(line):
+    """The short line on standard output; everything, steps and studies, on standard error before it."""
+    print(json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(short_line(line)), flush=True)
+
+
 def run_scan(a):
     """--workload scan: the batched scan as the JSON line's headline (see scan_study)."""
     import torch
@@ -402,7 +440,7 @@ def run_scan(a):
         "detail": out, "launch_shape": shape, "autotune": tuned,
     }
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print_line(line)
     return 0
 
 
@@ -743,7 +781,7 @@ def run_ours(a):
                    "warmup_steps": warm, "timed_steps": [brief(i) for i in infos]},
     }
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print_line(line)
     gsys.close()
     if dist is not None:
         dist.destroy_process_group()
