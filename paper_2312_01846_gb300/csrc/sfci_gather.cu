@@ -1540,7 +1540,7 @@ RowPlanArgs row_plan_args(const SysDev &d, const GatherShape &p, long long n) {
     ra.half = (unsigned long long)(0.55 * 1.45 * kGSlots);
     ra.fill = 0.65 * kGSlots;
     // at most 120 rows in a group (7 bits), and fewer than its key bits can number
-    ra.w_fixed = std::max(32u, (unsigned)(2 * ra.half / std::min(120, (1 << (32 - p.bb)) - 2) + 1));
+    ra.w_fixed = std::max(32u, (unsigned)(2 * ra.half / std::min(120ull, (1ull << (32 - p.bb)) - 2ull) + 1));
     return ra;
 }
 
