@@ -297,8 +297,8 @@ struct RowArgs {
     unsigned *id_b;         // [distinct] its beta index
     unsigned long long *bstr;     // [distinct]
     uint2 *hops;            // [distinct * sb] beta index of the hop, b n + j | sign << 31
-    unsigned long long *queue;    // and behind it the pairs of determinants that share a row
-    int count_pairs;
+    unsigned long long *queue;    // and behind it the pairs of determinants that share a row, the units
+    int count;                    // both are wanted
     double *g1, *g2;
 };
 
@@ -360,6 +360,7 @@ __global__ void __launch_bounds__(kT) rows_strings_kernel(RowArgs A) {
     const int lane = threadIdx.x & 31;
     unsigned char *occ = lists[threadIdx.x >> 5], *vir = occ + 64;
     const unsigned nd = (unsigned)A.b_id[d.cb], runs = (unsigned)A.run_of[A.n];
+    unsigned long long pairs = 0ull, units = 0ull;  // (lane 0's)
     for (unsigned w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nd + runs; w += (gridDim.x * blockDim.x) >> 5) {
         if (w >= nd) {
             const unsigned run = w - nd;
@@ -367,7 +368,8 @@ __global__ void __launch_bounds__(kT) rows_strings_kernel(RowArgs A) {
             if (lane == 0) {
                 const unsigned m = A.run_off[run + 1] - A.run_off[run];
                 const RowUnits u = row_units(d, m);
-                if (A.count_pairs && m > 1u) atomicAdd(A.queue + 1, (unsigned long long)m * (m - 1u) / 2ull);
+                pairs += (unsigned long long)m * (m - 1u) / 2ull;
+                units += u.n1 + u.n2 + u.n3;
                 A.run_str[run] = str;
                 A.units[run] = u.n1 + u.n2 + u.n3;
             }
@@ -388,6 +390,10 @@ __global__ void __launch_bounds__(kT) rows_strings_kernel(RowArgs A) {
             A.hops[(size_t)w * d.sb + x] =
                 make_uint2((unsigned)string_rank(str ^ (1ull << j) ^ (1ull << b), bt, d.ks), (unsigned)(b * d.n + j) | sg << 31);
         }
+    }
+    if (A.count && units) {
+        if (pairs) atomicAdd(A.queue + 1, pairs);
+        atomicAdd(A.queue + 2, units);
     }
 }
 
@@ -841,7 +847,7 @@ size_t rows_place(char *base, RowArgs &A, size_t &scan_ws, size_t &partial, cons
         o = a256(o + count * sizeof(*p));
     };
     const size_t nn = size_t(n), ca = size_t(d.ca), cb = size_t(d.cb), nd = std::min(nn, cb);
-    take(A.queue, 2);        // (the queue, the pairs and b_seen are cleared together)
+    take(A.queue, 3);        // (the queue, the counts behind it and b_seen are cleared together)
     take(A.b_seen, cb);
     take(A.row_run, ca);
     take(A.b_id, cb + 1);
@@ -862,18 +868,6 @@ size_t rows_place(char *base, RowArgs &A, size_t &scan_ws, size_t &partial, cons
     return o;
 }
 
-// Pairs by rows: strings are numbered in 26 bits, their hops in 32.  A determinant is compared
-// with all of its row, 0.6 to 1.2 ps a pair, where the lookups take 7 to 16 ps for each of its
-// excitations (28 orbitals, 7 + 7 electrons, level-like vectors: 3e5 determinants 20.5 ms and
-// 78 by lookups, 5.8e5 34 and 145; up to 587 000 strings by the last line).
-bool rows_taken(const SysDev &d, long long n) {
-    const double exc = (double)d.sb + (double)d.po_b * d.pv_b;
-    return n > 0 && n < (1ll << 31) && d.ca <= (1ull << 26) && d.cb <= (1ull << 26) &&
-           std::min((double)n, (double)d.cb) * std::max(d.sb, 1) < 4294967296.0 &&
-           (double)d.sa + (double)d.po_a * d.pv_a < 2147483648.0 &&
-           std::min((double)n, (double)d.cb) <= 4096.0 + 128.0 * exc;
-}
-
 // Up to so many pairs within rows, and whether n determinants may have more: 26 per beta excitation
 // of each determinant is where one row of 28 orbitals breaks even.  28 orbitals, 7 beta electrons:
 // 5.8e5 determinants on one row 106 ms by rows and 43 by lookups, on four rows (with 7 alpha
@@ -883,6 +877,34 @@ double row_pairs_limit(const SysDev &d, long long n) {
 }
 bool row_pairs_may_exceed(const SysDev &d, long long n) {
     return 0.5 * std::min((double)n, (double)d.cb) * (double)n > row_pairs_limit(d, n);
+}
+
+// Up to so many units, and whether n determinants may have more.  A unit takes some 9 ns of the chip
+// even where it finds nothing (more with more beta electrons on the diagonal), and a row of one
+// determinant has a unit per 256 alpha excitations; a lookup takes 10.5 ps, a determinant's other
+// work there 45 ns (23 without beta hops), and no call less than one warp's lookups in turn, 50 ns
+// each.  Where the opposite-spin lookups are few, the rows lose: 28 orbitals, 7 alpha electrons, 1e5
+// determinants on as many rows and none, 1, 2, 3 beta electrons: 20.9, 19.9, 18.9, 18.8 ms by rows,
+// 9.4, 11.1, 15.0, 18.1 by lookups; 20 to a row 1.2 (1 to 3 electrons) and 10.5, 14.8, 18.1.
+double row_units_limit(const SysDev &d, long long n) {
+    const double exc = (double)d.sa + d.sb + (double)d.po_a * d.pv_a + (double)d.po_b * d.pv_b + (double)d.sa * d.sb;
+    return ((double)n * ((d.sb == 0 ? 23.0 : 45.0) + 0.0105 * exc) + 50.0 * exc) / (9.2 + 0.08 * d.nb);
+}
+bool row_units_may_exceed(const SysDev &d, long long n) {  // (as many where there is one beta string)
+    const double hops = (double)d.sa + (double)d.po_a * d.pv_a;
+    return (double)n * (1.0 + std::ceil(hops / kT) + (d.sb ? std::ceil((double)d.sa / kT) : 0.0)) > row_units_limit(d, n);
+}
+
+// Pairs by rows: strings are numbered in 26 bits, their hops in 32.  A determinant is compared
+// with all of its row, 0.6 to 1.2 ps a pair, where the lookups take 7 to 16 ps for each of its
+// excitations (28 orbitals, 7 + 7 electrons, level-like vectors: 3e5 determinants 20.5 ms and
+// 78 by lookups, 5.8e5 34 and 145; up to 587 000 strings by the last line).
+bool rows_taken(const SysDev &d, long long n) {
+    const double exc = (double)d.sb + (double)d.po_b * d.pv_b;
+    return n > 0 && n < (1ll << 31) && d.ca <= (1ull << 26) && d.cb <= (1ull << 26) &&
+           std::min((double)n, (double)d.cb) * std::max(d.sb, 1) < 4294967296.0 &&
+           (double)d.sa + (double)d.po_a * d.pv_a < 2147483648.0 &&
+           std::min((double)n, (double)d.cb) <= 4096.0 + 128.0 * exc && !(d.cb == 1 && row_units_may_exceed(d, n));
 }
 
 int sms() {
@@ -957,7 +979,7 @@ sfci_status sfci_rdm12(const sfci_system *s, const uint64_t *rank, const double 
         size_t ignore;
         rows_place(w, A, ignore, ignore, d, n);
         A.d = d, A.rank = r, A.coef = coef, A.n = (unsigned)n, A.flag = flag, A.g1 = rdm1, A.g2 = rdm2;
-        A.count_pairs = row_pairs_may_exceed(d, n);
+        A.count = row_pairs_may_exceed(d, n) || row_units_may_exceed(d, n);
         SFCI_CUDA(cudaMemsetAsync(A.queue, 0, size_t((char *)A.row_run - (char *)A.queue), st));
         SFCI_CUDA(cudaMemsetAsync(A.row_run, 0xff, size_t(d.ca) * 4, st));
         const unsigned g = (unsigned)std::min<long long>((n + kT - 1) / kT, sms() * 8ll);
@@ -970,11 +992,12 @@ sfci_status sfci_rdm12(const sfci_system *s, const uint64_t *rank, const double 
         const size_t bts = size_t(d.n + 1) * d.ks * 8;
         count_launch();
         rows_strings_kernel<<<(unsigned)std::min<long long>((n + kT / 64 - 1) / (kT / 64), sms() * 8ll), kT, bts, st>>>(A);
-        if (A.count_pairs) {
-            unsigned long long pairs = 0;
-            SFCI_CUDA(cudaMemcpyAsync(&pairs, A.queue + 1, 8, cudaMemcpyDeviceToHost, st));
+        if (A.count) {
+            unsigned long long has[2] = {0, 0};  // pairs, units
+            SFCI_CUDA(cudaMemcpyAsync(has, A.queue + 1, 16, cudaMemcpyDeviceToHost, st));
             SFCI_CUDA(cudaStreamSynchronize(st));
-            if ((double)pairs > row_pairs_limit(d, n)) {  // (the table takes the rows' place in the workspace)
+            // (the table takes the rows' place in the workspace)
+            if ((double)has[0] > row_pairs_limit(d, n) || (double)has[1] > row_units_limit(d, n)) {
                 by_rows = false;
                 if ((e = norm_and_check()) != SFCI_OK) return e;
             }
