@@ -373,24 +373,28 @@ namespace {
 // sigma by target rows in the bytes [w, w + room) of the workspace, for a validated
 // input; unsorted entries leave to out_rank / out_coef, their number to *n_out (on the device
 // at *n_dev).
-// *done = false: its lists do not fit there (or the system is outside its limits).
+// *done = false: its lists do not fit there, the table is faster, or the system is outside its limits.
 //
 // The table path keeps every entry in a global hash table (32 bytes a slot, two to four
 // slots an entry): a clear, scattered atomics, a finish and an extraction, all over the
-// table: 6000 determinants of 20 orbitals, 3e7 entries, took 27.3 ms, 601 of them
+// table: 6000 determinants of 20 orbitals, 2.2e7 entries, took 27.3 ms, 601 of them
 // 2.82 ms; by rows 5.99 ms and 1.10 ms, of which sorting the entries is the largest part.
 sfci_status sigma_rows(const sfci_system *s, const unsigned long long *rank, const double *coef, long long n, double eps,
                        int fix_shift, unsigned long long *out_rank, double *out_coef, long long out_cap, char *w,
-                       size_t room, const unsigned long long **n_dev, unsigned long long *n_out, bool *done, cudaStream_t st) {
+                       size_t room, unsigned long long slots, const unsigned long long **n_dev, unsigned long long *n_out,
+                       bool *done, cudaStream_t st) {
     *done = false;
     const SysDev &d = s->d;
     GatherShape gs{};
-    if (!gather_shape(d, &gs) || !gather_numbers(d, n, 0)) return SFCI_OK;
+    if (!gather_shape(d, &gs) || !gather_numbers(d, n, 0) || !gather_beats_table(d, n, slots)) return SFCI_OK;
     GatherBufs b{};
     const size_t head = 8192, rps = a256((size_t(d.ca) + 1) * 4);
     const size_t size_a = gather_place_sources(nullptr, b, d, gs, n);
     size_t at = head + rps + size_a;
-    if (at > room) return SFCI_OK;
+    // (what surely does not fit is not prepared for nothing: 0.1 to 0.5 ms; a beta string is shared
+    // by at most one source of each row)
+    const size_t nd_least = ((size_t)n + d.ca - 1) / d.ca;
+    if (at + gather_place_tables(nullptr, b, d, gs, nd_least, n) + gather_lists_least(d, gs, n) > room) return SFCI_OK;
     // head: counters of the gather kernel (zeroed), rows' weights seen so far (none)
     struct Words {
         unsigned long long out, tau, mark, live, nonzero, read;
@@ -418,7 +422,7 @@ sfci_status sigma_rows(const sfci_system *s, const unsigned long long *rank, con
     SFCI_CUDA(gather_tables(d, gs, n, (unsigned)nd, s->pair_int, rp, b, ra, st));
     GatherCounts gn{};
     SFCI_CUDA(gather_counts(d, b, &gn, st));
-    if (!gn.fit() || at + gather_place_lists(nullptr, b, gs, gn) > room) return SFCI_OK;
+    if (!gn.fit() || !gather_beats_table(d, n, gn) || at + gather_place_lists(nullptr, b, gs, gn) > room) return SFCI_OK;
     gather_place_lists(w + at, b, gs, gn);
     SFCI_CUDA(gather_lists(d, gs, gn.act, gn.parts, s->pair_int, rp, b, ra, st));
     GatherArgs A{};
@@ -507,7 +511,7 @@ sfci_status sfci_sigma(const sfci_system *s, const uint64_t *in_rank, const doub
     const unsigned long long *n_rows = nullptr;
     if (n_in > 0) {
         const sfci_status r = sigma_rows(s, ir, in_coef, n_in, eps, t.fix_shift, reinterpret_cast<unsigned long long *>(out_rank),
-                                         out_coef, out_cap, w, L.status, &n_rows, &hn, &by_rows, st);
+                                         out_coef, out_cap, w, L.status, L.slots, &n_rows, &hn, &by_rows, st);
         if (r != SFCI_OK) {
             *n_out = 0;
             return r;

@@ -1531,6 +1531,38 @@ bool gather_pays(const SysDev &d, long long n, const GatherCounts &c) {
     return (double)c.visits <= 0.65 * elements && (c.units >= 152 || elements <= 5e5 * (double)c.units);
 }
 
+// The standalone sigma's hash table has no preparation, but a warp per source (0.13 us an element in
+// turn: 1.9 ms for 30 sources of 7876, by rows 0.5) and slots to clear and read (32 bytes each).  It
+// is left to
+//  * few elements a source and few slots: 28 orbitals, 1 + 1 electrons, 30 determinants 0.22 ms, by
+//    rows 0.29; 20 orbitals, 5 electrons of one spin, 85 determinants 0.28 and 0.39; but 12
+//    orbitals, 6 + 6 (1817 excitations), 20 determinants 0.50 and 0.39;
+//  * elements of one spin alone (records or own doubles, no table of singles to share), until the
+//    slots cost more: 28 orbitals, 7 electrons, 872 determinants (2^23 slots) 0.98 and 2.13, 8636
+//    (2^22) 1.41 and 1.84, but (2^26) 4.03 and 3.48; 24 orbitals, 12 electrons, 300 determinants
+//    (2^22) 1.02 and 0.91, 1000 1.19 and 1.30.
+bool gather_beats_table(const SysDev &d, long long n, unsigned long long slots) {
+    if (d.n_conn <= 1150 && slots <= 1ull << 20) return false;
+    return (d.sa > 0 && d.sb > 0) || slots > 1ull << 23 || (double)n * (double)(d.n_conn + 1) < 2e6;
+}
+
+// and to heavy rows whose classes visit sources more often than there are elements, a few
+// milliseconds of visits at least (the plan is made for nothing then: about 0.7 ms).  28 orbitals,
+// 1 + 7 electrons: 1.07 visits an element (1e4 determinants) 14.5 ms by rows, 9.7 by the table, 1.16
+// (3e4) 38.8 and 22.2; 29 orbitals, 1 + 10: 0.92 (3000) 8.7 and 9.1, 2.1 (8000) 32 and 22, 3.1 (25000)
+// 189 and 57; 26 orbitals, 2 + 9: 0.79 (1e4) 19.9 and 21.3.
+bool gather_beats_table(const SysDev &d, long long n, const GatherCounts &c) {
+    return (double)c.visits <= std::max((double)n * (double)(d.n_conn + 1), 8e7);
+}
+
+// What the lists take at least, whatever the rows: a source is listed under C(n_alpha, 2) substrings
+// of C(n - n_alpha + 2, 2) rows each, is one hop away from s_a rows, and has its own records.
+size_t gather_lists_least(const SysDev &d, const GatherShape &p, long long n) {
+    const double rows2 = 0.5 * (d.n - d.na + 2) * (d.n - d.na + 1);
+    const double rec = (double)n * ((d.ss_any ? d.po_a * rows2 : 0.0) + d.sa + d.sb + 1.0);
+    return (size_t)(rec * (p.bb > kGLog ? 24.0 : 12.0) + (d.ab_any ? 16.0 * (double)n * d.sa : 0.0));
+}
+
 RowPlanArgs row_plan_args(const SysDev &d, const GatherShape &p, long long n) {
     RowPlanArgs ra{};
     // a warp makes 128 to 1024 list items: as many warps as the chip holds twice, where there are enough

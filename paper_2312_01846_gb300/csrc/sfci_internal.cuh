@@ -723,6 +723,10 @@ bool gather_shape(const SysDev &d, GatherShape *p);  // false: the system is out
 // whether sigma by target rows is faster than the buckets: before anything is prepared, and as planned
 bool gather_pays(const SysDev &d, long long n);
 bool gather_pays(const SysDev &d, long long n, const GatherCounts &c);
+// the same against sfci_sigma's hash table (of so many slots)
+bool gather_beats_table(const SysDev &d, long long n, unsigned long long slots);
+bool gather_beats_table(const SysDev &d, long long n, const GatherCounts &c);
+size_t gather_lists_least(const SysDev &d, const GatherShape &p, long long n);  // bytes, a lower bound
 // its buffers in three parts, each placed when the counts it depends on are known: bytes
 // taken, pointers from base on (base null: sizes only)
 size_t gather_place_sources(char *base, GatherBufs &b, const SysDev &d, const GatherShape &p, long long n);
