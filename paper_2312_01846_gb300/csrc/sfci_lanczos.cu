@@ -940,7 +940,14 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
             return SFCI_E_NOMEM;
         }
         fits(false, 0.0);  // (budget)
-        sfci_status f = need + bucket_bytes(z) > budget ? free_bucket_buffers(z) : SFCI_OK;
+        // (what is held with the grown buffer: a stream that the buckets made longer counts as it is)
+        const auto over = [&] {
+            return row_bytes(z) + bucket_bytes(z) + (double)z->sig_key.bytes + (double)z->sig_val.bytes - (double)buf.bytes +
+                   headroom * (double)want > budget;
+        };
+        sfci_status f = over() ? free_bucket_buffers(z) : SFCI_OK;
+        if (f == SFCI_OK && over() && &buf != &z->sig_key && &buf != &z->sig_val)
+            f = free_buffers(z, {&z->sig_key, &z->sig_val});
         if (f == SFCI_OK) f = ensure(buf, want, z->st, what, headroom);
         if (f == SFCI_E_NOMEM && bucket_bytes(z) > 0.0) {
             cudaGetLastError();

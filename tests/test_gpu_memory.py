@@ -100,6 +100,18 @@ def test_short_after_long(sf, inputs):
     ref.close()
 
 
+def test_stream_of_the_buckets_counts(sf, inputs):
+    """The same where the stream is longer than the rows want it (how long the buckets make it
+    depends on the order in which it fills): it counts as it is."""
+    _, vecs = inputs
+    for _ in range(16):
+        lz = _solver(sf, inputs, share=SHARE)
+        assert _step(sf, lz, vecs[KEEP])[0] == 0
+        assert _step(sf, lz, vecs[SHORT])[0] == 1
+        assert lz.debug_memory() <= SHARE
+        lz.close()
+
+
 def test_allocation_time(sf, inputs):
     """ms_alloc: what a step by rows spends on growing its buffers, and nothing once they have grown."""
     _, vecs = inputs
