@@ -1503,6 +1503,10 @@ bool gather_numbers(const SysDev &d, long long n, unsigned long long nd) {
            (double)n * (d.po_a + 1.0) + std::min((double)n, (double)nd) * (d.sb + 1.0) < k32;
 }
 
+// A chip that a few units leave idle: 3.5 ns per element of a unit (30 rows of 9e5 elements: 3.8 ms,
+// buckets 3.1).
+bool enough_units(double units, double elements) { return units >= 152.0 || elements <= 5e5 * units; }
+
 // Sigma by target rows against the buckets (330 systems of 8 to 64 orbitals with random and with
 // level-like vectors, 10 to 3e5 determinants, both ways timed).  Besides its elements, 16 ps each
 // against 31 to 39, the row path pays for
@@ -1512,11 +1516,16 @@ bool gather_numbers(const SysDev &d, long long n, unsigned long long nd) {
 //    1e4 35 and 24, 1e5 100 and 98; with 7 + 7 (1.2e6 rows) rows win from one determinant on (0.8 and 1.9).
 //    Without opposite-spin elements (no singles of one spin) all are records or own doubles, and
 //    the buckets win from 1e7 elements on (28 orbitals, 7 electrons: 1.70 ms and 2.58).
-bool gather_pays(const SysDev &d, long long n) {
+//    Beside other solvers of a batch their work hides most of these, all of them with one spin.  Six
+//    steps of batches of 24 orbitals: 8 systems of 7 + 0 electrons, 500 determinants 17.7 ms by rows,
+//    10.3 by buckets; 4 of 10 + 10, 50 determinants 18.0 and 13.9; but 8 of 8 + 8, 8 determinants 12.5
+//    and 17.3, 16 of 7 + 7, 300 determinants 34.8 and 47.2.
+bool gather_pays(const SysDev &d, long long n, bool beside) {
     const double ca = (double)d.ca, subs = d.na + d.po_a, hops = 1.0 + d.sa + (double)d.po_a * d.pv_a;
     const double elements = (double)n * (double)(d.n_conn + 1);
-    if ((d.sa == 0 || d.sb == 0) && elements > 1e7) return false;
-    return ca * (8.0 + 3.65 * subs) + 250.0 * std::min(ca, n * hops) <= 1.2e9 + 4.0 * elements;
+    if ((d.sa == 0 || d.sb == 0) && (beside || elements > 1e7)) return false;
+    if (d.cb <= kGSlots && !enough_units(ca, elements)) return false;  // (no row has classes)
+    return ca * (8.0 + 3.65 * subs) + 250.0 * std::min(ca, n * hops) <= (beside ? 0.3e9 : 1.2e9) + 4.0 * elements;
 }
 
 //  * every class of a heavy row that a source is read for, 12 to 44 ps: where few rows hold most
@@ -1524,11 +1533,9 @@ bool gather_pays(const SysDev &d, long long n) {
 //    0.65 visits per element (truncated Lanczos vectors of 28 orbitals: 0.01 to 0.42, rows 815 ms
 //    and buckets 973 at 0.42; ten rows of 2500 sources of 29 orbitals, 1 + 10 electrons: 4.4,
 //    105 ms and 14).
-//  * a chip that a few units leave idle: 3.5 ns per element of a unit (30 rows of 9e5 elements:
-//    3.8 ms, buckets 3.1).
 bool gather_pays(const SysDev &d, long long n, const GatherCounts &c) {
     const double elements = (double)n * (double)(d.n_conn + 1);
-    return (double)c.visits <= 0.65 * elements && (c.units >= 152 || elements <= 5e5 * (double)c.units);
+    return (double)c.visits <= 0.65 * elements && enough_units((double)c.units, elements);
 }
 
 // The standalone sigma's hash table has no preparation, but a warp per source (0.13 us an element in

@@ -581,10 +581,11 @@ size_t aligned_dots_ws_bytes(int nvec);
 cudaError_t aligned_dots(const VecRef *vecs, double *const *sig, int nvec, double *out_dev, void *ws,
                          cudaStream_t st);
 
-// sfci_lanczos.cu: sfci_lanczos_create with the device bytes a batch leaves the solver (0: no batch)
+// sfci_lanczos.cu: sfci_lanczos_create with the device bytes a batch leaves the solver (0: no batch);
+// beside: others of the batch step at the same time
 sfci_status lanczos_create(sfci_lanczos **out, const sfci_system *sys, const sfci_params *params,
                            const uint64_t *init_rank, const double *init_coef, int64_t n_init, void *stream,
-                           int64_t share);
+                           int64_t share, bool beside);
 
 // sfci_gather.cu -- sigma by target rows (see the file's header)
 constexpr int kGatherMaxElectrons = 12;  // per spin
@@ -721,7 +722,7 @@ struct GatherArgs {
 };
 bool gather_shape(const SysDev &d, GatherShape *p);  // false: the system is outside the gather's limits
 // whether sigma by target rows is faster than the buckets: before anything is prepared, and as planned
-bool gather_pays(const SysDev &d, long long n);
+bool gather_pays(const SysDev &d, long long n, bool beside);
 bool gather_pays(const SysDev &d, long long n, const GatherCounts &c);
 // the same against sfci_sigma's hash table (of so many slots)
 bool gather_beats_table(const SysDev &d, long long n, unsigned long long slots);

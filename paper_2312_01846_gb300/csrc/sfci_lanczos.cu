@@ -265,6 +265,7 @@ struct sfci_lanczos {
     // sigma by target rows (sfci_gather.cu)
     bool gather_ok = false;             // the system is within its limits
     int64_t share = 0;                  // device bytes a batch leaves this solver (0: no batch)
+    bool beside = false;                // others of the batch step at the same time
     int64_t alloc_limit = 0;            // a row gather buffer above it counts as out of memory (tests; 0: off)
     GatherShape gs{};
     Buf ga, gb, gc, vrp, seen;          // work arrays by the stage that sizes them; row pointers of each w_j;
@@ -898,7 +899,7 @@ double sigma_budget(const sfci_lanczos *z) {
 // the system is outside its limits, or the space too large for so short a vector.
 bool gather_wanted(const sfci_lanczos *z) {
     return z->gather_ok && z->p.bucket_elems == 0 && z->p.mem_budget == 0 && z->p.ovf_max_log2 == 0 &&
-           z->p.emit_warps == 0 && z->p.flags == 0 && gather_pays(z->sys->d, z->wn[z->idx]);
+           z->p.emit_warps == 0 && z->p.flags == 0 && gather_pays(z->sys->d, z->wn[z->idx], z->beside);
 }
 
 // sigma_i = H w_i by target rows, with sigma recorded at every basis entry;
@@ -1193,7 +1194,7 @@ namespace sfci {
 // sfci_lanczos_create; share > 0: the device bytes a batch leaves this solver's sigma
 sfci_status lanczos_create(sfci_lanczos **out, const sfci_system *sys, const sfci_params *params,
                            const uint64_t *init_rank, const double *init_coef, int64_t n_init, void *stream,
-                           int64_t share) {
+                           int64_t share, bool beside) {
     if (!out || !sys || !params) {
         set_error("null argument");
         return SFCI_E_INVALID;
@@ -1215,6 +1216,7 @@ sfci_status lanczos_create(sfci_lanczos **out, const sfci_system *sys, const sfc
     z->sys = sys;
     z->p = *params;
     z->share = share;
+    z->beside = beside;
     z->st = static_cast<cudaStream_t>(stream);
     z->NL = params->n_lanczos;
     z->nkeep = params->n_keep;
@@ -1300,7 +1302,7 @@ extern "C" {
 sfci_status sfci_lanczos_create(sfci_lanczos **out, const sfci_system *sys,
                                 const sfci_params *params, const uint64_t *init_rank,
                                 const double *init_coef, int64_t n_init, void *stream) {
-    return lanczos_create(out, sys, params, init_rank, init_coef, n_init, stream, 0);
+    return lanczos_create(out, sys, params, init_rank, init_coef, n_init, stream, 0, false);
 }
 
 sfci_status sfci_lanczos_step(sfci_lanczos *z, sfci_step_info *info) {

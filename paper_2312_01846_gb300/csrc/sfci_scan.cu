@@ -122,6 +122,8 @@ sfci_status sfci_scan_create(sfci_scan **out, int32_t count, const sfci_system *
         work[i] = (double)params[i].n_keep * (double)(systems[i]->d.n_conn + 1);
         total += work[i];
     }
+    int nw = workers > 0 ? workers : std::min(count, 8);
+    nw = std::max(1, std::min(nw, count));
     size_t free_b = 0, tot_b = 0;
     cudaMemGetInfo(&free_b, &tot_b);
     for (int i = 0; i < count; ++i) {
@@ -134,7 +136,7 @@ sfci_status sfci_scan_create(sfci_scan **out, int32_t count, const sfci_system *
             return cuda_fail(e, "sfci_scan_create");
         }
         const sfci_status r = lanczos_create(&s->lz[i], systems[i], &params[i], init_rank[i], init_coef[i],
-                                             n_init[i], s->streams[i], share);
+                                             n_init[i], s->streams[i], share, nw > 1);
         if (r != SFCI_OK) {
             const std::string msg = "instance " + std::to_string(i) + ": " + sfci_last_error();
             destroy_scan(s);
@@ -145,8 +147,6 @@ sfci_status sfci_scan_create(sfci_scan **out, int32_t count, const sfci_system *
     s->order.resize(count);
     for (int i = 0; i < count; ++i) s->order[i] = i;
     std::stable_sort(s->order.begin(), s->order.end(), [&](int a, int b) { return work[a] > work[b]; });
-    int nw = workers > 0 ? workers : std::min(count, 8);
-    nw = std::max(1, std::min(nw, count));
     try {
         for (int w = 0; w < nw; ++w) s->workers.emplace_back(worker_main, s);
     } catch (...) {

@@ -44,6 +44,32 @@ def test_solver_past_the_limit(sf):
     assert _by_rows(sf, lambda: solver._run(sf, d, 900, 3, solver.AUFBAU))[0] == 0
 
 
+# a batch, where the others' work hides what the buckets wait for
+@pytest.mark.parametrize("n,na,nb,dets,alone,beside", [
+    (24, 7, 0, 400, 1, 0),      # elements of one spin
+    (24, 10, 10, 50, 1, 0),     # 2e6 rows for 50 determinants
+    (24, 8, 8, 8, 1, 1),
+    (14, 4, 4, 500, 1, 1),
+])
+def test_scan_takes_the_faster_path(sf, n, na, nb, dets, alone, beside):
+    d = single._molecule(n, na, nb)
+    r, c = _rows_vector(d, min(3 * dets, math.comb(n, na)), dets)
+    out = []
+    for workers, want in ((1, alone), (2, beside)):
+        systems = [sf.System.from_dict(d) for _ in range(2)]
+        scan = sf.Scan([(s, r, c, dets) for s in systems], n_lanczos=3, workers=workers)
+        rows, infos = _by_rows(sf, scan.step)
+        assert rows == (2 + sum(i["redo"] for i in infos) if want else 0)
+        for i in range(2):
+            rk, cf = scan.vector(i)
+            out.append((infos[i]["a"], sf.to_u64(rk), cf.cpu().numpy().view(np.uint64)))
+        scan.close()
+        for s in systems:
+            s.close()
+    for a, rk, cf in out[1:]:
+        assert a == out[0][0] and np.array_equal(rk, out[0][1]) and np.array_equal(cf, out[0][2])
+
+
 def _restarts(sf, d, init, count, **kw):
     """Rows taken and launches of `count` restarts from one vector, and the last step's vector."""
     s = sf.System.from_dict(d)
