@@ -583,12 +583,14 @@ __global__ void row_units_kernel(RowPlan rp, const unsigned long long *aw, const
         if (w > rp.half) {
             const unsigned n = row_classes(rp, w);
             nu[k] = n;
+            if (rp.bb <= kGLog) continue;  // (one class)
             const unsigned long long v = nab[k] + 4ull * (src[row[k] + 1] - src[row[k]]);
             const bool seen = rp.seen[2 * weight_bin(w) + 1] > kSeenEnough;
             const unsigned m = seen ? n : class_count(rp, -rp.cb * expm1(-(double)w / rp.cb));
             if (m > 1u) sum += seen ? m * v : m * v * 23ull / 32ull;
         } else nu[k] = k == 0 || aw[k - 1] > rp.half || wpre[k - 1] / rp.half != wpre[k] / rp.half;
     }
+    if (rp.bb <= kGLog) return;
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
     if ((threadIdx.x & 31) == 0 && sum) atomicAdd(visits, sum);
 }
