@@ -199,7 +199,7 @@ sfci_status sfci_truncate_topk_noalloc(const uint64_t *rank, const double *coef,
  * ovf_max_log2 not 0), a spin has more than 12 electrons or 2^26 strings, its lists do
  * not fit in memory, or the buckets are faster: a short vector in a space of many alpha
  * strings, or most of its entries on few alpha strings of a large space.  Both sum
- * exactly: the results are the same bits. */
+ * exactly: vectors, matrix elements and energies are the same bits (n_sigma: see there). */
 typedef struct sfci_params {
     int64_t n_keep;         /* N_d: entries kept per basis vector (Eq. 11)          */
     int64_t table_capacity; /* slots of sigma's hash table; 0 = sized automatically */
@@ -241,7 +241,9 @@ typedef struct sfci_step_info {
     double u_norm;     /* ||u_{i+1}|| before truncation (0 at a cycle end)          */
     double t00;        /* <w_0|H|w_0> of this cycle                                 */
     int64_t n_in;      /* entries of w_i                                            */
-    int64_t n_sigma;   /* entries of sigma_i after the screen                       */
+    int64_t n_sigma;   /* entries of sigma_i after the screen; the buckets may count
+                          entries whose every product is exactly zero (or below
+                          eps_element), by target rows such entries do not exist  */
     int64_t n_kept;    /* entries of the next basis vector                          */
     int64_t n_elements;/* intermediate elements enumerated for sigma_i              */
     int64_t n_psi;     /* non-zero entries of Psi = sum_j x_j w_j (cycle end)         */

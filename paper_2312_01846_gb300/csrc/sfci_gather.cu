@@ -89,7 +89,7 @@ __device__ unsigned long long unrank_one(unsigned long long r, int n, int m, con
     return s;
 }
 
-// the next string of the same electron count (Eq. 12's index plus one)
+// the next string of the same electron count (Eq. 12's index plus one): Gosper's step
 __device__ __forceinline__ unsigned long long next_string(unsigned long long x) {
     if (!x) return x;
     const int t = __ffsll((long long)x) - 1;
@@ -628,20 +628,6 @@ __global__ void write_units_kernel(RowPlan rp, const unsigned long long *aw, con
 }
 
 // ------------------------------------------------------------- row lists
-
-// Part q of nq as a member of one of min(nq, blocks) teams: blocks first,
-// first + step, ... are its team's; it is member `member` of `size` there.
-// (Parts left over when the teams do not divide nq get no block.)
-struct Team {
-    unsigned first, step, member, size;
-    __device__ __forceinline__ Team(unsigned q, unsigned nq, unsigned blocks) {
-        size = blocks > 0u && blocks < nq ? nq / blocks : 1u;
-        step = nq / size;
-        first = q / size;
-        member = q - first * size;
-        if (first >= step) first = 0x4000000u;
-    }
-};
 
 // which of the segments starting at cs (ascending over the lanes, ~0 past the
 // last) holds element e0 + lane (every lane calls it)

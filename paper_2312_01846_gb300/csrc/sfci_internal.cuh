@@ -552,9 +552,9 @@ cudaError_t exclusive_scan(const unsigned *in, long long m, unsigned long long *
                            cudaStream_t st);
 cudaError_t exclusive_scan(const unsigned long long *in, long long m, unsigned long long *out, void *ws,
                            cudaStream_t st);
-// four arrays of m counts, one behind the other, in the same launches (ws: 4 scan_ws_bytes(m))
 // sig[j][0..n[j]) = 0
 cudaError_t zero_vectors(double *const *sig, const long long *n, int nvec, cudaStream_t st);
+// four arrays of m counts, one behind the other, in the same launches (ws: 4 scan_ws_bytes(m))
 cudaError_t exclusive_scan4(const unsigned *in, long long m, unsigned long long *const out[4], void *ws,
                             cudaStream_t st);
 cudaError_t sort_overflow(const Buckets &bk, const unsigned *count, unsigned lo, unsigned nb,
@@ -784,7 +784,6 @@ cudaError_t select_split(Items it, long long k,
                          unsigned long long *cand_key, double *cand_val, long long cand_cap,
                          unsigned long long *cand_n, void *ws, size_t ws_bytes, SplitResult *res_host,
                          cudaStream_t st);
-size_t sort_workspace_bytes(long long n);
 // stable LSD radix sort of (key, val) by key on the low `bits` bits; result in
 // key/val (uses ws as ping-pong buffers); n read from the device when n_dev
 size_t sort_pairs_bytes(long long cap);

@@ -276,7 +276,6 @@ constexpr int kT = 256;
 constexpr unsigned kChunk = 2048;       // determinants of a row in the table at once
 constexpr unsigned kSlots = 4096;
 constexpr unsigned kNone = 0xffffffffu;
-constexpr unsigned kGrab = 1;  // units taken from the queue at a time (4: 0.7 ms more at 3e5 determinants)
 
 struct RowArgs {
     SysDev d;
@@ -508,10 +507,10 @@ __global__ void __launch_bounds__(kT, 5) rdm_rows_kernel(const __grid_constant__
         __syncwarp();
     };
     for (;;) {
-        __syncthreads();
-        if (warp == 0) {
+        __syncthreads();  // (the unit before is done with the shared memory)
+        if (warp == 0) {  // (one unit at a time: four take 0.7 ms more at 3e5 determinants)
             unsigned long long u = 0ull;
-            if (lane == 0) u = atomicAdd(A.queue, (unsigned long long)kGrab);
+            if (lane == 0) u = atomicAdd(A.queue, 1ull);
             u = __shfl_sync(kFull, u, 0);
             unsigned lo = 0, hi = runs;  // the last run whose units start at or before u
             while (u < total && hi - lo > 1u) {
@@ -523,260 +522,256 @@ __global__ void __launch_bounds__(kT, 5) rdm_rows_kernel(const __grid_constant__
             if (lane == 0) S.u0 = u, S.run = lo;
         }
         __syncthreads();
-        const unsigned long long u0 = S.u0, u1 = u0 + kGrab < total ? u0 + kGrab : total;
-        if (u0 >= total) break;
-        unsigned run = S.run;
-        for (unsigned long long u = u0; u < u1; ++u) {
-            while (u >= __ldg(&A.uoff[run + 1])) ++run;
-            const unsigned base = __ldg(&A.run_off[run]), m = __ldg(&A.run_off[run + 1]) - base;
-            const unsigned long long str = __ldg(&A.run_str[run]);
-            const RowUnits U = row_units(d, m);
-            unsigned long long q = u - __ldg(&A.uoff[run]);
-            __syncthreads();  // (the unit before is done with the shared memory)
-            if (q >= U.n1 + U.n2) {
-                // ---- pairs within the row: tile e against the strings f < e of four tiles
-                q -= U.n1 + U.n2;
-                const unsigned te = (unsigned)(q / U.nf), f0 = (unsigned)(q % U.nf) * kTileF;
-                if (f0 > te * kT) continue;
-                have_run = kNone;
-                unsigned long long *fs = reinterpret_cast<unsigned long long *>(S.keys);
-                double *fc = reinterpret_cast<double *>(fs + kTileF);
-                unsigned long long *es = reinterpret_cast<unsigned long long *>(S.pos);
-                double *ec = reinterpret_cast<double *>(es + kT);
-                const unsigned e = te * kT + tid, nf = min(kTileF, m - f0), ne = min((unsigned)kT, m - te * kT);
-                for (unsigned f = tid; f < nf; f += kT) {
-                    fs[f] = __ldg(&A.bstr[__ldg(&A.s_id[base + f0 + f])]);
-                    fc[f] = __ldg(&A.coef[base + f0 + f]);
-                }
-                if (e < m) {
-                    es[tid] = __ldg(&A.bstr[__ldg(&A.s_id[base + e])]);
-                    ec[tid] = __ldg(&A.coef[base + e]);
-                }
-                __syncthreads();
-                {
-                    const unsigned long long be = e < m ? es[tid] : 0ull;
-                    const unsigned fe = e < m ? min(nf, e > f0 ? e - f0 : 0u) : 0u;
-                    const unsigned all = __reduce_max_sync(kFull, fe);
-                    const unsigned local = (unsigned)tid << 16;
-                    auto pair = [&](unsigned long long x) {
-                        const unsigned le = (unsigned)x >> 16, lf = (unsigned)x & 0xffffu;
-                        const double ce = ec[le], cf = fc[lf];
-                        if (ce != 0.0 && cf != 0.0) same_spin_pair(A.g1, A.g2, n, es[le], fs[lf], str, ce * cf);
-                    };
-                    if (n <= 32)
-                        for (unsigned f = 0; f < all; ++f)
-                            push(f < fe && __popc((unsigned)be ^ (unsigned)fs[f]) <= 4, local | f, pair);
-                    else
-                        for (unsigned f = 0; f < all; ++f) push(f < fe && __popcll(be ^ fs[f]) <= 4, local | f, pair);
-                    finish(pair);
-                }
-                if (f0 == 0u) {
-                    // D' = D: a thread per pair of beta orbitals (p < q: both occupied; p = q:
-                    // one) and one for the row's weight, along the tile
-                    for (int x = tid; x <= n * n; x += kT) {
-                        const int p = x / n, r = x - p * n;
-                        if (x < n * n && r < p) continue;
-                        const unsigned long long both = x < n * n ? (1ull << p | 1ull << r) : 0ull;
-                        double w = 0.0;
-                        for (unsigned f = 0; f < ne; ++f)
-                            if ((es[f] & both) == both && ec[f] != 0.0) w = __fma_rn(ec[f], ec[f], w);
-                        if (w == 0.0) continue;
-                        if (x == n * n) {
-                            for (unsigned long long k = str; k; k &= k - 1ull) {
-                                const int i = __ffsll((long long)k) - 1;
-                                if (staged) diag[n * n + i * n + i] += w;
-                                else acc(A.g1, size_t(i) * n + i, w);
-                                for (unsigned long long l = k & (k - 1ull); l; l &= l - 1ull) {
-                                    const int j = __ffsll((long long)l) - 1;
-                                    if (staged) diag[n * n + i * n + j] += w;
-                                    else same(i, j, w);
-                                }
-                            }
-                        } else if (p == r) {
-                            if (staged) diag[x] += w;
-                            else acc(A.g1, size_t(p) * n + p, w);
-                            for (unsigned long long k = str; k; k &= k - 1ull) {
-                                const int i = __ffsll((long long)k) - 1;
-                                if (staged) diag[2 * n * n + i * n + p] += w;
-                                else acc(A.g2, i * N3 + i * N2 + p * N1 + p, 0.5 * w);
-                            }
-                        } else {
-                            if (staged) diag[x] += w;
-                            else same(p, r, w);
-                        }
-                    }
-                }
-                continue;
+        const unsigned long long u = S.u0;
+        if (u >= total) break;
+        const unsigned run = S.run;
+        const unsigned base = __ldg(&A.run_off[run]), m = __ldg(&A.run_off[run + 1]) - base;
+        const unsigned long long str = __ldg(&A.run_str[run]);
+        const RowUnits U = row_units(d, m);
+        unsigned long long q = u - __ldg(&A.uoff[run]);
+        if (q >= U.n1 + U.n2) {
+            // ---- pairs within the row: tile e against the strings f < e of four tiles
+            q -= U.n1 + U.n2;
+            const unsigned te = (unsigned)(q / U.nf), f0 = (unsigned)(q % U.nf) * kTileF;
+            if (f0 > te * kT) continue;
+            have_run = kNone;
+            unsigned long long *fs = reinterpret_cast<unsigned long long *>(S.keys);
+            double *fc = reinterpret_cast<double *>(fs + kTileF);
+            unsigned long long *es = reinterpret_cast<unsigned long long *>(S.pos);
+            double *ec = reinterpret_cast<double *>(es + kT);
+            const unsigned e = te * kT + tid, nf = min(kTileF, m - f0), ne = min((unsigned)kT, m - te * kT);
+            for (unsigned f = tid; f < nf; f += kT) {
+                fs[f] = __ldg(&A.bstr[__ldg(&A.s_id[base + f0 + f])]);
+                fc[f] = __ldg(&A.coef[base + f0 + f]);
             }
-            const bool opposite = q < U.n1;
-            if (!opposite) q -= U.n1;
-            const unsigned parts = opposite ? U.p1 : U.p2, nbat = opposite ? U.nb1 : U.nb2;
-            const unsigned t = (unsigned)(q / ((unsigned long long)parts * nbat));
-            const unsigned rem = (unsigned)(q - (unsigned long long)t * parts * nbat), batch = rem / parts, part = rem % parts;
-            const unsigned t0 = t * kChunk, mc = min(kChunk, m - t0);
-            // ---- the row's table and orbital lists
-            if (have_run != run || have_t != t) {
-                have_run = run, have_t = t;
-                unsigned size = 256u;
-                while (size < 4u * mc && size < kSlots) size *= 2u;
-                mask = size - 1u;
-                shift = 33 - __ffs((int)size);
-                for (unsigned h = tid; h < size; h += kT) S.keys[h] = kNone;
-                if (tid < n) {
-                    const int below = __popcll(str & ((1ull << tid) - 1ull));
-                    if ((str >> tid) & 1ull) S.occ[below] = (unsigned char)tid;
-                    else S.vir[tid - below] = (unsigned char)tid;
-                }
-                __syncthreads();
-                for (unsigned f = tid; f < mc; f += kT) {
-                    const unsigned key = __ldg(&A.s_b[base + t0 + f]);
-                    unsigned h = (key * 0x9E3779B1u) >> shift;
-                    while (atomicCAS(&S.keys[h], kNone, key) != kNone) h = (h + 1u) & mask;
-                    S.pos[h] = (unsigned short)f;
-                    if (m <= kFew) S.str[f] = __ldg(&A.bstr[__ldg(&A.s_id[base + f])]);
-                }
+            if (e < m) {
+                es[tid] = __ldg(&A.bstr[__ldg(&A.s_id[base + e])]);
+                ec[tid] = __ldg(&A.coef[base + e]);
             }
-            // ---- a batch of rows one or two hops away: hop from them to this row
-            const unsigned x = batch * kT + tid, n_hops = opposite ? d.sa : d.sa + d.po_a * d.pv_a;
-            unsigned cnt = 0, off = 0, hop = 0;
-            unsigned long long from = 0ull;
-            if (x < n_hops) {
-                int i1, a1, i2 = 0, a2 = 0;
-                const bool one = x < (unsigned)d.sa;
-                if (one) {
-                    a1 = S.occ[x / d.va], i1 = S.vir[x % d.va];
-                    from = str ^ (1ull << a1) ^ (1ull << i1);
-                } else {
-                    const unsigned y = x - d.sa;
-                    const unsigned char *po = d.pairs + 2 * (d.pair_off[0] + y / d.pv_a), *pv = d.pairs + 2 * (d.pair_off[1] + y % d.pv_a);
-                    a1 = S.occ[po[0]], a2 = S.occ[po[1]], i1 = S.vir[pv[0]], i2 = S.vir[pv[1]];
-                    from = str ^ (1ull << a1) ^ (1ull << i1) ^ (1ull << a2) ^ (1ull << i2);
-                }
-                const unsigned o = __ldg(&A.row_run[string_rank(from, bt, d.ks)]);
-                if (o != kNone) {
-                    off = __ldg(&A.run_off[o]);
-                    const unsigned mo = __ldg(&A.run_off[o + 1]) - off;
-                    if (mo < m || (mo == m && o < run)) cnt = mo;
-                }
-                hop = (unsigned)(a1 * n + i1) | (unsigned)parity64(from & between_mask(i1, a1)) << 31;
-            }
-            unsigned inc = cnt;
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(kFull, inc, o);
-                if (lane >= o) inc += y;
-            }
-            if (lane == 31) S.wsum[warp] = inc;
             __syncthreads();
-            for (int w = 0; w < warp; ++w) inc += S.wsum[w];
-            S.start[tid] = inc - cnt;
-            S.off[tid] = off - (inc - cnt);
-            S.hop[tid] = opposite ? hop : x;
-            if (tid == kT - 1) S.start[kT] = inc;
-            __syncthreads();
-            const unsigned tot = S.start[kT];
-            const unsigned lo = (unsigned)((unsigned long long)tot * part / parts), hi = (unsigned)((unsigned long long)tot * (part + 1) / parts);
-            if (lo == hi) continue;
-            auto segment = [&](unsigned at) {
-                unsigned o = 0;
-                for (unsigned step = kT / 2; step; step >>= 1)
-                    if (S.start[o + step] <= at) o += step;
-                return o;
-            };
-            if (opposite && m <= kFew && m < 2u * d.sb) {
+            {
+                const unsigned long long be = e < m ? es[tid] : 0ull;
+                const unsigned fe = e < m ? min(nf, e > f0 ? e - f0 : 0u) : 0u;
+                const unsigned all = __reduce_max_sync(kFull, fe);
+                const unsigned local = (unsigned)tid << 16;
                 auto pair = [&](unsigned long long x) {
-                    const unsigned s = (unsigned)(x >> 32), hp = S.hop[(unsigned)x >> 16 & 0xffffu], f = (unsigned)x & 0xffffu;
-                    const double c1 = __ldg(&A.coef[s]), c2 = __ldg(&A.coef[base + f]);
-                    if (c1 == 0.0 || c2 == 0.0) return;
-                    const unsigned long long b1 = __ldg(&A.bstr[__ldg(&A.s_id[s])]), b2 = S.str[f];
-                    const int j = __ffsll((long long)(b1 & ~b2)) - 1, b = __ffsll((long long)(b2 & ~b1)) - 1;
-                    const double v = c1 * c2;
-                    acc(A.g2, size_t(hp & 0x7fffffffu) * N2 + b * n + j,
-                        (hp >> 31 ^ (unsigned)parity64(b1 & between_mask(j, b))) ? -v : v);
+                    const unsigned le = (unsigned)x >> 16, lf = (unsigned)x & 0xffffu;
+                    const double ce = ec[le], cf = fc[lf];
+                    if (ce != 0.0 && cf != 0.0) same_spin_pair(A.g1, A.g2, n, es[le], fs[lf], str, ce * cf);
                 };
-                // a warp takes up to 32 determinants and runs through the row for each, end to end
-                const unsigned per = min(32u, (hi - lo + kT / 32 - 1u) / (kT / 32));
-                for (unsigned p0 = lo + warp * per; p0 < hi; p0 += per * (kT / 32)) {
-                    const unsigned k = min(per, hi - p0);
-                    unsigned o = 0, s = 0;
-                    unsigned long long bs = 0ull;
-                    if ((unsigned)lane < k) {
-                        o = segment(p0 + lane), s = S.off[o] + p0 + lane;
-                        bs = __ldg(&A.bstr[__ldg(&A.s_id[s])]);
-                    }
-                    unsigned l = (unsigned)lane / m, y = (unsigned)lane % m;
-                    const unsigned dl = 32u / m, dy = 32u % m;
-                    for (unsigned r = 0; r < k * m; r += 32u) {
-                        const unsigned src = l < k ? l : 0u;
-                        const unsigned long long b1 = __shfl_sync(kFull, bs, src);
-                        const unsigned s1 = __shfl_sync(kFull, s, src), o1 = __shfl_sync(kFull, o, src);
-                        push(l < k && __popcll(b1 ^ S.str[y]) == 2, (unsigned long long)s1 << 32 | o1 << 16 | y, pair);
-                        l += dl, y += dy;
-                        if (y >= m) y -= m, ++l;
-                    }
-                }
+                if (n <= 32)
+                    for (unsigned f = 0; f < all; ++f)
+                        push(f < fe && __popc((unsigned)be ^ (unsigned)fs[f]) <= 4, local | f, pair);
+                else
+                    for (unsigned f = 0; f < all; ++f) push(f < fe && __popcll(be ^ fs[f]) <= 4, local | f, pair);
                 finish(pair);
-            } else if (opposite) {
-                // a warp takes up to 32 determinants and runs through their hops end to end
-                const unsigned per = min(32u, (hi - lo + kT / 32 - 1u) / (kT / 32));
-                for (unsigned p0 = lo + warp * per; p0 < hi; p0 += per * (kT / 32)) {
-                    const unsigned k = min(per, hi - p0);
-                    unsigned id = 0, hp = 0;
-                    double c = 0.0;
-                    if ((unsigned)lane < k) {
-                        const unsigned o = segment(p0 + lane), s = S.off[o] + p0 + lane;
-                        id = __ldg(&A.s_id[s]) * (unsigned)d.sb, hp = S.hop[o];
-                        c = __ldg(&A.coef[s]);
-                    }
-                    unsigned l = (unsigned)lane / d.sb, y = (unsigned)lane % d.sb;
-                    const unsigned dl = 32u / d.sb, dy = 32u % d.sb;
-                    for (unsigned r = 0; r < k * d.sb; r += 32u) {
-                        const bool in = l < k;
-                        const unsigned src = in ? l : 0u;
-                        const unsigned id1 = __shfl_sync(kFull, id, src), hp1 = __shfl_sync(kFull, hp, src);
-                        const double c1 = __shfl_sync(kFull, c, src);
-                        if (in) {
-                            const uint2 e = __ldg(&A.hops[(size_t)id1 + y]);
-                            const int f = row_find(S.keys, mask, shift, e.x);
-                            if (f >= 0) {
-                                const double c2 = __ldg(&A.coef[base + t0 + S.pos[f]]);
-                                if (c1 != 0.0 && c2 != 0.0) {
-                                    const double v = c1 * c2;
-                                    acc(A.g2, size_t(hp1 & 0x7fffffffu) * N2 + (e.y & 0x7fffffffu), (hp1 ^ e.y) >> 31 ? -v : v);
-                                }
+            }
+            if (f0 == 0u) {
+                // D' = D: a thread per pair of beta orbitals (p < q: both occupied; p = q:
+                // one) and one for the row's weight, along the tile
+                for (int x = tid; x <= n * n; x += kT) {
+                    const int p = x / n, r = x - p * n;
+                    if (x < n * n && r < p) continue;
+                    const unsigned long long both = x < n * n ? (1ull << p | 1ull << r) : 0ull;
+                    double w = 0.0;
+                    for (unsigned f = 0; f < ne; ++f)
+                        if ((es[f] & both) == both && ec[f] != 0.0) w = __fma_rn(ec[f], ec[f], w);
+                    if (w == 0.0) continue;
+                    if (x == n * n) {
+                        for (unsigned long long k = str; k; k &= k - 1ull) {
+                            const int i = __ffsll((long long)k) - 1;
+                            if (staged) diag[n * n + i * n + i] += w;
+                            else acc(A.g1, size_t(i) * n + i, w);
+                            for (unsigned long long l = k & (k - 1ull); l; l &= l - 1ull) {
+                                const int j = __ffsll((long long)l) - 1;
+                                if (staged) diag[n * n + i * n + j] += w;
+                                else same(i, j, w);
                             }
                         }
-                        l += dl, y += dy;
-                        if (y >= (unsigned)d.sb) y -= d.sb, ++l;
-                    }
-                }
-            } else {
-                // a pair: source in the upper half, its hop and its place in the table in the lower
-                auto pair = [&](unsigned long long x) {
-                    const unsigned s = (unsigned)(x >> 32), y = S.hop[(unsigned)x >> 16 & 0xffffu], f = (unsigned)x & 0xffffu;
-                    const double c1 = __ldg(&A.coef[s]), c2 = __ldg(&A.coef[base + t0 + f]);
-                    if (c1 == 0.0 || c2 == 0.0) return;
-                    unsigned long long a = str;
-                    if (y < (unsigned)d.sa) {
-                        a ^= (1ull << S.occ[y / d.va]) ^ (1ull << S.vir[y % d.va]);
+                    } else if (p == r) {
+                        if (staged) diag[x] += w;
+                        else acc(A.g1, size_t(p) * n + p, w);
+                        for (unsigned long long k = str; k; k &= k - 1ull) {
+                            const int i = __ffsll((long long)k) - 1;
+                            if (staged) diag[2 * n * n + i * n + p] += w;
+                            else acc(A.g2, i * N3 + i * N2 + p * N1 + p, 0.5 * w);
+                        }
                     } else {
-                        const unsigned z = y - d.sa;
-                        const unsigned char *po = d.pairs + 2 * (d.pair_off[0] + z / d.pv_a), *pv = d.pairs + 2 * (d.pair_off[1] + z % d.pv_a);
-                        a ^= (1ull << S.occ[po[0]]) ^ (1ull << S.occ[po[1]]) ^ (1ull << S.vir[pv[0]]) ^ (1ull << S.vir[pv[1]]);
+                        if (staged) diag[x] += w;
+                        else same(p, r, w);
                     }
-                    same_spin_pair(A.g1, A.g2, n, a, str, __ldg(&A.bstr[__ldg(&A.s_id[s])]), c1 * c2);
-                };
-                for (unsigned i0 = lo + warp * 32; i0 < hi; i0 += kT) {
-                    const unsigned it = i0 + lane;
-                    unsigned o = 0, s = 0;
-                    int f = -1;
-                    if (it < hi) {
-                        o = segment(it), s = S.off[o] + it;
-                        f = row_find(S.keys, mask, shift, __ldg(&A.s_b[s]));
-                    }
-                    push(f >= 0, (unsigned long long)s << 32 | o << 16 | (f >= 0 ? S.pos[f] : 0), pair);
                 }
-                finish(pair);
             }
+            continue;
+        }
+        const bool opposite = q < U.n1;
+        if (!opposite) q -= U.n1;
+        const unsigned parts = opposite ? U.p1 : U.p2, nbat = opposite ? U.nb1 : U.nb2;
+        const unsigned t = (unsigned)(q / ((unsigned long long)parts * nbat));
+        const unsigned rem = (unsigned)(q - (unsigned long long)t * parts * nbat), batch = rem / parts, part = rem % parts;
+        const unsigned t0 = t * kChunk, mc = min(kChunk, m - t0);
+        // ---- the row's table and orbital lists
+        if (have_run != run || have_t != t) {
+            have_run = run, have_t = t;
+            unsigned size = 256u;
+            while (size < 4u * mc && size < kSlots) size *= 2u;
+            mask = size - 1u;
+            shift = 33 - __ffs((int)size);
+            for (unsigned h = tid; h < size; h += kT) S.keys[h] = kNone;
+            if (tid < n) {
+                const int below = __popcll(str & ((1ull << tid) - 1ull));
+                if ((str >> tid) & 1ull) S.occ[below] = (unsigned char)tid;
+                else S.vir[tid - below] = (unsigned char)tid;
+            }
+            __syncthreads();
+            for (unsigned f = tid; f < mc; f += kT) {
+                const unsigned key = __ldg(&A.s_b[base + t0 + f]);
+                unsigned h = (key * 0x9E3779B1u) >> shift;
+                while (atomicCAS(&S.keys[h], kNone, key) != kNone) h = (h + 1u) & mask;
+                S.pos[h] = (unsigned short)f;
+                if (m <= kFew) S.str[f] = __ldg(&A.bstr[__ldg(&A.s_id[base + f])]);
+            }
+        }
+        // ---- a batch of rows one or two hops away: hop from them to this row
+        const unsigned x = batch * kT + tid, n_hops = opposite ? d.sa : d.sa + d.po_a * d.pv_a;
+        unsigned cnt = 0, off = 0, hop = 0;
+        unsigned long long from = 0ull;
+        if (x < n_hops) {
+            int i1, a1, i2 = 0, a2 = 0;
+            const bool one = x < (unsigned)d.sa;
+            if (one) {
+                a1 = S.occ[x / d.va], i1 = S.vir[x % d.va];
+                from = str ^ (1ull << a1) ^ (1ull << i1);
+            } else {
+                const unsigned y = x - d.sa;
+                const unsigned char *po = d.pairs + 2 * (d.pair_off[0] + y / d.pv_a), *pv = d.pairs + 2 * (d.pair_off[1] + y % d.pv_a);
+                a1 = S.occ[po[0]], a2 = S.occ[po[1]], i1 = S.vir[pv[0]], i2 = S.vir[pv[1]];
+                from = str ^ (1ull << a1) ^ (1ull << i1) ^ (1ull << a2) ^ (1ull << i2);
+            }
+            const unsigned o = __ldg(&A.row_run[string_rank(from, bt, d.ks)]);
+            if (o != kNone) {
+                off = __ldg(&A.run_off[o]);
+                const unsigned mo = __ldg(&A.run_off[o + 1]) - off;
+                if (mo < m || (mo == m && o < run)) cnt = mo;
+            }
+            hop = (unsigned)(a1 * n + i1) | (unsigned)parity64(from & between_mask(i1, a1)) << 31;
+        }
+        unsigned inc = cnt;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) S.wsum[warp] = inc;
+        __syncthreads();
+        for (int w = 0; w < warp; ++w) inc += S.wsum[w];
+        S.start[tid] = inc - cnt;
+        S.off[tid] = off - (inc - cnt);
+        S.hop[tid] = opposite ? hop : x;
+        if (tid == kT - 1) S.start[kT] = inc;
+        __syncthreads();
+        const unsigned tot = S.start[kT];
+        const unsigned lo = (unsigned)((unsigned long long)tot * part / parts), hi = (unsigned)((unsigned long long)tot * (part + 1) / parts);
+        if (lo == hi) continue;
+        auto segment = [&](unsigned at) {
+            unsigned o = 0;
+            for (unsigned step = kT / 2; step; step >>= 1)
+                if (S.start[o + step] <= at) o += step;
+            return o;
+        };
+        if (opposite && m <= kFew && m < 2u * d.sb) {
+            auto pair = [&](unsigned long long x) {
+                const unsigned s = (unsigned)(x >> 32), hp = S.hop[(unsigned)x >> 16 & 0xffffu], f = (unsigned)x & 0xffffu;
+                const double c1 = __ldg(&A.coef[s]), c2 = __ldg(&A.coef[base + f]);
+                if (c1 == 0.0 || c2 == 0.0) return;
+                const unsigned long long b1 = __ldg(&A.bstr[__ldg(&A.s_id[s])]), b2 = S.str[f];
+                const int j = __ffsll((long long)(b1 & ~b2)) - 1, b = __ffsll((long long)(b2 & ~b1)) - 1;
+                const double v = c1 * c2;
+                acc(A.g2, size_t(hp & 0x7fffffffu) * N2 + b * n + j,
+                    (hp >> 31 ^ (unsigned)parity64(b1 & between_mask(j, b))) ? -v : v);
+            };
+            // a warp takes up to 32 determinants and runs through the row for each, end to end
+            const unsigned per = min(32u, (hi - lo + kT / 32 - 1u) / (kT / 32));
+            for (unsigned p0 = lo + warp * per; p0 < hi; p0 += per * (kT / 32)) {
+                const unsigned k = min(per, hi - p0);
+                unsigned o = 0, s = 0;
+                unsigned long long bs = 0ull;
+                if ((unsigned)lane < k) {
+                    o = segment(p0 + lane), s = S.off[o] + p0 + lane;
+                    bs = __ldg(&A.bstr[__ldg(&A.s_id[s])]);
+                }
+                unsigned l = (unsigned)lane / m, y = (unsigned)lane % m;
+                const unsigned dl = 32u / m, dy = 32u % m;
+                for (unsigned r = 0; r < k * m; r += 32u) {
+                    const unsigned src = l < k ? l : 0u;
+                    const unsigned long long b1 = __shfl_sync(kFull, bs, src);
+                    const unsigned s1 = __shfl_sync(kFull, s, src), o1 = __shfl_sync(kFull, o, src);
+                    push(l < k && __popcll(b1 ^ S.str[y]) == 2, (unsigned long long)s1 << 32 | o1 << 16 | y, pair);
+                    l += dl, y += dy;
+                    if (y >= m) y -= m, ++l;
+                }
+            }
+            finish(pair);
+        } else if (opposite) {
+            // a warp takes up to 32 determinants and runs through their hops end to end
+            const unsigned per = min(32u, (hi - lo + kT / 32 - 1u) / (kT / 32));
+            for (unsigned p0 = lo + warp * per; p0 < hi; p0 += per * (kT / 32)) {
+                const unsigned k = min(per, hi - p0);
+                unsigned id = 0, hp = 0;
+                double c = 0.0;
+                if ((unsigned)lane < k) {
+                    const unsigned o = segment(p0 + lane), s = S.off[o] + p0 + lane;
+                    id = __ldg(&A.s_id[s]) * (unsigned)d.sb, hp = S.hop[o];
+                    c = __ldg(&A.coef[s]);
+                }
+                unsigned l = (unsigned)lane / d.sb, y = (unsigned)lane % d.sb;
+                const unsigned dl = 32u / d.sb, dy = 32u % d.sb;
+                for (unsigned r = 0; r < k * d.sb; r += 32u) {
+                    const bool in = l < k;
+                    const unsigned src = in ? l : 0u;
+                    const unsigned id1 = __shfl_sync(kFull, id, src), hp1 = __shfl_sync(kFull, hp, src);
+                    const double c1 = __shfl_sync(kFull, c, src);
+                    if (in) {
+                        const uint2 e = __ldg(&A.hops[(size_t)id1 + y]);
+                        const int f = row_find(S.keys, mask, shift, e.x);
+                        if (f >= 0) {
+                            const double c2 = __ldg(&A.coef[base + t0 + S.pos[f]]);
+                            if (c1 != 0.0 && c2 != 0.0) {
+                                const double v = c1 * c2;
+                                acc(A.g2, size_t(hp1 & 0x7fffffffu) * N2 + (e.y & 0x7fffffffu), (hp1 ^ e.y) >> 31 ? -v : v);
+                            }
+                        }
+                    }
+                    l += dl, y += dy;
+                    if (y >= (unsigned)d.sb) y -= d.sb, ++l;
+                }
+            }
+        } else {
+            // a pair: source in the upper half, its hop and its place in the table in the lower
+            auto pair = [&](unsigned long long x) {
+                const unsigned s = (unsigned)(x >> 32), y = S.hop[(unsigned)x >> 16 & 0xffffu], f = (unsigned)x & 0xffffu;
+                const double c1 = __ldg(&A.coef[s]), c2 = __ldg(&A.coef[base + t0 + f]);
+                if (c1 == 0.0 || c2 == 0.0) return;
+                unsigned long long a = str;
+                if (y < (unsigned)d.sa) {
+                    a ^= (1ull << S.occ[y / d.va]) ^ (1ull << S.vir[y % d.va]);
+                } else {
+                    const unsigned z = y - d.sa;
+                    const unsigned char *po = d.pairs + 2 * (d.pair_off[0] + z / d.pv_a), *pv = d.pairs + 2 * (d.pair_off[1] + z % d.pv_a);
+                    a ^= (1ull << S.occ[po[0]]) ^ (1ull << S.occ[po[1]]) ^ (1ull << S.vir[pv[0]]) ^ (1ull << S.vir[pv[1]]);
+                }
+                same_spin_pair(A.g1, A.g2, n, a, str, __ldg(&A.bstr[__ldg(&A.s_id[s])]), c1 * c2);
+            };
+            for (unsigned i0 = lo + warp * 32; i0 < hi; i0 += kT) {
+                const unsigned it = i0 + lane;
+                unsigned o = 0, s = 0;
+                int f = -1;
+                if (it < hi) {
+                    o = segment(it), s = S.off[o] + it;
+                    f = row_find(S.keys, mask, shift, __ldg(&A.s_b[s]));
+                }
+                push(f >= 0, (unsigned long long)s << 32 | o << 16 | (f >= 0 ? S.pos[f] : 0), pair);
+            }
+            finish(pair);
         }
     }
     if (!staged) return;

@@ -22,7 +22,7 @@
 // What bounds it: at 3e6 items (48 MB) launches and the chain of passes, not
 // bandwidth; the 2e5 largest of 3e6, sorted: 554 us with one-block scans over
 // all counters and a pick launch per pass, 379 us so.  Where the capacity is
-// far above the count, the kernels follow the count: an unsorted sigma of 3e7
+// far above the count, the kernels follow the count: an unsorted sigma of 2.2e7
 // entries 60.2 ms when sorting over the capacity, 27.3 ms so.  A step on the
 // whole 4900-determinant space: 1066 us with 30 launches a sort, 839 us so.
 // With a pass of up to 256 tiles in one launch and only the partial sums that are
@@ -1005,8 +1005,6 @@ size_t sort_pairs_bytes(long long cap) {
     const long long ntiles = (cap + kTile - 1) / kTile;
     return a256(size_t(cap) * 8) * 2 + sort_counts_bytes(ntiles) + a256(sizeof(SortState));
 }
-
-size_t sort_workspace_bytes(long long n) { return sort_pairs_bytes(n); }
 
 namespace {
 cudaError_t small_sort(unsigned long long *key, double *val, long long cap, const unsigned long long *n_dev, int bits,
