@@ -568,13 +568,13 @@ __device__ __forceinline__ unsigned row_classes(const RowPlan &r, unsigned long 
 // it is the first of its group: the light rows whose weight prefix starts in
 // one window of half a group)
 // visits: sources that its classes read, summed over the heavy rows; own ones count four
-// times (their segments are longer).  A row of a weight that no sigma has shown yet counts
-// 23 / 32 of the classes it would have if its elements were scattered over all strings: the
-// first plan's guess is for vectors like Lanczos', and scattered ones split each class again
-// and again.
+// times (their segments are longer).  The first plan's guess of a row's classes is for vectors
+// like Lanczos', whose sources share beta strings; scattered ones (hardly a beta string twice)
+// split each class again and again: a row of theirs, of a weight that no sigma has shown yet,
+// counts 23 / 32 of the classes it would have if its elements were scattered over all strings.
 __global__ void row_units_kernel(RowPlan rp, const unsigned long long *aw, const unsigned long long *wpre,
                                  const unsigned long long *n_act, const unsigned *nab, const unsigned *row,
-                                 const unsigned *src, unsigned *nu, unsigned long long *visits) {
+                                 const unsigned *src, unsigned *nu, bool scattered, unsigned long long *visits) {
     const unsigned long long A = *n_act;
     unsigned long long sum = 0ull;
     for (unsigned long long k = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; k < A;
@@ -585,9 +585,9 @@ __global__ void row_units_kernel(RowPlan rp, const unsigned long long *aw, const
             nu[k] = n;
             if (rp.bb <= kGLog) continue;  // (one class)
             const unsigned long long v = nab[k] + 4ull * (src[row[k] + 1] - src[row[k]]);
-            const bool seen = rp.seen[2 * weight_bin(w) + 1] > kSeenEnough;
-            const unsigned m = seen ? n : class_count(rp, -rp.cb * expm1(-(double)w / rp.cb));
-            if (m > 1u) sum += seen ? m * v : m * v * 23ull / 32ull;
+            const bool guess = scattered && rp.seen[2 * weight_bin(w) + 1] <= kSeenEnough;
+            const unsigned m = guess ? class_count(rp, -rp.cb * expm1(-(double)w / rp.cb)) : n;
+            if (m > 1u) sum += guess ? m * v * 23ull / 32ull : m * v;
         } else nu[k] = k == 0 || aw[k - 1] > rp.half || wpre[k - 1] / rp.half != wpre[k] / rp.half;
     }
     if (rp.bb <= kGLog) return;
@@ -1518,9 +1518,10 @@ bool gather_pays(const SysDev &d, long long n, bool beside) {
 
 //  * every class of a heavy row that a source is read for, 12 to 44 ps: where few rows hold most
 //    sources, classes outnumber the excitations of a string and most visits find nothing.  Up to
-//    0.65 visits per element (truncated Lanczos vectors of 28 orbitals: 0.01 to 0.42, rows 815 ms
-//    and buckets 973 at 0.42; ten rows of 2500 sources of 29 orbitals, 1 + 10 electrons: 4.4,
-//    105 ms and 14).
+//    0.65 visits per element.  Truncated Lanczos vectors of 28 orbitals, 7 + 7 electrons, 1e5 to 1e6
+//    determinants 0.06 to 0.38, rows 0.68 to 0.81 of the buckets' time (1e6: 680 to 770 ms and 980);
+//    22 orbitals, 3 + 9 0.43 to 0.53, 0.68; 28 orbitals, 3 + 8 0.96 to 1.5, 1.7 to 2.2; 2 + 9 1.2 to
+//    2.2, 2.4 to 3.8; scattered vectors of 29 orbitals, 1 + 10 electrons 3.1 to 4.4, 7 to 11.
 bool gather_pays(const SysDev &d, long long n, const GatherCounts &c) {
     const double elements = (double)n * (double)(d.n_conn + 1);
     return (double)c.visits <= 0.65 * elements && enough_units((double)c.units, elements);
@@ -1669,7 +1670,7 @@ cudaError_t gather_tables(const SysDev &d, const GatherShape &p, long long n, un
     if (e != cudaSuccess) return e;
     count_launch();
     row_units_kernel<<<grid_for(d.ca, 256), 256, 0, st>>>(row_plan(d, p, b, ra), b.aw, b.wpre, b.apos + d.ca, b.nab,
-                                                          b.act_row, rp, b.nu, b.words + 8);
+                                                          b.act_row, rp, b.nu, 4.0 * nd > 3.0 * (double)n, b.words + 8);
     unsigned long long *const out[4] = {b.rec_off, b.ab_off, b.poff, b.uoff};  // nrec | nab | np | nu
     return exclusive_scan4(b.nrec, (long long)d.ca, out, b.scan_ws, st);
 }

@@ -138,6 +138,18 @@ def test_sigma(sf, name):
     s.close()
 
 
+def test_solver_takes_rows_for_its_vectors(sf):
+    """The vectors of a solver's own first steps, whose sources share beta strings: planned as if they
+    were scattered, the second has 1.9 visits an element (0.3 in truth: 6 ms by rows, 10 by buckets)."""
+    s = sf.System.from_dict(single._molecule(28, 2, 9))
+    lz = sf.Lanczos(s, np.zeros(1, dtype=np.uint64), np.ones(1), 16000, n_lanczos=3)
+    rows, infos = _by_rows(sf, lambda: [lz.step() for _ in range(2)])
+    lz.close()
+    s.close()
+    assert infos[1]["n_in"] > 15000
+    assert rows == 2 + sum(i["redo"] for i in infos)
+
+
 # the standalone sigma: few elements a source, elements of one spin (both while the table is small),
 # and heavy rows whose classes visit sources more often than there are elements
 @pytest.mark.parametrize("n,na,nb,rows,dets,caps,by_rows", [
