@@ -233,8 +233,9 @@ def sfci_sigma(sys: System, rank, coef, eps_screen=0.0, out_cap=None, stream=Non
     if out_cap is not None:
         cap = int(out_cap)
     else:
-        room = _SIGMA_ROOM if _rows_possible(sys) else _SIGMA_ROOM_TABLE
-        cap = max(1024, min(r.numel() * (sys.n_conn + 1), room))
+        cap = max(1024, r.numel() * (sys.n_conn + 1))
+        if cap > _SIGMA_ROOM_TABLE:
+            cap = min(cap, _SIGMA_ROOM if _rows_possible(sys) else _SIGMA_ROOM_TABLE)
     first = True
     for _ in range(16):
         try:

@@ -419,7 +419,7 @@ sfci_status sigma_rows(const sfci_system *s, const unsigned long long *rank, con
     gather_place_tables(w + at, b, d, gs, nd, n);
     at += size_b;
     const RowPlanArgs ra = row_plan_args(d, gs, n);
-    SFCI_CUDA(gather_tables(d, gs, n, (unsigned)nd, s->pair_int, rp, b, ra, st));
+    SFCI_CUDA(gather_tables(d, gs, n, (unsigned)nd, s->pair_int, rp, b, ra, true, st));
     GatherCounts gn{};
     SFCI_CUDA(gather_counts(d, b, &gn, st));
     if (!gn.fit() || !gather_beats_table(d, n, gn) || at + gather_place_lists(nullptr, b, gs, gn) > room) return SFCI_OK;

@@ -568,10 +568,14 @@ __device__ __forceinline__ unsigned row_classes(const RowPlan &r, unsigned long 
 // it is the first of its group: the light rows whose weight prefix starts in
 // one window of half a group)
 // visits: sources that its classes read, summed over the heavy rows; own ones count four
-// times (their segments are longer).  The first plan's guess of a row's classes is for vectors
-// like Lanczos', whose sources share beta strings; scattered ones (hardly a beta string twice)
-// split each class again and again: a row of theirs, of a weight that no sigma has shown yet,
-// counts 23 / 32 of the classes it would have if its elements were scattered over all strings.
+// times (their segments are longer).
+// The guess of row_classes is for vectors like Lanczos', whose sources share beta strings.  Where
+// they do not (scattered), and no sigma has shown yet what the rows hold, a row's elements count as
+// scattered over all strings: planned by the other guess its classes split again and again (3e5
+// determinants drawn from 2e4 rows of 28 orbitals: the first sigma 825 ms, 532 so, by buckets 627).
+// That is the most a row can hold, so a quarter more than a class should hold is left in one (two
+// took 2 % of a sigma of 73 determinants; with every class 18 % fuller they overflow: 30000 of 28
+// orbitals, 1 + 7 electrons 23.9 and 37.7 ms), and its visits count 23 / 32.
 __global__ void row_units_kernel(RowPlan rp, const unsigned long long *aw, const unsigned long long *wpre,
                                  const unsigned long long *n_act, const unsigned *nab, const unsigned *row,
                                  const unsigned *src, unsigned *nu, bool scattered, unsigned long long *visits) {
@@ -580,14 +584,19 @@ __global__ void row_units_kernel(RowPlan rp, const unsigned long long *aw, const
     for (unsigned long long k = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; k < A;
          k += (unsigned long long)gridDim.x * blockDim.x) {
         const unsigned long long w = aw[k];
-        if (w > rp.half) {
-            const unsigned n = row_classes(rp, w);
+        if (w > rp.half && rp.bb <= kGLog) {
+            nu[k] = 1u;  // (one table holds all strings)
+        } else if (w > rp.half) {
+            unsigned n;
+            if (scattered) {
+                const double most = -rp.cb * expm1(-(double)w / rp.cb);
+                n = most <= 1.25 * rp.fill ? 1u : class_count(rp, most);
+            } else {
+                n = row_classes(rp, w);
+            }
             nu[k] = n;
-            if (rp.bb <= kGLog) continue;  // (one class)
             const unsigned long long v = nab[k] + 4ull * (src[row[k] + 1] - src[row[k]]);
-            const bool guess = scattered && rp.seen[2 * weight_bin(w) + 1] <= kSeenEnough;
-            const unsigned m = guess ? class_count(rp, -rp.cb * expm1(-(double)w / rp.cb)) : n;
-            if (m > 1u) sum += guess ? m * v * 23ull / 32ull : m * v;
+            if (n > 1u) sum += scattered ? n * v * 23ull / 32ull : n * v;
         } else nu[k] = k == 0 || aw[k - 1] > rp.half || wpre[k - 1] / rp.half != wpre[k] / rp.half;
     }
     if (rp.bb <= kGLog) return;
@@ -1536,19 +1545,18 @@ bool gather_pays(const SysDev &d, long long n, const GatherCounts &c) {
 //  * elements of one spin alone (records or own doubles, no table of singles to share), until the
 //    slots cost more: 28 orbitals, 7 electrons, 872 determinants (2^23 slots) 0.98 and 2.13, 8636
 //    (2^22) 1.41 and 1.84, but (2^26) 4.03 and 3.48; 24 orbitals, 12 electrons, 300 determinants
-//    (2^22) 1.02 and 0.91, 1000 1.19 and 1.30.
+//    (2^22) 1.02 and 0.77, 2000 1.28 and 1.80.
 bool gather_beats_table(const SysDev &d, long long n, unsigned long long slots) {
     if (d.n_conn <= 1150 && slots <= 1ull << 20) return false;
     return (d.sa > 0 && d.sb > 0) || slots > 1ull << 23 || (double)n * (double)(d.n_conn + 1) < 2e6;
 }
 
-// and to heavy rows whose classes visit sources more often than there are elements, a few
-// milliseconds of visits at least (the plan is made for nothing then: about 0.7 ms).  28 orbitals,
-// 1 + 7 electrons: 1.07 visits an element (1e4 determinants) 14.5 ms by rows, 9.7 by the table, 1.16
-// (3e4) 38.8 and 22.2; 29 orbitals, 1 + 10: 0.92 (3000) 8.7 and 9.1, 2.1 (8000) 32 and 22, 3.1 (25000)
-// 189 and 57; 26 orbitals, 2 + 9: 0.79 (1e4) 19.9 and 21.3.
+// and to heavy rows whose classes visit sources more than twice as often as there are elements (the
+// plan, about 0.7 ms, is made for nothing then).  28 orbitals, 1 + 9 electrons: 1.3 visits an element
+// (5000 determinants) 8.9 ms by rows, 12.4 by the table, 2.3 (1e4) 20.9 and 20.1, 3.6 (2e4) 52 and 34; 29
+// orbitals, 1 + 10: 2.1 (8000) 21.4 and 22.1, 3.1 (25000) 115 and 57.
 bool gather_beats_table(const SysDev &d, long long n, const GatherCounts &c) {
-    return (double)c.visits <= std::max((double)n * (double)(d.n_conn + 1), 8e7);
+    return (double)c.visits <= 2.2 * (double)n * (double)(d.n_conn + 1);
 }
 
 // What the lists take at least, whatever the rows: a source is listed under C(n_alpha, 2) substrings
@@ -1634,7 +1642,7 @@ cudaError_t gather_sources(const SysDev &d, const GatherShape &p, const unsigned
 }
 
 cudaError_t gather_tables(const SysDev &d, const GatherShape &p, long long n, unsigned nd, const double *W,
-                          const unsigned *rp, const GatherBufs &b, const RowPlanArgs &ra, cudaStream_t st) {
+                          const unsigned *rp, const GatherBufs &b, const RowPlanArgs &ra, bool fresh, cudaStream_t st) {
     const size_t bts = size_t(d.n + 1) * d.ks * 8;
     count_launch();
     const size_t fields_smem = bts + (d.n <= kStageN ? size_t(2 * d.n + 1) * d.n * 8 : 0);
@@ -1668,9 +1676,13 @@ cudaError_t gather_tables(const SysDev &d, const GatherShape &p, long long n, un
                                                                b.act_row, b.act_str, b.aw, b.nrec, b.nab, b.np);
     e = exclusive_scan(static_cast<const unsigned long long *>(b.aw), (long long)d.ca, b.wpre, b.scan_ws, st);
     if (e != cudaSuccess) return e;
+    // (drawn at random, n sources have cb (1 - exp(-n / cb)) beta strings; a vector of many more
+    // than cb has them all, whatever it is)
+    const double cb = (double)d.cb, drawn = -cb * std::expm1(-(double)n / cb);
+    const bool scattered = fresh && (double)nd > 0.75 * drawn && (double)n < 1.5 * cb;
     count_launch();
     row_units_kernel<<<grid_for(d.ca, 256), 256, 0, st>>>(row_plan(d, p, b, ra), b.aw, b.wpre, b.apos + d.ca, b.nab,
-                                                          b.act_row, rp, b.nu, 4.0 * nd > 3.0 * (double)n, b.words + 8);
+                                                          b.act_row, rp, b.nu, scattered, b.words + 8);
     unsigned long long *const out[4] = {b.rec_off, b.ab_off, b.poff, b.uoff};  // nrec | nab | np | nu
     return exclusive_scan4(b.nrec, (long long)d.ca, out, b.scan_ws, st);
 }

@@ -746,9 +746,9 @@ cudaError_t launch_row_pointers(const SysDev &d, const unsigned long long *rank,
 cudaError_t gather_sources(const SysDev &d, const GatherShape &p, const unsigned long long *rank, const double *coef,
                            long long n, const GatherBufs &b, cudaStream_t st);
 // beta tables, substring lists, row plan (active rows in apos[ca], units in uoff[ca], list parts in poff[ca],
-// records in rec_off[ca], one-hop sources in ab_off[ca])
+// records in rec_off[ca], one-hop sources in ab_off[ca]); fresh: b.seen has nothing yet
 cudaError_t gather_tables(const SysDev &d, const GatherShape &p, long long n, unsigned nd, const double *W,
-                          const unsigned *rp, const GatherBufs &b, const RowPlanArgs &ra, cudaStream_t st);
+                          const unsigned *rp, const GatherBufs &b, const RowPlanArgs &ra, bool fresh, cudaStream_t st);
 cudaError_t gather_lists(const SysDev &d, const GatherShape &p, unsigned long long n_act, unsigned long long n_parts,
                          const double *W, const unsigned *rp, const GatherBufs &b, const RowPlanArgs &ra,
                          cudaStream_t st);

@@ -271,6 +271,7 @@ struct sfci_lanczos {
     Buf ga, gb, gc, vrp, seen;          // work arrays by the stage that sizes them; row pointers of each w_j;
                                         // elements and distinct entries by row weight
     std::vector<char> vrp_ok;           // row pointers of w_j are current
+    bool rows_seen = false;             // a sigma by rows has left its statistics
     long long no_rows_n = 0;            // the last input whose lists did not fit (0: none yet),
     double no_rows_budget = 0.0;        // in so many bytes
     int rows_skip = 0, rows_wait = 0;   // sigmas that still go to the buckets without a plan by rows; after the next
@@ -985,7 +986,7 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
     if ((r = grow(z->gb, size_b, "row gather tables", 1.1))) return r;
     gather_place_tables(static_cast<char *>(z->gb.p), b, d, gs, nd, n_in);
     const RowPlanArgs ra = row_plan_args(d, gs, n_in);
-    SFCI_CUDA(gather_tables(d, gs, n_in, (unsigned)nd, z->sys->pair_int, rp, b, ra, z->st));
+    SFCI_CUDA(gather_tables(d, gs, n_in, (unsigned)nd, z->sys->pair_int, rp, b, ra, !z->rows_seen, z->st));
     SFCI_CUDA(gather_counts(d, b, &z->host->counts, z->st));
     const GatherCounts gn = z->host->counts;
     if (!gn.fit()) return SFCI_OK;
@@ -1082,7 +1083,7 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
         while ((1ull << z->nb_log2) < gn.units) ++z->nb_log2;
         if (budget >= 0.0) z->budget_gb = budget / 1e9, z->free_gb = (budget - held) / 1e9, z->held_gb = held / 1e9;
         z->regions_gb = E * sizeof(Slot) / 1e9;  // what the elements would take as records
-        *done = true;
+        *done = z->rows_seen = true;
         count_row_sigma();
         return SFCI_OK;
     }

@@ -151,7 +151,7 @@ def test_solver_takes_rows_for_its_vectors(sf):
 
 
 # the standalone sigma: few elements a source, elements of one spin (both while the table is small),
-# and heavy rows whose classes visit sources more often than there are elements
+# and heavy rows whose classes visit sources more than twice as often as there are elements
 @pytest.mark.parametrize("n,na,nb,rows,dets,caps,by_rows", [
     (28, 1, 1, 28, 300, (1 << 19, (1 << 19) + 1), (0, 1)),
     (40, 1, 1, 40, 300, (1 << 19, 1 << 20), (1, 1)),
@@ -159,7 +159,8 @@ def test_solver_takes_rows_for_its_vectors(sf):
     (24, 0, 12, 1, 2000, (1 << 22, (1 << 22) + 1), (0, 1)),
     (24, 0, 12, 1, 300, (1 << 21, 1 << 22), (1, 1)),
     (28, 1, 7, 28, 3000, (18500000, 1 << 25), (1, 1)),
-    (28, 1, 7, 28, 10000, (31000000, 1 << 25), (0, 0)),
+    (28, 1, 9, 28, 5000, (48000000, 50000000), (1, 1)),
+    (28, 1, 9, 28, 12000, (110000000, 120000000), (0, 0)),
 ])
 def test_sigma_takes_the_faster_path(sf, n, na, nb, rows, dets, caps, by_rows):
     s = sf.System.from_dict(single._molecule(n, na, nb))
