@@ -930,14 +930,14 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
     };
     const bool have_a = z->ga.bytes >= size_a && z->vrp.bytes >= vrp_bytes &&
                         (double)std::min(z->sig_key.bytes, z->sig_val.bytes) >= 8.0 * sig_need;
-    double need = 1.25 * (double)size_a + (double)vrp_bytes + 1.1 * 16.0 * sig_need;  // (as grown below)
+    const double need = (double)size_a + (double)vrp_bytes + 16.0 * sig_need;
     if (!fits(have_a, need)) return SFCI_OK;
     SFCI_CUDA(cudaEventRecord(z->evp[0], z->st));
     z->ms_alloc = 0.0;
-    const auto grow = [&](sfci_lanczos::Buf &buf, size_t want, const char *what, double headroom) {
-        if (buf.p && buf.bytes >= want) return SFCI_OK;
+    const auto grow = [&](sfci_lanczos::Buf &buf, size_t bytes, const char *what, double headroom) {
+        if (buf.p && buf.bytes >= bytes) return SFCI_OK;
         const auto t0 = std::chrono::steady_clock::now();
-        if (z->alloc_limit > 0 && want > (size_t)z->alloc_limit) {
+        if (z->alloc_limit > 0 && bytes > (size_t)z->alloc_limit) {
             set_error(std::string(what) + ": above the allocation limit");
             return SFCI_E_NOMEM;
         }
@@ -945,16 +945,20 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
         // (what is held with the grown buffer: a stream that the buckets made longer counts as it is)
         const auto over = [&] {
             return row_bytes(z) + bucket_bytes(z) + (double)z->sig_key.bytes + (double)z->sig_val.bytes - (double)buf.bytes +
-                   headroom * (double)want > budget;
+                   headroom * (double)bytes > budget;
         };
         sfci_status f = over() ? free_bucket_buffers(z) : SFCI_OK;
-        if (f == SFCI_OK && over() && &buf != &z->sig_key && &buf != &z->sig_val)
-            f = free_buffers(z, {&z->sig_key, &z->sig_val});
-        if (f == SFCI_OK) f = ensure(buf, want, z->st, what, headroom);
+        const bool sig = &buf == &z->sig_key || &buf == &z->sig_val;
+        if (f == SFCI_OK && over() && !sig) f = free_buffers(z, {&z->sig_key, &z->sig_val});
+        // (headroom where there is room for it; what is made after this buffer gives its own back)
+        if (f == SFCI_OK && over() && &buf == &z->gb) f = free_buffers(z, {&z->gc});
+        if (f == SFCI_OK && over() && (&buf == &z->ga || &buf == &z->vrp)) f = free_buffers(z, {&z->gb, &z->gc});
+        if (over()) headroom = 1.0;
+        if (f == SFCI_OK) f = ensure(buf, bytes, z->st, what, headroom);
         if (f == SFCI_E_NOMEM && bucket_bytes(z) > 0.0) {
             cudaGetLastError();
             f = free_bucket_buffers(z);
-            if (f == SFCI_OK) f = ensure(buf, want, z->st, what, headroom);
+            if (f == SFCI_OK) f = ensure(buf, bytes, z->st, what, headroom);
         }
         z->ms_alloc += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         return f;
@@ -982,7 +986,7 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
     const unsigned long long nd = z->host->nd, runs = z->host->runs;
     const size_t size_b = gather_place_tables(nullptr, b, d, gs, nd, n_in);
     const bool have_b = have_a && z->gb.bytes >= size_b;
-    if (!gather_numbers(d, n_in, nd) || !fits(have_b, need += 1.1 * (double)size_b)) return SFCI_OK;
+    if (!gather_numbers(d, n_in, nd) || !fits(have_b, need + (double)size_b)) return SFCI_OK;
     if ((r = grow(z->gb, size_b, "row gather tables", 1.1))) return r;
     gather_place_tables(static_cast<char *>(z->gb.p), b, d, gs, nd, n_in);
     const RowPlanArgs ra = row_plan_args(d, gs, n_in);
@@ -995,7 +999,7 @@ sfci_status sum_rows(sfci_lanczos *z, int i, double *tau_io, unsigned long long 
         return SFCI_OK;
     }
     const size_t size_c = gather_place_lists(nullptr, b, gs, gn);
-    if (!fits(have_b && z->gc.bytes >= size_c, need += 1.1 * (double)size_c)) return SFCI_OK;
+    if (!fits(have_b && z->gc.bytes >= size_c, need + (double)size_b + (double)size_c)) return SFCI_OK;
     if ((r = grow(z->gc, size_c, "row gather lists", 1.1))) return r;
     gather_place_lists(static_cast<char *>(z->gc.p), b, gs, gn);
     SFCI_CUDA(gather_lists(d, gs, gn.act, gn.parts, z->sys->pair_int, rp, b, ra, z->st));
