@@ -890,6 +890,20 @@ bool row_units_may_exceed(const SysDev &d, long long n) {  // (as many where the
     return (double)n * (1.0 + std::ceil(hops / kT) + (d.sb ? std::ceil((double)d.sa / kT) : 0.0)) > row_units_limit(d, n);
 }
 
+// A call whose rows are few or small waits for its slowest unit: a thread steps through the row's
+// strings (up to 1024 of them) and through the tile for each of its places on the diagonal, 0.25 us a
+// step, after 45 us more of launches than the lookups need; these wait for one warp's lookups in
+// turn, 0.1 us each.  How uneven the rows are is not known: three times their mean.  One row of 1190
+// determinants of 17 orbitals, 4 electrons 429 us by rows, 88 by lookups; 4427 of 23 orbitals, 4
+// electrons 566 and 174.  (6463 systems of 8 to 34 orbitals: rows slower by a tenth or more in 467
+// without this line, in 154 with it.)
+bool rows_wait(const SysDev &d, long long n) {
+    const double exc = (double)d.sa + d.sb + (double)d.po_a * d.pv_a + (double)d.po_b * d.pv_b + (double)d.sa * d.sb;
+    const double m = std::min({(double)n, (double)d.cb, std::ceil(3.0 * (double)n / (double)d.ca)});
+    const double steps = std::ceil((d.n * d.n + 1.0) / kT) * std::min(m, (double)kT) + std::min(m, (double)kTileF);
+    return 90.0 + 0.25 * steps > 45.0 + 0.1 * exc + (double)n * (0.025 + 1.05e-5 * exc);
+}
+
 // Pairs by rows: strings are numbered in 26 bits, their hops in 32.  A determinant is compared
 // with all of its row, 0.6 to 1.2 ps a pair, where the lookups take 7 to 16 ps for each of its
 // excitations (28 orbitals, 7 + 7 electrons, level-like vectors: 3e5 determinants 20.5 ms and
@@ -899,7 +913,8 @@ bool rows_taken(const SysDev &d, long long n) {
     return n > 0 && n < (1ll << 31) && d.ca <= (1ull << 26) && d.cb <= (1ull << 26) &&
            std::min((double)n, (double)d.cb) * std::max(d.sb, 1) < 4294967296.0 &&
            (double)d.sa + (double)d.po_a * d.pv_a < 2147483648.0 &&
-           std::min((double)n, (double)d.cb) <= 4096.0 + 128.0 * exc && !(d.cb == 1 && row_units_may_exceed(d, n));
+           std::min((double)n, (double)d.cb) <= 4096.0 + 128.0 * exc && !(d.cb == 1 && row_units_may_exceed(d, n)) &&
+           !rows_wait(d, n);
 }
 
 int sms() {
